@@ -358,51 +358,59 @@ k_mg_scale(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, const 
 // Coarsest solve, one of its two products (n_c x n_c real V times the
 // complex block X, n_c x W):  Out = op(V) X, op(V) = V^T if trans, and if
 // cinv != nullptr each output row k of pole j is scaled by cinv[k*N + j].
-// 32 x 32-column tiles of Out per CTA (32 x 8 threads, 4 rows per thread).
-template <typename T>
-__global__ void __launch_bounds__(256)
+// (8 RT) x 16-column tiles of Out per CTA (16 x 8 threads, RT rows each).
+// Bound by the FP64 pipe of the SMs that have a tile (about 1.6 FMA per clock
+// and SM): with 32 x 32 tiles a 223 x 60 product ran on 14 of the 152 SMs and
+// took 141 us; RT = 1 spreads it over 112 CTAs.
+template <typename T, int RT>
+__global__ void __launch_bounds__(128)
 k_mg_coarse_gemm(int nc, int W, int Lp, int N, int trans, const T *__restrict__ V, const cplx<T> *__restrict__ X,
                  const cplx<T> *__restrict__ cinv, cplx<T> *__restrict__ Out, const int32_t *__restrict__ flag) {
     using C = cplx<T>;
-    __shared__ T sV[32][33];
-    __shared__ C sX[32][32];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int colb = blockIdx.x * 32, rowb = blockIdx.y * 32;
-    const int ccol = colb + tx;
-    C acc[4];
+    constexpr int TR = 8 * RT, TC = 16, TK = 32;
+    __shared__ T sV[TR][TK + 1];
+    __shared__ C sX[TK][TC];
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TC + tx;
+    const int rowb = blockIdx.y * TR;
+    const int ccol = blockIdx.x * TC + tx;
+    const bool live = ccol < W && flag[ccol] == 1;
+    if (!__syncthreads_or(live)) return;
+    C acc[RT];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[q] = mk((T)0, (T)0);
-    for (int k0 = 0; k0 < nc; k0 += 32) {
-        // sV[r][k] = op(V)[rowb + r][k0 + k]
-        for (int idx = ty * 32 + tx; idx < 32 * 32; idx += 256) {
-            const int r = idx / 32, k = idx % 32;
+    for (int q = 0; q < RT; ++q) acc[q] = mk((T)0, (T)0);
+    for (int k0 = 0; k0 < nc; k0 += TK) {
+        // sV[r][k] = op(V)[rowb + r][k0 + k]; lanes walk V's contiguous index
+#pragma unroll
+        for (int idx = tid; idx < TR * TK; idx += 128) {
+            const int r = trans ? idx % TR : idx / TK, k = trans ? idx / TR : idx % TK;
             const int gr = rowb + r, gk = k0 + k;
             T v = (T)0;
             if (gr < nc && gk < nc) v = trans ? V[(int64_t)gk * nc + gr] : V[(int64_t)gr * nc + gk];
             sV[r][k] = v;
         }
-        for (int k = ty; k < 32; k += 8) {
+#pragma unroll
+        for (int k = ty; k < TK; k += 8) {
             const int gk = k0 + k;
             sX[k][tx] = (gk < nc && ccol < W) ? X[(int64_t)gk * W + ccol] : mk((T)0, (T)0);
         }
         __syncthreads();
 #pragma unroll 8
-        for (int k = 0; k < 32; ++k) {
+        for (int k = 0; k < TK; ++k) {
             const C x = sX[k][tx];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const T v = sV[ty * 4 + q][k];
+            for (int q = 0; q < RT; ++q) {
+                const T v = sV[ty * RT + q][k];
                 acc[q].x = fma(v, x.x, acc[q].x);
                 acc[q].y = fma(v, x.y, acc[q].y);
             }
         }
         __syncthreads();
     }
-    if (ccol >= W || flag[ccol] != 1) return;
+    if (!live) return;
     const int j = ccol / Lp;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int r = rowb + ty * 4 + q;
+    for (int q = 0; q < RT; ++q) {
+        const int r = rowb + ty * RT + q;
         if (r >= nc) continue;
         C o = acc[q];
         if (cinv) o = cmul(o, cinv[(int64_t)r * N + j]);
@@ -559,15 +567,23 @@ void coarse_solve(Ctx &ctx, const KrylovDims &d, const MgSolve<T> &mg, const cpl
         }
     }
     const int nc = mg.nc, W = d.W();
-    dim3 grid((W + 31) / 32, (nc + 31) / 32), block(32, 8);
     const double bytes = (double)nc * nc * sizeof(T) + 2.0 * vec_bytes<T>(d, nc);
     const double flops = 4.0 * (double)nc * nc * W;
-    ctx.before(KC_MG_COARSE, bytes, flops);
-    k_mg_coarse_gemm<T><<<grid, block, 0, ctx.stream>>>(nc, W, d.Lp, d.N, 1, mg.V, Rv, mg.cinv, Y, flag);
-    ctx.after();
-    ctx.before(KC_MG_COARSE, bytes, flops);
-    k_mg_coarse_gemm<T><<<grid, block, 0, ctx.stream>>>(nc, W, d.Lp, d.N, 0, mg.V, Y, nullptr, Z, flag);
-    ctx.after();
+    // four rows per thread (fewer shared loads per FMA) once such tiles give
+    // every SM two CTAs, else one row per thread: four times the CTAs
+    const int gx = (W + 15) / 16;
+    const bool wide = (int64_t)gx * ((nc + 31) / 32) >= 2 * ctx.sm_count;
+    const dim3 grid(gx, wide ? (nc + 31) / 32 : (nc + 7) / 8), block(16, 8);
+    auto product = [&](int trans, const cplx<T> *X, const cplx<T> *cinv, cplx<T> *Out) {
+        ctx.before(KC_MG_COARSE, bytes, flops);
+        if (wide)
+            k_mg_coarse_gemm<T, 4><<<grid, block, 0, ctx.stream>>>(nc, W, d.Lp, d.N, trans, mg.V, X, cinv, Out, flag);
+        else
+            k_mg_coarse_gemm<T, 1><<<grid, block, 0, ctx.stream>>>(nc, W, d.Lp, d.N, trans, mg.V, X, cinv, Out, flag);
+        ctx.after();
+    };
+    product(1, Rv, mg.cinv, Y);
+    product(0, Y, nullptr, Z);
 }
 
 template <typename T>
