@@ -323,34 +323,14 @@ k_bcg_p(int n, int W, const cplx<T> *__restrict__ R, const cplx<T> *__restrict__
     }
 }
 
-// per-column scalar reductions (one warp per column, FP64 sums of the partials)
-template <typename T>
-__device__ __forceinline__ void warp_sum3(const T *part, int gy, int W, int col, double &s0, double &s1,
-                                          double &s2) {
-    const int lane = threadIdx.x & 31;
-    s0 = s1 = s2 = 0.0;
-    for (int g = lane; g < gy; g += 32) {
-        const T *o = part + ((int64_t)g * W + col) * 4;
-        s0 += (double)o[0];
-        s1 += (double)o[1];
-        s2 += (double)o[2];
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, off);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, off);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, off);
-    }
-}
-
+// per-column scalar reductions (one block per column, FP64 sums of the partials)
 // alpha = rho / (r^, v); ua = 2 coef alpha
 template <typename T>
 __global__ void k_bcg_alpha(int W, int gy, const T *__restrict__ part, KrylovScalars<T> s) {
-    const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (col >= W) return;
+    const int col = blockIdx.x;
     double s0, s1, s2;
-    warp_sum3(part, gy, W, col, s0, s1, s2);
-    if ((threadIdx.x & 31) == 0 && s.flag[col] == 1) {
+    col_sum3(part, gy, W, col, s0, s1, s2);
+    if (threadIdx.x == 0 && s.flag[col] == 1) {
         const double den = s0 * s0 + s1 * s1;
         if (!(den > 0.0) || !isfinite(den)) {
             s.flag[col] = 2;
@@ -369,11 +349,10 @@ __global__ void k_bcg_alpha(int W, int gy, const T *__restrict__ part, KrylovSca
 template <typename T>
 __global__ void k_bcg_omega(int W, int gy, const T *__restrict__ part, KrylovScalars<T> s, cplx<T> *__restrict__ omega,
                             cplx<T> *__restrict__ ua2) {
-    const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (col >= W) return;
+    const int col = blockIdx.x;
     double s0, s1, s2;
-    warp_sum3(part, gy, W, col, s0, s1, s2);
-    if ((threadIdx.x & 31) == 0 && s.flag[col] == 1) {
+    col_sum3(part, gy, W, col, s0, s1, s2);
+    if (threadIdx.x == 0 && s.flag[col] == 1) {
         double orr = 0.0, oi = 0.0;
         if (s2 > 0.0 && isfinite(s2)) {
             orr = s0 / s2;
@@ -431,7 +410,7 @@ void bicgstab_alpha(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb, BcgBuff
     k_bcg_dot<T, VC><<<grid, block, 0, ctx.stream>>>(d.n, W, bb.Rh, bb.V, nullptr, kb.s.flag, kb.s.part);
     ctx.after();
     ctx.before(KC_KRYLOV_REDUCE, (double)kb.gy * W * 4 * sizeof(T), 0);
-    k_bcg_alpha<T><<<(W * 32 + 255) / 256, 256, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s);
+    k_bcg_alpha<T><<<W, COL_SUM_THREADS, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s);
     ctx.after();
 }
 
@@ -457,7 +436,7 @@ void bicgstab_omega(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb, BcgBuff
     k_bcg_dot<T, VC><<<grid, block, 0, ctx.stream>>>(d.n, W, bb.Tt, kb.R, bb.Tt, kb.s.flag, kb.s.part);
     ctx.after();
     ctx.before(KC_KRYLOV_REDUCE, (double)kb.gy * W * 4 * sizeof(T), 0);
-    k_bcg_omega<T><<<(W * 32 + 255) / 256, 256, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s, bb.omega, bb.ua2);
+    k_bcg_omega<T><<<W, COL_SUM_THREADS, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s, bb.omega, bb.ua2);
     ctx.after();
 }
 

@@ -152,6 +152,70 @@ __device__ __forceinline__ void l2_prefetch_warp(const void *p, int64_t bytes, i
 }
 
 // ---------------------------------------------------------------------------
+// Per-column reduction of the Krylov kernels' partial sums (gy rows of W x 4
+// values): one block of COL_SUM_THREADS threads per column, FP64 sums in a
+// fixed order, valid in thread 0.  Latency-bound (a few hundred loads per
+// column): each thread issues the loads of four rows before it adds.  With
+// one warp per column and a serial loop over up to 38 rows per lane, a
+// reduction took 10-14 us (gy = 250..608); so it takes about 3 us.
+// ---------------------------------------------------------------------------
+constexpr int COL_SUM_THREADS = 128;
+__device__ __forceinline__ void ld_part3(const float *p, float v[3]) {
+    const float4 t = *reinterpret_cast<const float4 *>(p);
+    v[0] = t.x;
+    v[1] = t.y;
+    v[2] = t.z;
+}
+__device__ __forceinline__ void ld_part3(const double *p, double v[3]) {
+    const double2 t = *reinterpret_cast<const double2 *>(p);
+    v[0] = t.x;
+    v[1] = t.y;
+    v[2] = p[2];
+}
+template <typename T>
+__device__ __forceinline__ void col_sum3(const T *part, int gy, int W, int col, double &s0, double &s1, double &s2) {
+    constexpr int NT = COL_SUM_THREADS, U = 4;
+    const int tid = threadIdx.x;
+    s0 = s1 = s2 = 0.0;
+    for (int g0 = tid; g0 < gy; g0 += U * NT) {
+        T v[U][3];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int g = g0 + u * NT;
+            v[u][0] = v[u][1] = v[u][2] = (T)0;
+            if (g < gy) ld_part3(part + ((int64_t)g * W + col) * 4, v[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            s0 += (double)v[u][0];
+            s1 += (double)v[u][1];
+            s2 += (double)v[u][2];
+        }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, off);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+    }
+    __shared__ double red[NT / 32][3];
+    if ((tid & 31) == 0) {
+        red[tid >> 5][0] = s0;
+        red[tid >> 5][1] = s1;
+        red[tid >> 5][2] = s2;
+    }
+    __syncthreads();
+    if (tid == 0) {
+#pragma unroll
+        for (int w = 1; w < NT / 32; ++w) {
+            s0 += red[w][0];
+            s1 += red[w][1];
+            s2 += red[w][2];
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // kernel classes (profiling buckets of slrf_report)
 // ---------------------------------------------------------------------------
 enum KernelClass {

@@ -1046,34 +1046,14 @@ k_direction(int n, int W, int Lp, int N, const cplx<T> *__restrict__ R, const cp
 }
 
 // ---------------------------------------------------------------------------
-// per-column reductions (one warp per column, lanes over row groups, FP64)
+// per-column reductions (one block per column, FP64)
 // ---------------------------------------------------------------------------
 template <typename T>
-__device__ __forceinline__ void warp_sum3(const T *part, int gy, int W, int col, double &s0, double &s1,
-                                          double &s2) {
-    const int lane = threadIdx.x & 31;
-    s0 = s1 = s2 = 0.0;
-    for (int g = lane; g < gy; g += 32) {
-        const T *o = part + ((int64_t)g * W + col) * 4;
-        s0 += (double)o[0];
-        s1 += (double)o[1];
-        s2 += (double)o[2];
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, off);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, off);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, off);
-    }
-}
-
-template <typename T>
 __global__ void k_reduce_init(int W, int gy, const T *__restrict__ part, KrylovScalars<T> s) {
-    const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (col >= W) return;
+    const int col = blockIdx.x;
     double s0, s1, s2;
-    warp_sum3(part, gy, W, col, s0, s1, s2);
-    if ((threadIdx.x & 31) == 0) {
+    col_sum3(part, gy, W, col, s0, s1, s2);
+    if (threadIdx.x == 0) {
         s.rho[col] = mk((T)s0, (T)s1);
         s.bnorm2[col] = s2;
         s.rnorm2[col] = s2;
@@ -1084,11 +1064,10 @@ __global__ void k_reduce_init(int W, int gy, const T *__restrict__ part, KrylovS
 
 template <typename T>
 __global__ void k_reduce_alpha(int W, int gy, const T *__restrict__ part, KrylovScalars<T> s) {
-    const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (col >= W) return;
+    const int col = blockIdx.x;
     double s0, s1, s2;
-    warp_sum3(part, gy, W, col, s0, s1, s2);
-    if ((threadIdx.x & 31) == 0 && s.flag[col] == 1) {
+    col_sum3(part, gy, W, col, s0, s1, s2);
+    if (threadIdx.x == 0 && s.flag[col] == 1) {
         const double den = s0 * s0 + s1 * s1;
         const double rr = (double)s.rho[col].x, ri = (double)s.rho[col].y;
         if (!(den > 0.0) || !isfinite(den)) {
@@ -1107,11 +1086,10 @@ __global__ void k_reduce_alpha(int W, int gy, const T *__restrict__ part, Krylov
 template <typename T>
 __global__ void k_reduce_beta(int W, int gy, const T *__restrict__ part, KrylovScalars<T> s, double tol2,
                               int maxit) {
-    const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (col >= W) return;
+    const int col = blockIdx.x;
     double s0, s1, s2;
-    warp_sum3(part, gy, W, col, s0, s1, s2);
-    if ((threadIdx.x & 31) == 0 && s.flag[col] == 1) {
+    col_sum3(part, gy, W, col, s0, s1, s2);
+    if (threadIdx.x == 0 && s.flag[col] == 1) {
         const int it = s.iters[col] + 1;
         s.iters[col] = it;
         s.rnorm2[col] = s2;
@@ -1150,12 +1128,11 @@ __global__ void k_count_active(int W, const int32_t *__restrict__ flag, int32_t 
 
 template <typename T>
 __global__ void k_reduce_mu(int W, int gy, const T *__restrict__ part, cplx<T> *__restrict__ mu, int Lp, int m) {
-    const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (col >= W) return;
+    const int col = blockIdx.x;
     double s0, s1, s2;
-    warp_sum3(part, gy, W, col, s0, s1, s2);
+    col_sum3(part, gy, W, col, s0, s1, s2);
     const int j = col / Lp, c = col - j * Lp;
-    if ((threadIdx.x & 31) == 0 && c < m) mu[j * m + c] = mk((T)s0, (T)s1);
+    if (threadIdx.x == 0 && c < m) mu[j * m + c] = mk((T)s0, (T)s1);
 }
 
 // ---------------------------------------------------------------------------
@@ -1199,7 +1176,7 @@ template <typename T>
 void krylov_reduce_init(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb) {
     const int W = d.W();
     ctx.before(KC_KRYLOV_REDUCE, (double)kb.gy * W * 4 * sizeof(T), 0);
-    k_reduce_init<T><<<(W * 32 + 255) / 256, 256, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s);
+    k_reduce_init<T><<<W, COL_SUM_THREADS, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s);
     ctx.after();
 }
 
@@ -1268,7 +1245,7 @@ template <typename T>
 void krylov_reduce_alpha(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb) {
     const int W = d.W();
     ctx.before(KC_KRYLOV_REDUCE, (double)kb.gy * W * 4 * sizeof(T), 0);
-    k_reduce_alpha<T><<<(W * 32 + 255) / 256, 256, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s);
+    k_reduce_alpha<T><<<W, COL_SUM_THREADS, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s);
     ctx.after();
 }
 
@@ -1312,7 +1289,7 @@ template <typename T>
 void krylov_reduce_beta(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb, double tol2, int maxit) {
     const int W = d.W();
     ctx.before(KC_KRYLOV_REDUCE, (double)kb.gy * W * 4 * sizeof(T), 0);
-    k_reduce_beta<T><<<(W * 32 + 255) / 256, 256, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s, tol2, maxit);
+    k_reduce_beta<T><<<W, COL_SUM_THREADS, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s, tol2, maxit);
     ctx.after();
 }
 
@@ -1343,7 +1320,7 @@ template <typename T>
 void krylov_reduce_mu(Ctx &ctx, const KrylovDims &d, const T *part, int gy, cplx<T> *mu) {
     const int W = d.W();
     ctx.before(KC_KRYLOV_REDUCE, (double)gy * W * 4 * sizeof(T), 0);
-    k_reduce_mu<T><<<(W * 32 + 255) / 256, 256, 0, ctx.stream>>>(W, gy, part, mu, d.Lp, d.m);
+    k_reduce_mu<T><<<W, COL_SUM_THREADS, 0, ctx.stream>>>(W, gy, part, mu, d.Lp, d.m);
     ctx.after();
 }
 
