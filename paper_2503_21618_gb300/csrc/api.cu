@@ -1572,8 +1572,7 @@ slrf_status rr_step(slrf_handle *h, int m, const double *U, int64_t ldu, double 
     spmm_real(ctx, h->A, m, U, ldu, nullptr, 0, W1, m);
     CKS(gram(h, n, m, U, ldu, W1, m, G, true));
     small_colscale(ctx, m, G, s);
-    small_chol_upper(ctx, m, G, R1, pin_status, shift);
-    small_triinv_upper(ctx, m, R1, T1);
+    small_chol_inv(ctx, m, G, R1, T1, st, pin_status, shift);
     // Q1 = (U S) R1^{-1}: the column scaling S makes the split operand well scaled
     CKS(tall_product(h, n, m, m, U, ldu, s, T1, m, Q1, m));
     CK(cudaEventRecord(h->ev_poll, ctx.stream));
@@ -1596,8 +1595,7 @@ slrf_status rr_step(slrf_handle *h, int m, const double *U, int64_t ldu, double 
         double *Q2 = as<double>(h->rQ2);
         spmm_real(ctx, h->A, m, Q1, m, nullptr, 0, W1, m);
         CKS(gram(h, n, m, Q1, m, W1, m, G, true));
-        small_chol_upper(ctx, m, G, G, st + 2, 0.0);
-        small_triinv_upper(ctx, m, G, T1);
+        small_chol_inv(ctx, m, G, G, T1, st + 2, nullptr, 0.0);
         CKS(tall_product(h, n, m, m, Q1, m, nullptr, T1, m, Q2, m));
         CK(cudaMemcpyAsync(Q1, Q2, (size_t)n * m * sizeof(double), cudaMemcpyDeviceToDevice, ctx.stream));
         h->shifted_cholqr += 1;
@@ -1607,13 +1605,12 @@ slrf_status rr_step(slrf_handle *h, int m, const double *U, int64_t ldu, double 
     // pass 2: G2 = Q1^T B Q1, R2 = chol, T2 = R2^{-1}
     spmm_real(ctx, h->A, m, Q1, m, nullptr, 0, W1, m);
     CKS(gram(h, n, m, Q1, m, W1, m, G, true));
-    small_chol_upper(ctx, m, G, G, st + 1, 0.0);
-    small_triinv_upper(ctx, m, G, T2);
+    small_chol_inv(ctx, m, G, G, T2, st + 1, nullptr, 0.0);
     // projected A: A_hat = T2^T (Q1^T A Q1) T2
     spmm_real(ctx, h->A, m, Q1, m, W1, m, nullptr, 0);
     CKS(gram(h, n, m, Q1, m, W1, m, Ah1, true));
     dgemm(ctx, 0, 0, m, m, m, Ah1, m, T2, m, 0.0, R1, m, 1, nullptr, KC_SMALL_DENSE);
-    dgemm(ctx, 1, 0, m, m, m, T2, m, R1, m, 0.0, Ah, m, 1, nullptr, KC_SMALL_DENSE);
+    dgemm(ctx, 1, 0, m, m, m, T2, m, R1, m, 0.0, Ah, m, 1, nullptr, KC_SMALL_DENSE, true);
     ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
     k_symmetrize<<<(unsigned)((m2 + 255) / 256), 256, 0, ctx.stream>>>(m, Ah);
     ctx.after();

@@ -147,30 +147,56 @@ __global__ void k_split_reduce(int M, int N, int split, const double *__restrict
     *o = (beta != 0.0 ? beta * *o : 0.0) + s;
 }
 
-// Small products (the m x m x m GEMMs of the projection): one output per
-// thread, 16 x 16 tiles staged in shared memory, so an m = 150 product runs on
-// 100 CTAs instead of the 9 that the 64 x 64 tiling of k_dgemm gives it.
+// Small products (the m x m x m GEMMs of the projection) on 8 x 8 output
+// tiles: 64 outputs times a four-way split of each K chunk per CTA, the next
+// chunk's loads in flight during the FMAs, the four sums added in a fixed
+// order.  Bound by the FP64 pipe (~1.6 FMAs per clock and SM), so the tiles
+// are small enough that the most loaded SM has little more than the average:
+// m = 150 on 100 CTAs of 16 x 16 took 17 us, on 361 of 8 x 8 about 10 us.
+// symmetric: the result is known to be symmetric (X^T X, X^T S X): only the
+// tiles on and above the diagonal are computed, and mirrored.
 template <int OPA, int OPB>
 __global__ void __launch_bounds__(256)
 k_dgemm_small(int M, int N, int K, const double *__restrict__ A, int64_t lda, const double *__restrict__ B,
-              int64_t ldb, double beta, double *__restrict__ C, int64_t ldc) {
-    __shared__ double As[16][17], Bs[16][17];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int i = blockIdx.y * 16 + ty, j = blockIdx.x * 16 + tx;
-    double s = 0.0;
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        const int ka = k0 + tx, kb = k0 + ty;
-        As[ty][tx] = (i < M && ka < K) ? (OPA ? A[(int64_t)ka * lda + i] : A[(int64_t)i * lda + ka]) : 0.0;
-        Bs[ty][tx] = (kb < K && j < N) ? (OPB ? B[(int64_t)j * ldb + kb] : B[(int64_t)kb * ldb + j]) : 0.0;
+              int64_t ldb, double beta, double *__restrict__ C, int64_t ldc, int symmetric) {
+    constexpr int T = 8, KC = 32;
+    __shared__ double As[KC][T + 1], Bs[KC][T + 1], red[3][T * T];
+    if (symmetric && blockIdx.x < blockIdx.y) return;
+    const int tid = threadIdx.x;
+    const int i0 = blockIdx.y * T, j0 = blockIdx.x * T;
+    // this thread's element of each staged chunk (lanes along the contiguous index)
+    const int ai = OPA ? tid & 7 : tid >> 5, ak = OPA ? tid >> 3 : tid & 31;
+    const int bj = OPB ? tid >> 5 : tid & 7, bk = OPB ? tid & 31 : tid >> 3;
+    auto load_a = [&](int k0) {
+        const int i = i0 + ai, k = k0 + ak;
+        return i < M && k < K ? (OPA ? A[(int64_t)k * lda + i] : A[(int64_t)i * lda + k]) : 0.0;
+    };
+    auto load_b = [&](int k0) {
+        const int j = j0 + bj, k = k0 + bk;
+        return j < N && k < K ? (OPB ? B[(int64_t)j * ldb + k] : B[(int64_t)k * ldb + j]) : 0.0;
+    };
+    const int o = tid & 63, kq = tid >> 6, i = o >> 3, j = o & 7;
+    double s = 0.0, av = load_a(0), bv = load_b(0);
+    for (int k0 = 0; k0 < K; k0 += KC) {
+        As[ak][ai] = av;
+        Bs[bk][bj] = bv;
         __syncthreads();
+        if (k0 + KC < K) {
+            av = load_a(k0 + KC);
+            bv = load_b(k0 + KC);
+        }
 #pragma unroll
-        for (int k = 0; k < 16; ++k) s = fma(As[ty][k], Bs[k][tx], s);
+        for (int kk = 0; kk < KC / 4; ++kk) s = fma(As[kq * (KC / 4) + kk][i], Bs[kq * (KC / 4) + kk][j], s);
         __syncthreads();
     }
-    if (i < M && j < N) {
-        double *o = C + (int64_t)i * ldc + j;
-        *o = (beta != 0.0 ? beta * *o : 0.0) + s;
-    }
+    if (kq) red[kq - 1][o] = s;
+    __syncthreads();
+    const int gi = i0 + i, gj = j0 + j;
+    if (kq || gi >= M || gj >= N || (symmetric && gi > gj)) return;
+    s = ((s + red[0][o]) + red[1][o]) + red[2][o];
+    double *c = C + (int64_t)gi * ldc + gj;
+    *c = (beta != 0.0 ? beta * *c : 0.0) + s;
+    if (symmetric && gi != gj) C[(int64_t)gj * ldc + gi] = s;
 }
 
 int gram_split(const Ctx &ctx, int m, int64_t n) {
@@ -183,13 +209,14 @@ int gram_split(const Ctx &ctx, int m, int64_t n) {
 }
 
 void dgemm(Ctx &ctx, int opA, int opB, int M, int N, int K, const double *A, int64_t lda, const double *B,
-           int64_t ldb, double beta, double *C, int64_t ldc, int split, double *work, int kc) {
+           int64_t ldb, double beta, double *C, int64_t ldc, int split, double *work, int kc, bool symmetric) {
     if (M <= 0 || N <= 0) return;
     if (split < 1 || !work) split = 1;
     if (split == 1 && M <= 1024 && N <= 1024 && K <= 4096) {
-        const dim3 grid((N + 15) / 16, (M + 15) / 16), block(16, 16);
+        const dim3 grid((N + 7) / 8, (M + 7) / 8);
+        const int sym = symmetric && beta == 0.0 && M == N ? 1 : 0;
         ctx.before(kc, 8.0 * ((double)M * K + (double)K * N + (double)M * N), 2.0 * M * N * (double)K);
-#define LS(a, b) k_dgemm_small<a, b><<<grid, block, 0, ctx.stream>>>(M, N, K, A, lda, B, ldb, beta, C, ldc)
+#define LS(a, b) k_dgemm_small<a, b><<<grid, 256, 0, ctx.stream>>>(M, N, K, A, lda, B, ldb, beta, C, ldc, sym)
         if (opA == 0 && opB == 0) LS(0, 0);
         else if (opA == 1 && opB == 0) LS(1, 0);
         else if (opA == 0 && opB == 1) LS(0, 1);

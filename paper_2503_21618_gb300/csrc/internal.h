@@ -305,10 +305,11 @@ void spmm_real(Ctx &ctx, const DevPencil &A, int m, const double *X, int64_t ldx
 // C = op(A) op(B) (+ beta C), row-major; opA/opB: 0 = N, 1 = T.
 // Dimensions: op(A) is M x K, op(B) is K x N.  split > 1 splits K into
 // `split` slices whose partial products go to work[split][M][N] and are then
-// summed in a fixed order.
+// summed in a fixed order.  symmetric: the m x m result is known to be
+// symmetric (small products compute its upper tiles and mirror them).
 void dgemm(Ctx &ctx, int opA, int opB, int M, int N, int K, const double *A, int64_t lda,
            const double *B, int64_t ldb, double beta, double *C, int64_t ldc, int split = 1,
-           double *work = nullptr, int kc = KC_TALL_GEMM);
+           double *work = nullptr, int kc = KC_TALL_GEMM, bool symmetric = false);
 // Choose a split for a Gram of n rows.
 int gram_split(const Ctx &ctx, int m, int64_t n);
 // Residual of the Ritz pairs: Rout = BX diag(theta) - AX (if Rout != nullptr),
@@ -347,10 +348,12 @@ void ozaki_tall(Ctx &ctx, int64_t n, int k, int m, const double *A, int64_t lda,
 // All m x m matrices row-major, device.  status: device int, set nonzero on
 // failure (Cholesky pivot <= 0 or non-finite).
 void small_colscale(Ctx &ctx, int m, double *G, double *s);        // s = 1/sqrt(diag G); G = S G S
-// G + s I = R^T R (R upper) into R (may alias G); s = 0, or shift_on_fail if
-// the unshifted factorisation breaks down (*status = -1 then).
-void small_chol_upper(Ctx &ctx, int m, const double *G, double *R, int32_t *status, double shift_on_fail);
-void small_triinv_upper(Ctx &ctx, int m, const double *R, double *Rinv);
+// G + s I = R^T R (R upper) into R (may alias G) and Rinv = R^{-1}; s = 0, or
+// shift_on_fail if the unshifted factorisation breaks down (*status = -1
+// then; needs R != G).  status: device word; out_status: a copy of it, may be
+// a mapped host word, or nullptr.
+void small_chol_inv(Ctx &ctx, int m, const double *G, double *R, double *Rinv, int32_t *status, int32_t *out_status,
+                    double shift_on_fail);
 void small_scale_rows(Ctx &ctx, int m, const double *s, double *T);  // T = diag(s) T
 // Symmetric eigensolver: lam ascending, Q eigenvectors (columns).  mode 1:
 // FP32 Jacobi followed by FP64 refinement; 0: FP64 Jacobi.

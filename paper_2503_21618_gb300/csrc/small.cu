@@ -30,30 +30,24 @@ namespace slrf {
 // ---------------------------------------------------------------------------
 // column scaling of a Gram matrix: s_i = 1/sqrt(g_ii), G <- S G S
 // ---------------------------------------------------------------------------
-__global__ void k_colscale(int m, double *__restrict__ G, double *__restrict__ s) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= (int64_t)m * m) return;
-    const int i = (int)(e / m), j = (int)(e % m);
-    const double gi = G[(int64_t)i * m + i], gj = G[(int64_t)j * m + j];
-    const double si = gi > 0.0 ? 1.0 / sqrt(gi) : 0.0;
-    const double sj = gj > 0.0 ? 1.0 / sqrt(gj) : 0.0;
-    // every thread reads the diagonal before any writes it: write to a copy
-    // is avoided by updating the diagonal last (see k_colscale_diag).
-    if (i != j) G[e] *= si * sj;
-    if (i == j) s[i] = si;
-}
-__global__ void k_colscale_diag(int m, double *__restrict__ G, const double *__restrict__ s) {
+__global__ void k_colscale_diag(int m, const double *__restrict__ G, double *__restrict__ s) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m) G[(int64_t)i * m + i] *= s[i] * s[i];
+    if (i >= m) return;
+    const double g = G[(int64_t)i * m + i];
+    s[i] = g > 0.0 ? 1.0 / sqrt(g) : 0.0;
+}
+__global__ void k_colscale(int m, double *__restrict__ G, const double *__restrict__ s) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e < (int64_t)m * m) G[e] *= s[e / m] * s[e % m];
 }
 
 void small_colscale(Ctx &ctx, int m, double *G, double *s) {
     const int64_t tot = (int64_t)m * m;
+    ctx.before(KC_SMALL_DENSE, 16.0 * m, m);
+    k_colscale_diag<<<(m + 63) / 64, 64, 0, ctx.stream>>>(m, G, s);
+    ctx.after();
     ctx.before(KC_SMALL_DENSE, 16.0 * tot, tot);
     k_colscale<<<(unsigned)((tot + 255) / 256), 256, 0, ctx.stream>>>(m, G, s);
-    ctx.after();
-    ctx.before(KC_SMALL_DENSE, 16.0 * m, m);
-    k_colscale_diag<<<(m + 255) / 256, 256, 0, ctx.stream>>>(m, G, s);
     ctx.after();
 }
 
@@ -70,59 +64,43 @@ void small_scale_rows(Ctx &ctx, int m, const double *s, double *T) {
 }
 
 // ---------------------------------------------------------------------------
-// Cholesky G + shift I = R^T R (R upper), one block, right-looking.  G is read
-// and left untouched; R is written to Rg.  If the factorisation of G breaks
-// down (a pivot <= shift_on_fail, or non-finite) and shift_on_fail > 0, it is
-// redone on G + shift_on_fail I (shifted Cholesky-QR) and *status = -1; an
-// unrecoverable breakdown (pivot <= 0 with no shift) sets *status = k + 1
-// (k = failing pivot).
+// Shifted refactorisation after a breakdown (*status > 0 on entry, else it
+// returns): G + shift I = R^T R (R upper), one block, right-looking.  G is
+// read and left untouched.  *status = -1 on success; an unrecoverable
+// breakdown (a pivot not above 0) sets *status = k + 1, k the failing pivot.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_chol_upper(int m, const double *__restrict__ G, double *__restrict__ Rg,
-                                                      int32_t *__restrict__ status, int use_smem,
-                                                      double shift_on_fail, int only_if_failed) {
+__global__ void __launch_bounds__(1024) k_chol_shifted(int m, const double *__restrict__ G, double *__restrict__ Rg,
+                                                        int32_t *__restrict__ status, int32_t *__restrict__ out_status,
+                                                        int use_smem, double shift) {
     extern __shared__ double sm[];
+    if (*(volatile int32_t *)status <= 0) return;
     double *A = use_smem ? sm : Rg;
     const int tid = threadIdx.x, bs = blockDim.x;
     __shared__ int bad;
     __shared__ double dinv;
-    double shift = 0.0;
-    int first = 0;
-    if (only_if_failed) {   // the blocked form's breakdown fallback: shifted factor only
-        if (*(volatile int32_t *)status <= 0) return;
-        first = 1;
-        shift = shift_on_fail;
-    }
-    for (int attempt = first; attempt < 2; ++attempt) {
-        for (int e = tid; e < m * m; e += bs) A[e] = G[e] + ((e / m == e % m) ? shift : 0.0);
-        if (tid == 0) bad = 0;
-        __syncthreads();
-        // unshifted: a pivot at or below the shift (a numerically dependent
-        // column of the column-scaled Gram) counts as a breakdown too
-        const double pmin = attempt == 0 ? shift_on_fail : 0.0;
-        for (int k = 0; k < m; ++k) {
-            if (tid == 0) {
-                const double d = A[k * m + k];
-                if (!(d > pmin) || !isfinite(d)) {
-                    bad = k + 1;
-                } else {
-                    const double r = sqrt(d);
-                    A[k * m + k] = r;
-                    dinv = 1.0 / r;
-                }
+    for (int e = tid; e < m * m; e += bs) A[e] = G[e] + ((e / m == e % m) ? shift : 0.0);
+    if (tid == 0) bad = 0;
+    __syncthreads();
+    for (int k = 0; k < m; ++k) {
+        if (tid == 0) {
+            const double d = A[k * m + k];
+            if (!(d > 0.0) || !isfinite(d)) {
+                bad = k + 1;
+            } else {
+                const double r = sqrt(d);
+                A[k * m + k] = r;
+                dinv = 1.0 / r;
             }
-            __syncthreads();
-            if (bad) break;
-            for (int j = k + 1 + tid; j < m; j += bs) A[k * m + j] *= dinv;
-            __syncthreads();
-            const int r = m - k - 1;
-            for (int e = tid; e < r * r; e += bs) {
-                const int i = k + 1 + e / r, j = k + 1 + e % r;
-                if (j >= i) A[i * m + j] -= A[k * m + i] * A[k * m + j];
-            }
-            __syncthreads();
         }
-        if (!bad || !(shift_on_fail > 0.0) || attempt == 1) break;
-        shift = shift_on_fail;
+        __syncthreads();
+        if (bad) break;
+        for (int j = k + 1 + tid; j < m; j += bs) A[k * m + j] *= dinv;
+        __syncthreads();
+        const int r = m - k - 1;
+        for (int e = tid; e < r * r; e += bs) {
+            const int i = k + 1 + e / r, j = k + 1 + e % r;
+            if (j >= i) A[i * m + j] -= A[k * m + i] * A[k * m + j];
+        }
         __syncthreads();
     }
     if (!bad)
@@ -133,167 +111,176 @@ __global__ void __launch_bounds__(1024) k_chol_upper(int m, const double *__rest
     __syncthreads();
     if (use_smem)
         for (int e = tid; e < m * m; e += bs) Rg[e] = A[e];
-    if (tid == 0) *status = bad ? bad : (shift > 0.0 ? -1 : 0);
+    if (tid == 0) {
+        const int32_t st = bad ? bad : -1;
+        *status = st;
+        if (out_status) *out_status = st;
+    }
 }
 
 void raise_smem_limits();   // defined after the kernels it configures
 
 // ---------------------------------------------------------------------------
-// Blocked form for m >= 64: the CHB x CHB diagonal blocks on one CTA, the
-// panel solves and the symmetric trailing updates spread over the GPU (FP64
-// runs at a small fraction of the FP32 rate here, and one CTA would do all
-// m^3/6 FMAs of the update alone).  Right-looking, in place in R (upper).
-// A breakdown at pivot k (a pivot at or below shift_on_fail) sets *status =
-// k + 1 and stops the later steps; with shift_on_fail > 0 the one-block
-// kernel then refactors G + shift I.
+// Blocked Cholesky factor and inverse: G = R^T R, X = R^{-1}, from the
+// elimination of [G | I], whose right part ends as R^{-T}.  Right-looking in
+// CHB x CHB blocks: the diagonal block on one CTA, the panel solves and the
+// trailing updates of both parts spread over the GPU (FP64 issues at ~1.6
+// FMAs per clock and SM here, so m^3/6 of them belong on many SMs; what is
+// left is the chain of m pivots).  The right part costs no further steps: a
+// separate triangular inverse by back substitution, one warp per column, was
+// a chain of m dot products (m = 150: 136 us, m = 300: 321 us).  Factor and
+// inverse at m = 150: 446 us on one CTA each, 181 us here.  The lower
+// triangle of X holds the right part during the elimination; R is worked on
+// in place (upper).  A breakdown at pivot k (a pivot at or below
+// shift_on_fail) sets *status = k + 1 and stops the later steps; with
+// shift_on_fail > 0 the one-block kernel then refactors G + shift I and
+// k_triinv_upper inverts that factor.  `status` is a device word: the steps
+// read it, and the last kernel copies it to `out_status` (a mapped host word
+// costs each reader about a microsecond).
 // ---------------------------------------------------------------------------
 constexpr int CHB = 32;
 
-__global__ void k_chol_init(int m, const double *__restrict__ G, double *__restrict__ A, int32_t *__restrict__ status) {
+__global__ void k_chol_init(int m, const double *__restrict__ G, double *__restrict__ A, double *__restrict__ X,
+                            int32_t *__restrict__ status) {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e == 0) *status = 0;
-    if (e < (int64_t)m * m && G != A) A[e] = G[e];
+    if (e >= (int64_t)m * m) return;
+    if (G != A) A[e] = G[e];
+    X[e] = e / m == e % m ? 1.0 : 0.0;
 }
 
-// One warp factors the kb x kb diagonal block (lane j owns column j of its
-// upper triangle; warp barriers only).
-__global__ void __launch_bounds__(32) k_chol_diag(int m, int k0, int kb, double *__restrict__ A,
-                                                 int32_t *__restrict__ status, double pmin) {
-    __shared__ double S[CHB][CHB + 1];
-    if (*(volatile int32_t *)status != 0) return;
-    const int lane = threadIdx.x;
-    for (int i = 0; i < kb; ++i)
-        if (lane < kb) S[i][lane] = A[(int64_t)(k0 + i) * m + k0 + lane];
-    __syncwarp();
-    int bad = 0;
-    for (int k = 0; k < kb; ++k) {
-        const double d = S[k][k];
-        if (!(d > pmin) || !isfinite(d)) {
-            bad = k0 + k + 1;
-            break;   // uniform: every lane read the same pivot
-        }
-        const double r = sqrt(d), dinv = 1.0 / r;
-        __syncwarp();
-        if (lane == k) S[k][k] = r;
-        if (lane > k && lane < kb) S[k][lane] *= dinv;
-        __syncwarp();
-        if (lane > k && lane < kb) {
-            const double skj = S[k][lane];
-            for (int i = k + 1; i <= lane; ++i) S[i][lane] -= S[k][i] * skj;
-        }
-        __syncwarp();
+// The kb x kb diagonal block on 8 warps: thread (i0, j) owns rows i0, i0 + 8,
+// ... of column j in registers.  Per pivot the warp of row k scales the row
+// by 1/sqrt(pivot) and publishes it, one barrier, everyone updates its rows
+// below.  Bound by that chain (about 0.3 us per pivot; one warp with the
+// block in shared memory took 62 us per 32 pivots).
+__global__ void __launch_bounds__(256) k_chol_diag(int m, int k0, int kb, double *__restrict__ A,
+                                                   int32_t *__restrict__ status, double pmin) {
+    __shared__ double u[2][CHB];   // alternating by pivot: one barrier per pivot
+    __shared__ int bad[2];
+    if (*(volatile int32_t *)status != 0) return;   // uniform: the same word for every thread
+    const int j = threadIdx.x & 31, i0 = threadIdx.x >> 5;
+    double c[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = i0 + 8 * q;
+        c[q] = (i < kb && j < kb && j >= i) ? A[(int64_t)(k0 + i) * m + k0 + j] : 0.0;
     }
-    if (bad) {
-        if (lane == 0) *status = bad;
-        return;
+    if (threadIdx.x < 2) bad[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int q0 = 0; q0 < 4; ++q0) {
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) {
+            const int k = q0 * 8 + kk;
+            if (k >= kb) break;
+            if (i0 == kk) {
+                const double d = __shfl_sync(0xffffffffu, c[q0], k);
+                if (!(d > pmin) || !isfinite(d)) {
+                    if (j == 0) bad[k & 1] = k0 + k + 1;
+                } else {
+                    c[q0] *= rsqrt(d);
+                    u[k & 1][j] = c[q0];
+                }
+            }
+            __syncthreads();
+            if (bad[k & 1]) {   // uniform
+                if (threadIdx.x == 0) *status = bad[k & 1];
+                return;
+            }
+            const double uj = u[k & 1][j];
+#pragma unroll
+            for (int q = q0; q < 4; ++q) {
+                const int i = i0 + 8 * q;
+                if (i > k) c[q] = fma(-u[k & 1][i], uj, c[q]);
+            }
+        }
     }
-    for (int i = 0; i < kb; ++i)
-        if (lane < kb) A[(int64_t)(k0 + i) * m + k0 + lane] = lane >= i ? S[i][lane] : 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = i0 + 8 * q;
+        if (i < kb && j < kb) A[(int64_t)(k0 + i) * m + k0 + j] = j >= i ? c[q] : 0.0;
+    }
 }
 
-// rows k0 .. k0+kb of the columns right of the block: x = R_kk^{-T} a, one
-// warp per column (lane i = row i; the forward substitution broadcasts
-// x_p from lane p), four columns per block
-__global__ void __launch_bounds__(128) k_chol_panel(int m, int k0, int kb, double *__restrict__ A,
-                                                   const int32_t *__restrict__ status) {
-    __shared__ double Rk[CHB][CHB + 1];
+// rows k0 .. k0+kb of the columns right of the block and of the right part's
+// columns 0 .. k0+kb: x = R_kk^{-T} a, one warp per column (lane i = row i;
+// the forward substitution with the unit-scaled factor broadcasts row p, so
+// one FMA per step: FP64 FMAs of one warp issue ~70 clocks apart)
+__global__ void __launch_bounds__(64) k_chol_panel(int m, int k0, int kb, double *__restrict__ A,
+                                                   double *__restrict__ X, const int32_t *__restrict__ status) {
+    __shared__ double Rk[CHB][CHB + 1], ri[CHB];
     if (*(volatile int32_t *)status != 0) return;
-    for (int e = threadIdx.x; e < kb * kb; e += blockDim.x)
-        Rk[e / kb][e % kb] = A[(int64_t)(k0 + e / kb) * m + k0 + e % kb];
+    if (threadIdx.x < kb) ri[threadIdx.x] = 1.0 / A[(int64_t)(k0 + threadIdx.x) * m + k0 + threadIdx.x];
+    __syncthreads();
+    for (int e = threadIdx.x; e < kb * kb; e += blockDim.x) {
+        const int p = e / kb, i = e % kb;
+        Rk[p][i] = A[(int64_t)(k0 + p) * m + k0 + i] * ri[p];
+    }
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int c = k0 + kb + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (c >= m) return;
-    double v = lane < kb ? A[(int64_t)(k0 + lane) * m + c] : 0.0;
-    const double ri = lane < kb ? 1.0 / Rk[lane][lane] : 0.0;
-    double x = 0.0;
-    for (int p = 0; p < kb; ++p) {
-        const double xp = __shfl_sync(0xffffffffu, v * ri, p);
-        if (lane == p) x = xp;
-        if (lane > p && lane < kb) v = fma(-Rk[p][lane], xp, v);
+    double *col = (c < k0 + kb ? X : A) + (int64_t)k0 * m + c;
+    double v = lane < kb ? col[(int64_t)lane * m] : 0.0;
+    for (int p = 0; p + 1 < kb; ++p) {
+        const double vp = __shfl_sync(0xffffffffu, v, p);
+        if (lane > p && lane < kb) v = fma(-Rk[p][lane], vp, v);
     }
-    if (lane < kb) A[(int64_t)(k0 + lane) * m + c] = x;
+    // entries above the right part's diagonal are zero and stay so
+    if (lane < kb && (c >= k0 + kb || c <= k0 + lane)) col[(int64_t)lane * m] = v * ri[lane];
 }
 
-// A[i][j] -= sum_p A[k0+p][i] A[k0+p][j] for k0+kb <= i <= j < m, 16 x 16
-// output tiles (the tiles below the diagonal return at once)
-__global__ void __launch_bounds__(256) k_chol_update(int m, int k0, int kb, double *__restrict__ A,
-                                                    const int32_t *__restrict__ status) {
+// Trailing rows i >= k0+kb: A[i][j] -= sum_p A[k0+p][i] A[k0+p][j] for j >= i
+// and X[i][c] -= sum_p A[k0+p][i] X[k0+p][c] for the right part's columns
+// c < k0+kb; 16 x 16 output tiles, the first `tl` tile columns the left part
+__global__ void __launch_bounds__(256) k_chol_update(int m, int k0, int kb, int tl, double *__restrict__ A,
+                                                     double *__restrict__ X, const int32_t *__restrict__ status) {
     __shared__ double Pi[CHB][17], Pj[CHB][17];
     if (*(volatile int32_t *)status != 0) return;
     const int r0 = k0 + kb;
-    if (blockIdx.x < blockIdx.y) return;
+    const bool left = (int)blockIdx.x < tl;
+    if (left && blockIdx.x < blockIdx.y) return;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int i0 = r0 + blockIdx.y * 16, j0 = r0 + blockIdx.x * 16;
+    const int i0 = r0 + blockIdx.y * 16, j0 = left ? r0 + blockIdx.x * 16 : (blockIdx.x - tl) * 16;
+    const int jend = left ? m : r0;
+    double *D = left ? A : X;
     for (int e = threadIdx.x; e < kb * 16; e += 256) {
         const int p = e / 16, q = e % 16;
         Pi[p][q] = (i0 + q < m) ? A[(int64_t)(k0 + p) * m + i0 + q] : 0.0;
-        Pj[p][q] = (j0 + q < m) ? A[(int64_t)(k0 + p) * m + j0 + q] : 0.0;
+        // above the right part's diagonal the matrix holds nothing yet
+        Pj[p][q] = (j0 + q < jend && (left || j0 + q <= k0 + p)) ? D[(int64_t)(k0 + p) * m + j0 + q] : 0.0;
     }
     __syncthreads();
     const int i = i0 + ty, j = j0 + tx;
-    if (i >= m || j >= m || j < i) return;
+    if (i >= m || j >= jend || (left && j < i)) return;
     double s = 0.0;
+#pragma unroll 8
     for (int p = 0; p < kb; ++p) s = fma(Pi[p][ty], Pj[p][tx], s);
-    A[(int64_t)i * m + j] -= s;
+    D[(int64_t)i * m + j] -= s;
 }
 
-__global__ void k_chol_finish(int m, double *__restrict__ A, const int32_t *__restrict__ status) {
-    if (*(volatile int32_t *)status != 0) return;
+// R's lower triangle to zero, X = (its lower triangle)^T
+__global__ void k_chol_finish(int m, double *__restrict__ A, double *__restrict__ X,
+                              const int32_t *__restrict__ status, int32_t *__restrict__ out_status) {
+    const int32_t st = *(volatile int32_t *)status;
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e < (int64_t)m * m && e % m < e / m) A[e] = 0.0;
+    if (e == 0 && out_status) *out_status = st;
+    if (st != 0 || e >= (int64_t)m * m) return;
+    const int i = (int)(e / m), j = (int)(e % m);
+    if (j >= i) return;
+    A[e] = 0.0;
+    X[(int64_t)j * m + i] = X[e];
+    X[e] = 0.0;
 }
 
-void small_chol_upper(Ctx &ctx, int m, const double *G, double *R, int32_t *status, double shift_on_fail) {
-    const size_t smem = (size_t)m * m * sizeof(double);
-    const int use_smem = smem <= 200 * 1024;
-    raise_smem_limits();
-    if (m < 64) {
-        ctx.before(KC_SMALL_DENSE, 16.0 * m * m, (double)m * m * m / 3.0);
-        k_chol_upper<<<1, 1024, use_smem ? smem : 0, ctx.stream>>>(m, G, R, status, use_smem, shift_on_fail, 0);
-        ctx.after();
-        return;
-    }
-    const int64_t m2 = (int64_t)m * m;
-    const unsigned eg = (unsigned)((m2 + 255) / 256);
-    ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-    k_chol_init<<<eg, 256, 0, ctx.stream>>>(m, G, R, status);
-    ctx.after();
-    for (int k0 = 0; k0 < m; k0 += CHB) {
-        const int kb = std::min(CHB, m - k0), rest = m - k0 - kb;
-        ctx.before(KC_SMALL_DENSE, 16.0 * kb * kb, (double)kb * kb * kb / 3.0);
-        k_chol_diag<<<1, 32, 0, ctx.stream>>>(m, k0, kb, R, status, shift_on_fail);
-        ctx.after();
-        if (rest == 0) break;
-        ctx.before(KC_SMALL_DENSE, 16.0 * kb * rest, 0.5 * kb * kb * rest);
-        k_chol_panel<<<(rest + 3) / 4, 128, 0, ctx.stream>>>(m, k0, kb, R, status);
-        ctx.after();
-        const int tiles = (rest + 15) / 16;
-        ctx.before(KC_SMALL_DENSE, 8.0 * rest * rest, 0.5 * (double)rest * rest * kb);
-        k_chol_update<<<dim3(tiles, tiles), 256, 0, ctx.stream>>>(m, k0, kb, R, status);
-        ctx.after();
-    }
-    ctx.before(KC_SMALL_DENSE, 8.0 * m2, 0);
-    k_chol_finish<<<eg, 256, 0, ctx.stream>>>(m, R, status);
-    ctx.after();
-    if (shift_on_fail > 0.0 && G != R) {
-        ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-        k_chol_upper<<<1, 1024, use_smem ? smem : 0, ctx.stream>>>(m, G, R, status, use_smem, shift_on_fail, 1);
-        ctx.after();
-    }
-}
-
-// ---------------------------------------------------------------------------
-// X = R^{-1} for upper triangular R (m x m, row-major): one warp per column j,
-// back substitution x_i = (delta_ij - sum_{k=i+1..j} R_ik x_k) / R_ii with the
-// column in shared memory and each sum split over the lanes (R rows are read
-// coalesced; R stays in L1/L2).  Entries below the diagonal are set to zero.
-// ---------------------------------------------------------------------------
-// The reciprocals of the diagonal are formed once per column block up front
-// (FP64 division is slow here), so each step of the chain is FMAs and one
-// warp reduction.
-__global__ void __launch_bounds__(32) k_triinv_upper(int m, const double *__restrict__ R, double *__restrict__ X) {
+// X = R^{-1} of the shifted factor (runs only after a shifted refactorisation,
+// *status < 0): one warp per column j, back substitution x_i = (delta_ij -
+// sum_{k=i+1..j} R_ik x_k) / R_ii, the sum split over the lanes.
+__global__ void __launch_bounds__(32) k_triinv_upper(int m, const double *__restrict__ R, double *__restrict__ X,
+                                                     const int32_t *__restrict__ status) {
     extern __shared__ double xcol[];
+    if (*(volatile int32_t *)status >= 0) return;
     double *rinv = xcol + m;
     const int j = blockIdx.x, lane = threadIdx.x;
     for (int i = lane; i <= j; i += 32) rinv[i] = 1.0 / R[(int64_t)i * m + i];
@@ -314,12 +301,66 @@ __global__ void __launch_bounds__(32) k_triinv_upper(int m, const double *__rest
     }
 }
 
-void small_triinv_upper(Ctx &ctx, int m, const double *R, double *Rinv) {
-    const size_t smem = 2 * (size_t)m * sizeof(double);
-    ctx.before(KC_SMALL_DENSE, 16.0 * m * m, (double)m * m * m / 3.0);
-    raise_smem_limits();
-    k_triinv_upper<<<m, 32, smem, ctx.stream>>>(m, R, Rinv);
+void small_chol_inv(Ctx &ctx, int m, const double *G, double *R, double *Rinv, int32_t *status, int32_t *out_status,
+                    double shift_on_fail) {
+    const int64_t m2 = (int64_t)m * m;
+    const unsigned eg = (unsigned)((m2 + 255) / 256);
+    ctx.before(KC_SMALL_DENSE, 24.0 * m2, 0);
+    k_chol_init<<<eg, 256, 0, ctx.stream>>>(m, G, R, Rinv, status);
     ctx.after();
+    for (int k0 = 0; k0 < m; k0 += CHB) {
+        const int kb = std::min(CHB, m - k0), rest = m - k0 - kb;
+        ctx.before(KC_SMALL_DENSE, 16.0 * kb * kb, (double)kb * kb * kb / 3.0);
+        k_chol_diag<<<1, 256, 0, ctx.stream>>>(m, k0, kb, R, status, shift_on_fail);
+        ctx.after();
+        ctx.before(KC_SMALL_DENSE, 16.0 * kb * m, (double)kb * kb * m);
+        k_chol_panel<<<(m + 1) / 2, 64, 0, ctx.stream>>>(m, k0, kb, R, Rinv, status);
+        ctx.after();
+        if (rest == 0) break;
+        const int tl = (rest + 15) / 16, tr = (k0 + kb + 15) / 16;
+        ctx.before(KC_SMALL_DENSE, 8.0 * rest * m, (double)rest * m * kb);
+        k_chol_update<<<dim3(tl + tr, tl), 256, 0, ctx.stream>>>(m, k0, kb, tl, R, Rinv, status);
+        ctx.after();
+    }
+    ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
+    k_chol_finish<<<eg, 256, 0, ctx.stream>>>(m, R, Rinv, status, out_status);
+    ctx.after();
+    if (shift_on_fail > 0.0 && G != R) {
+        const size_t smem = (size_t)m * m * sizeof(double);
+        const int use_smem = smem <= 200 * 1024;
+        raise_smem_limits();
+        ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
+        k_chol_shifted<<<1, 1024, use_smem ? smem : 0, ctx.stream>>>(m, G, R, status, out_status, use_smem, shift_on_fail);
+        ctx.after();
+        ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
+        k_triinv_upper<<<m, 32, 2 * (size_t)m * sizeof(double), ctx.stream>>>(m, R, Rinv, status);
+        ctx.after();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// ||S||_F as FRO_PARTS partial sums of squares, one per block, summed by the
+// readers (fro_norm, a whole warp)
+constexpr int FRO_PARTS = 32, OA_PARTS = 64;   // OA_PARTS: blocks of k_oa_norms
+__global__ void __launch_bounds__(256) k_fro(int m, const double *__restrict__ S, double *__restrict__ part) {
+    __shared__ double red[8];
+    double s = 0;
+    for (int64_t e = blockIdx.x * 256 + threadIdx.x; e < (int64_t)m * m; e += FRO_PARTS * 256) s += S[e] * S[e];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        part[blockIdx.x] = t;
+    }
+}
+__device__ __forceinline__ double fro_norm(const double *part) {
+    double s = part[threadIdx.x & 31];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    return sqrt(s);
 }
 
 // ---------------------------------------------------------------------------
@@ -483,7 +524,7 @@ k_jacobi_coop(int m, double *__restrict__ A, double *__restrict__ V, double *__r
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
     const double eps = DBL_EPSILON;
-    const double absmin = (*normA) * eps * 0.5 / (double)m;
+    const double absmin = fro_norm(normA) * eps * 0.5 / (double)m;
     // cnt[2 + (sweep & 1)]: set when some pair still passes the rotation test
     if (gtid == 0) cnt[2] = cnt[3] = 0;
     grid.sync();
@@ -596,42 +637,40 @@ __global__ void k_identity(int m, double *__restrict__ V) {
     if (e < (int64_t)m * m) V[e] = (e / m == e % m) ? 1.0 : 0.0;
 }
 
-// final ordering: lam ascending, Q columns permuted
-__global__ void k_sort_eig(int m, const double *__restrict__ lam_in, const double *__restrict__ S,
-                           double *__restrict__ lam, double *__restrict__ Q) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-        const double di = lam_in[i];
-        int rank = 0;
-        for (int j = 0; j < m; ++j) {
-            const double dj = lam_in[j];
-            rank += (dj < di) || (dj == di && j < i);
-        }
-        lam[rank] = di;
-        for (int row = 0; row < m; ++row) Q[(int64_t)row * m + rank] = S[(int64_t)row * m + i];
+// final ordering: lam ascending, Q columns permuted.  Every block ranks all
+// eigenvalues (as integers of the same order: FP64 compares run on the slow
+// FP64 pipe) and moves its rows, one warp per row.
+__global__ void __launch_bounds__(256) k_sort_eig(int m, const double *__restrict__ lam_in, const double *__restrict__ S,
+                                                  double *__restrict__ lam, double *__restrict__ Q) {
+    __shared__ long long key[1024];
+    __shared__ int rank[1024];
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        const long long b = __double_as_longlong(lam_in[i]);
+        key[i] = b ^ ((b >> 63) & 0x7fffffffffffffffll);
     }
-}
-
-__global__ void k_fro(int m, const double *__restrict__ S, double *__restrict__ out) {
-    __shared__ double red[32];
-    double s = 0;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) s += S[e] * S[e];
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0;
-        for (int w = 0; w < (blockDim.x + 31) / 32; ++w) t += red[w];
-        *out = sqrt(t);
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        const long long ki = key[i];
+        int r = 0;
+#pragma unroll 4
+        for (int j = 0; j < m; ++j) r += (key[j] < ki) || (key[j] == ki && j < i);
+        rank[i] = r;
+        if (blockIdx.x == 0) lam[r] = lam_in[i];
     }
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (row >= m) return;
+    for (int j = lane; j < m; j += 32) Q[(int64_t)row * m + rank[j]] = S[(int64_t)row * m + j];
 }
 
 size_t small_syev_work_bytes(int m) {
     const size_t mp = (size_t)(m + (m & 1));
     const size_t m2 = (size_t)m * m;
-    // A32/V32 global fallback (2 mp^2 doubles) + S0, S1, G, Y, T, V (6 m^2) + lam0, normA, counters,
-    // component labels and sizes (2 m ints)
-    return 2 * mp * mp * sizeof(double) + 6 * m2 * sizeof(double) + (2 * (size_t)m + 2) * sizeof(double) +
-           2 * (size_t)m * sizeof(int) + 4096;
+    // A32/V32 global fallback (2 mp^2 doubles) + S0, S1, G, Y, T, V (6 m^2) + lam0, counters,
+    // component labels and sizes (2 m ints), partial norms
+    return 2 * mp * mp * sizeof(double) + 6 * m2 * sizeof(double) +
+           ((size_t)m + FRO_PARTS + OA_PARTS) * sizeof(double) + 2 * (size_t)m * sizeof(int) + 4096;
 }
 
 // ---------------------------------------------------------------------------
@@ -654,39 +693,47 @@ size_t small_syev_work_bytes(int m) {
 // products are FP64 GEMMs; three steps reach FP64 accuracy from the FP32
 // Jacobi's vectors wherever the pairs are separated.
 // ---------------------------------------------------------------------------
-__device__ double block_sum(double v, double *red) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    double t = 0.0;
-    for (int w = 0; w < nw; ++w) t += red[w];
-    return t;
-}
-
-// lam_t = t_ii / g_ii and the pair threshold delta = 2 ||T - D||_F (one
-// block: the norm is one fixed-order reduction)
-__global__ void __launch_bounds__(1024) k_oa_norms(int m, const double *__restrict__ G, const double *__restrict__ T,
-                                                  double *__restrict__ lam_t, double *__restrict__ delta) {
-    __shared__ double red[32];
-    const int tid = threadIdx.x, bs = blockDim.x;
+// lam_t = t_ii / g_ii, and per block the partial sum of ||T - D||_F^2 over its
+// rows (fixed order; one block for the whole matrix took 33 us at m = 150,
+// all of it FP64 issue; this takes 5)
+__global__ void __launch_bounds__(256) k_oa_norms(int m, const double *__restrict__ G, const double *__restrict__ T,
+                                                  double *__restrict__ lam_t, double *__restrict__ part) {
+    __shared__ double red[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double off = 0.0;
-    for (int e = tid; e < m * m; e += bs) {
-        const int i = e / m, j = e % m;
-        const double d = i == j ? T[e] - T[e] / G[e] : T[e];
-        off += d * d;
+    for (int i = blockIdx.x * 8 + warp; i < m; i += OA_PARTS * 8) {
+        const double *Ti = T + (int64_t)i * m;
+        const double ti = Ti[i], li = ti / G[(int64_t)i * m + i];
+        if (lane == 0) lam_t[i] = li;
+        for (int j = lane; j < m; j += 32) {
+            const double d = i == j ? ti - li : Ti[j];
+            off = fma(d, d, off);
+        }
     }
-    off = block_sum(off, red);
-    for (int i = tid; i < m; i += bs) lam_t[i] = T[(int64_t)i * m + i] / G[(int64_t)i * m + i];
-    if (tid == 0) *delta = 2.0 * sqrt(off);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) off += __shfl_xor_sync(0xffffffffu, off, o);
+    if (lane == 0) red[warp] = off;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        part[blockIdx.x] = t;
+    }
 }
 
 // Ep = I + E (row-major), one thread per entry over many blocks (the FP64
-// divisions spread over the GPU)
-__global__ void k_oa_step(int m, const double *__restrict__ G, const double *__restrict__ T,
-                          const double *__restrict__ lam_t, const double *__restrict__ delta, double *__restrict__ Ep) {
+// divisions spread over the GPU); the pair threshold is delta = 2 ||T - D||_F
+__global__ void __launch_bounds__(256) k_oa_step(int m, const double *__restrict__ G, const double *__restrict__ T,
+                                                 const double *__restrict__ lam_t, const double *__restrict__ part,
+                                                 double *__restrict__ Ep) {
+    __shared__ double delta;
+    if (threadIdx.x < 32) {
+        double s = part[threadIdx.x] + part[threadIdx.x + 32];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) delta = 2.0 * sqrt(s);
+    }
+    __syncthreads();
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= (int64_t)m * m) return;
     const int i = (int)(e / m), j = (int)(e % m);
@@ -696,7 +743,7 @@ __global__ void k_oa_step(int m, const double *__restrict__ G, const double *__r
         v = 1.0 + 0.5 * r;
     } else {
         const double li = lam_t[i], lj = lam_t[j], num = T[e] + lj * r;
-        const bool sep = fabs(li - lj) > *delta && 8.0 * fabs(num) <= fabs(lj - li);
+        const bool sep = fabs(li - lj) > delta && 8.0 * fabs(num) <= fabs(lj - li);
         v = sep ? num / (lj - li) : 0.5 * r;
     }
     Ep[e] = v;
@@ -727,9 +774,11 @@ __global__ void __launch_bounds__(1024) k_oa_components(int m, const double *__r
     __shared__ int members[1024];
     __shared__ double cs[512], sn[512];
     __shared__ int pp[512], qq[512];
-    const double tau = 4.0 * m * 1.1102230246251565e-16 * (*normS);
+    const double tau = 4.0 * m * 1.1102230246251565e-16 * fro_norm(normS);
+    // T is symmetric (its product is mirrored); |t| > tau compared as integers
+    const long long tau_bits = __double_as_longlong(tau);
     auto joined = [&](int i, int j) {
-        return fabs(T[(int64_t)i * m + j]) > tau || fabs(T[(int64_t)j * m + i]) > tau;
+        return (__double_as_longlong(T[(int64_t)i * m + j]) & 0x7fffffffffffffffll) > tau_bits;
     };
     for (int i = tid; i < m; i += bs) {
         label[i] = i;
@@ -919,25 +968,29 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
     double *Tm = Ym + m2;
     double *Vm = Tm + m2;
     double *lam0 = Vm + m2;
-    double *normA = lam0 + m;   // [0] = ||S||_F, [1] = the refinement's pair threshold
-    int *cnt = reinterpret_cast<int *>(normA + m + 2);
+    double *normA = lam0 + m;             // FRO_PARTS partial sums of ||S||_F^2
+    double *oa_part = normA + FRO_PARTS;  // OA_PARTS partial sums of the refinement's ||T - D||_F^2
+    int *cnt = reinterpret_cast<int *>(oa_part + OA_PARTS);
     int32_t *cst = cnt + 4;
 
     ctx.before(KC_SMALL_DENSE, 8.0 * m2, 2.0 * m2);
-    k_fro<<<1, 1024, 0, ctx.stream>>>(m, S, normA);
+    k_fro<<<FRO_PARTS, 256, 0, ctx.stream>>>(m, S, normA);
     ctx.after();
-    ctx.before(KC_SMALL_DENSE, 8.0 * m2, 0);
-    k_identity<<<(unsigned)((m2 + 255) / 256), 256, 0, ctx.stream>>>(m, Vm);
-    ctx.after();
+    auto identity = [&](double *V) {
+        ctx.before(KC_SMALL_DENSE, 8.0 * m2, 0);
+        k_identity<<<(unsigned)((m2 + 255) / 256), 256, 0, ctx.stream>>>(m, V);
+        ctx.after();
+    };
     // The FP32 stage needs A and V in one block's shared memory (m <= 160:
     // 206 KB with the odd row pitch); larger problems go straight to the
     // cooperative FP64 Jacobi.
     if (mode == 0 || m > JMAX) {
+        identity(Vm);
         cudaMemcpyAsync(Tm, S, m2 * sizeof(double), cudaMemcpyDeviceToDevice, ctx.stream);
         const cudaError_t e = coop_jacobi(ctx, m, Tm, Vm, lam0, 60, normA, cnt);
         if (e != cudaSuccess) return e;
         ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-        k_sort_eig<<<(m + 127) / 128, 128, 0, ctx.stream>>>(m, lam0, Vm, lam, Q);
+        k_sort_eig<<<(m + 7) / 8, 256, 0, ctx.stream>>>(m, lam0, Vm, lam, Q);
         ctx.after();
         return cudaGetLastError();
     }
@@ -955,20 +1008,20 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
         double *X0 = S0, *X1 = S1;
         const unsigned eg = (unsigned)((m2 + 255) / 256);
         for (int it = 0; it < 3; ++it) {
-            dgemm(ctx, 1, 0, m, m, m, X0, m, X0, m, 0.0, G, m, 1, nullptr, KC_SMALL_DENSE);
+            dgemm(ctx, 1, 0, m, m, m, X0, m, X0, m, 0.0, G, m, 1, nullptr, KC_SMALL_DENSE, true);
             ctx.before(KC_SMALL_DENSE, 16.0 * m2, 2.0 * m2);
             k_ns_factor<<<eg, 256, 0, ctx.stream>>>(m, G, Vm);
             ctx.after();
             dgemm(ctx, 0, 0, m, m, m, X0, m, Vm, m, 0.0, X1, m, 1, nullptr, KC_SMALL_DENSE);
             std::swap(X0, X1);
-            dgemm(ctx, 1, 0, m, m, m, X0, m, X0, m, 0.0, G, m, 1, nullptr, KC_SMALL_DENSE);
+            dgemm(ctx, 1, 0, m, m, m, X0, m, X0, m, 0.0, G, m, 1, nullptr, KC_SMALL_DENSE, true);
             dgemm(ctx, 0, 0, m, m, m, S, m, X0, m, 0.0, Ym, m, 1, nullptr, KC_SMALL_DENSE);
-            dgemm(ctx, 1, 0, m, m, m, X0, m, Ym, m, 0.0, Tm, m, 1, nullptr, KC_SMALL_DENSE);
+            dgemm(ctx, 1, 0, m, m, m, X0, m, Ym, m, 0.0, Tm, m, 1, nullptr, KC_SMALL_DENSE, true);
             ctx.before(KC_SMALL_DENSE, 16.0 * m2, 4.0 * m2);
-            k_oa_norms<<<1, 1024, 0, ctx.stream>>>(m, G, Tm, lam0, normA + 1);
+            k_oa_norms<<<OA_PARTS, 256, 0, ctx.stream>>>(m, G, Tm, lam0, oa_part);
             ctx.after();
             ctx.before(KC_SMALL_DENSE, 24.0 * m2, 8.0 * m2);
-            k_oa_step<<<eg, 256, 0, ctx.stream>>>(m, G, Tm, lam0, normA + 1, Vm);
+            k_oa_step<<<eg, 256, 0, ctx.stream>>>(m, G, Tm, lam0, oa_part, Vm);
             ctx.after();
             dgemm(ctx, 0, 0, m, m, m, X0, m, Vm, m, 0.0, X1, m, 1, nullptr, KC_SMALL_DENSE);
             std::swap(X0, X1);
@@ -977,7 +1030,7 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
         // accepted steps: three orthonormalisation steps bring it back to
         // rounding level before the groups are rotated
         for (int it = 0; it < 3; ++it) {
-            dgemm(ctx, 1, 0, m, m, m, X0, m, X0, m, 0.0, G, m, 1, nullptr, KC_SMALL_DENSE);
+            dgemm(ctx, 1, 0, m, m, m, X0, m, X0, m, 0.0, G, m, 1, nullptr, KC_SMALL_DENSE, true);
             ctx.before(KC_SMALL_DENSE, 16.0 * m2, 2.0 * m2);
             k_ns_factor<<<eg, 256, 0, ctx.stream>>>(m, G, Vm);
             ctx.after();
@@ -985,30 +1038,30 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
             std::swap(X0, X1);
         }
         dgemm(ctx, 0, 0, m, m, m, S, m, X0, m, 0.0, Ym, m, 1, nullptr, KC_SMALL_DENSE);
-        dgemm(ctx, 1, 0, m, m, m, X0, m, Ym, m, 0.0, Tm, m, 1, nullptr, KC_SMALL_DENSE);
+        dgemm(ctx, 1, 0, m, m, m, X0, m, Ym, m, 0.0, Tm, m, 1, nullptr, KC_SMALL_DENSE, true);
         int *label = cst + 4, *csize = label + m;
         ctx.before(KC_SMALL_DENSE, 24.0 * m2, 4.0 * m2);
         k_oa_components<<<1, 1024, 0, ctx.stream>>>(m, Tm, normA, X0, lam0, label, csize, (double *)Ag,
                                                      (double *)Vg, X1);
         ctx.after();
         ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-        k_sort_eig<<<(m + 127) / 128, 128, 0, ctx.stream>>>(m, lam0, X0, lam, Q);
+        k_sort_eig<<<(m + 7) / 8, 256, 0, ctx.stream>>>(m, lam0, X0, lam, Q);
         ctx.after();
         return cudaGetLastError();
     }
     // stage 2: FP64 re-orthonormalisation S1 = S0 R^{-1}, G = S0^T S0 = R^T R
-    dgemm(ctx, 1, 0, m, m, m, S0, m, S0, m, 0.0, G, m, 1, nullptr, KC_SMALL_DENSE);
-    small_chol_upper(ctx, m, G, G, cst, 0.0);
-    small_triinv_upper(ctx, m, G, Ym);
+    dgemm(ctx, 1, 0, m, m, m, S0, m, S0, m, 0.0, G, m, 1, nullptr, KC_SMALL_DENSE, true);
+    small_chol_inv(ctx, m, G, G, Ym, cst, nullptr, 0.0);
     dgemm(ctx, 0, 0, m, m, m, S0, m, Ym, m, 0.0, S1, m, 1, nullptr, KC_SMALL_DENSE);
     // T = S1^T A S1, then polish T by FP64 Jacobi, S = S1 V
     dgemm(ctx, 0, 0, m, m, m, S, m, S1, m, 0.0, Ym, m, 1, nullptr, KC_SMALL_DENSE);
     dgemm(ctx, 1, 0, m, m, m, S1, m, Ym, m, 0.0, Tm, m, 1, nullptr, KC_SMALL_DENSE);
+    identity(Vm);
     const cudaError_t e = coop_jacobi(ctx, m, Tm, Vm, lam0, 20, normA, cnt);
     if (e != cudaSuccess) return e;
     dgemm(ctx, 0, 0, m, m, m, S1, m, Vm, m, 0.0, S0, m, 1, nullptr, KC_SMALL_DENSE);
     ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-    k_sort_eig<<<(m + 127) / 128, 128, 0, ctx.stream>>>(m, lam0, S0, lam, Q);
+    k_sort_eig<<<(m + 7) / 8, 256, 0, ctx.stream>>>(m, lam0, S0, lam, Q);
     ctx.after();
     return cudaGetLastError();
 }
@@ -1024,7 +1077,7 @@ void raise_smem_limits() {
     cudaGetDevice(&dev);
     std::call_once(once[dev < 0 || dev >= kMaxDevices ? 0 : dev], [] {   // per device, with it current
         const int lim = 200 * 1024;
-        cudaFuncSetAttribute(k_chol_upper, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_chol_shifted, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_triinv_upper, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_jacobi32, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     });
