@@ -1066,13 +1066,6 @@ slrf_status mg_prepare(slrf_handle *h, const slrf_filter *f, const KrylovDims &d
     mg.Minv = nullptr;
     if (e_inv >= 0) {
         if constexpr (sizeof(T) == 4) {
-            if (!h->cublas) {
-                if (cublasCreate(&h->cublas) != CUBLAS_STATUS_SUCCESS) {
-                    h->cublas = nullptr;
-                    g_last_error = "cublasCreate failed";
-                    return SLRF_ECUDA;
-                }
-            }
             const size_t inv_bytes = (size_t)N * nc * nc * sizeof(cplx<T>);
             const size_t inv_off = (inv_bytes + 255) / 256 * 256;
             CKS(ensure(h, h->mgInv, inv_off + coarse_inverse_work_bytes(nc, N)));
@@ -1084,20 +1077,14 @@ slrf_status mg_prepare(slrf_handle *h, const slrf_filter *f, const KrylovDims &d
             }
             if (key != h->inv_key || h->inv_buf != h->mgInv.p) {
                 const MgLevel<T> &Le = mg.lv[e_inv];
-                const int rc = coarse_inverse(h->ctx, h->cublas, nc, make_poleset<float>(f), Le.gptr, Le.gcol,
-                                              reinterpret_cast<const float2 *>(Le.ab), Minv,
-                                              reinterpret_cast<char *>(h->mgInv.p) + inv_off);
-                if (rc != 0) {
-                    h->inv_key.clear();
-                    g_last_error = "coarse inverse: cuBLAS status " + std::to_string(rc);
-                    return SLRF_ECUDA;
-                }
+                coarse_inverse(h->ctx, nc, make_poleset<float>(f), Le.gptr, Le.gcol,
+                               reinterpret_cast<const float2 *>(Le.ab), Minv,
+                               reinterpret_cast<char *>(h->mgInv.p) + inv_off);
                 h->inv_key = key;
                 h->inv_buf = h->mgInv.p;
                 h->inv_pan_ok = false;
             }
             mg.Minv = reinterpret_cast<const cplx<T> *>(Minv);
-            mg.cublas = h->cublas;
             mg.Mpan = nullptr;
             if (h->opts.mg_exact_tc && coarse_tc_fits(d.Lp)) {
                 CKS(ensure(h, h->mgInvPan, coarse_tc_panel_bytes(nc, N)));
@@ -1110,7 +1097,12 @@ slrf_status mg_prepare(slrf_handle *h, const slrf_filter *f, const KrylovDims &d
                 mg.Mpan = h->mgInvPan.p;
                 mg.ct_work = h->mgCtWork.p;
                 mg.ct_err = h->d_pin + 1;
+            } else if (!h->cublas && cublasCreate(&h->cublas) != CUBLAS_STATUS_SUCCESS) {
+                h->cublas = nullptr;
+                g_last_error = "cublasCreate failed";
+                return SLRF_ECUDA;
             }
+            mg.cublas = h->cublas;
         }
         mg_dinv<T>(h->ctx, mg, make_poleset<T>(f));
         return SLRF_OK;

@@ -12,18 +12,23 @@
 // as one batched complex GEMM per visit.  The inverse is symmetrised, so the
 // cycle stays a complex symmetric operator, as COCG requires.
 //
-// Blocked Gauss-Jordan (column-major view, blocks of CB rows/columns K, the
-// rest R), per block step, in place:
-//   P = M_KK^{-1} (one CTA per matrix, Gauss-Jordan in shared memory)
-//   T = P M_K*            C = M_*K
-//   M -= C T              (rank-CB update of the whole matrix)
-//   M_K* = T,  M_*K = -C P,  M_KK = P
-// after the last block M holds M^{-1}.  The GEMMs are plain complex FP32
-// GEMMs (cuBLAS, batched over the poles).
+// The elimination is the symmetric sweep in blocks of CB rows K (the rest R),
+// which keeps M complex symmetric, so only its block upper triangle is held
+// and half the arithmetic of Gauss-Jordan is done:
+//   P = M_KK^{-1},  T = P M_KR,  M_RR -= M_KR^T T,  M_KR = T,  M_KK = -P;
+// after the last block M holds -M^{-1}.  M is padded to whole blocks with the
+// identity.  Two launches per block: the panel (T, every block column its own
+// CTA), and the update, one CTA per 64 x 64 tile, whose first CTA takes the
+// next diagonal block and sweeps it in registers while the others work, so
+// the chain of 64 pivots (~11 us) hides behind the update.  Bound by FP32
+// arithmetic: 4 N n^3 flops (n = 1283, N = 4: 34 GF, 0.45 ms at 75 TFLOP/s);
+// cuBLAS complex GEMMs on the whole matrix, with the diagonal blocks and
+// block copies in launches of their own, took 3.9 ms there, this 1.7 ms.
 #include <cublas_v2.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "internal.h"
 
@@ -31,16 +36,18 @@ namespace slrf {
 
 namespace {
 
-constexpr int CB = 64;   // block size of the elimination
+constexpr int CB = 64;   // block size of the sweep
 
-// M_j = A - sigma_j B on the level's CSR pattern of (a, b) pairs, dense n x n
-__global__ void k_dense_shift(int n, int N, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
+// M_j = A - sigma_j B on the level's CSR pattern of (a, b) pairs, dense, np x
+// np (rows and columns from n on: the identity)
+__global__ void k_dense_shift(int n, int np, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
                               const float2 *__restrict__ ab, PoleSet<float> ps, float2 *__restrict__ M) {
     const int row = blockIdx.x;
     const int j = blockIdx.y;
-    float2 *Mr = M + ((int64_t)j * n + row) * n;
-    for (int c = threadIdx.x; c < n; c += blockDim.x) Mr[c] = make_float2(0.f, 0.f);
+    float2 *Mr = M + ((int64_t)j * np + row) * np;
+    for (int c = threadIdx.x; c < np; c += blockDim.x) Mr[c] = make_float2(row >= n && c == row ? 1.f : 0.f, 0.f);
     __syncthreads();
+    if (row >= n) return;
     const float sr = ps.re[j], si = ps.im[j];
     for (int k = ptr[row] + threadIdx.x; k < ptr[row + 1]; k += blockDim.x) {
         const float2 w = ab[k];
@@ -48,147 +55,271 @@ __global__ void k_dense_shift(int n, int N, const int32_t *__restrict__ ptr, con
     }
 }
 
-// In-place inverse of the b x b diagonal block at (k0, k0) of each of the
-// N matrices (column-major, leading dimension n), copied out to P (b x b,
-// column-major, ld CB) -- Gauss-Jordan without pivoting in shared memory.
-// 1024 threads, thread (r, c0) owns rows r and columns c0, c0 + 16, ...: no
-// index division in the elimination loop, four entries per thread.
-__global__ void __launch_bounds__(1024) k_block_inverse(int n, int b, int k0, const float2 *__restrict__ M,
-                                                       float2 *__restrict__ P) {
-    __shared__ float2 S[CB][CB + 1];   // S[r][c]
-    __shared__ float2 rowk[CB], colk[CB];
-    const int j = blockIdx.x;
-    const float2 *Mj = M + (int64_t)j * n * n;
-    const int r = threadIdx.x & (CB - 1), c0 = threadIdx.x >> 6;   // c0 in [0, 16)
-    for (int c = c0; c < b; c += 16)
-        if (r < b) S[r][c] = Mj[(int64_t)(k0 + c) * n + k0 + r];
-    __syncthreads();
-    for (int k = 0; k < b; ++k) {
-        if (threadIdx.x < b) {
-            rowk[threadIdx.x] = S[k][threadIdx.x];
-            colk[threadIdx.x] = S[threadIdx.x][k];
-        }
-        __syncthreads();
-        const float2 p = rowk[k];
-        const float den = p.x * p.x + p.y * p.y;
-        const float2 pinv = make_float2(p.x / den, -p.y / den);
-        if (r < b) {
-            const float2 cr = colk[r];
-            for (int c = c0; c < b; c += 16) {
-                float2 v;
-                if (r == k && c == k) {
-                    v = pinv;
-                } else if (r == k) {
-                    v = cmul(rowk[c], pinv);
-                } else if (c == k) {
-                    v = cmul(cr, pinv);
-                    v.x = -v.x;
-                    v.y = -v.y;
-                } else {
-                    v = csub(S[r][c], cmul(cr, cmul(rowk[c], pinv)));
+// Thread (ty, tx) of 16 x 16 holds of a CB x CB tile the rows 4 ty .. 4 ty+3
+// and the columns 2 tx, 2 tx + 1, 2 tx + 32, 2 tx + 33: a row's operands are
+// one broadcast and the columns' two conflict-free 16-byte shared loads.
+__device__ __forceinline__ int tile_col(int tx, int q) { return 2 * tx + 32 * (q >> 1) + (q & 1); }
+
+// acc += A^T B over the CB rows of two staged CB x CB panels
+__device__ __forceinline__ void tile_product(const float2 (*A)[CB], const float2 (*B)[CB], int ty, int tx,
+                                             float2 (&acc)[4][4]) {
+#pragma unroll 4
+    for (int k = 0; k < CB; ++k) {
+        const float4 a01 = *reinterpret_cast<const float4 *>(&A[k][4 * ty]);
+        const float4 a23 = *reinterpret_cast<const float4 *>(&A[k][4 * ty + 2]);
+        const float4 b01 = *reinterpret_cast<const float4 *>(&B[k][2 * tx]);
+        const float4 b23 = *reinterpret_cast<const float4 *>(&B[k][2 * tx + 32]);
+        const float2 a[4] = {make_float2(a01.x, a01.y), make_float2(a01.z, a01.w), make_float2(a23.x, a23.y),
+                             make_float2(a23.z, a23.w)};
+        const float2 b[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w), make_float2(b23.x, b23.y),
+                             make_float2(b23.z, b23.w)};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[i][q] = cfma(a[i], b[q], acc[i][q]);
+    }
+}
+
+// The symmetric sweep of all CB pivots of a tile in registers: S -> -S^{-1}.
+// Per pivot the owners publish its row (= its column), one barrier.
+__device__ __forceinline__ void tile_sweep(float2 (&S)[4][4], float2 (*row)[CB], int ty, int tx) {
+    for (int k4 = 0; k4 < CB / 4; ++k4)
+#pragma unroll
+        for (int ki = 0; ki < 4; ++ki) {
+            const int k = 4 * k4 + ki;
+            float2 *rk = row[ki & 1];
+            if (ty == k4)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) rk[tile_col(tx, q)] = S[ki][q];
+            __syncthreads();
+            const float2 p = rk[k];
+            const float den = p.x * p.x + p.y * p.y;
+            const float2 pinv = make_float2(p.x / den, -p.y / den);
+            float2 w[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) w[q] = cmul(pinv, rk[tile_col(tx, q)]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 ri = rk[4 * ty + i];
+                const bool prow = ty == k4 && i == ki;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const bool pcol = tile_col(tx, q) == k;
+                    const float2 v = csub(S[i][q], cmul(ri, w[q]));
+                    const float2 c = prow ? w[q] : cmul(pinv, ri);
+                    const float2 d = make_float2(-pinv.x, -pinv.y);
+                    S[i][q] = prow && pcol ? d : (prow || pcol ? c : v);
                 }
-                S[r][c] = v;
             }
         }
+}
+
+// Sweep of the diagonal block at k0: M_KK = -P, and P beside it
+__device__ __forceinline__ void sweep_store(float2 (&S)[4][4], float2 (*row)[CB], int np, int k0, float2 *__restrict__ M,
+                                            float2 *__restrict__ P, int ty, int tx) {
+    tile_sweep(S, row, ty, tx);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = 4 * ty + i, c = tile_col(tx, q);
+            M[(int64_t)(k0 + r) * np + k0 + c] = S[i][q];
+            P[r * CB + c] = make_float2(-S[i][q].x, -S[i][q].y);
+        }
+}
+
+__global__ void __launch_bounds__(256) k_first_block(int np, float2 *__restrict__ M, float2 *__restrict__ P) {
+    __shared__ float2 row[2][CB];
+    float2 *Mj = M + (int64_t)blockIdx.x * np * np;
+    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+    float2 S[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) S[i][q] = Mj[(int64_t)(4 * ty + i) * np + tile_col(tx, q)];
+    sweep_store(S, row, np, 0, Mj, P + (int64_t)blockIdx.x * CB * CB, ty, tx);
+}
+
+// Panel of block K: the old rows M_K* (from the upper triangle: M_KJ for J >
+// K, M_JK^T for J < K) to Cp, T = P M_K* to Tp and in place of the old block.
+__global__ void __launch_bounds__(256, 3) k_sweep_panel(int np, int K, float2 *__restrict__ M,
+                                                        const float2 *__restrict__ P, float2 *__restrict__ Cp,
+                                                        float2 *__restrict__ Tp) {
+    extern __shared__ __align__(16) float2 sm[];
+    float2(*sP)[CB] = reinterpret_cast<float2(*)[CB]>(sm);
+    float2(*sC)[CB] = sP + CB;
+    const int J = (int)blockIdx.x + ((int)blockIdx.x >= K ? 1 : 0), j = blockIdx.y;
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    float2 *Mj = M + (int64_t)j * np * np;
+    float2 *C = Cp + (int64_t)j * CB * np, *T = Tp + (int64_t)j * CB * np;
+    const int k0 = K * CB, c0 = J * CB;
+    for (int e = tid; e < CB * CB; e += 256) {
+        const int r = e / CB, c = e % CB;
+        sP[r][c] = P[(int64_t)j * CB * CB + e];   // symmetric
+        // the tile is read along its rows; below the diagonal it is transposed
+        if (J > K) sC[r][c] = Mj[(int64_t)(k0 + r) * np + c0 + c];
+        else sC[c][r ^ (c & 15)] = Mj[(int64_t)(c0 + r) * np + k0 + c];   // swizzled against bank conflicts
+    }
+    __syncthreads();
+    if (J < K) {   // undo the swizzle, row by row
+        for (int r = tid >> 5; r < CB; r += 8) {
+            const int l = tid & 31;
+            const float2 v0 = sC[r][l ^ (r & 15)], v1 = sC[r][(l + 32) ^ (r & 15)];
+            __syncwarp();
+            sC[r][l] = v0;
+            sC[r][l + 32] = v1;
+        }
         __syncthreads();
     }
-    float2 *Pj = P + (int64_t)j * CB * CB;
-    for (int c = c0; c < b; c += 16)
-        if (r < b) Pj[c * CB + r] = S[r][c];
+    for (int e = tid; e < CB * CB; e += 256) C[(int64_t)(e / CB) * np + c0 + e % CB] = sC[e / CB][e % CB];
+    float2 acc[4][4] = {};
+    tile_product(sP, sC, ty, tx, acc);   // P^T = P
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = 4 * ty + i, c = tile_col(tx, q);
+            T[(int64_t)r * np + c0 + c] = acc[i][q];
+            if (J > K) Mj[(int64_t)(k0 + r) * np + c0 + c] = acc[i][q];
+            else Mj[(int64_t)(c0 + c) * np + k0 + r] = acc[i][q];
+        }
 }
 
-// dst(r, c) = scale * src(r, c) for an rows x cols column-major block of
-// each of N matrices
-__global__ void k_copy_block(int N, int rows, int cols, const float2 *__restrict__ src, int64_t lds, int64_t ss,
-                             float2 *__restrict__ dst, int64_t ldd, int64_t sd, float scale) {
-    const int64_t tot = (int64_t)rows * cols;
+// M_IJ -= Cp_I^T T_J for the tiles I <= J off block K; the first CTA of each
+// matrix takes the next diagonal block and sweeps it.
+__global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, float2 *__restrict__ M,
+                                                         float2 *__restrict__ P, const float2 *__restrict__ Cp,
+                                                         const float2 *__restrict__ Tp) {
+    extern __shared__ __align__(16) float2 sm[];
+    float2(*sA)[CB] = reinterpret_cast<float2(*)[CB]>(sm);
+    float2(*sB)[CB] = sA + CB;
     const int j = blockIdx.y;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(e % rows), c = (int)(e / rows);
-        const float2 v = src[j * ss + (int64_t)c * lds + r];
-        dst[j * sd + (int64_t)c * ldd + r] = make_float2(scale * v.x, scale * v.y);
+    // tile t of the upper triangle of the nb - 1 blocks other than K
+    const bool next = K + 1 < nb;
+    int I, J;
+    {
+        int t = blockIdx.x;
+        const int q = nb - 1;
+        // the next diagonal block (position K among the others) comes first
+        const int td = next ? K * q - K * (K - 1) / 2 : -1;
+        if (next) t = t == 0 ? td : (t <= td ? t - 1 : t);
+        int i = 0, rem = t;
+        while (rem >= q - i) {
+            rem -= q - i;
+            ++i;
+        }
+        I = i;
+        J = i + rem;
+        if (I >= K) ++I;
+        if (J >= K) ++J;
+    }
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    float2 *Mj = M + (int64_t)j * np * np;
+    const float2 *C = Cp + (int64_t)j * CB * np + I * CB, *T = Tp + (int64_t)j * CB * np + J * CB;
+    float2 *D = Mj + (int64_t)I * CB * np + J * CB;
+    float2 m[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 v = *reinterpret_cast<const float4 *>(D + (int64_t)(4 * ty + i) * np + 2 * tx + 32 * h);
+            m[i][2 * h] = make_float2(v.x, v.y);
+            m[i][2 * h + 1] = make_float2(v.z, v.w);
+        }
+    for (int e = tid; e < CB * CB / 2; e += 256) {
+        const int r = e / (CB / 2), c = e % (CB / 2) * 2;
+        *reinterpret_cast<float4 *>(&sA[r][c]) = *reinterpret_cast<const float4 *>(C + (int64_t)r * np + c);
+        float4 v = *reinterpret_cast<const float4 *>(T + (int64_t)r * np + c);
+        *reinterpret_cast<float4 *>(&sB[r][c]) = make_float4(-v.x, -v.y, -v.z, -v.w);
+    }
+    __syncthreads();
+    tile_product(sA, sB, ty, tx, m);
+    if (next && blockIdx.x == 0) {
+        __syncthreads();   // the panels' shared memory holds the pivot rows from here
+        sweep_store(m, sA, np, (K + 1) * CB, Mj, P + (int64_t)j * CB * CB, ty, tx);
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            *reinterpret_cast<float4 *>(D + (int64_t)(4 * ty + i) * np + 2 * tx + 32 * h) =
+                make_float4(m[i][2 * h].x, m[i][2 * h].y, m[i][2 * h + 1].x, m[i][2 * h + 1].y);
+}
+
+// Minv = -M from M's upper triangle (n x n, symmetric), 32 x 32 tiles
+__global__ void __launch_bounds__(256) k_sweep_finish(int n, int np, const float2 *__restrict__ M,
+                                                      float2 *__restrict__ Minv) {
+    __shared__ float2 s[32][33];
+    if (blockIdx.x < blockIdx.y) return;
+    const float2 *Mj = M + (int64_t)blockIdx.z * np * np;
+    float2 *O = Minv + (int64_t)blockIdx.z * n * n;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+#pragma unroll
+    for (int i = ty; i < 32; i += 8) {
+        const int r = r0 + i, c = c0 + tx;
+        // inside a diagonal block both halves are swept; its upper one counts
+        const float2 v = r <= c ? Mj[(int64_t)r * np + c] : Mj[(int64_t)c * np + r];
+        s[i][tx] = make_float2(-v.x, -v.y);
+        if (r < n && c < n) O[(int64_t)r * n + c] = s[i][tx];
+    }
+    if (blockIdx.x == blockIdx.y) return;
+    __syncthreads();
+#pragma unroll
+    for (int i = ty; i < 32; i += 8) {
+        const int r = c0 + i, c = r0 + tx;
+        if (r < n && c < n) O[(int64_t)r * n + c] = s[tx][i];
     }
 }
 
-// M <- (M + M^T) / 2 for each matrix (upper triangle pairs)
-__global__ void k_symmetrize_c(int n, float2 *__restrict__ M) {
-    const int j = blockIdx.y;
-    float2 *Mj = M + (int64_t)j * n * n;
-    const int64_t tot = (int64_t)n * n;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(e / n), c = (int)(e % n);
-        if (c <= r) continue;
-        const float2 a = Mj[(int64_t)r * n + c], b = Mj[(int64_t)c * n + r];
-        const float2 m = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y + b.y));
-        Mj[(int64_t)r * n + c] = m;
-        Mj[(int64_t)c * n + r] = m;
-    }
+constexpr size_t SWEEP_SMEM = 2 * CB * CB * sizeof(float2);
+
+// The kernels' shared-memory limit, raised once per device
+void raise_sweep_smem() {
+    static std::once_flag once[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::call_once(once[dev < 0 || dev >= 64 ? 0 : dev], [] {
+        cudaFuncSetAttribute(k_sweep_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SWEEP_SMEM);
+        cudaFuncSetAttribute(k_sweep_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SWEEP_SMEM);
+    });
 }
 
 }  // namespace
 
 size_t coarse_inverse_work_bytes(int n, int N) {
-    return (2 * (size_t)N * n * CB + (size_t)N * CB * CB) * sizeof(float2) + 1024;
+    const size_t np = (size_t)(n + CB - 1) / CB * CB;
+    return (size_t)N * (np * np + 2 * np * CB + CB * CB) * sizeof(float2);
 }
 
-int coarse_inverse(Ctx &ctx, void *cublas, int n, const PoleSet<float> &ps, const int32_t *ptr, const int32_t *col,
-                   const float2 *ab, float2 *Minv, void *work) {
-    cublasHandle_t hb = reinterpret_cast<cublasHandle_t>(cublas);
-    const int N = ps.N;
-    const int64_t nn = (int64_t)n * n;
-    float2 *T = reinterpret_cast<float2 *>(work);          // N x (CB x n), ld CB
-    float2 *C = T + (size_t)N * n * CB;                      // N x (n x CB), ld n
-    float2 *P = C + (size_t)N * n * CB;                      // N x (CB x CB), ld CB
-    cublasStatus_t st = cublasSetStream(hb, ctx.stream);
-    if (st != CUBLAS_STATUS_SUCCESS) return (int)st;
-    ctx.before(KC_MG_COARSE, (double)N * nn * 8, 0);
-    k_dense_shift<<<dim3(n, N), 128, 0, ctx.stream>>>(n, N, ptr, col, ab, ps, Minv);
+void coarse_inverse(Ctx &ctx, int n, const PoleSet<float> &ps, const int32_t *ptr, const int32_t *col,
+                    const float2 *ab, float2 *Minv, void *work) {
+    const int N = ps.N, nb = (n + CB - 1) / CB, np = nb * CB;
+    float2 *M = reinterpret_cast<float2 *>(work);             // N x (np x np), block upper triangle
+    float2 *Cp = M + (size_t)N * np * np;                     // N x (CB x np)
+    float2 *Tp = Cp + (size_t)N * np * CB;                    // N x (CB x np)
+    float2 *P = Tp + (size_t)N * np * CB;                     // N x (CB x CB)
+    raise_sweep_smem();
+    ctx.before(KC_MG_COARSE, 8.0 * N * np * np, 0);
+    k_dense_shift<<<dim3(np, N), 128, 0, ctx.stream>>>(n, np, ptr, col, ab, ps, M);
     ctx.after();
-    const cuComplex one = make_cuComplex(1.f, 0.f), mone = make_cuComplex(-1.f, 0.f),
-                    zero = make_cuComplex(0.f, 0.f);
-    const unsigned cgrid = (unsigned)std::min<int64_t>(((int64_t)n * CB + 255) / 256, 4096);
-    for (int k0 = 0; k0 < n; k0 += CB) {
-        const int b = std::min(CB, n - k0);
-        ctx.before(KC_MG_COARSE, (double)N * b * b * 16, 8.0 * N * b * b * b);
-        k_block_inverse<<<N, 1024, 0, ctx.stream>>>(n, b, k0, Minv, P);
-        ctx.after();
-        // T = P M_K*  (b x n)
-        ctx.before(KC_MG_COARSE, (double)N * b * n * 16, 8.0 * N * b * b * n);
-        st = cublasCgemmStridedBatched(hb, CUBLAS_OP_N, CUBLAS_OP_N, b, n, b, &one, P, CB, (int64_t)CB * CB,
-                                       Minv + k0, n, nn, &zero, T, CB, (int64_t)CB * n, N);
-        ctx.after();
-        if (st != CUBLAS_STATUS_SUCCESS) return (int)st;
-        // C = M_*K  (n x b)
-        ctx.before(KC_MG_COARSE, (double)N * b * n * 16, 0);
-        k_copy_block<<<dim3(cgrid, N), 256, 0, ctx.stream>>>(N, n, b, Minv + (int64_t)k0 * n, n, nn, C, n,
-                                                             (int64_t)n * CB, 1.f);
-        ctx.after();
-        // M -= C T
-        ctx.before(KC_MG_COARSE, (double)N * nn * 16, 8.0 * N * b * (double)nn);
-        st = cublasCgemmStridedBatched(hb, CUBLAS_OP_N, CUBLAS_OP_N, n, n, b, &mone, C, n, (int64_t)n * CB, T, CB,
-                                       (int64_t)CB * n, &one, Minv, n, nn, N);
-        ctx.after();
-        if (st != CUBLAS_STATUS_SUCCESS) return (int)st;
-        // M_K* = T
-        ctx.before(KC_MG_COARSE, (double)N * b * n * 16, 0);
-        k_copy_block<<<dim3(cgrid, N), 256, 0, ctx.stream>>>(N, b, n, T, CB, (int64_t)CB * n, Minv + k0, n, nn, 1.f);
-        ctx.after();
-        // M_*K = -C P
-        ctx.before(KC_MG_COARSE, (double)N * b * n * 16, 8.0 * N * b * b * n);
-        st = cublasCgemmStridedBatched(hb, CUBLAS_OP_N, CUBLAS_OP_N, n, b, b, &mone, C, n, (int64_t)n * CB, P, CB,
-                                       (int64_t)CB * CB, &zero, Minv + (int64_t)k0 * n, n, nn, N);
-        ctx.after();
-        if (st != CUBLAS_STATUS_SUCCESS) return (int)st;
-        // M_KK = P
-        ctx.before(KC_MG_COARSE, (double)N * b * b * 16, 0);
-        k_copy_block<<<dim3(1, N), 256, 0, ctx.stream>>>(N, b, b, P, CB, (int64_t)CB * CB, Minv + (int64_t)k0 * n + k0,
-                                                         n, nn, 1.f);
-        ctx.after();
-    }
-    ctx.before(KC_MG_COARSE, (double)N * nn * 16, 0);
-    k_symmetrize_c<<<dim3((unsigned)std::min<int64_t>((nn + 255) / 256, 4096), N), 256, 0, ctx.stream>>>(n, Minv);
+    ctx.before(KC_MG_COARSE, 16.0 * N * CB * CB, 8.0 * N * CB * CB * CB);
+    k_first_block<<<N, 256, 0, ctx.stream>>>(np, M, P);
     ctx.after();
-    return (int)CUBLAS_STATUS_SUCCESS;
+    if (nb > 1)
+        for (int K = 0; K < nb; ++K) {
+            ctx.before(KC_MG_COARSE, 24.0 * N * CB * np, 8.0 * N * CB * CB * (double)np);
+            k_sweep_panel<<<dim3(nb - 1, N), 256, SWEEP_SMEM, ctx.stream>>>(np, K, M, P, Cp, Tp);
+            ctx.after();
+            ctx.before(KC_MG_COARSE, 8.0 * N * np * (double)np, 4.0 * N * CB * (double)np * np);
+            k_sweep_update<<<dim3((nb - 1) * nb / 2, N), 256, SWEEP_SMEM, ctx.stream>>>(np, nb, K, M, P, Cp, Tp);
+            ctx.after();
+        }
+    ctx.before(KC_MG_COARSE, 12.0 * N * n * (double)n, 0);
+    const unsigned g = (unsigned)((n + 31) / 32);
+    k_sweep_finish<<<dim3(g, g, N), 256, 0, ctx.stream>>>(n, np, M, Minv);
+    ctx.after();
 }
 
 int coarse_inverse_apply(Ctx &ctx, void *cublas, const KrylovDims &d, int n, const float2 *Minv, const float2 *R,

@@ -227,11 +227,11 @@ void mg_dinv(Ctx &ctx, MgSolve<T> &mg, const PoleSet<T> &ps);
 
 // ---------------------------------------------------------------- coarse.cu
 // Dense shifted inverses of one level: Minv_j = (A - sigma_j B)^{-1}, j < N,
-// n x n each (symmetric), from the level's CSR pairs, by blocked Gauss-Jordan
-// (GEMMs through cuBLAS handle `cublas`); work: coarse_inverse_work_bytes.
+// n x n each (symmetric), from the level's CSR pairs, by a blocked symmetric
+// sweep; work: coarse_inverse_work_bytes.
 size_t coarse_inverse_work_bytes(int n, int N);
-int coarse_inverse(Ctx &ctx, void *cublas, int n, const PoleSet<float> &ps, const int32_t *ptr, const int32_t *col,
-                   const float2 *ab, float2 *Minv, void *work);
+void coarse_inverse(Ctx &ctx, int n, const PoleSet<float> &ps, const int32_t *ptr, const int32_t *col,
+                    const float2 *ab, float2 *Minv, void *work);
 // Z_j = Minv_j R_j for every pole's columns of the level block (layout of the state)
 int coarse_inverse_apply(Ctx &ctx, void *cublas, const KrylovDims &d, int n, const float2 *Minv, const float2 *R,
                          float2 *Z);
