@@ -1495,14 +1495,15 @@ slrf_status krylov_solve(slrf_handle *h, const slrf_filter *f, int m, const doub
 
 // G = X^T Y with the handle's Gram method (Ozaki digits on the tcgen05 or the
 // mma.sync tensor path, or FP64) (symmetric: Y = B X with B symmetric, so only
-// the upper tiles are computed)
+// the upper tiles are computed; same_x: X is the last call's, its digits are
+// kept)
 slrf_status gram(slrf_handle *h, int64_t n, int m, const double *X, int64_t ldx, const double *Y, int64_t ldy,
-                 double *G, bool symmetric = false) {
+                 double *G, bool symmetric = false, bool same_x = false) {
     Ctx &ctx = h->ctx;
     if (h->opts.gram_ozaki) {
         CKS(ensure(h, h->rOz, ozaki_gram_work_bytes(n, m, ctx.sm_count)));
         ozaki_gram(ctx, n, m, X, ldx, Y, ldy, G, h->rOz.p, symmetric,
-                   h->opts.gram_ozaki == 2 ? h->d_pin + 1 : nullptr);
+                   h->opts.gram_ozaki == 2 ? h->d_pin + 1 : nullptr, same_x);
         return SLRF_OK;
     }
     const int split = gram_split(ctx, m, n);
@@ -1600,7 +1601,7 @@ slrf_status rr_step(slrf_handle *h, int m, const double *U, int64_t ldu, double 
     small_chol_inv(ctx, m, G, G, T2, st + 1, nullptr, 0.0);
     // projected A: A_hat = T2^T (Q1^T A Q1) T2
     spmm_real(ctx, h->A, m, Q1, m, W1, m, nullptr, 0);
-    CKS(gram(h, n, m, Q1, m, W1, m, Ah1, true));
+    CKS(gram(h, n, m, Q1, m, W1, m, Ah1, true, true));   // Q1's digits are those of the last Gram
     dgemm(ctx, 0, 0, m, m, m, Ah1, m, T2, m, 0.0, R1, m, 1, nullptr, KC_SMALL_DENSE);
     dgemm(ctx, 1, 0, m, m, m, T2, m, R1, m, 0.0, Ah, m, 1, nullptr, KC_SMALL_DENSE, true);
     ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);

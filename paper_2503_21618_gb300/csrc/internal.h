@@ -332,8 +332,10 @@ size_t ozaki_gram_work_bytes(int64_t n, int m, int sm_count);
 // the tiles on and above the diagonal are computed and mirrored.
 // tc_err != nullptr selects the tensor-core (tcgen05, bf16 digits) form; it
 // receives a nonzero code if one of that kernel's bounded waits gives up.
+// same_x: X, n, m and work are those of the last call and X's digits are still
+// in work (tensor-core form only).
 void ozaki_gram(Ctx &ctx, int64_t n, int m, const double *X, int64_t ldx, const double *Y, int64_t ldy, double *G,
-                void *work, bool symmetric = false, int32_t *tc_err = nullptr);
+                void *work, bool symmetric = false, int32_t *tc_err = nullptr, bool same_x = false);
 // C = (A diag(cs)) B, A n x k, B k x m, C n x m (row-major, leading dims),
 // cs = nullptr for no column scaling; FP64-accurate from exact digit
 // products.  tc_err != nullptr (and k <= 512) selects the tcgen05 form (bf16
