@@ -1880,12 +1880,7 @@ slrf_status precond_apply_t(slrf_handle *h, const slrf_filter *f, KrylovDims &d,
     kb.dinv = as<cplx<T>>(h->kDinv);
     kb.s.part = as<T>(h->kPart);
     kb.s.flag = as<int32_t>(h->kFlags);
-    std::vector<int32_t> flags(W);
-    for (int col = 0; col < W; ++col) flags[col] = (col % d.Lp) < d.m ? 1 : 0;
-    std::vector<cplx<T>> sg(SLRF_MAX_POLES);
-    for (int j = 0; j < N; ++j) sg[j] = mk((T)f->sigma_re[j], (T)f->sigma_im[j]);
-    CK(cudaMemcpyAsync(kb.s.flag, flags.data(), W * sizeof(int32_t), cudaMemcpyHostToDevice, ctx.stream));
-    CK(cudaMemcpyAsync(h->kSig.p, sg.data(), N * sizeof(cplx<T>), cudaMemcpyHostToDevice, ctx.stream));
+    krylov_set_columns<T>(ctx, d, make_poleset<T>(f), kb.s.flag, as<cplx<T>>(h->kSig));
     const cplx<T> *sig = as<cplx<T>>(h->kSig);
     h->inv_key.clear();
     h->ctx.reset_counters();
@@ -1913,7 +1908,7 @@ slrf_status precond_apply_t(slrf_handle *h, const slrf_filter *f, KrylovDims &d,
     }
     if (mu) krylov_reduce_mu<T>(ctx, d, kb.s.part, kb.gy, mu);
     if (mg_levels) *mg_levels = use_mg ? mg_of<T>(h).nlev : 0;
-    CK(cudaStreamSynchronize(ctx.stream));   // the host vectors above are pageable
+    CK(cudaStreamSynchronize(ctx.stream));
     CK(cudaGetLastError());
     return SLRF_OK;
 }
@@ -2550,25 +2545,18 @@ slrf_status slrf_shifted_spmm(slrf_handle *h, const slrf_filter *f, int32_t prec
     CKS(ensure(h, h->kPart, (size_t)gy * W * 4 * esz));
     CKS(ensure(h, h->kSig, SLRF_MAX_POLES * 2 * esz));
     CKS(ensure(h, h->kFlags, (size_t)W * 2 * sizeof(int32_t) + 64));
-    std::vector<int32_t> flags(W);
-    for (int col = 0; col < W; ++col) flags[col] = (col % ldp) < m ? 1 : 0;
-    CK(cudaMemcpyAsync(h->kFlags.p, flags.data(), W * 4, cudaMemcpyHostToDevice, ctx.stream));
     h->ctx.reset_counters();
-    CK(cudaStreamSynchronize(ctx.stream));
     *(volatile int32_t *)(h->h_pin + 1) = 0;
+    int32_t *flag = as<int32_t>(h->kFlags);
     if (prec == SLRF_PREC_MIXED) {
-        std::vector<float2> sg(d.N);
-        for (int j = 0; j < d.N; ++j) sg[j] = make_float2((float)f->sigma_re[j], (float)f->sigma_im[j]);
-        CK(cudaMemcpyAsync(h->kSig.p, sg.data(), d.N * sizeof(float2), cudaMemcpyHostToDevice, ctx.stream));
-        krylov_spmm<float>(ctx, d, h->A, as<float2>(h->kSig), (const float2 *)P, (float2 *)Q, as<int32_t>(h->kFlags),
-                           as<float>(h->kPart), gy);
+        krylov_set_columns<float>(ctx, d, make_poleset<float>(f), flag, as<float2>(h->kSig));
+        krylov_spmm<float>(ctx, d, h->A, as<float2>(h->kSig), (const float2 *)P, (float2 *)Q, flag, as<float>(h->kPart),
+                           gy);
         if (mu) krylov_reduce_mu<float>(ctx, d, as<float>(h->kPart), gy, (float2 *)mu);
     } else if (prec == SLRF_PREC_FP64) {
-        std::vector<double2> sg(d.N);
-        for (int j = 0; j < d.N; ++j) sg[j] = make_double2(f->sigma_re[j], f->sigma_im[j]);
-        CK(cudaMemcpyAsync(h->kSig.p, sg.data(), d.N * sizeof(double2), cudaMemcpyHostToDevice, ctx.stream));
-        krylov_spmm<double>(ctx, d, h->A, as<double2>(h->kSig), (const double2 *)P, (double2 *)Q,
-                            as<int32_t>(h->kFlags), as<double>(h->kPart), gy);
+        krylov_set_columns<double>(ctx, d, make_poleset<double>(f), flag, as<double2>(h->kSig));
+        krylov_spmm<double>(ctx, d, h->A, as<double2>(h->kSig), (const double2 *)P, (double2 *)Q, flag,
+                            as<double>(h->kPart), gy);
         if (mu) krylov_reduce_mu<double>(ctx, d, as<double>(h->kPart), gy, (double2 *)mu);
     } else {
         return SLRF_EINVAL;

@@ -129,6 +129,11 @@ int krylov_row_groups(const Ctx &ctx, const KrylovDims &d, int prec_fp32);
 template <typename T>
 void krylov_dinv(Ctx &ctx, const DevPencil &A, const PoleSet<T> &ps, int precond, cplx<T> *dinv);
 
+// flag = 1 for the columns c < m of every pole, else 0; sig = the poles
+// (written by a kernel: the step calls upload nothing and do not wait for it)
+template <typename T>
+void krylov_set_columns(Ctx &ctx, const KrylovDims &d, const PoleSet<T> &ps, int32_t *flag, cplx<T> *sig);
+
 // r = p = z = M^{-1} b from a real block shared by all poles (rhs: n x m, ld)
 // or, if rhs_c != nullptr, a complex block per pole (layout of the state).
 template <typename T>

@@ -1126,6 +1126,14 @@ __global__ void k_count_active(int W, const int32_t *__restrict__ flag, int32_t 
     if (threadIdx.x == 0) *count = tot;
 }
 
+// Flags of a block whose m columns of every pole are all active, and the poles
+template <typename T>
+__global__ void k_set_columns(int W, int Lp, int m, PoleSet<T> ps, int32_t *__restrict__ flag, cplx<T> *__restrict__ sig) {
+    const int col = blockIdx.x * blockDim.x + threadIdx.x;
+    if (col < W) flag[col] = col % Lp < m ? 1 : 0;
+    if (col < ps.N) sig[col] = mk(ps.re[col], ps.im[col]);
+}
+
 template <typename T>
 __global__ void k_reduce_mu(int W, int gy, const T *__restrict__ part, cplx<T> *__restrict__ mu, int Lp, int m) {
     const int col = blockIdx.x;
@@ -1242,6 +1250,14 @@ void krylov_spmm(Ctx &ctx, const KrylovDims &d, const DevPencil &A, const cplx<T
 }
 
 template <typename T>
+void krylov_set_columns(Ctx &ctx, const KrylovDims &d, const PoleSet<T> &ps, int32_t *flag, cplx<T> *sig) {
+    const int W = d.W();
+    ctx.before(KC_OTHER, 4.0 * W, 0);
+    k_set_columns<T><<<(W + 127) / 128, 128, 0, ctx.stream>>>(W, d.Lp, d.m, ps, flag, sig);
+    ctx.after();
+}
+
+template <typename T>
 void krylov_reduce_alpha(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb) {
     const int W = d.W();
     ctx.before(KC_KRYLOV_REDUCE, (double)kb.gy * W * 4 * sizeof(T), 0);
@@ -1331,6 +1347,7 @@ void krylov_reduce_mu(Ctx &ctx, const KrylovDims &d, const T *part, int gy, cplx
     template void krylov_reduce_init<T>(Ctx &, const KrylovDims &, KrylovBuffers<T> &);                       \
     template void krylov_spmm<T>(Ctx &, const KrylovDims &, const DevPencil &, const cplx<T> *,               \
                                  const cplx<T> *, cplx<T> *, const int32_t *, T *, int);                       \
+    template void krylov_set_columns<T>(Ctx &, const KrylovDims &, const PoleSet<T> &, int32_t *, cplx<T> *);  \
     template void krylov_reduce_alpha<T>(Ctx &, const KrylovDims &, KrylovBuffers<T> &);                      \
     template void krylov_update<T>(Ctx &, const KrylovDims &, KrylovBuffers<T> &);                            \
     template void krylov_reduce_beta<T>(Ctx &, const KrylovDims &, KrylovBuffers<T> &, double, int);          \
