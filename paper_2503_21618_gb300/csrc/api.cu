@@ -800,6 +800,10 @@ slrf_status mg_upload(slrf_handle *h, const HostHierarchy &H, const MgStaged &S,
             L0.ab = reinterpret_cast<const cplx<T> *>(A.rg_rows > 1 ? (const void *)A.rg_ab32 : (const void *)A.ab32);
         else
             L0.ab = reinterpret_cast<const cplx<T> *>(A.rg_rows > 1 ? (const void *)A.rg_ab64 : (const void *)A.ab64);
+        L0.row_nnz = A.nnz;
+        L0.row_ptr = A.rowptr;
+        L0.row_col = A.col;
+        L0.row_ab = reinterpret_cast<const cplx<T> *>(sizeof(T) == 4 ? (const void *)A.ab32 : (const void *)A.ab64);
         L0.diag_a = A.diag_a;
         L0.diag_b = A.diag_b;
         for (int l = 0; l < nlev; ++l) {

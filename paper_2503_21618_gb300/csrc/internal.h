@@ -192,6 +192,10 @@ template <typename T> struct MgLevel {
     const int32_t *gptr = nullptr, *gcol = nullptr;
     const cplx<T> *ab = nullptr;              // R (a, b) pairs per union entry
     const double *diag_a = nullptr, *diag_b = nullptr;
+    // level 0: plain rows (R = 1) of the same pencil, for the FP64 cycle
+    int64_t row_nnz = 0;
+    const int32_t *row_ptr = nullptr, *row_col = nullptr;
+    const cplx<T> *row_ab = nullptr;
     int64_t p_nnz = 0, r_nnz = 0;
     const int32_t *pptr = nullptr, *pcol = nullptr, *rptr = nullptr, *rcol = nullptr;
     const T *pval = nullptr, *rval = nullptr;

@@ -21,7 +21,10 @@
 //   z  = D (2 r - M y - F e),  r^T z        k_mg_sspmm<UP>    (fine row groups)
 // with y = D r formed once (fused into the Krylov update that produces r).
 // (P^T (I - M D) = -((M - D^{-1}) P)^T D and (I - D M) P = -D F.)  The fine
-// level is read twice and written once per cycle.
+// level is read twice and written once per cycle.  The FP64 cycle is bound by
+// the FMA pipe instead and takes the second end unfolded, z1 = y + P e in
+// place and z = z1 + D (r - M z1) on plain rows: F has about six entries per
+// row where P has two, and the row groups pad a third of both.
 // Coarser levels run nu sweeps on each side and gamma coarse visits
 // (gamma = 2: W-cycle) with materialised iterates.
 #include <cuda_runtime.h>
@@ -134,9 +137,10 @@ __device__ __forceinline__ void seg_accum(int e0, int e1, const int32_t *__restr
 // ---------------------------------------------------------------------------
 // 40 registers, 6 resident CTAs per SM: measured on the 2D bench, the finest
 // UP product of row groups runs faster there (282 us per launch, with some
-// spills) than at 64 registers and 4 CTAs without spills (323 us).
+// spills) than at 64 registers and 4 CTAs without spills (323 us).  FP64 is
+// bound by its FMA pipe and needs fewer warps: 4 CTAs.
 template <typename T, int VC, int R, int MODE>
-__global__ void __launch_bounds__(32 * TY, 6)
+__global__ void __launch_bounds__(32 * TY, sizeof(T) == 4 ? 6 : 4)
 k_mg_sspmm(int n, int W, int Lp, int N, int ngroups, const int32_t *__restrict__ gptr,
            const int32_t *__restrict__ ucol, const cplx<T> *__restrict__ uab, const cplx<T> *__restrict__ sig,
            const cplx<T> *__restrict__ dinv, const cplx<T> *__restrict__ X, const cplx<T> *__restrict__ Rv,
@@ -651,9 +655,11 @@ void mg_dinv(Ctx &ctx, MgSolve<T> &mg, const PoleSet<T> &ps) {
     }
     MgLevel<T> &L0 = mg.lv[0];
     if (mg.nlev > 1) {
-        const int64_t ns = L0.fu_nnz * L0.R + L0.fd_nnz;
+        // the FP64 cycle uses the down pairs (the last) only
+        const int64_t s0 = sizeof(T) == 8 ? L0.fu_nnz * L0.R : 0, ns = L0.fu_nnz * L0.R + L0.fd_nnz - s0;
         ctx.before(KC_KRYLOV_INIT, (double)ns * (32 + sizeof(cplx<T>)), 0);
-        k_mg_fold<T><<<(unsigned)((ns + 255) / 256), 256, 0, ctx.stream>>>(ns, L0.f_q, L0.rho / mg.omega, L0.f_ab);
+        k_mg_fold<T><<<(unsigned)((ns + 255) / 256), 256, 0, ctx.stream>>>(ns, L0.f_q + 2 * s0, L0.rho / mg.omega,
+                                                                          L0.f_ab + s0);
         ctx.after();
     }
 }
@@ -688,9 +694,17 @@ void mg_apply(Ctx &ctx, const KrylovDims &d, MgSolve<T> &mg, const cplx<T> *sig,
     launch_sspmm<T, MG_DOWN>(ctx, d, KC_MG_FINE, Lc.n, 1, Lc.n, L.fd_ptr, L.fd_col, L.f_ab + L.fu_nnz * L.R,
                              L.fd_nnz, L.n, gyd, sig, L.dinv, Y0, nullptr, Lc.r, flag, nullptr);
     cplx<T> *e = cycle<T>(ctx, d, mg, 1, gy, sig, flag);
-    // z = D (2 r - M y - F e), r^T z
-    launch_sspmm<T, MG_UP>(ctx, d, KC_MG_FINE, L.n, L.R, L.ngroups, L.gptr, L.gcol, L.ab, L.nnz_union, L.n, gy, sig,
-                           L.dinv, Y0, R0, Z0, flag, part, L.fu_ptr, L.fu_col, L.f_ab, L.fu_nnz, e, Lc.n);
+    if constexpr (sizeof(T) == 8) {
+        // y is scratch (the caller's T0, or the Krylov update's own block)
+        cplx<T> *z1 = const_cast<cplx<T> *>(Y0);
+        launch_xfer<T, MG_PROLONG_ADD>(ctx, d, L.n, Lc.n, L.p_nnz, L.pptr, L.pcol, L.pval, gy, e, z1, flag);
+        launch_sspmm<T, MG_SMOOTH>(ctx, d, KC_MG_FINE, L.n, 1, L.n, L.row_ptr, L.row_col, L.row_ab, L.row_nnz, L.n, gy,
+                                   sig, L.dinv, z1, R0, Z0, flag, part);
+    } else {
+        // z = D (2 r - M y - F e), r^T z
+        launch_sspmm<T, MG_UP>(ctx, d, KC_MG_FINE, L.n, L.R, L.ngroups, L.gptr, L.gcol, L.ab, L.nnz_union, L.n, gy, sig,
+                               L.dinv, Y0, R0, Z0, flag, part, L.fu_ptr, L.fu_col, L.f_ab, L.fu_nnz, e, Lc.n);
+    }
 }
 
 template <typename T>
