@@ -4,18 +4,20 @@
 // the eigenvalue problem A_hat s_i = theta_i B_hat s_i" once B_hat = I).
 //
 // FP64 arithmetic runs at a small fraction of the FP32 rate on this GPU, so
-// the eigensolver has two modes:
+// the modes of the eigensolver are:
 //  0. cyclic parallel Jacobi in FP64 (round-robin pair ordering, all m/2
 //     rotations of a round applied at once) as ONE cooperative multi-block
 //     kernel: each round is "rotations -> row phase -> grid barrier -> column
 //     phase -> grid barrier", so the O(m^3) rotation work of a sweep is spread
 //     over many SMs;
-//  1. the same Jacobi in FP32 in one block's shared memory first (fast, gives
-//     eigenvectors S0 good to ~1e-6), then S0 is re-orthonormalised in FP64
-//     (Cholesky of S0^T S0 ~ I), T = S0^T A S0 is formed by FP64 GEMMs, and the
-//     cooperative FP64 Jacobi polishes the nearly diagonal T in 2-3 sweeps
-//     (Jacobi converges quadratically; unlike first-order refinement it is
-//     robust to clustered and graded spectra).
+//  2. (default, m <= 448) the same Jacobi in FP32 in one block's shared memory
+//     (m <= 160) or in double-float on a thread-block cluster first, the
+//     vectors then refined by FP64 products (Ogita-Aishima) and groups of
+//     close eigenvalues diagonalised in FP64;
+//  1. (m <= 160) FP32 Jacobi, FP64 re-orthonormalisation (Cholesky of S0^T S0 ~
+//     I), and the cooperative FP64 Jacobi polishes the nearly diagonal T =
+//     S0^T A S0 in 2-3 sweeps (Jacobi converges quadratically; unlike
+//     first-order refinement it is robust to clustered and graded spectra).
 #include <cuda_runtime.h>
 #include <cooperative_groups.h>
 #include <float.h>
@@ -507,14 +509,361 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *__restri
 }
 
 // ---------------------------------------------------------------------------
+// Cyclic Jacobi for JMAX < m <= JDF_MAX on one thread-block cluster, in
+// double-float arithmetic (hi + lo FP32 pairs, ~46 bits).
+//
+// The FP64 Jacobi over the whole GPU (k_jacobi_coop) is bound by its grid
+// barriers and the FP64 pipe (32 ms at m = 300; this kernel 11.6).  FP32 rotations would do for
+// the accuracy, since the vectors are refined in FP64 afterwards, but the
+// eigenvectors' signs come out of the rotation path: where two diagonal
+// entries are close an FP32 rounding turns a rotation by 45 degrees the other
+// way.  In double-float the path is the FP64 one (a decision differs only
+// where the FP64 one is within ~1e-13), at ten FP32 instructions per
+// operation on a pipe eighty times as fast.
+//
+// All m/2 rotations of a round (rr_pair) are applied at once, A in the shared
+// memory of the C CTAs.  Position k of a round holds the pair (a_k, b_k).  A CTA
+// owns a contiguous range of positions and the two full rows of each; from one
+// round to the next the upper rows move down one position and the lower rows
+// up one, so per round a CTA hands one row to each neighbour (DSMEM) and the
+// rest stay where they are.  Per round:
+//   update    the 2 x 2 blocks (k, l) of the own positions k and all l, rows
+//             and columns in one pass (A is kept in full, so the columns of a
+//             block are two contiguous runs); block barrier
+//   rotations of the next round from the own rows and the diagonal, which
+//             every CTA keeps in full (updated in closed form); they go to all
+//             CTAs while the boundary rows move; one cluster barrier
+// The eigenvectors are not formed here: the rotations are logged (FP32) and
+// k_jacobi_vectors applies them to the rows of I afterwards, every row on its
+// own SM.  A rotation is skipped below rel_tol of sqrt(|a_pp a_qq|); the
+// sweeps stop once every rotation of a sweep was below sqrt(rel_tol).
+// Output: lam (FP64, unsorted), the log and *nrounds.
+// ---------------------------------------------------------------------------
+constexpr int JDF_MAX = 448;      // a CTA's rows of an 8-CTA cluster in 227 KB
+constexpr int JDF_CTAS = 8;
+constexpr int JDF_SWEEPS = 20;
+constexpr int JDF_THREADS = 512;
+
+// double-float: the rounded operations are spelled out, so that no
+// multiplication and addition of the error terms is contracted
+struct df {
+    float h, l;
+};
+__device__ __forceinline__ df df_renorm(float h, float l) {
+    const float s = __fadd_rn(h, l);
+    return {s, __fsub_rn(l, __fsub_rn(s, h))};
+}
+__device__ __forceinline__ df df_of(double x) {
+    const float h = (float)x;
+    return {h, (float)(x - (double)h)};
+}
+__device__ __forceinline__ df df_neg(df a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ df df_add(df a, df b) {
+    const float s = __fadd_rn(a.h, b.h), v = __fsub_rn(s, a.h);
+    float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, v)), __fsub_rn(b.h, v));
+    e = __fadd_rn(e, __fadd_rn(a.l, b.l));
+    return df_renorm(s, e);
+}
+__device__ __forceinline__ df df_mul(df a, df b) {
+    const float p = __fmul_rn(a.h, b.h);
+    float e = fmaf(a.h, b.h, -p);
+    e = fmaf(a.h, b.l, e);
+    e = fmaf(a.l, b.h, e);
+    return df_renorm(p, e);
+}
+// c x - s z
+__device__ __forceinline__ df df_rot(df c, df x, df s, df z) {
+    const float p = __fmul_rn(c.h, x.h), q = __fmul_rn(s.h, z.h);
+    float pl = fmaf(c.h, x.h, -p), ql = fmaf(s.h, z.h, -q);
+    pl = fmaf(c.h, x.l, pl);
+    ql = fmaf(s.h, z.l, ql);
+    pl = fmaf(c.l, x.h, pl);
+    ql = fmaf(s.l, z.h, ql);
+    const float d = __fsub_rn(p, q), v = __fsub_rn(d, p);
+    float e = __fsub_rn(__fsub_rn(p, __fsub_rn(d, v)), __fadd_rn(q, v));
+    e = __fadd_rn(e, __fsub_rn(pl, ql));
+    return df_renorm(d, e);
+}
+__device__ __forceinline__ df df_div(df a, df b) {
+    const float q = a.h / b.h;
+    const df r = df_add(a, df_neg(df_mul({q, 0.f}, b)));
+    return df_renorm(q, r.h / b.h);
+}
+__device__ __forceinline__ df df_sqrt(df a) {
+    const float y = rsqrtf(a.h), s = __fmul_rn(a.h, y);
+    const df r = df_add(a, df_neg(df_mul({s, 0.f}, {s, 0.f})));
+    return df_renorm(s, 0.5f * y * r.h);
+}
+__device__ __forceinline__ df df_rsqrt(df a) {
+    const float y = rsqrtf(a.h);
+    const df r = df_add({1.f, 0.f}, df_neg(df_mul(a, df_mul({y, 0.f}, {y, 0.f}))));
+    return df_renorm(y, 0.5f * y * r.h);
+}
+
+// index of the upper (a) and lower (b) row of position k in round r
+__device__ __forceinline__ int rr_top(int k, int r, int mp) {
+    const int x = k - 1 + r;
+    return k == 0 ? 0 : (x >= mp - 1 ? x - (mp - 1) : x) + 1;
+}
+__device__ __forceinline__ int rr_bot(int k, int r, int mp) {
+    const int x = mp - 2 - k + r;
+    return (x >= mp - 1 ? x - (mp - 1) : x) + 1;
+}
+
+struct JacobiShape {
+    int mp, npair, ld, maxcnt;
+    __host__ __device__ JacobiShape(int m, int C) {
+        mp = m + (m & 1);
+        npair = mp / 2;
+        ld = mp;   // even: rows of 8-byte pairs start on 16 bytes
+        maxcnt = (npair + C - 1) / C;
+    }
+    // rows (two free ones for arrivals), rotations and diagonal changes of two rounds, diagonal, row slots
+    __host__ __device__ size_t bytes() const {
+        return (size_t)(2 * maxcnt + 2) * ld * 8 + (size_t)npair * 48 + (size_t)ld * 8 + (size_t)maxcnt * 16;
+    }
+};
+
+__global__ void __launch_bounds__(JDF_THREADS, 1)
+k_jacobi_df(int m, const double *__restrict__ S, const double *__restrict__ fro_part, double *__restrict__ lam,
+            float2 *__restrict__ rlog, int *__restrict__ nrounds, float rel_tol) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks(), c = (int)cl.block_rank();
+    const JacobiShape sh(m, C);
+    const int mp = sh.mp, npair = sh.npair, ld = sh.ld;
+    extern __shared__ float4 jsm4[];
+    float4 *par = jsm4;                                   // [2][npair]: c, s as (hi, lo)
+    df *rows = reinterpret_cast<df *>(par + 2 * npair);
+    df *pda = rows + (size_t)(2 * sh.maxcnt + 2) * ld;    // [2][npair]: change of a_aa
+    df *diag = pda + 2 * npair;
+    int *slots = reinterpret_cast<int *>(diag + ld);      // [2][upper, lower][maxcnt]
+    __shared__ int nbfree[2][2];    // free slot of the lower / upper neighbour, by round parity
+    __shared__ int myfree[2][2];    // own free slots for an upper / a lower row, by round parity
+    __shared__ int mx[2];           // largest relative pivot of a sweep (float bits), by sweep parity
+    __shared__ int allmx[JDF_CTAS]; // the CTAs' mx of the sweep that ends
+    __shared__ float absmin;
+    __shared__ int scale;           // ||S||_F < 2^scale; A holds S 2^-scale
+    const int tid = threadIdx.x, bs = blockDim.x;
+    const int lane = tid & 31, warp = tid >> 5, nwarp = bs >> 5;
+    const int k0 = c * npair / C, k1 = (c + 1) * npair / C, cnt = k1 - k0;
+    const bool last = c == C - 1;
+    auto slot_of = [&](int par_, int low) { return slots + (par_ * 2 + low) * sh.maxcnt; };
+    cl.sync();   // every CTA runs before any writes to another's shared memory
+
+    if (warp == 0) {
+        const double f = fro_norm(fro_part);
+        if (lane == 0) {
+            scale = f > 0.0 && isfinite(f) ? ilogb(f) + 1 : 0;
+            absmin = (float)(scalbn(f, -scale) * (double)rel_tol / sqrt((double)m));
+            mx[0] = mx[1] = 0;
+            myfree[0][0] = 2 * cnt;
+            myfree[0][1] = 2 * cnt + 1;
+            if (c > 0) cl.map_shared_rank(&nbfree[0][1], c - 1)[0] = 2 * cnt + 1;   // where c - 1 sends a lower row
+            if (!last) cl.map_shared_rank(&nbfree[0][0], c + 1)[0] = 2 * cnt;       // where c + 1 sends an upper row
+        }
+    }
+    __syncthreads();
+    const double sc = scalbn(1.0, -scale);
+    // the upper rows of the CTA's positions, then the lower ones
+    for (int e = warp; e < 2 * cnt; e += nwarp) {
+        const int low = e >= cnt, k = k0 + (low ? e - cnt : e);
+        const int i = low ? rr_bot(k, 0, mp) : rr_top(k, 0, mp);
+        for (int j = lane; j < ld; j += 32)
+            rows[(size_t)e * ld + j] = i < m && j < m ? df_of(S[(int64_t)i * m + j] * sc) : df{0.f, 0.f};
+        if (lane == 0) slot_of(0, low)[k - k0] = e;
+    }
+    for (int i = tid; i < ld; i += bs) diag[i] = i < m ? df_of(S[(int64_t)i * m + i] * sc) : df{0.f, 0.f};
+    __syncthreads();
+
+    // rotation of position k (a = upper, b = lower index) from its pivot; to every CTA and the log of round g
+    auto rotation = [&](int k, int a, int b, df apq, int sweep, int64_t g, int pb) {
+        df cc = {1.f, 0.f}, ss = {0.f, 0.f}, da = {0.f, 0.f};
+        if (max(a, b) < m) {
+            const df app = diag[min(a, b)], aqq = diag[max(a, b)];
+            const float mag = sqrtf(fabsf(app.h * aqq.h));
+            if (fabsf(apq.h) > rel_tol * mag && fabsf(apq.h) > absmin) {
+                // t = sign(th) / (|th| + sqrt(1 + th^2)), th = (a_qq - a_pp) / (2 a_pq)
+                const df d = df_add(aqq, df_neg(app)), a2 = {2.f * apq.h, 2.f * apq.l};
+                const df ad = d.h < 0.f ? df_neg(d) : d, aa = a2.h < 0.f ? df_neg(a2) : a2;
+                const df h = df_sqrt(df_add(df_mul(ad, ad), df_mul(aa, aa)));
+                df t = df_div(aa, df_add(ad, h));
+                if (d.h != 0.f && (d.h > 0.f) != (apq.h > 0.f)) t = df_neg(t);
+                cc = df_rsqrt(df_add({1.f, 0.f}, df_mul(t, t)));
+                ss = df_mul(t, cc);
+                da = df_neg(df_mul(t, apq));
+                if (a > b) {
+                    ss = df_neg(ss);
+                    da = df_neg(da);
+                }
+                atomicMax(&mx[sweep & 1], __float_as_int(fabsf(apq.h) / (mag > 0.f ? mag : 1.f)));
+            }
+        }
+        const float4 v = make_float4(cc.h, cc.l, ss.h, ss.l);
+        for (int q = 0; q < C; ++q) {
+            cl.map_shared_rank(par + pb * npair + k, q)[0] = v;
+            cl.map_shared_rank(pda + pb * npair + k, q)[0] = da;
+        }
+        rlog[g * npair + k] = make_float2(cc.h, ss.h);
+    };
+    for (int j = tid; j < cnt; j += bs) {
+        const int k = k0 + j, a = rr_top(k, 0, mp), b = rr_bot(k, 0, mp);
+        rotation(k, a, b, rows[(size_t)slot_of(0, 0)[j] * ld + b], 0, 0, 0);
+    }
+    cl.sync();
+
+    int64_t g = 0;   // rounds applied
+    int cur = 0;
+    for (int sweep = 0; sweep < JDF_SWEEPS; ++sweep) {
+        for (int r = 0; r < mp - 1; ++r) {
+            const float4 *P = par + cur * npair;
+            const int *sT = slot_of(cur, 0), *sB = slot_of(cur, 1);
+            for (int l = tid; l < npair; l += bs) {
+                const df da = pda[cur * npair + l];
+                if (da.h != 0.f) {
+                    const int a = rr_top(l, r, mp), b = rr_bot(l, r, mp);
+                    diag[a] = df_add(diag[a], da);
+                    diag[b] = df_add(diag[b], df_neg(da));
+                }
+            }
+            // tasks (position j, 32 positions l), dealt to the warps
+            int j = warp, l0 = 0;
+            while (j >= cnt) {
+                j -= cnt;
+                l0 += 32;
+            }
+            while (l0 < npair) {
+                const int k = k0 + j, l = l0 + lane;
+                if (l < npair) {
+                    const float4 pk = P[k], pl = P[l];
+                    if (pk.z != 0.f || pl.z != 0.f) {
+                        df *ra = rows + (size_t)sT[j] * ld, *rb = rows + (size_t)sB[j] * ld;
+                        const int a = rr_top(l, r, mp), b = rr_bot(l, r, mp);
+                        if (l == k) {   // the pivot; the diagonal lives in diag
+                            ra[b] = {0.f, 0.f};
+                            rb[a] = {0.f, 0.f};
+                        } else {
+                            const df ck = {pk.x, pk.y}, sk = {pk.z, pk.w}, cl_ = {pl.x, pl.y}, sl = {pl.z, pl.w};
+                            const df xaa = ra[a], xab = ra[b], xba = rb[a], xbb = rb[b];
+                            const df yaa = df_rot(ck, xaa, sk, xba), yab = df_rot(ck, xab, sk, xbb);
+                            const df yba = df_rot(sk, xaa, df_neg(ck), xba), ybb = df_rot(sk, xab, df_neg(ck), xbb);
+                            ra[a] = df_rot(cl_, yaa, sl, yab);
+                            ra[b] = df_rot(sl, yaa, df_neg(cl_), yab);
+                            rb[a] = df_rot(cl_, yba, sl, ybb);
+                            rb[b] = df_rot(sl, yba, df_neg(cl_), ybb);
+                        }
+                    }
+                }
+                j += nwarp;
+                while (j >= cnt) {
+                    j -= cnt;
+                    l0 += 32;
+                }
+            }
+            __syncthreads();
+            ++g;
+            const int nxt = cur ^ 1, r1 = r + 1 == mp - 1 ? 0 : r + 1, s1 = r1 ? sweep : sweep + 1;
+            // rotations of the next round, at the positions after the move
+            for (int jj = tid; jj < cnt; jj += bs) {
+                const int k = k0 + jj, a = rr_top(k, r1, mp), b = rr_bot(k, r1, mp);
+                df apq;
+                if (c == 0 && jj == 0) apq = rows[(size_t)sT[0] * ld + b];
+                else if (jj + 1 < cnt) apq = rows[(size_t)sT[jj + 1] * ld + b];
+                else if (last) apq = rows[(size_t)sB[jj] * ld + b];
+                else apq = rows[(size_t)sB[jj - 1] * ld + a];   // the upper row is on its way: the lower one's entry
+                rotation(k, a, b, apq, s1, g, nxt);
+            }
+            // the rows' new slots
+            int *nT = slot_of(nxt, 0), *nB = slot_of(nxt, 1);
+            for (int jj = bs - 1 - tid; jj < cnt; jj += bs) {
+                nT[jj] = c == 0 && jj == 0 ? sT[0] : jj + 1 < cnt ? sT[jj + 1] : last ? sB[cnt - 1] : myfree[cur][0];
+                nB[jj] = jj > 0 ? sB[jj - 1] : c == 0 ? sT[1] : myfree[cur][1];
+            }
+            if (warp == nwarp / 2 && c > 0) {          // the lowest upper row to the lower neighbour
+                const float4 *src = reinterpret_cast<const float4 *>(rows + (size_t)sT[0] * ld);
+                float4 *dst = reinterpret_cast<float4 *>(cl.map_shared_rank(rows, c - 1) + (size_t)nbfree[cur][0] * ld);
+                for (int q = lane; q < ld / 2; q += 32) dst[q] = src[q];
+            }
+            if (warp == nwarp / 2 + 1 && !last) {      // the highest lower row to the upper neighbour
+                const float4 *src = reinterpret_cast<const float4 *>(rows + (size_t)sB[cnt - 1] * ld);
+                float4 *dst = reinterpret_cast<float4 *>(cl.map_shared_rank(rows, c + 1) + (size_t)nbfree[cur][1] * ld);
+                for (int q = lane; q < ld / 2; q += 32) dst[q] = src[q];
+            }
+            if (warp == nwarp / 2 + 2 && lane == 0) {
+                const int fT = c == 0 ? sB[cnt - 1] : sT[0], fB = last ? sT[0] : sB[cnt - 1];
+                myfree[nxt][0] = fT;
+                myfree[nxt][1] = fB;
+                if (c > 0) cl.map_shared_rank(&nbfree[nxt][1], c - 1)[0] = fB;
+                if (!last) cl.map_shared_rank(&nbfree[nxt][0], c + 1)[0] = fT;
+            }
+            if (tid == bs - 1) {
+                if (r == 0) mx[(sweep + 1) & 1] = 0;
+                if (r == mp - 2)
+                    for (int q = 0; q < C; ++q) cl.map_shared_rank(&allmx[c], q)[0] = mx[sweep & 1];
+            }
+            cl.sync();
+            cur = nxt;
+        }
+        float top = 0.f;
+        for (int q = 0; q < C; ++q) top = fmaxf(top, __int_as_float(allmx[q]));
+        if (top < sqrtf(rel_tol)) break;
+    }
+    if (c == 0) {
+        for (int i = tid; i < m; i += bs) lam[i] = scalbn((double)diag[i].h + (double)diag[i].l, scale);
+        if (tid == 0) *nrounds = (int)g;
+    }
+}
+
+// Q = the product of the logged rotations, row by row of I (one warp per row,
+// the row in shared memory; the next round's rotations are loaded ahead)
+__global__ void __launch_bounds__(32) k_jacobi_vectors(int m, const float2 *__restrict__ rlog,
+                                                       const int *__restrict__ nrounds, double *__restrict__ Q) {
+    extern __shared__ float vrow[];
+    const int mp = m + (m & 1), npair = mp / 2;
+    constexpr int U = (JDF_MAX / 2 + 31) / 32;
+    const int lane = threadIdx.x, row = blockIdx.x;
+    for (int i = lane; i < mp; i += 32) vrow[i] = i == row ? 1.f : 0.f;
+    const int n = *nrounds, nu = (npair + 31) / 32;
+    float2 w[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if (u < nu) w[u] = lane + 32 * u < npair && n > 0 ? rlog[lane + 32 * u] : make_float2(1.f, 0.f);
+    __syncwarp();
+    int r = 0;
+    for (int g = 0; g < n; ++g) {
+        float2 next[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (u < nu) {
+                const int k = lane + 32 * u;
+                next[u] = k < npair && g + 1 < n ? rlog[(int64_t)(g + 1) * npair + k] : make_float2(1.f, 0.f);
+                if (w[u].y != 0.f) {
+                    const int a = rr_top(k, r, mp), b = rr_bot(k, r, mp);
+                    const float x = vrow[a], y = vrow[b];
+                    vrow[a] = w[u].x * x - w[u].y * y;
+                    vrow[b] = w[u].y * x + w[u].x * y;
+                }
+            }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (u < nu) w[u] = next[u];
+        if (++r == mp - 1) r = 0;
+    }
+    for (int i = lane; i < m; i += 32) Q[(int64_t)row * m + i] = (double)vrow[i];
+}
+
+// ---------------------------------------------------------------------------
 // cooperative FP64 Jacobi on a global m x m matrix A (overwritten; diag = lam)
-// accumulating V <- V J.  cnt[4] (device): rotation counters of the last two
+// accumulating V <- V J.  Pairs whose |a_pq| is below eps abs_factor ||A||_F
+// are left alone.  cnt[4] (device): rotation counters of the last two
 // sweeps (0, 1) and their pre-check flags (2, 3).  All blocks
 // compute the same rotations from the same data, so no broadcast is needed.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
 k_jacobi_coop(int m, double *__restrict__ A, double *__restrict__ V, double *__restrict__ lam, int max_sweeps,
-              const double *__restrict__ normA, int *__restrict__ cnt, int32_t *__restrict__ info) {
+              const double *__restrict__ normA, double abs_factor, int *__restrict__ cnt,
+              int32_t *__restrict__ info) {
     namespace cg = cooperative_groups;
     cg::grid_group grid = cg::this_grid();
     const int mp = m + (m & 1);
@@ -524,7 +873,7 @@ k_jacobi_coop(int m, double *__restrict__ A, double *__restrict__ V, double *__r
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
     const double eps = DBL_EPSILON;
-    const double absmin = fro_norm(normA) * eps * 0.5 / (double)m;
+    const double absmin = fro_norm(normA) * eps * abs_factor;
     // cnt[2 + (sweep & 1)]: set when some pair still passes the rotation test
     if (gtid == 0) cnt[2] = cnt[3] = 0;
     grid.sync();
@@ -664,13 +1013,20 @@ __global__ void __launch_bounds__(256) k_sort_eig(int m, const double *__restric
     for (int j = lane; j < m; j += 32) Q[(int64_t)row * m + rank[j]] = S[(int64_t)row * m + j];
 }
 
-size_t small_syev_work_bytes(int m) {
+static size_t syev_base_bytes(int m) {
     const size_t mp = (size_t)(m + (m & 1));
     const size_t m2 = (size_t)m * m;
-    // A32/V32 global fallback (2 mp^2 doubles) + S0, S1, G, Y, T, V (6 m^2) + lam0, counters,
-    // component labels and sizes (2 m ints), partial norms
-    return 2 * mp * mp * sizeof(double) + 6 * m2 * sizeof(double) +
-           ((size_t)m + FRO_PARTS + OA_PARTS) * sizeof(double) + 2 * (size_t)m * sizeof(int) + 4096;
+    // group blocks (2 mp^2 doubles) + S0, S1, G, Y, T, V (6 m^2) + lam0, partial norms, counters,
+    // component labels and sizes (2 m ints)
+    const size_t b = 2 * mp * mp * sizeof(double) + 6 * m2 * sizeof(double) +
+                     ((size_t)m + FRO_PARTS + OA_PARTS) * sizeof(double) + 2 * (size_t)m * sizeof(int) + 4096;
+    return (b + 255) / 256 * 256;
+}
+size_t small_syev_work_bytes(int m) {
+    // the double-float Jacobi's rotation log (one entry per pair and round)
+    const size_t mp = (size_t)(m + (m & 1));
+    const size_t log = m <= JMAX || m > JDF_MAX ? 0 : (JDF_SWEEPS * (mp - 1) + 1) * (mp / 2) * sizeof(float2);
+    return syev_base_bytes(m) + log;
 }
 
 // ---------------------------------------------------------------------------
@@ -925,7 +1281,7 @@ static std::mutex g_coop_mutex;
 // few co-resident blocks, say) must not leave the caller polishing an
 // unrotated matrix.
 static cudaError_t coop_jacobi(Ctx &ctx, int m, double *A, double *V, double *lam, int max_sweeps,
-                               const double *normA, int *cnt) {
+                               const double *normA, double abs_factor, int *cnt) {
     static const int per_sm = [] {
         int b = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_jacobi_coop, 256, 0);
@@ -935,7 +1291,7 @@ static cudaError_t coop_jacobi(Ctx &ctx, int m, double *A, double *V, double *la
     int blocks = (int)std::min<int64_t>((work + 255) / 256, std::min(per_sm * ctx.sm_count, ctx.sm_count));
     if (blocks < 1) blocks = 1;
     int32_t *info = nullptr;
-    void *args[] = {&m, &A, &V, &lam, &max_sweeps, (void *)&normA, &cnt, &info};
+    void *args[] = {&m, &A, &V, &lam, &max_sweeps, (void *)&normA, &abs_factor, &cnt, &info};
     thread_local cudaEvent_t done = nullptr;
     if (!done) {
         const cudaError_t e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
@@ -971,7 +1327,8 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
     double *normA = lam0 + m;             // FRO_PARTS partial sums of ||S||_F^2
     double *oa_part = normA + FRO_PARTS;  // OA_PARTS partial sums of the refinement's ||T - D||_F^2
     int *cnt = reinterpret_cast<int *>(oa_part + OA_PARTS);
-    int32_t *cst = cnt + 4;
+    int32_t *cst = cnt + 4;   // cnt[6]: rounds of the double-float Jacobi
+    float2 *rlog = reinterpret_cast<float2 *>(w + syev_base_bytes(m));
 
     ctx.before(KC_SMALL_DENSE, 8.0 * m2, 2.0 * m2);
     k_fro<<<FRO_PARTS, 256, 0, ctx.stream>>>(m, S, normA);
@@ -981,25 +1338,47 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
         k_identity<<<(unsigned)((m2 + 255) / 256), 256, 0, ctx.stream>>>(m, V);
         ctx.after();
     };
-    // The FP32 stage needs A and V in one block's shared memory (m <= 160:
-    // 206 KB with the odd row pitch); larger problems go straight to the
-    // cooperative FP64 Jacobi.
-    if (mode == 0 || m > JMAX) {
+    // The one-block FP32 stage takes m <= JMAX (A and V in its shared memory),
+    // the double-float cluster m <= JDF_MAX; beyond that, and without the
+    // refinement, the cooperative FP64 Jacobi.
+    if (mode == 0 || m > JDF_MAX || (mode == 1 && m > JMAX)) {
         identity(Vm);
         cudaMemcpyAsync(Tm, S, m2 * sizeof(double), cudaMemcpyDeviceToDevice, ctx.stream);
-        const cudaError_t e = coop_jacobi(ctx, m, Tm, Vm, lam0, 60, normA, cnt);
+        const cudaError_t e = coop_jacobi(ctx, m, Tm, Vm, lam0, 60, normA, 0.5 / m, cnt);
         if (e != cudaSuccess) return e;
         ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
         k_sort_eig<<<(m + 7) / 8, 256, 0, ctx.stream>>>(m, lam0, Vm, lam, Q);
         ctx.after();
         return cudaGetLastError();
     }
-    // stage 1: FP32 Jacobi in shared memory
+    // stage 1: eigenvectors to single precision
     raise_smem_limits();
-    ctx.before(KC_SMALL_DENSE, 24.0 * m2, 9.0 * (double)m * m2 * 8);
-    const size_t smem32 = 2 * (size_t)m * (m | 1) * sizeof(float);
-    k_jacobi32<<<1, 1024, smem32, ctx.stream>>>(m, S, lam0, S0, 40, 1e-6f);
-    ctx.after();
+    if (m <= JMAX) {
+        ctx.before(KC_SMALL_DENSE, 24.0 * m2, 9.0 * (double)m * m2 * 8);
+        const size_t smem32 = 2 * (size_t)m * (m | 1) * sizeof(float);
+        k_jacobi32<<<1, 1024, smem32, ctx.stream>>>(m, S, lam0, S0, 40, 1e-6f);
+        ctx.after();
+    } else {
+        ctx.before(KC_SMALL_DENSE, 12.0 * m2, 9.0 * (double)m * m2 * 8);
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = JDF_CTAS;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.gridDim = dim3(JDF_CTAS);
+        cfg.blockDim = dim3(JDF_THREADS);
+        cfg.dynamicSmemBytes = JacobiShape(m, JDF_CTAS).bytes();
+        cfg.stream = ctx.stream;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        const cudaError_t je =
+            cudaLaunchKernelEx(&cfg, k_jacobi_df, m, S, (const double *)normA, lam0, rlog, cnt + 6, 1e-10f);
+        ctx.after();
+        if (je != cudaSuccess) return je;
+        ctx.before(KC_SMALL_DENSE, 8.0 * m2, 3.0 * (double)m * m2 * 8);
+        k_jacobi_vectors<<<m, 32, mp * sizeof(float), ctx.stream>>>(m, rlog, cnt + 6, S0);
+        ctx.after();
+    }
     if (mode == 2) {
         // stage 2: three rounds of an orthonormalisation step and a
         // refinement step X <- X (I + E) from the FP64 products G = X^T X and
@@ -1039,6 +1418,19 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
         }
         dgemm(ctx, 0, 0, m, m, m, S, m, X0, m, 0.0, Ym, m, 1, nullptr, KC_SMALL_DENSE);
         dgemm(ctx, 1, 0, m, m, m, X0, m, Ym, m, 0.0, Tm, m, 1, nullptr, KC_SMALL_DENSE, true);
+        if (m > JMAX) {
+            // a large group of close eigenvalues is too much for one block:
+            // the cooperative Jacobi rotates whatever the refinement left
+            // above rounding level (it returns after one look if nothing is)
+            identity(Vm);
+            const cudaError_t e = coop_jacobi(ctx, m, Tm, Vm, lam0, 60, normA, 2.0 * m, cnt);
+            if (e != cudaSuccess) return e;
+            dgemm(ctx, 0, 0, m, m, m, X0, m, Vm, m, 0.0, X1, m, 1, nullptr, KC_SMALL_DENSE);
+            ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
+            k_sort_eig<<<(m + 7) / 8, 256, 0, ctx.stream>>>(m, lam0, X1, lam, Q);
+            ctx.after();
+            return cudaGetLastError();
+        }
         int *label = cst + 4, *csize = label + m;
         ctx.before(KC_SMALL_DENSE, 24.0 * m2, 4.0 * m2);
         k_oa_components<<<1, 1024, 0, ctx.stream>>>(m, Tm, normA, X0, lam0, label, csize, (double *)Ag,
@@ -1057,7 +1449,7 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
     dgemm(ctx, 0, 0, m, m, m, S, m, S1, m, 0.0, Ym, m, 1, nullptr, KC_SMALL_DENSE);
     dgemm(ctx, 1, 0, m, m, m, S1, m, Ym, m, 0.0, Tm, m, 1, nullptr, KC_SMALL_DENSE);
     identity(Vm);
-    const cudaError_t e = coop_jacobi(ctx, m, Tm, Vm, lam0, 20, normA, cnt);
+    const cudaError_t e = coop_jacobi(ctx, m, Tm, Vm, lam0, 20, normA, 0.5 / m, cnt);
     if (e != cudaSuccess) return e;
     dgemm(ctx, 0, 0, m, m, m, S1, m, Vm, m, 0.0, S0, m, 1, nullptr, KC_SMALL_DENSE);
     ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
@@ -1080,6 +1472,7 @@ void raise_smem_limits() {
         cudaFuncSetAttribute(k_chol_shifted, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_triinv_upper, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_jacobi32, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        cudaFuncSetAttribute(k_jacobi_df, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     });
 }
 
