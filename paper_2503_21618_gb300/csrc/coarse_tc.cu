@@ -192,7 +192,8 @@ k_inv_apply_tc(int n, int Lp, int64_t nks, int ntra, int ntrb, const __nv_bfloat
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const unsigned a0 = smem_addr(stg + (size_t)st * stage), b0 = a0 + CT_PARTS * CT_ABLK;
+            const unsigned sa = smem_addr(stg + (size_t)st * stage);
+            const uint64_t a0 = umma_desc(sa), b0 = umma_desc(sa + CT_PARTS * CT_ABLK);
 #pragma unroll
             for (int k16 = 0; k16 < 2; ++k16)
 #pragma unroll
@@ -200,9 +201,8 @@ k_inv_apply_tc(int n, int Lp, int64_t nks, int ntra, int ntrb, const __nv_bfloat
                     // (s, t) = (0,0) (0,1) (1,0) (0,2) (1,1) (2,0)
                     const int s = p < 1 ? 0 : (p < 3 ? p - 1 : p - 3);
                     const int t = p < 1 ? 0 : (p < 3 ? 2 - p : 5 - p);
-                    const uint64_t ad = umma_desc(a0 + s * CT_ABLK + k16 * 256u);
-                    const uint64_t bd = umma_desc(b0 + t * bblk + k16 * 256u);
-                    umma_bf16(tmem, ad, bd, idesc, (first && k16 == 0 && p == 0) ? 0u : 1u);
+                    umma_bf16(tmem, umma_desc_at(a0, s * CT_ABLK + k16 * 256u), umma_desc_at(b0, t * bblk + k16 * 256u),
+                              idesc, (first && k16 == 0 && p == 0) ? 0u : 1u);
                 }
             first = false;
             umma_commit(empty + st);
