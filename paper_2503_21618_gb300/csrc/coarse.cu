@@ -23,7 +23,7 @@
 // the chain of 64 pivots (~11 us) hides behind the update.  Bound by FP32
 // arithmetic: 4 N n^3 flops (n = 1283, N = 4: 34 GF, 0.45 ms at 75 TFLOP/s);
 // cuBLAS complex GEMMs on the whole matrix, with the diagonal blocks and
-// block copies in launches of their own, took 3.9 ms there, this 1.7 ms.
+// block copies in launches of their own, took 3.9 ms there, this 1.2 ms.
 #include <cublas_v2.h>
 #include <cuda_runtime.h>
 
@@ -81,37 +81,50 @@ __device__ __forceinline__ void tile_product(const float2 (*A)[CB], const float2
 }
 
 // The symmetric sweep of all CB pivots of a tile in registers: S -> -S^{-1}.
-// Per pivot the owners publish its row (= its column), one barrier.
+// Per pivot the owners publish its row (= its column), one barrier, everyone
+// updates, and the owners of the pivot's row and column overwrite theirs (the
+// indices of a column's owners are fixed at compile time but for one lane
+// number, so nothing is selected in the common path).
 __device__ __forceinline__ void tile_sweep(float2 (&S)[4][4], float2 (*row)[CB], int ty, int tx) {
-    for (int k4 = 0; k4 < CB / 4; ++k4)
 #pragma unroll
-        for (int ki = 0; ki < 4; ++ki) {
-            const int k = 4 * k4 + ki;
-            float2 *rk = row[ki & 1];
-            if (ty == k4)
+    for (int half = 0; half < 2; ++half)
+        for (int k8 = 0; k8 < CB / 8; ++k8)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) rk[tile_col(tx, q)] = S[ki][q];
-            __syncthreads();
-            const float2 p = rk[k];
-            const float den = p.x * p.x + p.y * p.y;
-            const float2 pinv = make_float2(p.x / den, -p.y / den);
-            float2 w[4];
+            for (int ki = 0; ki < 4; ++ki) {
+                const int k4 = 8 * half + k8, k = 4 * k4 + ki;
+                constexpr int Q0[2] = {0, 2};
+                const int qk = Q0[half] + (ki & 1), kx = (k & 31) >> 1;   // column k: registers S[.][qk] of lane tx = kx
+                float2 *rk = row[ki & 1];
+                if (ty == k4) {
+                    *reinterpret_cast<float4 *>(rk + 2 * tx) = make_float4(S[ki][0].x, S[ki][0].y, S[ki][1].x, S[ki][1].y);
+                    *reinterpret_cast<float4 *>(rk + 2 * tx + 32) =
+                        make_float4(S[ki][2].x, S[ki][2].y, S[ki][3].x, S[ki][3].y);
+                }
+                __syncthreads();
+                const float2 p = rk[k];
+                const float4 c01 = *reinterpret_cast<const float4 *>(rk + 2 * tx);
+                const float4 c23 = *reinterpret_cast<const float4 *>(rk + 2 * tx + 32);
+                const float4 r01 = *reinterpret_cast<const float4 *>(rk + 4 * ty);
+                const float4 r23 = *reinterpret_cast<const float4 *>(rk + 4 * ty + 2);
+                const float di = __frcp_rn(p.x * p.x + p.y * p.y);
+                const float2 pinv = make_float2(p.x * di, -p.y * di);
+                const float2 w[4] = {cmul(pinv, make_float2(c01.x, c01.y)), cmul(pinv, make_float2(c01.z, c01.w)),
+                                     cmul(pinv, make_float2(c23.x, c23.y)), cmul(pinv, make_float2(c23.z, c23.w))};
+                const float2 r[4] = {make_float2(r01.x, r01.y), make_float2(r01.z, r01.w), make_float2(r23.x, r23.y),
+                                     make_float2(r23.z, r23.w)};
 #pragma unroll
-            for (int q = 0; q < 4; ++q) w[q] = cmul(pinv, rk[tile_col(tx, q)]);
+                for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float2 ri = rk[4 * ty + i];
-                const bool prow = ty == k4 && i == ki;
+                    for (int q = 0; q < 4; ++q) S[i][q] = cfma(make_float2(-r[i].x, -r[i].y), w[q], S[i][q]);
+                if (tx == kx)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const bool pcol = tile_col(tx, q) == k;
-                    const float2 v = csub(S[i][q], cmul(ri, w[q]));
-                    const float2 c = prow ? w[q] : cmul(pinv, ri);
-                    const float2 d = make_float2(-pinv.x, -pinv.y);
-                    S[i][q] = prow && pcol ? d : (prow || pcol ? c : v);
+                    for (int i = 0; i < 4; ++i) S[i][qk] = cmul(pinv, r[i]);
+                if (ty == k4) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) S[ki][q] = w[q];
+                    if (tx == kx) S[ki][qk] = make_float2(-pinv.x, -pinv.y);
                 }
             }
-        }
 }
 
 // Sweep of the diagonal block at k0: M_KK = -P, and P beside it
@@ -129,7 +142,7 @@ __device__ __forceinline__ void sweep_store(float2 (&S)[4][4], float2 (*row)[CB]
 }
 
 __global__ void __launch_bounds__(256) k_first_block(int np, float2 *__restrict__ M, float2 *__restrict__ P) {
-    __shared__ float2 row[2][CB];
+    __shared__ __align__(16) float2 row[2][CB];
     float2 *Mj = M + (int64_t)blockIdx.x * np * np;
     const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
     float2 S[4][4];
@@ -141,48 +154,67 @@ __global__ void __launch_bounds__(256) k_first_block(int np, float2 *__restrict_
 }
 
 // Panel of block K: the old rows M_K* (from the upper triangle: M_KJ for J >
-// K, M_JK^T for J < K) to Cp, T = P M_K* to Tp and in place of the old block.
-__global__ void __launch_bounds__(256, 3) k_sweep_panel(int np, int K, float2 *__restrict__ M,
-                                                        const float2 *__restrict__ P, float2 *__restrict__ Cp,
-                                                        float2 *__restrict__ Tp) {
+// K, M_JK^T for J < K) to Cp, T = P M_K* to Tp and in place of the old block;
+// one CTA per matrix and 32 columns.
+constexpr int PC = 32, PLD = PC + 2;   // columns of a panel CTA, their pitch
+__global__ void __launch_bounds__(256) k_sweep_panel(int np, int K, float2 *__restrict__ M,
+                                                     const float2 *__restrict__ P, float2 *__restrict__ Cp,
+                                                     float2 *__restrict__ Tp) {
     extern __shared__ __align__(16) float2 sm[];
     float2(*sP)[CB] = reinterpret_cast<float2(*)[CB]>(sm);
-    float2(*sC)[CB] = sP + CB;
-    const int J = (int)blockIdx.x + ((int)blockIdx.x >= K ? 1 : 0), j = blockIdx.y;
+    float2(*sC)[PLD] = reinterpret_cast<float2(*)[PLD]>(sm + CB * CB);
+    const int j = blockIdx.x, Jh = blockIdx.y >> 1, J = Jh + (Jh >= K ? 1 : 0);
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
     float2 *Mj = M + (int64_t)j * np * np;
     float2 *C = Cp + (int64_t)j * CB * np, *T = Tp + (int64_t)j * CB * np;
-    const int k0 = K * CB, c0 = J * CB;
-    for (int e = tid; e < CB * CB; e += 256) {
-        const int r = e / CB, c = e % CB;
-        sP[r][c] = P[(int64_t)j * CB * CB + e];   // symmetric
-        // the tile is read along its rows; below the diagonal it is transposed
-        if (J > K) sC[r][c] = Mj[(int64_t)(k0 + r) * np + c0 + c];
-        else sC[c][r ^ (c & 15)] = Mj[(int64_t)(c0 + r) * np + k0 + c];   // swizzled against bank conflicts
-    }
+    const int k0 = K * CB, c0 = J * CB + (blockIdx.y & 1) * PC;
+#pragma unroll 8
+    for (int e = tid; e < CB * CB / 2; e += 256)
+        *reinterpret_cast<float4 *>(&sP[0][0] + 2 * e) =
+            *reinterpret_cast<const float4 *>(P + (int64_t)j * CB * CB + 2 * e);   // symmetric
+    if (J > K)
+#pragma unroll
+        for (int e = tid; e < CB * PC; e += 256)
+            sC[e / PC][e % PC] = Mj[(int64_t)(k0 + e / PC) * np + c0 + e % PC];
+    else
+#pragma unroll
+        for (int e = tid; e < CB * PC; e += 256)
+            sC[e % CB][e / CB] = Mj[(int64_t)(c0 + e / CB) * np + k0 + e % CB];
     __syncthreads();
-    if (J < K) {   // undo the swizzle, row by row
-        for (int r = tid >> 5; r < CB; r += 8) {
-            const int l = tid & 31;
-            const float2 v0 = sC[r][l ^ (r & 15)], v1 = sC[r][(l + 32) ^ (r & 15)];
-            __syncwarp();
-            sC[r][l] = v0;
-            sC[r][l + 32] = v1;
-        }
-        __syncthreads();
+#pragma unroll
+    for (int e = tid; e < CB * PC; e += 256) C[(int64_t)(e / PC) * np + c0 + e % PC] = sC[e / PC][e % PC];
+    float2 acc[4][2] = {};
+#pragma unroll 4
+    for (int k = 0; k < CB; ++k) {   // P^T = P
+        const float4 a01 = *reinterpret_cast<const float4 *>(&sP[k][4 * ty]);
+        const float4 a23 = *reinterpret_cast<const float4 *>(&sP[k][4 * ty + 2]);
+        const float4 b01 = *reinterpret_cast<const float4 *>(&sC[k][2 * tx]);
+        const float2 a[4] = {make_float2(a01.x, a01.y), make_float2(a01.z, a01.w), make_float2(a23.x, a23.y),
+                             make_float2(a23.z, a23.w)};
+        const float2 b[2] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w)};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) acc[i][q] = cfma(a[i], b[q], acc[i][q]);
     }
-    for (int e = tid; e < CB * CB; e += 256) C[(int64_t)(e / CB) * np + c0 + e % CB] = sC[e / CB][e % CB];
-    float2 acc[4][4] = {};
-    tile_product(sP, sC, ty, tx, acc);   // P^T = P
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i) {
+        const int r = 4 * ty + i, c = c0 + 2 * tx;
+        const float4 v = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+        *reinterpret_cast<float4 *>(T + (int64_t)r * np + c) = v;
+        if (J > K) *reinterpret_cast<float4 *>(Mj + (int64_t)(k0 + r) * np + c) = v;
+    }
+    if (J < K) {   // transposed, through shared memory
+        __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int r = 4 * ty + i, c = tile_col(tx, q);
-            T[(int64_t)r * np + c0 + c] = acc[i][q];
-            if (J > K) Mj[(int64_t)(k0 + r) * np + c0 + c] = acc[i][q];
-            else Mj[(int64_t)(c0 + c) * np + k0 + r] = acc[i][q];
-        }
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) sC[4 * ty + i][2 * tx + q] = acc[i][q];
+        __syncthreads();
+#pragma unroll
+        for (int e = tid; e < CB * PC; e += 256)
+            Mj[(int64_t)(c0 + e / CB) * np + k0 + e % CB] = sC[e % CB][e / CB];
+    }
 }
 
 // M_IJ -= Cp_I^T T_J for the tiles I <= J off block K; the first CTA of each
@@ -193,12 +225,12 @@ __global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, 
     extern __shared__ __align__(16) float2 sm[];
     float2(*sA)[CB] = reinterpret_cast<float2(*)[CB]>(sm);
     float2(*sB)[CB] = sA + CB;
-    const int j = blockIdx.y;
+    const int j = blockIdx.x;   // the matrices fastest: every first CTA starts at once
     // tile t of the upper triangle of the nb - 1 blocks other than K
     const bool next = K + 1 < nb;
     int I, J;
     {
-        int t = blockIdx.x;
+        int t = blockIdx.y;
         const int q = nb - 1;
         // the next diagonal block (position K among the others) comes first
         const int td = next ? K * q - K * (K - 1) / 2 : -1;
@@ -234,7 +266,7 @@ __global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, 
     }
     __syncthreads();
     tile_product(sA, sB, ty, tx, m);
-    if (next && blockIdx.x == 0) {
+    if (next && blockIdx.y == 0) {
         __syncthreads();   // the panels' shared memory holds the pivot rows from here
         sweep_store(m, sA, np, (K + 1) * CB, Mj, P + (int64_t)j * CB * CB, ty, tx);
         return;
@@ -274,6 +306,7 @@ __global__ void __launch_bounds__(256) k_sweep_finish(int n, int np, const float
 }
 
 constexpr size_t SWEEP_SMEM = 2 * CB * CB * sizeof(float2);
+constexpr size_t PANEL_SMEM = (CB * CB + CB * PLD) * sizeof(float2);
 
 // The kernels' shared-memory limit, raised once per device
 void raise_sweep_smem() {
@@ -281,7 +314,7 @@ void raise_sweep_smem() {
     int dev = 0;
     cudaGetDevice(&dev);
     std::call_once(once[dev < 0 || dev >= 64 ? 0 : dev], [] {
-        cudaFuncSetAttribute(k_sweep_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SWEEP_SMEM);
+        cudaFuncSetAttribute(k_sweep_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PANEL_SMEM);
         cudaFuncSetAttribute(k_sweep_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SWEEP_SMEM);
     });
 }
@@ -310,10 +343,10 @@ void coarse_inverse(Ctx &ctx, int n, const PoleSet<float> &ps, const int32_t *pt
     if (nb > 1)
         for (int K = 0; K < nb; ++K) {
             ctx.before(KC_MG_COARSE, 24.0 * N * CB * np, 8.0 * N * CB * CB * (double)np);
-            k_sweep_panel<<<dim3(nb - 1, N), 256, SWEEP_SMEM, ctx.stream>>>(np, K, M, P, Cp, Tp);
+            k_sweep_panel<<<dim3(N, 2 * (nb - 1)), 256, PANEL_SMEM, ctx.stream>>>(np, K, M, P, Cp, Tp);
             ctx.after();
             ctx.before(KC_MG_COARSE, 8.0 * N * np * (double)np, 4.0 * N * CB * (double)np * np);
-            k_sweep_update<<<dim3((nb - 1) * nb / 2, N), 256, SWEEP_SMEM, ctx.stream>>>(np, nb, K, M, P, Cp, Tp);
+            k_sweep_update<<<dim3(N, (nb - 1) * nb / 2), 256, SWEEP_SMEM, ctx.stream>>>(np, nb, K, M, P, Cp, Tp);
             ctx.after();
         }
     ctx.before(KC_MG_COARSE, 12.0 * N * n * (double)n, 0);
