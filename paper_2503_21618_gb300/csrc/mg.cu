@@ -362,16 +362,70 @@ k_mg_scale(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, const 
 // Coarsest solve, one of its two products (n_c x n_c real V times the
 // complex block X, n_c x W):  Out = op(V) X, op(V) = V^T if trans, and if
 // cinv != nullptr each output row k of pole j is scaled by cinv[k*N + j].
-// (8 RT) x 16-column tiles of Out per CTA (16 x 8 threads, RT rows each).
-// Bound by the FP64 pipe of the SMs that have a tile (about 1.6 FMA per clock
-// and SM): with 32 x 32 tiles a 223 x 60 product ran on 14 of the 152 SMs and
-// took 141 us; RT = 1 spreads it over 112 CTAs.
-template <typename T, int RT>
+// Bound by the FP64 pipe (two FMAs per clock and SM), so what counts is that
+// every SM has the same share.  Two forms:
+//  * k_mg_coarse_gemm: 32-row x 16-column tiles per CTA (16 x 8 threads, four
+//    rows each) from shared memory, where such tiles give every SM two CTAs;
+//  * k_mg_coarse_split: 4-row x 8-column tiles, the four warps of a CTA take a
+//    quarter of K each and read V and X directly (32 and 128 bytes per step).
+//    Nothing is staged, so there is no barrier but the final one, and 223 x 60
+//    makes 448 CTAs of a quarter's length: 19 us for the product against
+//    31 us with 8 x 16 tiles from shared memory (112 CTAs, a barrier and an
+//    exposed load every 32 steps) and 141 us with 32 x 32 tiles.
+template <typename T>
+__global__ void __launch_bounds__(128)
+k_mg_coarse_split(int nc, int W, int Lp, int N, int trans, const T *__restrict__ V, const cplx<T> *__restrict__ X,
+                  const cplx<T> *__restrict__ cinv, cplx<T> *__restrict__ Out, const int32_t *__restrict__ flag) {
+    using C = cplx<T>;
+    constexpr int KW = 4, U = 8;
+    __shared__ C red[KW][32];
+    const int lane = threadIdx.x & 31, wk = threadIdx.x >> 5;
+    const int row = blockIdx.y * 4 + (lane >> 3), col = blockIdx.x * 8 + (lane & 7);
+    const bool live = col < W && flag[col] == 1 && row < nc;
+    if (!__syncthreads_or(live)) return;
+    const int kc = (nc + KW - 1) / KW, k0 = wk * kc, k1 = min(nc, k0 + kc);
+    C acc = mk((T)0, (T)0);
+    if (live) {
+        const T *v = trans ? V + row : V + (int64_t)row * nc;
+        const int64_t vs = trans ? nc : 1;
+        const C *x = X + col;
+        int k = k0;
+        for (; k + U <= k1; k += U) {
+            T a[U];
+            C b[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                a[u] = __ldg(v + (k + u) * vs);
+                b[u] = x[(int64_t)(k + u) * W];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                acc.x = fma(a[u], b[u].x, acc.x);
+                acc.y = fma(a[u], b[u].y, acc.y);
+            }
+        }
+        for (; k < k1; ++k) {
+            const T a = __ldg(v + k * vs);
+            const C b = x[(int64_t)k * W];
+            acc.x = fma(a, b.x, acc.x);
+            acc.y = fma(a, b.y, acc.y);
+        }
+    }
+    red[wk][lane] = acc;
+    __syncthreads();
+    if (wk != 0 || !live) return;
+#pragma unroll
+    for (int w = 1; w < KW; ++w) acc = cadd(acc, red[w][lane]);
+    if (cinv) acc = cmul(acc, cinv[(int64_t)row * N + col / Lp]);
+    Out[(int64_t)row * W + col] = acc;
+}
+
+template <typename T>
 __global__ void __launch_bounds__(128)
 k_mg_coarse_gemm(int nc, int W, int Lp, int N, int trans, const T *__restrict__ V, const cplx<T> *__restrict__ X,
                  const cplx<T> *__restrict__ cinv, cplx<T> *__restrict__ Out, const int32_t *__restrict__ flag) {
     using C = cplx<T>;
-    constexpr int TR = 8 * RT, TC = 16, TK = 32;
+    constexpr int RT = 4, TR = 8 * RT, TC = 16, TK = 32;
     __shared__ T sV[TR][TK + 1];
     __shared__ C sX[TK][TC];
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TC + tx;
@@ -574,16 +628,17 @@ void coarse_solve(Ctx &ctx, const KrylovDims &d, const MgSolve<T> &mg, const cpl
     const double bytes = (double)nc * nc * sizeof(T) + 2.0 * vec_bytes<T>(d, nc);
     const double flops = 4.0 * (double)nc * nc * W;
     // four rows per thread (fewer shared loads per FMA) once such tiles give
-    // every SM two CTAs, else one row per thread: four times the CTAs
-    const int gx = (W + 15) / 16;
-    const bool wide = (int64_t)gx * ((nc + 31) / 32) >= 2 * ctx.sm_count;
-    const dim3 grid(gx, wide ? (nc + 31) / 32 : (nc + 7) / 8), block(16, 8);
+    // every SM two CTAs, else small tiles split over K
+    const dim3 tiles((W + 15) / 16, (nc + 31) / 32);
+    const bool wide = (int64_t)tiles.x * tiles.y >= 2 * ctx.sm_count;
     auto product = [&](int trans, const cplx<T> *X, const cplx<T> *cinv, cplx<T> *Out) {
         ctx.before(KC_MG_COARSE, bytes, flops);
         if (wide)
-            k_mg_coarse_gemm<T, 4><<<grid, block, 0, ctx.stream>>>(nc, W, d.Lp, d.N, trans, mg.V, X, cinv, Out, flag);
+            k_mg_coarse_gemm<T><<<tiles, dim3(16, 8), 0, ctx.stream>>>(nc, W, d.Lp, d.N, trans, mg.V, X, cinv, Out,
+                                                                       flag);
         else
-            k_mg_coarse_gemm<T, 1><<<grid, block, 0, ctx.stream>>>(nc, W, d.Lp, d.N, trans, mg.V, X, cinv, Out, flag);
+            k_mg_coarse_split<T><<<dim3((W + 7) / 8, (nc + 3) / 4), 128, 0, ctx.stream>>>(nc, W, d.Lp, d.N, trans,
+                                                                                          mg.V, X, cinv, Out, flag);
         ctx.after();
     };
     product(1, Rv, mg.cinv, Y);
