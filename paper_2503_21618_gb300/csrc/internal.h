@@ -1,6 +1,8 @@
 // Internal interfaces between the slrf translation units (not part of the ABI).
 #pragma once
 #include <cuda_runtime.h>
+
+#include <algorithm>
 #include <stdint.h>
 
 #include <vector>
@@ -125,6 +127,31 @@ struct KrylovBuffers {
 };
 
 int krylov_row_groups(const Ctx &ctx, const KrylovDims &d, int prec_fp32);
+
+// Block shape of the kernels whose thread (tx, ty) owns a column group and
+// every blockDim.y-th row: gx blocks of bx x 8 threads over the groups.  A
+// warp costs the FP64 pipe the same with 18 live lanes as with 32, so bx is the
+// multiple of four, at most 32, that leaves the fewest lanes over; warps then
+// span several rows.  At n = 10 000 with 4 poles of 36 columns: the update in
+// three blocks of 12 instead of two of 32 lanes 77 -> 39 us (a third of it
+// fewer operations), the shifted product, 6 x 24 instead of 5 x 32, 121 -> 107,
+// at the pipe's rate both times.  The widest shape within 1/32 of the best is
+// taken (longer runs per row).  Kernels bound by their gathers (FP32; the real
+// products A X, B X: 257 -> 287 us at n = 89 401, m = 150) keep a row per warp.
+struct ColShape {
+    int bx, gx;
+};
+inline ColShape col_shape(int groups, bool fp64) {
+    ColShape best{32, (groups + 31) / 32};
+    if (!fp64) return best;
+    int least = best.gx * 32;
+    for (int bx = 28; bx >= 4; bx -= 4) least = std::min(least, (groups + bx - 1) / bx * bx);
+    for (int bx = 32; bx >= 4; bx -= 4) {
+        const int gx = (groups + bx - 1) / bx;
+        if (32 * gx * bx <= 33 * least) return ColShape{bx, gx};
+    }
+    return best;
+}
 
 template <typename T>
 void krylov_dinv(Ctx &ctx, const DevPencil &A, const PoleSet<T> &ps, int precond, cplx<T> *dinv);

@@ -93,7 +93,7 @@ k_init(int n, int W, int Lp, int N, int m, const double *__restrict__ rhs, int64
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * 32 + tx;
+    const int cg = blockIdx.x * blockDim.x + tx;
     const int c0 = cg * VC;
     int j = 0, cl = 0;
     bool act[VC];
@@ -183,7 +183,7 @@ k_spmm_shifted_rb(int n, int W, int Lp, int rows_per_block, const int32_t *__res
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * 32 + tx;
+    const int cg = blockIdx.x * blockDim.x + tx;
     const int c0 = cg * VC;
     bool act = false;
     C s = mk((T)0, (T)0);
@@ -239,7 +239,7 @@ k_spmm_shifted_rb(int n, int W, int Lp, int rows_per_block, const int32_t *__res
             }
             CV<T, VC> q;
 #pragma unroll
-            for (int v = 0; v < VC; ++v) q.v[v] = csub(sa[v], cmul(s, sb[v]));
+            for (int v = 0; v < VC; ++v) q.v[v] = cfms(s, sb[v], sa[v]);
             stcv(Q + (int64_t)row * W + c0, q);
             const CV<T, VC> pr = ldcv(P + (int64_t)row * W + c0);
 #pragma unroll
@@ -284,7 +284,7 @@ k_spmm_shifted_rg(int n, int W, int Lp, int ngroups, int groups_per_block, const
     using AB = typename ABT<T>::type;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * 32 + tx;
+    const int cg = blockIdx.x * blockDim.x + tx;
     const int c0 = cg * VC;
     bool act = false;
     C s = mk((T)0, (T)0);
@@ -355,7 +355,7 @@ k_spmm_shifted_rg(int n, int W, int Lp, int ngroups, int groups_per_block, const
                 if (row >= n) break;
                 CV<T, VC> q;
 #pragma unroll
-                for (int v = 0; v < VC; ++v) q.v[v] = csub(sa[r][v], cmul(s, sb[r][v]));
+                for (int v = 0; v < VC; ++v) q.v[v] = cfms(s, sb[r][v], sa[r][v]);
                 stcv(Q + (int64_t)row * W + c0, q);
                 const CV<T, VC> pr = ldcv(P + (int64_t)row * W + c0);
 #pragma unroll
@@ -403,7 +403,7 @@ k_spmm_shifted_nb(int n, int W, int Lp, int ngroups, int groups_per_block, const
     constexpr int VC = 2;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * 32 + tx;
+    const int cg = blockIdx.x * blockDim.x + tx;
     const int c0 = cg * VC;
     bool act = false;
     float2 s = make_float2(0.f, 0.f);
@@ -468,7 +468,7 @@ k_spmm_shifted_nb(int n, int W, int Lp, int ngroups, int groups_per_block, const
                 if (row >= n) break;
                 CV<float, VC> q;
 #pragma unroll
-                for (int v = 0; v < VC; ++v) q.v[v] = csub(sa[r][v], cmul(s, sb[r][v]));
+                for (int v = 0; v < VC; ++v) q.v[v] = cfms(s, sb[r][v], sa[r][v]);
                 stcv(Q + (int64_t)row * W + c0, q);
                 const CV<float, VC> pr = ldcv(P + (int64_t)row * W + c0);
 #pragma unroll
@@ -514,7 +514,7 @@ k_spmm_shifted_sell(int n, int W, int Lp, int C, int nchunks, int chunks_per_blo
     constexpr int VC = 2;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * 32 + tx;
+    const int cg = blockIdx.x * blockDim.x + tx;
     const int c0 = cg * VC;
     bool act = false;
     float2 s = make_float2(0.f, 0.f);
@@ -572,7 +572,7 @@ k_spmm_shifted_sell(int n, int W, int Lp, int C, int nchunks, int chunks_per_blo
                 }
                 CV<float, VC> q;
 #pragma unroll
-                for (int v = 0; v < VC; ++v) q.v[v] = csub(sa[v], cmul(s, sb[v]));
+                for (int v = 0; v < VC; ++v) q.v[v] = cfms(s, sb[v], sa[v]);
                 stcv(Q + (int64_t)row * W + c0, q);
                 const CV<float, VC> pr = ldcv(P + (int64_t)row * W + c0);
 #pragma unroll
@@ -792,7 +792,7 @@ k_spmm_staged(int n, int W, int Lp, int ngroups, int gpb, int emax, const int32_
             float2 q[VC];
 #pragma unroll
             for (int v = 0; v < VC; ++v) {
-                q[v] = csub(sa[r][v], cmul(sg, sb[r][v]));
+                q[v] = cfms(sg, sb[r][v], sa[r][v]);
                 const float2 pr = xs[(size_t)dp * CW + v];
                 mu[v] = cfma(pr, q[v], mu[v]);
             }
@@ -899,7 +899,7 @@ k_update(int n, int W, int Lp, int N, cplx<T> *__restrict__ R, const cplx<T> *__
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ngl = Lp / VC;
-    const int cgl = blockIdx.x * 32 + tx;
+    const int cgl = blockIdx.x * blockDim.x + tx;
     const int c0 = cgl * VC;
     const bool live = cgl < ngl;
     unsigned actmask = 0;   // bit j*VC + v
@@ -938,15 +938,15 @@ k_update(int n, int W, int Lp, int N, cplx<T> *__restrict__ R, const cplx<T> *__
                     if (!(mj & (1u << v))) continue;
                     const C a = alpha[j * Lp + c0 + v];
                     const C w = ua[j * Lp + c0 + v];
-                    r.v[v] = csub(r.v[v], cmul(a, q.v[v]));
-                    u[v] += w.x * p.v[v].x - w.y * p.v[v].y;
+                    r.v[v] = cfms(a, q.v[v], r.v[v]);
+                    u[v] = fma(w.x, p.v[v].x, fma(-w.y, p.v[v].y, u[v]));
                     if (JAC) {
                         const C z = cmul(dv, r.v[v]);
                         const C rz = cmul(r.v[v], z);
                         acc[j][v][0] += rz.x;
                         acc[j][v][1] += rz.y;
                     }
-                    acc[j][v][2] += cabs2(r.v[v]);
+                    acc[j][v][2] = fma(r.v[v].x, r.v[v].x, fma(r.v[v].y, r.v[v].y, acc[j][v][2]));
                 }
                 stcv(R + base, r);
                 if (MGY) {
@@ -1007,7 +1007,7 @@ k_direction(int n, int W, int Lp, int N, const cplx<T> *__restrict__ R, const cp
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * 32 + tx;
+    const int cg = blockIdx.x * blockDim.x + tx;
     if (cg >= ng) return;
     const int c0 = cg * VC;
     const int j = c0 / Lp;
@@ -1172,7 +1172,8 @@ void krylov_init(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb, const doub
                  const cplx<double> *rhs_c) {
     constexpr int VC = VecN<T>::VC;
     const int W = d.W();
-    dim3 grid((W / VC + 31) / 32, kb.gy), block(32, TY);
+    const ColShape cs = col_shape(W / VC, sizeof(T) == 8);
+    dim3 grid(cs.gx, kb.gy), block(cs.bx, TY);
     const double vb = (double)d.n * W * sizeof(cplx<T>);
     ctx.before(KC_KRYLOV_INIT, 2 * vb + (double)d.n * d.m * 8, 0);
     k_init<T, VC><<<grid, block, 0, ctx.stream>>>(d.n, W, d.Lp, d.N, d.m, rhs, ldr, rhs_c, kb.dinv, kb.R, kb.P,
@@ -1193,7 +1194,8 @@ void krylov_spmm(Ctx &ctx, const KrylovDims &d, const DevPencil &A, const cplx<T
                  cplx<T> *Q, const int32_t *flag, T *part, int gy) {
     constexpr int VC = VecN<T>::VC;
     const int W = d.W();
-    dim3 grid((W / VC + 31) / 32, gy), block(32, TY);
+    const ColShape cs = col_shape(W / VC, sizeof(T) == 8);
+    dim3 grid(cs.gx, gy), block(cs.bx, TY);
     // algorithmic bytes: pattern + (a,b) pairs once, P read once and Q written
     // once for the active columns (converged columns are skipped)
     const double bytes = 4.0 * (d.n + 1) + (double)A.nnz * (4 + 2 * sizeof(T)) +
@@ -1273,7 +1275,8 @@ template <typename T, int NP>
 static void launch_update(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb) {
     constexpr int VC = VecN<T>::VC;
     const int W = d.W();
-    dim3 grid((d.Lp / VC + 31) / 32, kb.gy), block(32, TY);
+    const ColShape cs = col_shape(d.Lp / VC, sizeof(T) == 8);
+    dim3 grid(cs.gx, kb.gy), block(cs.bx, TY);
     const double vb = (double)d.n * W * d.frac * sizeof(cplx<T>);
     ctx.before(KC_KRYLOV_UPDATE,
                (kb.mgd ? 5 : 4) * vb + 2.0 * d.n * d.Lp * sizeof(T) + (double)d.n * d.N * sizeof(cplx<T>),
@@ -1317,7 +1320,8 @@ template <typename T>
 void krylov_direction(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb, int init) {
     constexpr int VC = VecN<T>::VC;
     const int W = d.W();
-    dim3 grid((W / VC + 31) / 32, kb.gy), block(32, TY);
+    const ColShape cs = col_shape(W / VC, sizeof(T) == 8);
+    dim3 grid(cs.gx, kb.gy), block(cs.bx, TY);
     const double vb = (double)d.n * W * d.frac * sizeof(cplx<T>);
     ctx.before(KC_KRYLOV_DIR, (init ? 2 : 3) * vb + (kb.Z ? 0.0 : (double)d.n * d.N * sizeof(cplx<T>)),
                10.0 * d.n * W * d.frac);

@@ -152,7 +152,7 @@ k_mg_sspmm(int n, int W, int Lp, int N, int ngroups, const int32_t *__restrict__
     constexpr int UNR = (MODE == MG_DOWN) ? 4 : 2;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * 32 + tx;
+    const int cg = blockIdx.x * blockDim.x + tx;
     const int c0 = cg * VC;
     bool act = false;
     int j = 0;
@@ -199,19 +199,29 @@ k_mg_sspmm(int n, int W, int Lp, int N, int ngroups, const int32_t *__restrict__
                 CV<T, VC> o;
                 if constexpr (MODE == MG_DOWN) {
 #pragma unroll
-                    for (int v = 0; v < VC; ++v) o.v[v] = csub(cmul(s, sb[r][v]), sa[r][v]);
+                    for (int v = 0; v < VC; ++v) {
+                        if constexpr (sizeof(T) == 8)
+                            o.v[v] = cfma(s, sb[r][v], mk(-sa[r][v].x, -sa[r][v].y));
+                        else
+                            o.v[v] = csub(cmul(s, sb[r][v]), sa[r][v]);
+                    }
                 } else {
                     const CV<T, VC> rr = ldcv(Rv + base);
                     if constexpr (MODE == MG_RESID) {
 #pragma unroll
-                        for (int v = 0; v < VC; ++v) o.v[v] = csub(rr.v[v], csub(sa[r][v], cmul(s, sb[r][v])));
+                        for (int v = 0; v < VC; ++v) {
+                            if constexpr (sizeof(T) == 8)
+                                o.v[v] = cfma(s, sb[r][v], csub(rr.v[v], sa[r][v]));
+                            else
+                                o.v[v] = csub(rr.v[v], csub(sa[r][v], cmul(s, sb[r][v])));
+                        }
                     } else {
                         const C d = dinv[(int64_t)row * N + j];
                         CV<T, VC> xr;
                         if constexpr (MODE == MG_SMOOTH) xr = ldcv(X + base);
 #pragma unroll
                         for (int v = 0; v < VC; ++v) {
-                            const C y = csub(sa[r][v], cmul(s, sb[r][v]));
+                            const C y = cfms(s, sb[r][v], sa[r][v]);
                             if constexpr (MODE == MG_SMOOTH)
                                 o.v[v] = cfma(d, csub(rr.v[v], y), xr.v[v]);
                             else
@@ -263,7 +273,7 @@ k_mg_xfer(int n_out, int W, int rows_per_block, const int32_t *__restrict__ ptr,
     constexpr int UNR = 4;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * 32 + tx;
+    const int cg = blockIdx.x * blockDim.x + tx;
     if (cg >= ng) return;
     const int c0 = cg * VC;
     if (!col_active<VC>(flag, c0)) return;
@@ -271,9 +281,11 @@ k_mg_xfer(int n_out, int W, int rows_per_block, const int32_t *__restrict__ ptr,
     const int r_end = min(n_out, r_begin + rows_per_block);
     for (int row = r_begin + ty; row < r_end; row += TY) {
         const int k0 = __ldg(ptr + row), k1 = __ldg(ptr + row + 1);
-        C acc[VC];
+        const int64_t base = (int64_t)row * W + c0;
+        CV<T, VC> acc;
 #pragma unroll
-        for (int v = 0; v < VC; ++v) acc[v] = mk((T)0, (T)0);
+        for (int v = 0; v < VC; ++v) acc.v[v] = mk((T)0, (T)0);
+        if (MODE == MG_PROLONG_ADD) acc = ldcv(Out + base);
         for (int k = k0; k < k1; k += UNR) {
             int cc[UNR];
             T w[UNR];
@@ -297,21 +309,11 @@ k_mg_xfer(int n_out, int W, int rows_per_block, const int32_t *__restrict__ ptr,
             for (int u = 0; u < UNR; ++u)
 #pragma unroll
                 for (int v = 0; v < VC; ++v) {
-                    acc[v].x = fma(w[u], x[u].v[v].x, acc[v].x);
-                    acc[v].y = fma(w[u], x[u].v[v].y, acc[v].y);
+                    acc.v[v].x = fma(w[u], x[u].v[v].x, acc.v[v].x);
+                    acc.v[v].y = fma(w[u], x[u].v[v].y, acc.v[v].y);
                 }
         }
-        const int64_t base = (int64_t)row * W + c0;
-        CV<T, VC> o;
-        if (MODE == MG_RESTRICT) {
-#pragma unroll
-            for (int v = 0; v < VC; ++v) o.v[v] = acc[v];
-        } else {
-            o = ldcv(Out + base);
-#pragma unroll
-            for (int v = 0; v < VC; ++v) o.v[v] = cadd(o.v[v], acc[v]);
-        }
-        stcv(Out + base, o);
+        stcv(Out + base, acc);
     }
 }
 
@@ -322,7 +324,7 @@ k_mg_jacobi0(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, cons
              cplx<T> *__restrict__ Out, const int32_t *__restrict__ flag) {
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * 32 + tx;
+    const int cg = blockIdx.x * blockDim.x + tx;
     if (cg >= ng) return;
     const int c0 = cg * VC;
     if (!col_active<VC>(flag, c0)) return;
@@ -344,7 +346,7 @@ k_mg_scale(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, const 
            cplx<T> *__restrict__ Out, const int32_t *__restrict__ flag) {
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * 32 + tx;
+    const int cg = blockIdx.x * blockDim.x + tx;
     if (cg >= ng) return;
     const int c0 = cg * VC;
     if (!col_active<VC>(flag, c0)) return;
@@ -484,7 +486,7 @@ k_mg_rz(int n, int W, const cplx<T> *__restrict__ Rv, const cplx<T> *__restrict_
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * 32 + tx;
+    const int cg = blockIdx.x * blockDim.x + tx;
     const int c0 = cg * VC;
     C rz[VC];
 #pragma unroll
@@ -567,7 +569,8 @@ void launch_sspmm(Ctx &ctx, const KrylovDims &d, int kc, int n_rows, int R, int 
     const int W = d.W();
     // gy is used as given: with partial dots every one of the gy partial rows
     // must be written (CTAs without row groups write zeros)
-    dim3 grid((W / VC + 31) / 32, gy), block(32, TY);
+    const ColShape cs = col_shape(W / VC, sizeof(T) == 8);
+    dim3 grid(cs.gx, gy), block(cs.bx, TY);
     const double vin = vec_bytes<T>(d, n_in), vout = vec_bytes<T>(d, n_rows);
     double bytes = 4.0 * (ngroups + 1) + (double)nnz_union * (4 + R * sizeof(cplx<T>)) + vin + vout;
     if (MODE == MG_RESID || MODE == MG_SMOOTH || MODE == MG_UP) bytes += vout;   // r of the rows
@@ -602,7 +605,8 @@ void launch_xfer(Ctx &ctx, const KrylovDims &d, int n_out, int n_in, int64_t nnz
     const int W = d.W();
     int gyy = std::min(gy, (n_out + TY - 1) / TY);
     if (gyy < 1) gyy = 1;
-    dim3 grid((W / VC + 31) / 32, gyy), block(32, TY);
+    const ColShape cs = col_shape(W / VC, sizeof(T) == 8);
+    dim3 grid(cs.gx, gyy), block(cs.bx, TY);
     const int rpb = (n_out + gyy - 1) / gyy;
     const double bytes = 4.0 * (n_out + 1) + (double)nnz * (4 + sizeof(T)) + vec_bytes<T>(d, n_in) +
                          (MODE == MG_RESTRICT ? 1 : 2) * vec_bytes<T>(d, n_out);
@@ -650,7 +654,8 @@ void launch_rz(Ctx &ctx, const KrylovDims &d, int gy, const cplx<T> *R, const cp
                T *part) {
     constexpr int VC = VecN<T>::VC;
     const int W = d.W();
-    dim3 grid((W / VC + 31) / 32, gy), block(32, TY);
+    const ColShape cs = col_shape(W / VC, sizeof(T) == 8);
+    dim3 grid(cs.gx, gy), block(cs.bx, TY);
     ctx.before(KC_MG_TRANSFER, 2 * vec_bytes<T>(d, d.n), 0);
     k_mg_rz<T, VC><<<grid, block, 0, ctx.stream>>>(d.n, W, R, Z, flag, part);
     ctx.after();
@@ -672,7 +677,8 @@ cplx<T> *cycle(Ctx &ctx, const KrylovDims &d, MgSolve<T> &mg, int l, int gy, con
     cplx<T> *z = L.z, *t = L.t;
     {
         const int W = d.W();
-        dim3 grid((W / VC + 31) / 32, gyl), block(32, TY);
+        const ColShape cs = col_shape(W / VC, sizeof(T) == 8);
+    dim3 grid(cs.gx, gyl), block(cs.bx, TY);
         ctx.before(KC_MG_TRANSFER, 2 * vec_bytes<T>(d, L.n) + (double)L.n * d.N * sizeof(cplx<T>), 0);
         k_mg_jacobi0<T, VC><<<grid, block, 0, ctx.stream>>>(L.n, W, d.Lp, d.N, L.dinv, L.r, z, flag);
         ctx.after();
@@ -724,7 +730,8 @@ void mg_scale(Ctx &ctx, const KrylovDims &d, const MgSolve<T> &mg, int gy, const
               const int32_t *flag) {
     constexpr int VC = VecN<T>::VC;
     const int W = d.W();
-    dim3 grid((W / VC + 31) / 32, gy), block(32, TY);
+    const ColShape cs = col_shape(W / VC, sizeof(T) == 8);
+    dim3 grid(cs.gx, gy), block(cs.bx, TY);
     ctx.before(KC_MG_TRANSFER, 2 * vec_bytes<T>(d, d.n) + (double)d.n * d.N * sizeof(cplx<T>), 0);
     k_mg_scale<T, VC><<<grid, block, 0, ctx.stream>>>(d.n, W, d.Lp, d.N, mg.lv[0].dinv, X, Y, flag);
     ctx.after();
