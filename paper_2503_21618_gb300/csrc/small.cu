@@ -375,42 +375,63 @@ __device__ __forceinline__ void rr_pair(int k, int r, int mp, int &a, int &b) {
 }
 
 // ---------------------------------------------------------------------------
-// FP32 cyclic Jacobi for m <= JMAX in one block: all m/2 rotations of a
-// round applied at once (rows, then columns), A and V in shared memory with
-// an odd row pitch (the column phase's lanes walk a column without bank
-// conflicts), every row and column loop unrolled to its fixed trip count
-// (predicated on m), and the pivot pair's zeroing folded into the column
-// phase (three block barriers per round).  A rotation is skipped below
-// rel_tol of sqrt(|a_pp a_qq|); the sweeps stop once every rotation of a
-// sweep was below sqrt(rel_tol) (quadratic convergence: the next sweep would
-// find nothing).  Output: lam ascending (FP64), Q (FP64, columns =
-// eigenvectors).
+// FP32 cyclic Jacobi for m <= JMAX in one block: all m/2 rotations of a round
+// applied at once, A in shared memory with an odd row pitch.  Bound by shared
+// memory: the 2 x 2 block (k, l) of two pairs takes its row and its column
+// rotation in one visit, so A is read and written once per round (rows, then
+// columns, then the columns of V took three times that: 1.52 ms at m = 150, 1.22 now),
+// and the vectors are not formed here: the rotations are logged and
+// k_jacobi_vectors applies them, every row on its own SM.  Two block barriers
+// per round: rotations, update.  A rotation is skipped below rel_tol of
+// sqrt(|a_pp a_qq|); the sweeps stop once every rotation of a sweep was below
+// sqrt(rel_tol) (quadratic convergence: the next sweep would find nothing).
+// Output: lam ascending (FP64), rank (the place of eigenvalue i in lam), the
+// log and *nrounds.
 // ---------------------------------------------------------------------------
 constexpr int JMAX = 160;
+constexpr int J32_SWEEPS = 40;
+
+// x' = c x - s y, y' = s x + c y
+__device__ __forceinline__ void rotate(float c, float s, float &x, float &y) {
+    const float u = x, v = y;
+    x = c * u - s * v;
+    y = s * u + c * v;
+}
+
+// Padded order, row pitch and threads of the one-block Jacobi
+struct Jacobi32Shape {
+    int mp, npair, ld, threads;
+    __host__ __device__ explicit Jacobi32Shape(int m) {
+        mp = m + (m & 1);
+        npair = mp / 2;
+        ld = mp + 1;
+        threads = (npair * npair + 31) / 32 * 32;
+        threads = threads < 128 ? 128 : (threads > 1024 ? 1024 : threads);
+    }
+    size_t bytes() const { return (size_t)mp * ld * sizeof(float); }
+};
 
 __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *__restrict__ S, double *__restrict__ lam,
-                                                  double *__restrict__ Q, int max_sweeps, float rel_tol) {
+                                                  int *__restrict__ rank, float2 *__restrict__ rlog,
+                                                  int *__restrict__ nrounds, float rel_tol) {
     extern __shared__ float jsm[];
-    const int ld = m | 1;
-    float *A = jsm, *V = jsm + (size_t)m * ld;
+    const Jacobi32Shape sh(m);
+    const int mp = sh.mp, npair = sh.npair, ld = sh.ld;
+    float *A = jsm;   // mp x mp: an odd order's last row and column are zero
     const int tid = threadIdx.x, bs = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5, nwarp = bs >> 5;
-    const int mp = m + (m & 1);
-    const int npair = mp / 2;
-    constexpr int NIT = (JMAX + 31) / 32;
-    __shared__ float cs[JMAX / 2], sn[JMAX / 2];
-    __shared__ int pp[JMAX / 2], qq[JMAX / 2];
-    __shared__ int nrot;
-    __shared__ float maxrel;
+    __shared__ float2 cs[JMAX / 2];    // c, s of a pair (1, 0: no rotation)
+    __shared__ int2 pq[JMAX / 2];
+    __shared__ int maxrel;             // largest relative pivot of the sweep (float bits)
     __shared__ double red[32];
     __shared__ float absmin;
     double fro = 0.0;
-    for (int e = tid; e < m * m; e += bs) {
-        const double v = S[e];
-        A[(e / m) * ld + e % m] = (float)v;
+    for (int e = tid; e < mp * mp; e += bs) {
+        const int i = e / mp, j = e - i * mp;
+        const double v = i < m && j < m ? S[(int64_t)i * m + j] : 0.0;
+        A[i * ld + j] = (float)v;
         fro += v * v;
     }
-    for (int e = tid; e < m * m; e += bs) V[(e / m) * ld + e % m] = (e / m == e % m) ? 1.f : 0.f;
     for (int off = 16; off > 0; off >>= 1) fro += __shfl_xor_sync(0xffffffffu, fro, off);
     if (lane == 0) red[warp] = fro;
     __syncthreads();
@@ -418,15 +439,15 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *__restri
         double t = 0;
         for (int w = 0; w < nwarp; ++w) t += red[w];
         absmin = (float)(sqrt(t) * (double)rel_tol / sqrt((double)m));
+        maxrel = 0;
     }
     __syncthreads();
-    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-        if (tid == 0) {
-            nrot = 0;
-            maxrel = 0.f;
-        }
-        __syncthreads();
-        for (int r = 0; r < mp - 1; ++r) {
+    // this thread's blocks (k, l): every bs-th of the npair x npair, l fastest
+    const int k_first = tid / npair, l_first = tid - k_first * npair;
+    const int dk = bs / npair, dl = bs - dk * npair;
+    int64_t g = 0;   // rounds applied
+    for (int sweep = 0; sweep < J32_SWEEPS; ++sweep) {
+        for (int r = 0; r < mp - 1; ++r, ++g) {
             if (tid < npair) {
                 int a, b;
                 rr_pair(tid, r, mp, a, b);
@@ -441,71 +462,61 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *__restri
                         const float t = (th >= 0.f ? 1.f : -1.f) / (fabsf(th) + sqrtf(1.f + th * th));
                         c = 1.f / sqrtf(1.f + t * t);
                         sv = t * c;
-                        atomicAdd(&nrot, 1);
                         const float rel = fabsf(apq) / (scale > 0.f ? scale : 1.f);
-                        atomicMax(reinterpret_cast<int *>(&maxrel), __float_as_int(rel));
+                        atomicMax(&maxrel, __float_as_int(rel));
                     }
                 }
-                cs[tid] = c;
-                sn[tid] = sv;
-                pp[tid] = p;
-                qq[tid] = (q < m && sv != 0.f) ? q : -1;
+                cs[tid] = make_float2(c, sv);
+                pq[tid] = make_int2(p, q);
+                rlog[g * npair + tid] = make_float2(a > b ? -c : c, sv);   // the sign: lower row first
             }
             __syncthreads();
-            // rows: A <- J^T A (warp per pair, lanes over columns)
-            for (int k = warp; k < npair; k += nwarp) {
-                const int q = qq[k];
-                if (q < 0) continue;
-                const int p = pp[k];
-                const float c = cs[k], sv = sn[k];
-                float *Ap = A + p * ld, *Aq = A + q * ld;
-#pragma unroll
-                for (int it = 0; it < NIT; ++it) {
-                    const int col = lane + 32 * it;
-                    if (col < m) {
-                        const float x = Ap[col], y = Aq[col];
-                        Ap[col] = c * x - sv * y;
-                        Aq[col] = sv * x + c * y;
+            for (int k = k_first, l = l_first; k < npair;) {
+                const float2 wk = cs[k], wl = cs[l];
+                if (wk.y != 0.f || wl.y != 0.f) {
+                    const int2 ik = pq[k], il = pq[l];
+                    float *Ap = A + ik.x * ld, *Aq = A + ik.y * ld;
+                    float xpp = Ap[il.x], xpq = Ap[il.y], xqp = Aq[il.x], xqq = Aq[il.y];
+                    if (wk.y != 0.f) {
+                        rotate(wk.x, wk.y, xpp, xqp);
+                        rotate(wk.x, wk.y, xpq, xqq);
                     }
+                    if (wl.y != 0.f) {
+                        rotate(wl.x, wl.y, xpp, xpq);
+                        rotate(wl.x, wl.y, xqp, xqq);
+                    }
+                    if (k == l) xpq = xqp = 0.f;
+                    Ap[il.x] = xpp;
+                    Ap[il.y] = xpq;
+                    Aq[il.x] = xqp;
+                    Aq[il.y] = xqq;
                 }
-            }
-            __syncthreads();
-            // columns: A <- A J, V <- V J; the pivot pair (p, q) / (q, p) becomes 0
-            for (int k = warp; k < npair; k += nwarp) {
-                const int q = qq[k];
-                if (q < 0) continue;
-                const int p = pp[k];
-                const float c = cs[k], sv = sn[k];
-#pragma unroll
-                for (int it = 0; it < NIT; ++it) {
-                    const int row = lane + 32 * it;
-                    if (row < m) {
-                        float *Ar = A + row * ld, *Vr = V + row * ld;
-                        const float x = Ar[p], y = Ar[q];
-                        Ar[p] = row == q ? 0.f : c * x - sv * y;
-                        Ar[q] = row == p ? 0.f : sv * x + c * y;
-                        const float vx = Vr[p], vy = Vr[q];
-                        Vr[p] = c * vx - sv * vy;
-                        Vr[q] = sv * vx + c * vy;
-                    }
+                k += dk;
+                l += dl;
+                if (l >= npair) {
+                    l -= npair;
+                    ++k;
                 }
             }
             __syncthreads();
         }
-        if (nrot == 0 || maxrel < sqrtf(rel_tol)) break;
+        const float top = __int_as_float(maxrel);   // 0: nothing rotated
+        if (top < sqrtf(rel_tol)) break;
+        __syncthreads();
+        if (tid == 0) maxrel = 0;
         __syncthreads();
     }
-    // sort eigenvalues ascending (rank sort), permute columns into Q (FP64)
     for (int i = tid; i < m; i += bs) {
         const float di = A[i * ld + i];
-        int rank = 0;
+        int k = 0;
         for (int j = 0; j < m; ++j) {
             const float dj = A[j * ld + j];
-            rank += (dj < di) || (dj == di && j < i);
+            k += (dj < di) || (dj == di && j < i);
         }
-        lam[rank] = (double)di;
-        for (int row = 0; row < m; ++row) Q[(int64_t)row * m + rank] = (double)V[row * ld + i];
+        rank[i] = k;
+        lam[k] = (double)di;
     }
+    if (tid == 0) *nrounds = (int)g;
 }
 
 // ---------------------------------------------------------------------------
@@ -543,6 +554,8 @@ constexpr int JDF_MAX = 448;      // a CTA's rows of an 8-CTA cluster in 227 KB
 constexpr int JDF_CTAS = 8;
 constexpr int JDF_SWEEPS = 20;
 constexpr int JDF_THREADS = 512;
+constexpr int JVEC_ROUNDS = 8;    // rounds of the log per stage of k_jacobi_vectors
+static_assert(JDF_MAX <= 2 * 32 * 7, "k_jacobi_vectors holds at most 7 positions per lane");
 
 // double-float: the rounded operations are spelled out, so that no
 // multiplication and addition of the error terms is contracted
@@ -814,43 +827,105 @@ k_jacobi_df(int m, const double *__restrict__ S, const double *__restrict__ fro_
     }
 }
 
-// Q = the product of the logged rotations, row by row of I (one warp per row,
-// the row in shared memory; the next round's rotations are loaded ahead)
+// Q = the product of the logged rotations, row by row of I, one warp per row.
+// A serial chain over the rounds, so the row stays in registers in the order of
+// the round's positions: a lane holds K consecutive ones (upper and lower
+// index), and from round to round the upper ones move down one position and the
+// lower ones up one (two shuffles).  The log streams through shared memory, G
+// rounds ahead.  0.18 us a round; with the row in shared memory, gathered by index, 0.64
+// (1.53 ms at m = 300, 0.42 now).
+// A log entry (c, s) rotates (upper, lower), or (lower, upper) if c < 0; column
+// i goes to column rank[i] of Q (rank = nullptr: i).
+template <int K>
 __global__ void __launch_bounds__(32) k_jacobi_vectors(int m, const float2 *__restrict__ rlog,
-                                                       const int *__restrict__ nrounds, double *__restrict__ Q) {
-    extern __shared__ float vrow[];
+                                                       const int *__restrict__ nrounds, const int *__restrict__ rank,
+                                                       double *__restrict__ Q) {
+    constexpr int G = JVEC_ROUNDS;
+    extern __shared__ float4 vsm4[];
     const int mp = m + (m & 1), npair = mp / 2;
-    constexpr int U = (JDF_MAX / 2 + 31) / 32;
     const int lane = threadIdx.x, row = blockIdx.x;
-    for (int i = lane; i < mp; i += 32) vrow[i] = i == row ? 1.f : 0.f;
-    const int n = *nrounds, nu = (npair + 31) / 32;
-    float2 w[U];
+    const int n = *nrounds, nch = (n + G - 1) / G;
+    const int stage = G * npair * (int)sizeof(float2);   // a multiple of 16
+    char *buf = reinterpret_cast<char *>(vsm4);
+    auto fetch = [&](int ch) {
+        if (ch < nch) {
+            // the last chunk's odd half of 16 bytes: the log has one more round
+            const int bytes = (min(G, n - ch * G) * npair * (int)sizeof(float2) + 15) / 16 * 16;
+            const char *src = reinterpret_cast<const char *>(rlog) + (int64_t)ch * stage;
+            const unsigned dst = smem_addr(buf + (ch & 1) * stage);
+            for (int o = lane * 16; o < bytes; o += 32 * 16)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + o), "l"(src + o) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float top[K], bot[K];
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-        if (u < nu) w[u] = lane + 32 * u < npair && n > 0 ? rlog[lane + 32 * u] : make_float2(1.f, 0.f);
-    __syncwarp();
-    int r = 0;
-    for (int g = 0; g < n; ++g) {
-        float2 next[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (u < nu) {
-                const int k = lane + 32 * u;
-                next[u] = k < npair && g + 1 < n ? rlog[(int64_t)(g + 1) * npair + k] : make_float2(1.f, 0.f);
-                if (w[u].y != 0.f) {
-                    const int a = rr_top(k, r, mp), b = rr_bot(k, r, mp);
-                    const float x = vrow[a], y = vrow[b];
-                    vrow[a] = w[u].x * x - w[u].y * y;
-                    vrow[b] = w[u].y * x + w[u].x * y;
-                }
-            }
-        __syncwarp();
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (u < nu) w[u] = next[u];
-        if (++r == mp - 1) r = 0;
+    for (int i = 0; i < K; ++i) {
+        const int k = lane * K + i;
+        top[i] = k < npair && rr_top(k, 0, mp) == row ? 1.f : 0.f;
+        bot[i] = k < npair && rr_bot(k, 0, mp) == row ? 1.f : 0.f;
     }
-    for (int i = lane; i < m; i += 32) Q[(int64_t)row * m + i] = (double)vrow[i];
+    fetch(0);
+    fetch(1);
+    for (int ch = 0; ch < nch; ++ch) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        const float2 *w = reinterpret_cast<const float2 *>(buf + (ch & 1) * stage) + lane * K;
+        const int rounds = min(G, n - ch * G);
+        for (int j = 0; j < rounds; ++j, w += npair) {
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                const float2 v = lane * K + i < npair ? w[i] : make_float2(1.f, 0.f);
+                const bool sw = v.x < 0.f;
+                float x = sw ? bot[i] : top[i], y = sw ? top[i] : bot[i];
+                rotate(fabsf(v.x), v.y, x, y);
+                top[i] = sw ? y : x;
+                bot[i] = sw ? x : y;
+            }
+            const float up = __shfl_down_sync(0xffffffffu, top[0], 1);      // next lane's first upper
+            const float dn = __shfl_up_sync(0xffffffffu, bot[K - 1], 1);    // previous lane's last lower
+            const float first = top[0], second = npair == 1 ? bot[0] : K > 1 ? top[K > 1 ? 1 : 0] : up;
+            float t[K];
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                t[i] = i + 1 < K ? top[i + 1 < K ? i + 1 : 0] : up;
+                if (lane * K + i == npair - 1) t[i] = bot[i];   // the last lower turns upper
+            }
+#pragma unroll
+            for (int i = K - 1; i > 0; --i) bot[i] = bot[i - 1];
+            bot[0] = dn;
+#pragma unroll
+            for (int i = 0; i < K; ++i) top[i] = t[i];
+            if (lane == 0) {       // position 0: the upper stays, the next upper turns lower
+                top[0] = first;
+                bot[0] = second;
+            }
+        }
+        __syncwarp();
+        fetch(ch + 2);
+    }
+    const int r = n % (mp - 1);
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        const int k = lane * K + i;
+        if (k >= npair) continue;
+        const int a = rr_top(k, r, mp), b = rr_bot(k, r, mp);
+        if (a < m) Q[(int64_t)row * m + (rank ? rank[a] : a)] = (double)top[i];
+        if (b < m) Q[(int64_t)row * m + (rank ? rank[b] : b)] = (double)bot[i];
+    }
+}
+
+void jacobi_vectors(Ctx &ctx, int m, const float2 *rlog, const int *nrounds, const int *rank, double *Q) {
+    const int npair = (m + 1) / 2;
+    const size_t smem = 2 * (size_t)JVEC_ROUNDS * npair * sizeof(float2);
+    ctx.before(KC_SMALL_DENSE, 8.0 * m * m, 3.0 * (double)m * m * m * 8);
+#define JV(K) case K: k_jacobi_vectors<K><<<m, 32, smem, ctx.stream>>>(m, rlog, nrounds, rank, Q); break
+    switch ((npair + 31) / 32) {
+        JV(1); JV(2); JV(3); JV(4); JV(5); JV(6);
+        default: k_jacobi_vectors<7><<<m, 32, smem, ctx.stream>>>(m, rlog, nrounds, rank, Q); break;
+    }
+#undef JV
+    ctx.after();
 }
 
 // ---------------------------------------------------------------------------
@@ -1023,10 +1098,11 @@ static size_t syev_base_bytes(int m) {
     return (b + 255) / 256 * 256;
 }
 size_t small_syev_work_bytes(int m) {
-    // the double-float Jacobi's rotation log (one entry per pair and round)
+    // the rotation log (one entry per pair and round, one round more)
     const size_t mp = (size_t)(m + (m & 1));
-    const size_t log = m <= JMAX || m > JDF_MAX ? 0 : (JDF_SWEEPS * (mp - 1) + 1) * (mp / 2) * sizeof(float2);
-    return syev_base_bytes(m) + log;
+    const size_t sweeps = m <= JMAX ? J32_SWEEPS : JDF_SWEEPS;
+    const size_t log = m > JDF_MAX ? 0 : (sweeps * (mp - 1) + 1) * (mp / 2) * sizeof(float2);
+    return syev_base_bytes(m) + log + 32;   // the log starts on 16 bytes and is read in 16s
 }
 
 // ---------------------------------------------------------------------------
@@ -1327,8 +1403,10 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
     double *normA = lam0 + m;             // FRO_PARTS partial sums of ||S||_F^2
     double *oa_part = normA + FRO_PARTS;  // OA_PARTS partial sums of the refinement's ||T - D||_F^2
     int *cnt = reinterpret_cast<int *>(oa_part + OA_PARTS);
-    int32_t *cst = cnt + 4;   // cnt[6]: rounds of the double-float Jacobi
-    float2 *rlog = reinterpret_cast<float2 *>(w + syev_base_bytes(m));
+    int32_t *cst = cnt + 4;   // cnt[6]: rounds of the Jacobi
+    int *label = cst + 4, *csize = label + m;   // label: the FP32 Jacobi's ranks first
+    // 16-byte aligned (work is a multiple of 8 bytes) for the vectors' bulk loads
+    float2 *rlog = reinterpret_cast<float2 *>((reinterpret_cast<uintptr_t>(w + syev_base_bytes(m)) + 15) / 16 * 16);
 
     ctx.before(KC_SMALL_DENSE, 8.0 * m2, 2.0 * m2);
     k_fro<<<FRO_PARTS, 256, 0, ctx.stream>>>(m, S, normA);
@@ -1354,10 +1432,11 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
     // stage 1: eigenvectors to single precision
     raise_smem_limits();
     if (m <= JMAX) {
-        ctx.before(KC_SMALL_DENSE, 24.0 * m2, 9.0 * (double)m * m2 * 8);
-        const size_t smem32 = 2 * (size_t)m * (m | 1) * sizeof(float);
-        k_jacobi32<<<1, 1024, smem32, ctx.stream>>>(m, S, lam0, S0, 40, 1e-6f);
+        const Jacobi32Shape sh(m);
+        ctx.before(KC_SMALL_DENSE, 8.0 * m2, 6.0 * (double)m * m2 * 8);
+        k_jacobi32<<<1, sh.threads, sh.bytes(), ctx.stream>>>(m, S, lam0, label, rlog, cnt + 6, 1e-6f);
         ctx.after();
+        jacobi_vectors(ctx, m, rlog, cnt + 6, label, S0);
     } else {
         ctx.before(KC_SMALL_DENSE, 12.0 * m2, 9.0 * (double)m * m2 * 8);
         cudaLaunchConfig_t cfg = {};
@@ -1375,9 +1454,7 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
             cudaLaunchKernelEx(&cfg, k_jacobi_df, m, S, (const double *)normA, lam0, rlog, cnt + 6, 1e-10f);
         ctx.after();
         if (je != cudaSuccess) return je;
-        ctx.before(KC_SMALL_DENSE, 8.0 * m2, 3.0 * (double)m * m2 * 8);
-        k_jacobi_vectors<<<m, 32, mp * sizeof(float), ctx.stream>>>(m, rlog, cnt + 6, S0);
-        ctx.after();
+        jacobi_vectors(ctx, m, rlog, cnt + 6, nullptr, S0);
     }
     if (mode == 2) {
         // stage 2: three rounds of an orthonormalisation step and a
@@ -1431,7 +1508,6 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
             ctx.after();
             return cudaGetLastError();
         }
-        int *label = cst + 4, *csize = label + m;
         ctx.before(KC_SMALL_DENSE, 24.0 * m2, 4.0 * m2);
         k_oa_components<<<1, 1024, 0, ctx.stream>>>(m, Tm, normA, X0, lam0, label, csize, (double *)Ag,
                                                      (double *)Vg, X1);
