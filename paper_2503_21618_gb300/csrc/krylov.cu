@@ -93,7 +93,7 @@ k_init(int n, int W, int Lp, int N, int m, const double *__restrict__ rhs, int64
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * blockDim.x + tx;
+    const int cg = blockIdx.x * block_cols<T>() + tx;
     const int c0 = cg * VC;
     int j = 0, cl = 0;
     bool act[VC];
@@ -183,7 +183,7 @@ k_spmm_shifted_rb(int n, int W, int Lp, int rows_per_block, const int32_t *__res
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * blockDim.x + tx;
+    const int cg = blockIdx.x * block_cols<T>() + tx;
     const int c0 = cg * VC;
     bool act = false;
     C s = mk((T)0, (T)0);
@@ -284,7 +284,7 @@ k_spmm_shifted_rg(int n, int W, int Lp, int ngroups, int groups_per_block, const
     using AB = typename ABT<T>::type;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * blockDim.x + tx;
+    const int cg = blockIdx.x * block_cols<T>() + tx;
     const int c0 = cg * VC;
     bool act = false;
     C s = mk((T)0, (T)0);
@@ -403,7 +403,7 @@ k_spmm_shifted_nb(int n, int W, int Lp, int ngroups, int groups_per_block, const
     constexpr int VC = 2;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * blockDim.x + tx;
+    const int cg = blockIdx.x * 32 + tx;
     const int c0 = cg * VC;
     bool act = false;
     float2 s = make_float2(0.f, 0.f);
@@ -514,7 +514,7 @@ k_spmm_shifted_sell(int n, int W, int Lp, int C, int nchunks, int chunks_per_blo
     constexpr int VC = 2;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * blockDim.x + tx;
+    const int cg = blockIdx.x * 32 + tx;
     const int c0 = cg * VC;
     bool act = false;
     float2 s = make_float2(0.f, 0.f);
@@ -899,7 +899,7 @@ k_update(int n, int W, int Lp, int N, cplx<T> *__restrict__ R, const cplx<T> *__
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ngl = Lp / VC;
-    const int cgl = blockIdx.x * blockDim.x + tx;
+    const int cgl = blockIdx.x * block_cols<T>() + tx;
     const int c0 = cgl * VC;
     const bool live = cgl < ngl;
     unsigned actmask = 0;   // bit j*VC + v
@@ -1007,7 +1007,7 @@ k_direction(int n, int W, int Lp, int N, const cplx<T> *__restrict__ R, const cp
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * blockDim.x + tx;
+    const int cg = blockIdx.x * block_cols<T>() + tx;
     if (cg >= ng) return;
     const int c0 = cg * VC;
     const int j = c0 / Lp;

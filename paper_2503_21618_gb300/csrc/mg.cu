@@ -152,7 +152,7 @@ k_mg_sspmm(int n, int W, int Lp, int N, int ngroups, const int32_t *__restrict__
     constexpr int UNR = (MODE == MG_DOWN) ? 4 : 2;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * blockDim.x + tx;
+    const int cg = blockIdx.x * block_cols<T>() + tx;
     const int c0 = cg * VC;
     bool act = false;
     int j = 0;
@@ -273,7 +273,7 @@ k_mg_xfer(int n_out, int W, int rows_per_block, const int32_t *__restrict__ ptr,
     constexpr int UNR = 4;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * blockDim.x + tx;
+    const int cg = blockIdx.x * block_cols<T>() + tx;
     if (cg >= ng) return;
     const int c0 = cg * VC;
     if (!col_active<VC>(flag, c0)) return;
@@ -324,7 +324,7 @@ k_mg_jacobi0(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, cons
              cplx<T> *__restrict__ Out, const int32_t *__restrict__ flag) {
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * blockDim.x + tx;
+    const int cg = blockIdx.x * block_cols<T>() + tx;
     if (cg >= ng) return;
     const int c0 = cg * VC;
     if (!col_active<VC>(flag, c0)) return;
@@ -346,7 +346,7 @@ k_mg_scale(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, const 
            cplx<T> *__restrict__ Out, const int32_t *__restrict__ flag) {
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * blockDim.x + tx;
+    const int cg = blockIdx.x * block_cols<T>() + tx;
     if (cg >= ng) return;
     const int c0 = cg * VC;
     if (!col_active<VC>(flag, c0)) return;
@@ -486,7 +486,7 @@ k_mg_rz(int n, int W, const cplx<T> *__restrict__ Rv, const cplx<T> *__restrict_
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
-    const int cg = blockIdx.x * blockDim.x + tx;
+    const int cg = blockIdx.x * block_cols<T>() + tx;
     const int c0 = cg * VC;
     C rz[VC];
 #pragma unroll
