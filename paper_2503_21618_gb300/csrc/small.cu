@@ -524,8 +524,8 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *__restri
 // double-float arithmetic (hi + lo FP32 pairs, ~46 bits).
 //
 // The FP64 Jacobi over the whole GPU (k_jacobi_coop) is bound by its grid
-// barriers and the FP64 pipe (32 ms at m = 300; this kernel 11.6).  FP32 rotations would do for
-// the accuracy, since the vectors are refined in FP64 afterwards, but the
+// barriers and the FP64 pipe (32 ms at m = 300).  FP32 rotations would do for the
+// accuracy, since the vectors are refined in FP64 afterwards, but the
 // eigenvectors' signs come out of the rotation path: where two diagonal
 // entries are close an FP32 rounding turns a rotation by 45 degrees the other
 // way.  In double-float the path is the FP64 one (a decision differs only
@@ -536,14 +536,19 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *__restri
 // memory of the C CTAs.  Position k of a round holds the pair (a_k, b_k).  A CTA
 // owns a contiguous range of positions and the two full rows of each; from one
 // round to the next the upper rows move down one position and the lower rows
-// up one, so per round a CTA hands one row to each neighbour (DSMEM) and the
-// rest stay where they are.  Per round:
-//   update    the 2 x 2 blocks (k, l) of the own positions k and all l, rows
-//             and columns in one pass (A is kept in full, so the columns of a
-//             block are two contiguous runs); block barrier
-//   rotations of the next round from the own rows and the diagonal, which
-//             every CTA keeps in full (updated in closed form); they go to all
-//             CTAs while the boundary rows move; one cluster barrier
+// up one, so per round a CTA hands one row to each neighbour and the rest stay
+// where they are.  Per round, between a block barrier (the inputs of the
+// rotations are taken) and a cluster barrier:
+//   update    (warps 1 ..) the 2 x 2 blocks (k, l) of the own positions k and
+//             all l, rows and columns in one pass (A is kept in full, so the
+//             columns of a block are two contiguous runs); the two rows that
+//             move are written straight into the neighbours' free rows (DSMEM)
+//   rotations (warp 0) of the next round, one lane per position, from the one
+//             2 x 2 block each depends on and the diagonal, which every CTA
+//             keeps in full (updated in closed form); they go to all CTAs
+// The chain of double-float square roots and divisions (~1 us) thus hides behind
+// the update: 8.3 ms at m = 300 on 16 CTAs, against 11.6 ms on 8 with it, and the
+// rows' move, after the update.
 // The eigenvectors are not formed here: the rotations are logged (FP32) and
 // k_jacobi_vectors applies them to the rows of I afterwards, every row on its
 // own SM.  A rotation is skipped below rel_tol of sqrt(|a_pp a_qq|); the
@@ -551,9 +556,10 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *__restri
 // Output: lam (FP64, unsorted), the log and *nrounds.
 // ---------------------------------------------------------------------------
 constexpr int JDF_MAX = 448;      // a CTA's rows of an 8-CTA cluster in 227 KB
-constexpr int JDF_CTAS = 8;
+constexpr int JDF_CTAS = 8, JDF_CTAS_WIDE = 16;
 constexpr int JDF_SWEEPS = 20;
-constexpr int JDF_THREADS = 512;
+constexpr int JDF_THREADS = 544;  // 16 warps for the update, one for the rotations
+static_assert(JDF_MAX <= 2 * 32 * JDF_CTAS, "one lane of warp 0 per position of a CTA");
 constexpr int JVEC_ROUNDS = 8;    // rounds of the log per stage of k_jacobi_vectors
 static_assert(JDF_MAX <= 2 * 32 * 7, "k_jacobi_vectors holds at most 7 positions per lane");
 
@@ -654,7 +660,7 @@ k_jacobi_df(int m, const double *__restrict__ S, const double *__restrict__ fro_
     __shared__ int nbfree[2][2];    // free slot of the lower / upper neighbour, by round parity
     __shared__ int myfree[2][2];    // own free slots for an upper / a lower row, by round parity
     __shared__ int mx[2];           // largest relative pivot of a sweep (float bits), by sweep parity
-    __shared__ int allmx[JDF_CTAS]; // the CTAs' mx of the sweep that ends
+    __shared__ int allmx[JDF_CTAS_WIDE]; // the CTAs' mx of the sweep that ends
     __shared__ float absmin;
     __shared__ int scale;           // ||S||_F < 2^scale; A holds S 2^-scale
     const int tid = threadIdx.x, bs = blockDim.x;
@@ -731,6 +737,41 @@ k_jacobi_df(int m, const double *__restrict__ S, const double *__restrict__ fro_
         for (int r = 0; r < mp - 1; ++r) {
             const float4 *P = par + cur * npair;
             const int *sT = slot_of(cur, 0), *sB = slot_of(cur, 1);
+            const int nxt = cur ^ 1, r1 = r + 1 == mp - 1 ? 0 : r + 1, s1 = r1 ? sweep : sweep + 1;
+            // Warp 0 forms the rotations of the next round: each needs one
+            // element as this round's update will leave it, so its block's
+            // inputs are taken before the update starts.  Element (a', b') of
+            // position k: rows and columns of the present positions kr and lc.
+            const bool mine = warp == 0 && lane < cnt;
+            df x00, x01, x10, x11;
+            float4 pr, pc;
+            bool row_low = false, col_low = true;
+            if (mine) {
+                const int k = k0 + lane;
+                int kr = lane + 1, lc = k - 1;                       // (a_{k+1}, b_{k-1})
+                if (k == 0) {                                        // (a_0, a_1)
+                    kr = 0;
+                    lc = 1;
+                    col_low = false;
+                } else if (lane + 1 == cnt) {
+                    row_low = true;
+                    if (last) {                                      // (b_k, b_{k-1})
+                        kr = lane;
+                    } else {                                         // (b_{k-1}, a_{k+1}): a_{k+1} is elsewhere
+                        kr = lane - 1;
+                        lc = k + 1;
+                        col_low = false;
+                    }
+                }
+                const df *ra = rows + (size_t)sT[kr] * ld, *rb = rows + (size_t)sB[kr] * ld;
+                const int a = rr_top(lc, r, mp), b = rr_bot(lc, r, mp);
+                x00 = ra[a];
+                x01 = ra[b];
+                x10 = rb[a];
+                x11 = rb[b];
+                pr = P[k0 + kr];
+                pc = P[lc];
+            }
             for (int l = tid; l < npair; l += bs) {
                 const df da = pda[cur * npair + l];
                 if (da.h != 0.f) {
@@ -739,70 +780,77 @@ k_jacobi_df(int m, const double *__restrict__ S, const double *__restrict__ fro_
                     diag[b] = df_add(diag[b], df_neg(da));
                 }
             }
-            // tasks (position j, 32 positions l), dealt to the warps
-            int j = warp, l0 = 0;
-            while (j >= cnt) {
-                j -= cnt;
-                l0 += 32;
-            }
-            while (l0 < npair) {
-                const int k = k0 + j, l = l0 + lane;
-                if (l < npair) {
-                    const float4 pk = P[k], pl = P[l];
-                    if (pk.z != 0.f || pl.z != 0.f) {
-                        df *ra = rows + (size_t)sT[j] * ld, *rb = rows + (size_t)sB[j] * ld;
-                        const int a = rr_top(l, r, mp), b = rr_bot(l, r, mp);
-                        if (l == k) {   // the pivot; the diagonal lives in diag
-                            ra[b] = {0.f, 0.f};
-                            rb[a] = {0.f, 0.f};
-                        } else {
-                            const df ck = {pk.x, pk.y}, sk = {pk.z, pk.w}, cl_ = {pl.x, pl.y}, sl = {pl.z, pl.w};
-                            const df xaa = ra[a], xab = ra[b], xba = rb[a], xbb = rb[b];
-                            const df yaa = df_rot(ck, xaa, sk, xba), yab = df_rot(ck, xab, sk, xbb);
-                            const df yba = df_rot(sk, xaa, df_neg(ck), xba), ybb = df_rot(sk, xab, df_neg(ck), xbb);
-                            ra[a] = df_rot(cl_, yaa, sl, yab);
-                            ra[b] = df_rot(sl, yaa, df_neg(cl_), yab);
-                            rb[a] = df_rot(cl_, yba, sl, ybb);
-                            rb[b] = df_rot(sl, yba, df_neg(cl_), ybb);
-                        }
+            __syncthreads();
+            if (warp == 0) {
+                if (mine) {
+                    const int k = k0 + lane;
+                    df apq;
+                    if (pr.z != 0.f || pc.z != 0.f) {
+                        const df ck = {pr.x, pr.y}, sk = {pr.z, pr.w}, cl_ = {pc.x, pc.y}, sl = {pc.z, pc.w};
+                        const df u = row_low ? sk : ck, v = row_low ? df_neg(ck) : sk;
+                        const df y0 = df_rot(u, x00, v, x10), y1 = df_rot(u, x01, v, x11);
+                        apq = col_low ? df_rot(sl, y0, df_neg(cl_), y1) : df_rot(cl_, y0, sl, y1);
+                    } else {
+                        apq = row_low ? (col_low ? x11 : x10) : (col_low ? x01 : x00);
                     }
+                    rotation(k, rr_top(k, r1, mp), rr_bot(k, r1, mp), apq, s1, g + 1, nxt);
                 }
-                j += nwarp;
+            } else {
+                // The update: tasks (position j, 32 positions l), dealt to the
+                // other warps.  The lowest upper row and the highest lower row
+                // are written where the neighbours expect them, every element.
+                df *const out_lo = c > 0 ? cl.map_shared_rank(rows, c - 1) + (size_t)nbfree[cur][0] * ld : nullptr;
+                df *const out_hi = last ? nullptr : cl.map_shared_rank(rows, c + 1) + (size_t)nbfree[cur][1] * ld;
+                int j = warp - 1, l0 = 0;
                 while (j >= cnt) {
                     j -= cnt;
                     l0 += 32;
                 }
+                while (l0 < npair) {
+                    const int k = k0 + j, l = l0 + lane;
+                    if (l < npair) {
+                        const float4 pk = P[k], pl = P[l];
+                        const bool to_lo = j == 0 && c > 0, to_hi = j == cnt - 1 && !last;
+                        if (pk.z != 0.f || pl.z != 0.f || to_lo || to_hi) {
+                            df *ra = rows + (size_t)sT[j] * ld, *rb = rows + (size_t)sB[j] * ld;
+                            df *wa = to_lo ? out_lo : ra, *wb = to_hi ? out_hi : rb;
+                            const int a = rr_top(l, r, mp), b = rr_bot(l, r, mp);
+                            if (l == k) {   // the pivot; the diagonal lives in diag
+                                wa[b] = {0.f, 0.f};
+                                wb[a] = {0.f, 0.f};
+                            } else {
+                                df xaa = ra[a], xab = ra[b], xba = rb[a], xbb = rb[b];
+                                if (pk.z != 0.f || pl.z != 0.f) {
+                                    const df ck = {pk.x, pk.y}, sk = {pk.z, pk.w}, cl_ = {pl.x, pl.y}, sl = {pl.z, pl.w};
+                                    const df yaa = df_rot(ck, xaa, sk, xba), yab = df_rot(ck, xab, sk, xbb);
+                                    const df yba = df_rot(sk, xaa, df_neg(ck), xba), ybb = df_rot(sk, xab, df_neg(ck), xbb);
+                                    xaa = df_rot(cl_, yaa, sl, yab);
+                                    xab = df_rot(sl, yaa, df_neg(cl_), yab);
+                                    xba = df_rot(cl_, yba, sl, ybb);
+                                    xbb = df_rot(sl, yba, df_neg(cl_), ybb);
+                                }
+                                wa[a] = xaa;
+                                wa[b] = xab;
+                                wb[a] = xba;
+                                wb[b] = xbb;
+                            }
+                        }
+                    }
+                    j += nwarp - 1;
+                    while (j >= cnt) {
+                        j -= cnt;
+                        l0 += 32;
+                    }
+                }
             }
-            __syncthreads();
             ++g;
-            const int nxt = cur ^ 1, r1 = r + 1 == mp - 1 ? 0 : r + 1, s1 = r1 ? sweep : sweep + 1;
-            // rotations of the next round, at the positions after the move
-            for (int jj = tid; jj < cnt; jj += bs) {
-                const int k = k0 + jj, a = rr_top(k, r1, mp), b = rr_bot(k, r1, mp);
-                df apq;
-                if (c == 0 && jj == 0) apq = rows[(size_t)sT[0] * ld + b];
-                else if (jj + 1 < cnt) apq = rows[(size_t)sT[jj + 1] * ld + b];
-                else if (last) apq = rows[(size_t)sB[jj] * ld + b];
-                else apq = rows[(size_t)sB[jj - 1] * ld + a];   // the upper row is on its way: the lower one's entry
-                rotation(k, a, b, apq, s1, g, nxt);
-            }
             // the rows' new slots
             int *nT = slot_of(nxt, 0), *nB = slot_of(nxt, 1);
             for (int jj = bs - 1 - tid; jj < cnt; jj += bs) {
                 nT[jj] = c == 0 && jj == 0 ? sT[0] : jj + 1 < cnt ? sT[jj + 1] : last ? sB[cnt - 1] : myfree[cur][0];
                 nB[jj] = jj > 0 ? sB[jj - 1] : c == 0 ? sT[1] : myfree[cur][1];
             }
-            if (warp == nwarp / 2 && c > 0) {          // the lowest upper row to the lower neighbour
-                const float4 *src = reinterpret_cast<const float4 *>(rows + (size_t)sT[0] * ld);
-                float4 *dst = reinterpret_cast<float4 *>(cl.map_shared_rank(rows, c - 1) + (size_t)nbfree[cur][0] * ld);
-                for (int q = lane; q < ld / 2; q += 32) dst[q] = src[q];
-            }
-            if (warp == nwarp / 2 + 1 && !last) {      // the highest lower row to the upper neighbour
-                const float4 *src = reinterpret_cast<const float4 *>(rows + (size_t)sB[cnt - 1] * ld);
-                float4 *dst = reinterpret_cast<float4 *>(cl.map_shared_rank(rows, c + 1) + (size_t)nbfree[cur][1] * ld);
-                for (int q = lane; q < ld / 2; q += 32) dst[q] = src[q];
-            }
-            if (warp == nwarp / 2 + 2 && lane == 0) {
+            if (warp == nwarp / 2 && lane == 0) {
                 const int fT = c == 0 ? sB[cnt - 1] : sT[0], fB = last ? sT[0] : sB[cnt - 1];
                 myfree[nxt][0] = fT;
                 myfree[nxt][1] = fB;
@@ -1387,6 +1435,37 @@ static cudaError_t coop_jacobi(Ctx &ctx, int m, double *A, double *V, double *la
     return cudaEventSynchronize(done);
 }
 
+// CTAs of the double-float Jacobi's cluster on the current device: 16 if the
+// device places clusters of that size (not a portable one), else 8.  The result
+// does not depend on it.
+static int jacobi_df_ctas() {
+    constexpr int kMaxDevices = 64;
+    static std::once_flag once[kMaxDevices];
+    static int ctas[kMaxDevices];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int i = dev < 0 || dev >= kMaxDevices ? 0 : dev;
+    std::call_once(once[i], [i] {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = JDF_CTAS_WIDE;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.gridDim = dim3(JDF_CTAS_WIDE);
+        cfg.blockDim = dim3(JDF_THREADS);
+        cfg.dynamicSmemBytes = JacobiShape(JDF_MAX, JDF_CTAS_WIDE).bytes();
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        const bool wide =
+            cudaFuncSetAttribute(k_jacobi_df, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&n, k_jacobi_df, &cfg) == cudaSuccess && n > 0;
+        if (!wide) cudaGetLastError();
+        ctas[i] = wide ? JDF_CTAS_WIDE : JDF_CTAS;
+    });
+    return ctas[i];
+}
+
 cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q, double *work, int mode) {
     const size_t m2 = (size_t)m * m;
     const size_t mp = (size_t)(m + (m & 1));
@@ -1442,11 +1521,12 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = JDF_CTAS;
+        const int ctas = jacobi_df_ctas();
+        attr.val.clusterDim.x = ctas;
         attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-        cfg.gridDim = dim3(JDF_CTAS);
+        cfg.gridDim = dim3(ctas);
         cfg.blockDim = dim3(JDF_THREADS);
-        cfg.dynamicSmemBytes = JacobiShape(m, JDF_CTAS).bytes();
+        cfg.dynamicSmemBytes = JacobiShape(m, ctas).bytes();
         cfg.stream = ctx.stream;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
