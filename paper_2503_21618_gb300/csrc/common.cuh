@@ -172,6 +172,19 @@ __device__ __forceinline__ void l2_prefetch_warp(const void *p, int64_t bytes, i
 template <typename T> __device__ __forceinline__ int block_cols() { return sizeof(T) == 4 ? 32 : blockDim.x; }
 
 // ---------------------------------------------------------------------------
+// Chained launches (launch_chained): the kernel may be scheduled while the one
+// before it still runs.  Its first statement waits until that one has finished
+// and its writes are visible, then lets the next one be scheduled.  Inputs that
+// earlier kernels of the chain write are plain pointers there, not const
+// __restrict__: a read-only load is only for data that nobody writes while the
+// kernel is on the device.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
 // Per-column reduction of the Krylov kernels' partial sums (gy rows of W x 4
 // values): one block of COL_SUM_THREADS threads per column, FP64 sums in a
 // fixed order, valid in thread 0.  Latency-bound (a few hundred loads per

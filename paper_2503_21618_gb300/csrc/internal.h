@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <stdint.h>
 
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
@@ -127,6 +128,27 @@ struct KrylovBuffers {
 };
 
 int krylov_row_groups(const Ctx &ctx, const KrylovDims &d, int prec_fp32);
+
+// Launch of a kernel that begins with chain_wait(): overlaps its launch and the
+// scheduling of its blocks with the end of the kernel before it on the stream.
+// The Krylov iteration and the cycle are chains of 15 to 20 short launches, each
+// waiting for the last: plain FP64 solve of the 1D pencil (n = 2000) 19.7 -> 17.5
+// ms, of the 2D pencil (n = 10 000) 102.7 -> 97.8.
+template <typename... KA, typename... A>
+inline void launch_chained(Ctx &ctx, void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem,
+                           A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = ctx.stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);   // an error stays as the stream's last error
+}
 
 // Block shape of the kernels whose thread (tx, ty) owns a column group and
 // every blockDim.y-th row: gx blocks of bx x 8 threads over the groups.  A

@@ -178,8 +178,9 @@ template <typename T, int VC, int UNR>
 __global__ void __launch_bounds__(32 * TY)
 k_spmm_shifted_rb(int n, int W, int Lp, int rows_per_block, const int32_t *__restrict__ rowptr,
                   const int32_t *__restrict__ col, const typename ABT<T>::type *__restrict__ ab,
-                  const cplx<T> *__restrict__ sig, const cplx<T> *__restrict__ P, cplx<T> *__restrict__ Q,
-                  const int32_t *__restrict__ flag, T *__restrict__ part) {
+                  const cplx<T> *sig, const cplx<T> *P, cplx<T> *__restrict__ Q,
+                  const int32_t *flag, T *__restrict__ part) {
+    chain_wait();
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
@@ -892,10 +893,11 @@ static void launch_staged(Ctx &ctx, const KrylovDims &d, const DevPencil &A, con
 // read here: the block the cycle's gathered products read.
 template <typename T, int VC, int NP, bool JAC, bool MGY>
 __global__ void __launch_bounds__(32 * TY)
-k_update(int n, int W, int Lp, int N, cplx<T> *__restrict__ R, const cplx<T> *__restrict__ P,
-         cplx<T> *__restrict__ Q, const cplx<T> *__restrict__ dinv, const cplx<T> *__restrict__ alpha,
-         const cplx<T> *__restrict__ ua, const int32_t *__restrict__ flag, T *__restrict__ U,
+k_update(int n, int W, int Lp, int N, cplx<T> *__restrict__ R, const cplx<T> *P,
+         cplx<T> *__restrict__ Q, const cplx<T> *__restrict__ dinv, const cplx<T> *alpha,
+         const cplx<T> *ua, const int32_t *flag, T *__restrict__ U,
          T *__restrict__ part) {
+    chain_wait();
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ngl = Lp / VC;
@@ -1001,9 +1003,10 @@ k_update(int n, int W, int Lp, int N, cplx<T> *__restrict__ R, const cplx<T> *__
 // ---------------------------------------------------------------------------
 template <typename T, int VC, bool MGZ>
 __global__ void __launch_bounds__(32 * TY)
-k_direction(int n, int W, int Lp, int N, const cplx<T> *__restrict__ R, const cplx<T> *__restrict__ Z,
-            cplx<T> *__restrict__ P, const cplx<T> *__restrict__ dinv, const cplx<T> *__restrict__ beta,
-            const int32_t *__restrict__ flag, int init) {
+k_direction(int n, int W, int Lp, int N, const cplx<T> *R, const cplx<T> *Z,
+            cplx<T> *__restrict__ P, const cplx<T> *__restrict__ dinv, const cplx<T> *beta,
+            const int32_t *flag, int init) {
+    chain_wait();
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
@@ -1049,7 +1052,8 @@ k_direction(int n, int W, int Lp, int N, const cplx<T> *__restrict__ R, const cp
 // per-column reductions (one block per column, FP64)
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void k_reduce_init(int W, int gy, const T *__restrict__ part, KrylovScalars<T> s) {
+__global__ void k_reduce_init(int W, int gy, const T *part, KrylovScalars<T> s) {
+    chain_wait();
     const int col = blockIdx.x;
     double s0, s1, s2;
     col_sum3(part, gy, W, col, s0, s1, s2);
@@ -1063,7 +1067,8 @@ __global__ void k_reduce_init(int W, int gy, const T *__restrict__ part, KrylovS
 }
 
 template <typename T>
-__global__ void k_reduce_alpha(int W, int gy, const T *__restrict__ part, KrylovScalars<T> s) {
+__global__ void k_reduce_alpha(int W, int gy, const T *part, KrylovScalars<T> s) {
+    chain_wait();
     const int col = blockIdx.x;
     double s0, s1, s2;
     col_sum3(part, gy, W, col, s0, s1, s2);
@@ -1084,8 +1089,9 @@ __global__ void k_reduce_alpha(int W, int gy, const T *__restrict__ part, Krylov
 }
 
 template <typename T>
-__global__ void k_reduce_beta(int W, int gy, const T *__restrict__ part, KrylovScalars<T> s, double tol2,
+__global__ void k_reduce_beta(int W, int gy, const T *part, KrylovScalars<T> s, double tol2,
                               int maxit) {
+    chain_wait();
     const int col = blockIdx.x;
     double s0, s1, s2;
     col_sum3(part, gy, W, col, s0, s1, s2);
@@ -1115,7 +1121,8 @@ __global__ void k_reduce_beta(int W, int gy, const T *__restrict__ part, KrylovS
     }
 }
 
-__global__ void k_count_active(int W, const int32_t *__restrict__ flag, int32_t *__restrict__ count) {
+__global__ void k_count_active(int W, const int32_t *flag, int32_t *__restrict__ count) {
+    chain_wait();
     __shared__ int tot;
     if (threadIdx.x == 0) tot = 0;
     __syncthreads();
@@ -1135,7 +1142,8 @@ __global__ void k_set_columns(int W, int Lp, int m, PoleSet<T> ps, int32_t *__re
 }
 
 template <typename T>
-__global__ void k_reduce_mu(int W, int gy, const T *__restrict__ part, cplx<T> *__restrict__ mu, int Lp, int m) {
+__global__ void k_reduce_mu(int W, int gy, const T *part, cplx<T> *__restrict__ mu, int Lp, int m) {
+    chain_wait();
     const int col = blockIdx.x;
     double s0, s1, s2;
     col_sum3(part, gy, W, col, s0, s1, s2);
@@ -1185,7 +1193,7 @@ template <typename T>
 void krylov_reduce_init(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb) {
     const int W = d.W();
     ctx.before(KC_KRYLOV_REDUCE, (double)kb.gy * W * 4 * sizeof(T), 0);
-    k_reduce_init<T><<<W, COL_SUM_THREADS, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s);
+    launch_chained(ctx, k_reduce_init<T>, W, COL_SUM_THREADS, 0, W, kb.gy, kb.s.part, kb.s);
     ctx.after();
 }
 
@@ -1249,7 +1257,7 @@ void krylov_spmm(Ctx &ctx, const KrylovDims &d, const DevPencil &A, const cplx<T
 #undef RGL
     } else {
         const int rpb = (d.n + gy - 1) / gy;
-        k_spmm_shifted_rb<T, VC, 4><<<grid, block, 0, ctx.stream>>>(d.n, W, d.Lp, rpb, A.rowptr, A.col, abp, sig, P,
+        launch_chained(ctx, k_spmm_shifted_rb<T, VC, 4>, grid, block, 0, d.n, W, d.Lp, rpb, A.rowptr, A.col, abp, sig, P,
                                                                      Q, flag, part);
     }
     ctx.after();
@@ -1267,7 +1275,7 @@ template <typename T>
 void krylov_reduce_alpha(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb) {
     const int W = d.W();
     ctx.before(KC_KRYLOV_REDUCE, (double)kb.gy * W * 4 * sizeof(T), 0);
-    k_reduce_alpha<T><<<W, COL_SUM_THREADS, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s);
+    launch_chained(ctx, k_reduce_alpha<T>, W, COL_SUM_THREADS, 0, W, kb.gy, kb.s.part, kb.s);
     ctx.after();
 }
 
@@ -1282,15 +1290,15 @@ static void launch_update(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb) {
                (kb.mgd ? 5 : 4) * vb + 2.0 * d.n * d.Lp * sizeof(T) + (double)d.n * d.N * sizeof(cplx<T>),
                16.0 * d.n * W * d.frac);
     if (kb.Z && kb.mgd)
-        k_update<T, VC, NP, false, true><<<grid, block, 0, ctx.stream>>>(d.n, W, d.Lp, d.N, kb.R, kb.P, kb.Q, kb.mgd,
+        launch_chained(ctx, k_update<T, VC, NP, false, true>, grid, block, 0, d.n, W, d.Lp, d.N, kb.R, kb.P, kb.Q, kb.mgd,
                                                                           kb.s.alpha, kb.s.ua, kb.s.flag, kb.Uacc,
                                                                           kb.s.part);
     else if (kb.Z)
-        k_update<T, VC, NP, false, false><<<grid, block, 0, ctx.stream>>>(d.n, W, d.Lp, d.N, kb.R, kb.P, kb.Q,
+        launch_chained(ctx, k_update<T, VC, NP, false, false>, grid, block, 0, d.n, W, d.Lp, d.N, kb.R, kb.P, kb.Q,
                                                                            kb.dinv, kb.s.alpha, kb.s.ua, kb.s.flag,
                                                                            kb.Uacc, kb.s.part);
     else
-        k_update<T, VC, NP, true, false><<<grid, block, 0, ctx.stream>>>(d.n, W, d.Lp, d.N, kb.R, kb.P, kb.Q, kb.dinv,
+        launch_chained(ctx, k_update<T, VC, NP, true, false>, grid, block, 0, d.n, W, d.Lp, d.N, kb.R, kb.P, kb.Q, kb.dinv,
                                                                           kb.s.alpha, kb.s.ua, kb.s.flag, kb.Uacc,
                                                                           kb.s.part);
     ctx.after();
@@ -1312,7 +1320,7 @@ template <typename T>
 void krylov_reduce_beta(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb, double tol2, int maxit) {
     const int W = d.W();
     ctx.before(KC_KRYLOV_REDUCE, (double)kb.gy * W * 4 * sizeof(T), 0);
-    k_reduce_beta<T><<<W, COL_SUM_THREADS, 0, ctx.stream>>>(W, kb.gy, kb.s.part, kb.s, tol2, maxit);
+    launch_chained(ctx, k_reduce_beta<T>, W, COL_SUM_THREADS, 0, W, kb.gy, kb.s.part, kb.s, tol2, maxit);
     ctx.after();
 }
 
@@ -1326,17 +1334,17 @@ void krylov_direction(Ctx &ctx, const KrylovDims &d, KrylovBuffers<T> &kb, int i
     ctx.before(KC_KRYLOV_DIR, (init ? 2 : 3) * vb + (kb.Z ? 0.0 : (double)d.n * d.N * sizeof(cplx<T>)),
                10.0 * d.n * W * d.frac);
     if (kb.Z)
-        k_direction<T, VC, true><<<grid, block, 0, ctx.stream>>>(d.n, W, d.Lp, d.N, kb.R, kb.Z, kb.P, kb.dinv,
+        launch_chained(ctx, k_direction<T, VC, true>, grid, block, 0, d.n, W, d.Lp, d.N, kb.R, kb.Z, kb.P, kb.dinv,
                                                                  kb.s.beta, kb.s.flag, init);
     else
-        k_direction<T, VC, false><<<grid, block, 0, ctx.stream>>>(d.n, W, d.Lp, d.N, kb.R, kb.Z, kb.P, kb.dinv,
+        launch_chained(ctx, k_direction<T, VC, false>, grid, block, 0, d.n, W, d.Lp, d.N, kb.R, kb.Z, kb.P, kb.dinv,
                                                                   kb.s.beta, kb.s.flag, init);
     ctx.after();
 }
 
 void krylov_count_active(Ctx &ctx, int W, const int32_t *flag, int32_t *count) {
     ctx.before(KC_KRYLOV_REDUCE, 4.0 * W, 0);
-    k_count_active<<<1, 256, 0, ctx.stream>>>(W, flag, count);
+    launch_chained(ctx, k_count_active, 1, 256, 0, W, flag, count);
     ctx.after();
 }
 
@@ -1344,7 +1352,7 @@ template <typename T>
 void krylov_reduce_mu(Ctx &ctx, const KrylovDims &d, const T *part, int gy, cplx<T> *mu) {
     const int W = d.W();
     ctx.before(KC_KRYLOV_REDUCE, (double)gy * W * 4 * sizeof(T), 0);
-    k_reduce_mu<T><<<W, COL_SUM_THREADS, 0, ctx.stream>>>(W, gy, part, mu, d.Lp, d.m);
+    launch_chained(ctx, k_reduce_mu<T>, W, COL_SUM_THREADS, 0, W, gy, part, mu, d.Lp, d.m);
     ctx.after();
 }
 

@@ -143,10 +143,11 @@ template <typename T, int VC, int R, int MODE>
 __global__ void __launch_bounds__(32 * TY, sizeof(T) == 4 ? 6 : 4)
 k_mg_sspmm(int n, int W, int Lp, int N, int ngroups, const int32_t *__restrict__ gptr,
            const int32_t *__restrict__ ucol, const cplx<T> *__restrict__ uab, const cplx<T> *__restrict__ sig,
-           const cplx<T> *__restrict__ dinv, const cplx<T> *__restrict__ X, const cplx<T> *__restrict__ Rv,
-           cplx<T> *__restrict__ Out, const int32_t *__restrict__ flag, T *__restrict__ part,
+           const cplx<T> *__restrict__ dinv, const cplx<T> *X, const cplx<T> *Rv,
+           cplx<T> *__restrict__ Out, const int32_t *flag, T *__restrict__ part,
            const int32_t *__restrict__ g2ptr, const int32_t *__restrict__ u2col, const cplx<T> *__restrict__ u2ab,
-           const cplx<T> *__restrict__ X2) {
+           const cplx<T> *X2) {
+    chain_wait();
     using C = cplx<T>;
     constexpr bool DOTS = MODE == MG_SMOOTH || MODE == MG_UP;
     constexpr int UNR = (MODE == MG_DOWN) ? 4 : 2;
@@ -268,7 +269,8 @@ k_mg_sspmm(int n, int W, int Lp, int N, int ngroups, const int32_t *__restrict__
 template <typename T, int VC, int MODE>
 __global__ void __launch_bounds__(32 * TY)
 k_mg_xfer(int n_out, int W, int rows_per_block, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
-          const T *__restrict__ val, const cplx<T> *__restrict__ X, cplx<T> *Out, const int32_t *__restrict__ flag) {
+          const T *__restrict__ val, const cplx<T> *X, cplx<T> *Out, const int32_t *flag) {
+    chain_wait();
     using C = cplx<T>;
     constexpr int UNR = 4;
     const int tx = threadIdx.x, ty = threadIdx.y;
@@ -320,8 +322,9 @@ k_mg_xfer(int n_out, int W, int rows_per_block, const int32_t *__restrict__ ptr,
 // out = D r (first pre-smoothing sweep from a zero iterate)
 template <typename T, int VC>
 __global__ void __launch_bounds__(32 * TY)
-k_mg_jacobi0(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, const cplx<T> *__restrict__ Rv,
-             cplx<T> *__restrict__ Out, const int32_t *__restrict__ flag) {
+k_mg_jacobi0(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, const cplx<T> *Rv,
+             cplx<T> *__restrict__ Out, const int32_t *flag) {
+    chain_wait();
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
     const int cg = blockIdx.x * block_cols<T>() + tx;
@@ -342,8 +345,9 @@ k_mg_jacobi0(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, cons
 // y = D x on the finest level (the block the DOWN / UP products gather)
 template <typename T, int VC>
 __global__ void __launch_bounds__(32 * TY)
-k_mg_scale(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, const cplx<T> *__restrict__ Xv,
-           cplx<T> *__restrict__ Out, const int32_t *__restrict__ flag) {
+k_mg_scale(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, const cplx<T> *Xv,
+           cplx<T> *__restrict__ Out, const int32_t *flag) {
+    chain_wait();
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
     const int cg = blockIdx.x * block_cols<T>() + tx;
@@ -376,8 +380,9 @@ k_mg_scale(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, const 
 //    exposed load every 32 steps) and 141 us with 32 x 32 tiles.
 template <typename T>
 __global__ void __launch_bounds__(128)
-k_mg_coarse_split(int nc, int W, int Lp, int N, int trans, const T *__restrict__ V, const cplx<T> *__restrict__ X,
-                  const cplx<T> *__restrict__ cinv, cplx<T> *__restrict__ Out, const int32_t *__restrict__ flag) {
+k_mg_coarse_split(int nc, int W, int Lp, int N, int trans, const T *__restrict__ V, const cplx<T> *X,
+                  const cplx<T> *cinv, cplx<T> *__restrict__ Out, const int32_t *flag) {
+    chain_wait();
     using C = cplx<T>;
     constexpr int KW = 4, U = 8;
     __shared__ C red[KW][32];
@@ -424,8 +429,9 @@ k_mg_coarse_split(int nc, int W, int Lp, int N, int trans, const T *__restrict__
 
 template <typename T>
 __global__ void __launch_bounds__(128)
-k_mg_coarse_gemm(int nc, int W, int Lp, int N, int trans, const T *__restrict__ V, const cplx<T> *__restrict__ X,
-                 const cplx<T> *__restrict__ cinv, cplx<T> *__restrict__ Out, const int32_t *__restrict__ flag) {
+k_mg_coarse_gemm(int nc, int W, int Lp, int N, int trans, const T *__restrict__ V, const cplx<T> *X,
+                 const cplx<T> *cinv, cplx<T> *__restrict__ Out, const int32_t *flag) {
+    chain_wait();
     using C = cplx<T>;
     constexpr int RT = 4, TR = 8 * RT, TC = 16, TK = 32;
     __shared__ T sV[TR][TK + 1];
@@ -481,8 +487,9 @@ k_mg_coarse_gemm(int nc, int W, int Lp, int N, int trans, const T *__restrict__ 
 // partial r^T z per column (used when the hierarchy is a single level)
 template <typename T, int VC>
 __global__ void __launch_bounds__(32 * TY)
-k_mg_rz(int n, int W, const cplx<T> *__restrict__ Rv, const cplx<T> *__restrict__ Z, const int32_t *__restrict__ flag,
+k_mg_rz(int n, int W, const cplx<T> *Rv, const cplx<T> *Z, const int32_t *flag,
         T *__restrict__ part) {
+    chain_wait();
     using C = cplx<T>;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int ng = W / VC;
@@ -578,7 +585,7 @@ void launch_sspmm(Ctx &ctx, const KrylovDims &d, int kc, int n_rows, int R, int 
     if (MODE == MG_UP) bytes += 4.0 * (ngroups + 1) + (double)nnz2 * (4 + R * sizeof(cplx<T>)) + vec_bytes<T>(d, n2);
     ctx.before(kc, bytes, 8.0 * (double)(nnz_union + nnz2) * R * W * d.frac);
 #define SSP(RR)                                                                                                     \
-    k_mg_sspmm<T, VC, RR, MODE><<<grid, block, 0, ctx.stream>>>(n_rows, W, d.Lp, d.N, ngroups, gptr, gcol, ab, sig, \
+    launch_chained(ctx, k_mg_sspmm<T, VC, RR, MODE>, grid, block, 0, n_rows, W, d.Lp, d.N, ngroups, gptr, gcol, ab, sig, \
                                                                dinv, X, Rv, Out, flag, part, g2ptr, g2col, ab2, X2)
     switch (R) {
         case 1: SSP(1); break;
@@ -611,7 +618,7 @@ void launch_xfer(Ctx &ctx, const KrylovDims &d, int n_out, int n_in, int64_t nnz
     const double bytes = 4.0 * (n_out + 1) + (double)nnz * (4 + sizeof(T)) + vec_bytes<T>(d, n_in) +
                          (MODE == MG_RESTRICT ? 1 : 2) * vec_bytes<T>(d, n_out);
     ctx.before(KC_MG_TRANSFER, bytes, 4.0 * (double)nnz * W * d.frac);
-    k_mg_xfer<T, VC, MODE><<<grid, block, 0, ctx.stream>>>(n_out, W, rpb, ptr, col, val, X, Out, flag);
+    launch_chained(ctx, k_mg_xfer<T, VC, MODE>, grid, block, 0, n_out, W, rpb, ptr, col, val, X, Out, flag);
     ctx.after();
 }
 
@@ -638,10 +645,10 @@ void coarse_solve(Ctx &ctx, const KrylovDims &d, const MgSolve<T> &mg, const cpl
     auto product = [&](int trans, const cplx<T> *X, const cplx<T> *cinv, cplx<T> *Out) {
         ctx.before(KC_MG_COARSE, bytes, flops);
         if (wide)
-            k_mg_coarse_gemm<T><<<tiles, dim3(16, 8), 0, ctx.stream>>>(nc, W, d.Lp, d.N, trans, mg.V, X, cinv, Out,
+            launch_chained(ctx, k_mg_coarse_gemm<T>, tiles, dim3(16, 8), 0, nc, W, d.Lp, d.N, trans, mg.V, X, cinv, Out,
                                                                        flag);
         else
-            k_mg_coarse_split<T><<<dim3((W + 7) / 8, (nc + 3) / 4), 128, 0, ctx.stream>>>(nc, W, d.Lp, d.N, trans,
+            launch_chained(ctx, k_mg_coarse_split<T>, dim3((W + 7) / 8, (nc + 3) / 4), 128, 0, nc, W, d.Lp, d.N, trans,
                                                                                           mg.V, X, cinv, Out, flag);
         ctx.after();
     };
@@ -657,7 +664,7 @@ void launch_rz(Ctx &ctx, const KrylovDims &d, int gy, const cplx<T> *R, const cp
     const ColShape cs = col_shape(W / VC, sizeof(T) == 8);
     dim3 grid(cs.gx, gy), block(cs.bx, TY);
     ctx.before(KC_MG_TRANSFER, 2 * vec_bytes<T>(d, d.n), 0);
-    k_mg_rz<T, VC><<<grid, block, 0, ctx.stream>>>(d.n, W, R, Z, flag, part);
+    launch_chained(ctx, k_mg_rz<T, VC>, grid, block, 0, d.n, W, R, Z, flag, part);
     ctx.after();
 }
 
@@ -680,7 +687,7 @@ cplx<T> *cycle(Ctx &ctx, const KrylovDims &d, MgSolve<T> &mg, int l, int gy, con
         const ColShape cs = col_shape(W / VC, sizeof(T) == 8);
     dim3 grid(cs.gx, gyl), block(cs.bx, TY);
         ctx.before(KC_MG_TRANSFER, 2 * vec_bytes<T>(d, L.n) + (double)L.n * d.N * sizeof(cplx<T>), 0);
-        k_mg_jacobi0<T, VC><<<grid, block, 0, ctx.stream>>>(L.n, W, d.Lp, d.N, L.dinv, L.r, z, flag);
+        launch_chained(ctx, k_mg_jacobi0<T, VC>, grid, block, 0, L.n, W, d.Lp, d.N, L.dinv, L.r, z, flag);
         ctx.after();
     }
     for (int s = 1; s < mg.nu; ++s) {
@@ -733,7 +740,7 @@ void mg_scale(Ctx &ctx, const KrylovDims &d, const MgSolve<T> &mg, int gy, const
     const ColShape cs = col_shape(W / VC, sizeof(T) == 8);
     dim3 grid(cs.gx, gy), block(cs.bx, TY);
     ctx.before(KC_MG_TRANSFER, 2 * vec_bytes<T>(d, d.n) + (double)d.n * d.N * sizeof(cplx<T>), 0);
-    k_mg_scale<T, VC><<<grid, block, 0, ctx.stream>>>(d.n, W, d.Lp, d.N, mg.lv[0].dinv, X, Y, flag);
+    launch_chained(ctx, k_mg_scale<T, VC>, grid, block, 0, d.n, W, d.Lp, d.N, mg.lv[0].dinv, X, Y, flag);
     ctx.after();
 }
 
