@@ -484,6 +484,13 @@ __global__ void k_symmetrize(int m, double *S) {
     S[(int64_t)i * m + j] = v;
     S[(int64_t)j * m + i] = v;
 }
+// out = (S + S^T) / 2
+__global__ void k_symmetrized(int m, const double *__restrict__ S, double *__restrict__ out) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= (int64_t)m * m) return;
+    const int i = (int)(e / m), j = (int)(e % m);
+    out[e] = i == j ? S[e] : 0.5 * (S[e] + S[(int64_t)j * m + i]);
+}
 
 // ---------------------------------------------------------------------------
 // row-group form of the pencil for the shifted SpMM
@@ -2637,9 +2644,8 @@ slrf_status slrf_syev(slrf_handle *h, int32_t m, const double *S, double *lam, d
     CKS(ensure(h, h->rSmall, small_syev_work_bytes(m) + (size_t)m * m * sizeof(double)));
     double *Sc = as<double>(h->rSmall);
     double *w = Sc + (size_t)m * m;
-    CK(cudaMemcpyAsync(Sc, S, (size_t)m * m * 8, cudaMemcpyDeviceToDevice, h->ctx.stream));
     h->ctx.before(KC_SMALL_DENSE, 16.0 * m * m, 0);
-    k_symmetrize<<<(unsigned)(((size_t)m * m + 255) / 256), 256, 0, h->ctx.stream>>>(m, Sc);
+    k_symmetrized<<<(unsigned)(((size_t)m * m + 255) / 256), 256, 0, h->ctx.stream>>>(m, S, Sc);
     h->ctx.after();
     CK(small_syev(h->ctx, m, Sc, lam, Q, w, h->opts.eig_refine));
     CK(cudaGetLastError());

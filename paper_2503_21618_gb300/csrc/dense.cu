@@ -192,8 +192,10 @@ __global__ void k_split_reduce(int M, int N, int split, const double *__restrict
 // tiles on and above the diagonal are computed, and mirrored.
 template <int OPA, int OPB>
 __global__ void __launch_bounds__(256)
-k_dgemm_small(int M, int N, int K, const double *__restrict__ A, int64_t lda, const double *__restrict__ B,
-              int64_t ldb, double beta, double *__restrict__ C, int64_t ldc, int symmetric) {
+k_dgemm_small(int M, int N, int K, const double *A, int64_t lda, const double *B,
+              int64_t ldb, double beta, double *__restrict__ C, int64_t ldc, int symmetric,
+              int ns) {
+    chain_wait();
     constexpr int T = 8, KC = 32;
     __shared__ double As[KC][T + 1], Bs[KC][T + 1], red[3][T * T];
     if (symmetric && blockIdx.x < blockIdx.y) return;
@@ -230,6 +232,7 @@ k_dgemm_small(int M, int N, int K, const double *__restrict__ A, int64_t lda, co
     if (kq || gi >= M || gj >= N || (symmetric && gi > gj)) return;
     s = ((s + red[0][o]) + red[1][o]) + red[2][o];
     double *c = C + (int64_t)gi * ldc + gj;
+    if (ns) s = (gi == gj ? 1.5 : 0.0) - 0.5 * s;
     *c = (beta != 0.0 ? beta * *c : 0.0) + s;
     if (symmetric && gi != gj) C[(int64_t)gj * ldc + gi] = s;
 }
@@ -243,6 +246,14 @@ int gram_split(const Ctx &ctx, int m, int64_t n) {
     return split;
 }
 
+void small_ns_factor(Ctx &ctx, int m, const double *X, double *E) {
+    const dim3 grid((m + 7) / 8, (m + 7) / 8);
+    ctx.before(KC_SMALL_DENSE, 16.0 * m * m, (double)m * m * m);
+    launch_chained(ctx, k_dgemm_small<1, 0>, grid, 256, 0, m, m, m, X, (int64_t)m, X, (int64_t)m, 0.0, E, (int64_t)m,
+                   1, 1);
+    ctx.after();
+}
+
 void dgemm(Ctx &ctx, int opA, int opB, int M, int N, int K, const double *A, int64_t lda, const double *B,
            int64_t ldb, double beta, double *C, int64_t ldc, int split, double *work, int kc, bool symmetric) {
     if (M <= 0 || N <= 0) return;
@@ -251,7 +262,7 @@ void dgemm(Ctx &ctx, int opA, int opB, int M, int N, int K, const double *A, int
         const dim3 grid((N + 7) / 8, (M + 7) / 8);
         const int sym = symmetric && beta == 0.0 && M == N ? 1 : 0;
         ctx.before(kc, 8.0 * ((double)M * K + (double)K * N + (double)M * N), 2.0 * M * N * (double)K);
-#define LS(a, b) k_dgemm_small<a, b><<<grid, 256, 0, ctx.stream>>>(M, N, K, A, lda, B, ldb, beta, C, ldc, sym)
+#define LS(a, b) launch_chained(ctx, k_dgemm_small<a, b>, grid, 256, 0, M, N, K, A, lda, B, ldb, beta, C, ldc, sym, 0)
         if (opA == 0 && opB == 0) LS(0, 0);
         else if (opA == 1 && opB == 0) LS(1, 0);
         else if (opA == 0 && opB == 1) LS(0, 1);

@@ -368,6 +368,8 @@ void spmm_real(Ctx &ctx, const DevPencil &A, int m, const double *X, int64_t ldx
 void dgemm(Ctx &ctx, int opA, int opB, int M, int N, int K, const double *A, int64_t lda,
            const double *B, int64_t ldb, double beta, double *C, int64_t ldc, int split = 1,
            double *work = nullptr, int kc = KC_TALL_GEMM, bool symmetric = false);
+// E = (3 I - X^T X) / 2 of an m x m matrix (m <= 1024)
+void small_ns_factor(Ctx &ctx, int m, const double *X, double *E);
 // Choose a split for a Gram of n rows.
 int gram_split(const Ctx &ctx, int m, int64_t n);
 // Residual of the Ritz pairs: Rout = BX diag(theta) - AX (if Rout != nullptr),

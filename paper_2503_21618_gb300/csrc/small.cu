@@ -32,13 +32,15 @@ namespace slrf {
 // ---------------------------------------------------------------------------
 // column scaling of a Gram matrix: s_i = 1/sqrt(g_ii), G <- S G S
 // ---------------------------------------------------------------------------
-__global__ void k_colscale_diag(int m, const double *__restrict__ G, double *__restrict__ s) {
+__global__ void k_colscale_diag(int m, const double *G, double *__restrict__ s) {
+    chain_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
     const double g = G[(int64_t)i * m + i];
     s[i] = g > 0.0 ? 1.0 / sqrt(g) : 0.0;
 }
-__global__ void k_colscale(int m, double *__restrict__ G, const double *__restrict__ s) {
+__global__ void k_colscale(int m, double *__restrict__ G, const double *s) {
+    chain_wait();
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e < (int64_t)m * m) G[e] *= s[e / m] * s[e % m];
 }
@@ -46,14 +48,15 @@ __global__ void k_colscale(int m, double *__restrict__ G, const double *__restri
 void small_colscale(Ctx &ctx, int m, double *G, double *s) {
     const int64_t tot = (int64_t)m * m;
     ctx.before(KC_SMALL_DENSE, 16.0 * m, m);
-    k_colscale_diag<<<(m + 63) / 64, 64, 0, ctx.stream>>>(m, G, s);
+    launch_chained(ctx, k_colscale_diag, (m + 63) / 64, 64, 0, m, G, s);
     ctx.after();
     ctx.before(KC_SMALL_DENSE, 16.0 * tot, tot);
-    k_colscale<<<(unsigned)((tot + 255) / 256), 256, 0, ctx.stream>>>(m, G, s);
+    launch_chained(ctx, k_colscale, (unsigned)((tot + 255) / 256), 256, 0, m, G, s);
     ctx.after();
 }
 
-__global__ void k_scale_rows(int m, const double *__restrict__ s, double *__restrict__ T) {
+__global__ void k_scale_rows(int m, const double *s, double *__restrict__ T) {
+    chain_wait();
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= (int64_t)m * m) return;
     T[e] *= s[e / m];
@@ -61,7 +64,7 @@ __global__ void k_scale_rows(int m, const double *__restrict__ s, double *__rest
 void small_scale_rows(Ctx &ctx, int m, const double *s, double *T) {
     const int64_t tot = (int64_t)m * m;
     ctx.before(KC_SMALL_DENSE, 16.0 * tot, tot);
-    k_scale_rows<<<(unsigned)((tot + 255) / 256), 256, 0, ctx.stream>>>(m, s, T);
+    launch_chained(ctx, k_scale_rows, (unsigned)((tot + 255) / 256), 256, 0, m, s, T);
     ctx.after();
 }
 
@@ -71,9 +74,10 @@ void small_scale_rows(Ctx &ctx, int m, const double *s, double *T) {
 // read and left untouched.  *status = -1 on success; an unrecoverable
 // breakdown (a pivot not above 0) sets *status = k + 1, k the failing pivot.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_chol_shifted(int m, const double *__restrict__ G, double *__restrict__ Rg,
+__global__ void __launch_bounds__(1024) k_chol_shifted(int m, const double *G, double *__restrict__ Rg,
                                                         int32_t *__restrict__ status, int32_t *__restrict__ out_status,
                                                         int use_smem, double shift) {
+    chain_wait();
     extern __shared__ double sm[];
     if (*(volatile int32_t *)status <= 0) return;
     double *A = use_smem ? sm : Rg;
@@ -142,8 +146,9 @@ void raise_smem_limits();   // defined after the kernels it configures
 // ---------------------------------------------------------------------------
 constexpr int CHB = 32;
 
-__global__ void k_chol_init(int m, const double *__restrict__ G, double *__restrict__ A, double *__restrict__ X,
+__global__ void k_chol_init(int m, const double *G, double *__restrict__ A, double *__restrict__ X,
                             int32_t *__restrict__ status) {
+    chain_wait();
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e == 0) *status = 0;
     if (e >= (int64_t)m * m) return;
@@ -158,6 +163,7 @@ __global__ void k_chol_init(int m, const double *__restrict__ G, double *__restr
 // block in shared memory took 62 us per 32 pivots).
 __global__ void __launch_bounds__(256) k_chol_diag(int m, int k0, int kb, double *__restrict__ A,
                                                    int32_t *__restrict__ status, double pmin) {
+    chain_wait();
     __shared__ double u[2][CHB];   // alternating by pivot: one barrier per pivot
     __shared__ int bad[2];
     if (*(volatile int32_t *)status != 0) return;   // uniform: the same word for every thread
@@ -210,7 +216,8 @@ __global__ void __launch_bounds__(256) k_chol_diag(int m, int k0, int kb, double
 // the forward substitution with the unit-scaled factor broadcasts row p, so
 // one FMA per step: FP64 FMAs of one warp issue ~70 clocks apart)
 __global__ void __launch_bounds__(64) k_chol_panel(int m, int k0, int kb, double *__restrict__ A,
-                                                   double *__restrict__ X, const int32_t *__restrict__ status) {
+                                                   double *__restrict__ X, const int32_t *status) {
+    chain_wait();
     __shared__ double Rk[CHB][CHB + 1], ri[CHB];
     if (*(volatile int32_t *)status != 0) return;
     if (threadIdx.x < kb) ri[threadIdx.x] = 1.0 / A[(int64_t)(k0 + threadIdx.x) * m + k0 + threadIdx.x];
@@ -237,7 +244,8 @@ __global__ void __launch_bounds__(64) k_chol_panel(int m, int k0, int kb, double
 // and X[i][c] -= sum_p A[k0+p][i] X[k0+p][c] for the right part's columns
 // c < k0+kb; 16 x 16 output tiles, the first `tl` tile columns the left part
 __global__ void __launch_bounds__(256) k_chol_update(int m, int k0, int kb, int tl, double *__restrict__ A,
-                                                     double *__restrict__ X, const int32_t *__restrict__ status) {
+                                                     double *__restrict__ X, const int32_t *status) {
+    chain_wait();
     __shared__ double Pi[CHB][17], Pj[CHB][17];
     if (*(volatile int32_t *)status != 0) return;
     const int r0 = k0 + kb;
@@ -264,7 +272,8 @@ __global__ void __launch_bounds__(256) k_chol_update(int m, int k0, int kb, int 
 
 // R's lower triangle to zero, X = (its lower triangle)^T
 __global__ void k_chol_finish(int m, double *__restrict__ A, double *__restrict__ X,
-                              const int32_t *__restrict__ status, int32_t *__restrict__ out_status) {
+                              const int32_t *status, int32_t *__restrict__ out_status) {
+    chain_wait();
     const int32_t st = *(volatile int32_t *)status;
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e == 0 && out_status) *out_status = st;
@@ -279,8 +288,9 @@ __global__ void k_chol_finish(int m, double *__restrict__ A, double *__restrict_
 // X = R^{-1} of the shifted factor (runs only after a shifted refactorisation,
 // *status < 0): one warp per column j, back substitution x_i = (delta_ij -
 // sum_{k=i+1..j} R_ik x_k) / R_ii, the sum split over the lanes.
-__global__ void __launch_bounds__(32) k_triinv_upper(int m, const double *__restrict__ R, double *__restrict__ X,
-                                                     const int32_t *__restrict__ status) {
+__global__ void __launch_bounds__(32) k_triinv_upper(int m, const double *R, double *__restrict__ X,
+                                                     const int32_t *status) {
+    chain_wait();
     extern __shared__ double xcol[];
     if (*(volatile int32_t *)status >= 0) return;
     double *rinv = xcol + m;
@@ -308,34 +318,34 @@ void small_chol_inv(Ctx &ctx, int m, const double *G, double *R, double *Rinv, i
     const int64_t m2 = (int64_t)m * m;
     const unsigned eg = (unsigned)((m2 + 255) / 256);
     ctx.before(KC_SMALL_DENSE, 24.0 * m2, 0);
-    k_chol_init<<<eg, 256, 0, ctx.stream>>>(m, G, R, Rinv, status);
+    launch_chained(ctx, k_chol_init, eg, 256, 0, m, G, R, Rinv, status);
     ctx.after();
     for (int k0 = 0; k0 < m; k0 += CHB) {
         const int kb = std::min(CHB, m - k0), rest = m - k0 - kb;
         ctx.before(KC_SMALL_DENSE, 16.0 * kb * kb, (double)kb * kb * kb / 3.0);
-        k_chol_diag<<<1, 256, 0, ctx.stream>>>(m, k0, kb, R, status, shift_on_fail);
+        launch_chained(ctx, k_chol_diag, 1, 256, 0, m, k0, kb, R, status, shift_on_fail);
         ctx.after();
         ctx.before(KC_SMALL_DENSE, 16.0 * kb * m, (double)kb * kb * m);
-        k_chol_panel<<<(m + 1) / 2, 64, 0, ctx.stream>>>(m, k0, kb, R, Rinv, status);
+        launch_chained(ctx, k_chol_panel, (m + 1) / 2, 64, 0, m, k0, kb, R, Rinv, status);
         ctx.after();
         if (rest == 0) break;
         const int tl = (rest + 15) / 16, tr = (k0 + kb + 15) / 16;
         ctx.before(KC_SMALL_DENSE, 8.0 * rest * m, (double)rest * m * kb);
-        k_chol_update<<<dim3(tl + tr, tl), 256, 0, ctx.stream>>>(m, k0, kb, tl, R, Rinv, status);
+        launch_chained(ctx, k_chol_update, dim3(tl + tr, tl), 256, 0, m, k0, kb, tl, R, Rinv, status);
         ctx.after();
     }
     ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-    k_chol_finish<<<eg, 256, 0, ctx.stream>>>(m, R, Rinv, status, out_status);
+    launch_chained(ctx, k_chol_finish, eg, 256, 0, m, R, Rinv, status, out_status);
     ctx.after();
     if (shift_on_fail > 0.0 && G != R) {
         const size_t smem = (size_t)m * m * sizeof(double);
         const int use_smem = smem <= 200 * 1024;
         raise_smem_limits();
         ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-        k_chol_shifted<<<1, 1024, use_smem ? smem : 0, ctx.stream>>>(m, G, R, status, out_status, use_smem, shift_on_fail);
+        launch_chained(ctx, k_chol_shifted, 1, 1024, use_smem ? smem : 0, m, G, R, status, out_status, use_smem, shift_on_fail);
         ctx.after();
         ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-        k_triinv_upper<<<m, 32, 2 * (size_t)m * sizeof(double), ctx.stream>>>(m, R, Rinv, status);
+        launch_chained(ctx, k_triinv_upper, m, 32, 2 * (size_t)m * sizeof(double), m, R, Rinv, status);
         ctx.after();
     }
 }
@@ -344,7 +354,8 @@ void small_chol_inv(Ctx &ctx, int m, const double *G, double *R, double *Rinv, i
 // ||S||_F as FRO_PARTS partial sums of squares, one per block, summed by the
 // readers (fro_norm, a whole warp)
 constexpr int FRO_PARTS = 32, OA_PARTS = 64;   // OA_PARTS: blocks of k_oa_norms
-__global__ void __launch_bounds__(256) k_fro(int m, const double *__restrict__ S, double *__restrict__ part) {
+__global__ void __launch_bounds__(256) k_fro(int m, const double *S, double *__restrict__ part) {
+    chain_wait();
     __shared__ double red[8];
     double s = 0;
     for (int64_t e = blockIdx.x * 256 + threadIdx.x; e < (int64_t)m * m; e += FRO_PARTS * 256) s += S[e] * S[e];
@@ -411,9 +422,10 @@ struct Jacobi32Shape {
     size_t bytes() const { return (size_t)mp * ld * sizeof(float); }
 };
 
-__global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *__restrict__ S, double *__restrict__ lam,
+__global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *S, double *__restrict__ lam,
                                                   int *__restrict__ rank, float2 *__restrict__ rlog,
                                                   int *__restrict__ nrounds, float rel_tol) {
+    chain_wait();
     extern __shared__ float jsm[];
     const Jacobi32Shape sh(m);
     const int mp = sh.mp, npair = sh.npair, ld = sh.ld;
@@ -885,9 +897,10 @@ k_jacobi_df(int m, const double *__restrict__ S, const double *__restrict__ fro_
 // A log entry (c, s) rotates (upper, lower), or (lower, upper) if c < 0; column
 // i goes to column rank[i] of Q (rank = nullptr: i).
 template <int K>
-__global__ void __launch_bounds__(32) k_jacobi_vectors(int m, const float2 *__restrict__ rlog,
-                                                       const int *__restrict__ nrounds, const int *__restrict__ rank,
+__global__ void __launch_bounds__(32) k_jacobi_vectors(int m, const float2 *rlog,
+                                                       const int *nrounds, const int *rank,
                                                        double *__restrict__ Q) {
+    chain_wait();
     constexpr int G = JVEC_ROUNDS;
     extern __shared__ float4 vsm4[];
     const int mp = m + (m & 1), npair = mp / 2;
@@ -967,10 +980,10 @@ void jacobi_vectors(Ctx &ctx, int m, const float2 *rlog, const int *nrounds, con
     const int npair = (m + 1) / 2;
     const size_t smem = 2 * (size_t)JVEC_ROUNDS * npair * sizeof(float2);
     ctx.before(KC_SMALL_DENSE, 8.0 * m * m, 3.0 * (double)m * m * m * 8);
-#define JV(K) case K: k_jacobi_vectors<K><<<m, 32, smem, ctx.stream>>>(m, rlog, nrounds, rank, Q); break
+#define JV(K) case K: launch_chained(ctx, k_jacobi_vectors<K>, m, 32, smem, m, rlog, nrounds, rank, Q); break
     switch ((npair + 31) / 32) {
         JV(1); JV(2); JV(3); JV(4); JV(5); JV(6);
-        default: k_jacobi_vectors<7><<<m, 32, smem, ctx.stream>>>(m, rlog, nrounds, rank, Q); break;
+        default: launch_chained(ctx, k_jacobi_vectors<7>, m, 32, smem, m, rlog, nrounds, rank, Q); break;
     }
 #undef JV
     ctx.after();
@@ -1105,6 +1118,7 @@ k_jacobi_coop(int m, double *__restrict__ A, double *__restrict__ V, double *__r
 }
 
 __global__ void k_identity(int m, double *__restrict__ V) {
+    chain_wait();
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e < (int64_t)m * m) V[e] = (e / m == e % m) ? 1.0 : 0.0;
 }
@@ -1112,8 +1126,9 @@ __global__ void k_identity(int m, double *__restrict__ V) {
 // final ordering: lam ascending, Q columns permuted.  Every block ranks all
 // eigenvalues (as integers of the same order: FP64 compares run on the slow
 // FP64 pipe) and moves its rows, one warp per row.
-__global__ void __launch_bounds__(256) k_sort_eig(int m, const double *__restrict__ lam_in, const double *__restrict__ S,
+__global__ void __launch_bounds__(256) k_sort_eig(int m, const double *lam_in, const double *S,
                                                   double *__restrict__ lam, double *__restrict__ Q) {
+    chain_wait();
     __shared__ long long key[1024];
     __shared__ int rank[1024];
     for (int i = threadIdx.x; i < m; i += blockDim.x) {
@@ -1176,8 +1191,9 @@ size_t small_syev_work_bytes(int m) {
 // lam_t = t_ii / g_ii, and per block the partial sum of ||T - D||_F^2 over its
 // rows (fixed order; one block for the whole matrix took 33 us at m = 150,
 // all of it FP64 issue; this takes 5)
-__global__ void __launch_bounds__(256) k_oa_norms(int m, const double *__restrict__ G, const double *__restrict__ T,
+__global__ void __launch_bounds__(256) k_oa_norms(int m, const double *G, const double *T,
                                                   double *__restrict__ lam_t, double *__restrict__ part) {
+    chain_wait();
     __shared__ double red[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double off = 0.0;
@@ -1203,9 +1219,10 @@ __global__ void __launch_bounds__(256) k_oa_norms(int m, const double *__restric
 
 // Ep = I + E (row-major), one thread per entry over many blocks (the FP64
 // divisions spread over the GPU); the pair threshold is delta = 2 ||T - D||_F
-__global__ void __launch_bounds__(256) k_oa_step(int m, const double *__restrict__ G, const double *__restrict__ T,
-                                                 const double *__restrict__ lam_t, const double *__restrict__ part,
+__global__ void __launch_bounds__(256) k_oa_step(int m, const double *G, const double *T,
+                                                 const double *lam_t, const double *part,
                                                  double *__restrict__ Ep) {
+    chain_wait();
     __shared__ double delta;
     if (threadIdx.x < 32) {
         double s = part[threadIdx.x] + part[threadIdx.x + 32];
@@ -1230,11 +1247,6 @@ __global__ void __launch_bounds__(256) k_oa_step(int m, const double *__restrict
 }
 
 // Newton-Schulz orthonormalisation factor: Ep = (3 I - G) / 2
-__global__ void k_ns_factor(int m, const double *__restrict__ G, double *__restrict__ Ep) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= (int64_t)m * m) return;
-    Ep[e] = (e / m == e % m ? 1.5 : 0.0) - 0.5 * G[e];
-}
 
 // After the refinement T = Q^T S Q is diagonal up to rounding except inside
 // groups of (nearly) equal eigenvalues.  Indices joined by an off-diagonal
@@ -1243,11 +1255,12 @@ __global__ void k_ns_factor(int m, const double *__restrict__ G, double *__restr
 // component of two or more is diagonalised by cyclic FP64 Jacobi and its
 // columns of Q rotated; lam receives the diagonal (unsorted).  Workspace:
 // label, size (m ints each), blk, W (m^2 doubles each), Qc (m^2 doubles).
-__global__ void __launch_bounds__(1024) k_oa_components(int m, const double *__restrict__ T,
-                                                       const double *__restrict__ normS, double *__restrict__ Q,
+__global__ void __launch_bounds__(1024) k_oa_components(int m, const double *T,
+                                                       const double *normS, double *__restrict__ Q,
                                                        double *__restrict__ lam, int *__restrict__ label,
                                                        int *__restrict__ size, double *__restrict__ blk,
                                                        double *__restrict__ Wm, double *__restrict__ Qc) {
+    chain_wait();
     const int tid = threadIdx.x, bs = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5, nwarp = bs >> 5;
     __shared__ int changed, k, nrot;
@@ -1488,11 +1501,11 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
     float2 *rlog = reinterpret_cast<float2 *>((reinterpret_cast<uintptr_t>(w + syev_base_bytes(m)) + 15) / 16 * 16);
 
     ctx.before(KC_SMALL_DENSE, 8.0 * m2, 2.0 * m2);
-    k_fro<<<FRO_PARTS, 256, 0, ctx.stream>>>(m, S, normA);
+    launch_chained(ctx, k_fro, FRO_PARTS, 256, 0, m, S, normA);
     ctx.after();
     auto identity = [&](double *V) {
         ctx.before(KC_SMALL_DENSE, 8.0 * m2, 0);
-        k_identity<<<(unsigned)((m2 + 255) / 256), 256, 0, ctx.stream>>>(m, V);
+        launch_chained(ctx, k_identity, (unsigned)((m2 + 255) / 256), 256, 0, m, V);
         ctx.after();
     };
     // The one-block FP32 stage takes m <= JMAX (A and V in its shared memory),
@@ -1504,7 +1517,7 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
         const cudaError_t e = coop_jacobi(ctx, m, Tm, Vm, lam0, 60, normA, 0.5 / m, cnt);
         if (e != cudaSuccess) return e;
         ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-        k_sort_eig<<<(m + 7) / 8, 256, 0, ctx.stream>>>(m, lam0, Vm, lam, Q);
+        launch_chained(ctx, k_sort_eig, (m + 7) / 8, 256, 0, m, lam0, Vm, lam, Q);
         ctx.after();
         return cudaGetLastError();
     }
@@ -1513,7 +1526,7 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
     if (m <= JMAX) {
         const Jacobi32Shape sh(m);
         ctx.before(KC_SMALL_DENSE, 8.0 * m2, 6.0 * (double)m * m2 * 8);
-        k_jacobi32<<<1, sh.threads, sh.bytes(), ctx.stream>>>(m, S, lam0, label, rlog, cnt + 6, 1e-6f);
+        launch_chained(ctx, k_jacobi32, 1, sh.threads, sh.bytes(), m, S, lam0, label, rlog, cnt + 6, 1e-6f);
         ctx.after();
         jacobi_vectors(ctx, m, rlog, cnt + 6, label, S0);
     } else {
@@ -1544,20 +1557,17 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
         double *X0 = S0, *X1 = S1;
         const unsigned eg = (unsigned)((m2 + 255) / 256);
         for (int it = 0; it < 3; ++it) {
-            dgemm(ctx, 1, 0, m, m, m, X0, m, X0, m, 0.0, G, m, 1, nullptr, KC_SMALL_DENSE, true);
-            ctx.before(KC_SMALL_DENSE, 16.0 * m2, 2.0 * m2);
-            k_ns_factor<<<eg, 256, 0, ctx.stream>>>(m, G, Vm);
-            ctx.after();
+            small_ns_factor(ctx, m, X0, Vm);
             dgemm(ctx, 0, 0, m, m, m, X0, m, Vm, m, 0.0, X1, m, 1, nullptr, KC_SMALL_DENSE);
             std::swap(X0, X1);
             dgemm(ctx, 1, 0, m, m, m, X0, m, X0, m, 0.0, G, m, 1, nullptr, KC_SMALL_DENSE, true);
             dgemm(ctx, 0, 0, m, m, m, S, m, X0, m, 0.0, Ym, m, 1, nullptr, KC_SMALL_DENSE);
             dgemm(ctx, 1, 0, m, m, m, X0, m, Ym, m, 0.0, Tm, m, 1, nullptr, KC_SMALL_DENSE, true);
             ctx.before(KC_SMALL_DENSE, 16.0 * m2, 4.0 * m2);
-            k_oa_norms<<<OA_PARTS, 256, 0, ctx.stream>>>(m, G, Tm, lam0, oa_part);
+            launch_chained(ctx, k_oa_norms, OA_PARTS, 256, 0, m, G, Tm, lam0, oa_part);
             ctx.after();
             ctx.before(KC_SMALL_DENSE, 24.0 * m2, 8.0 * m2);
-            k_oa_step<<<eg, 256, 0, ctx.stream>>>(m, G, Tm, lam0, oa_part, Vm);
+            launch_chained(ctx, k_oa_step, eg, 256, 0, m, G, Tm, lam0, oa_part, Vm);
             ctx.after();
             dgemm(ctx, 0, 0, m, m, m, X0, m, Vm, m, 0.0, X1, m, 1, nullptr, KC_SMALL_DENSE);
             std::swap(X0, X1);
@@ -1566,10 +1576,7 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
         // accepted steps: three orthonormalisation steps bring it back to
         // rounding level before the groups are rotated
         for (int it = 0; it < 3; ++it) {
-            dgemm(ctx, 1, 0, m, m, m, X0, m, X0, m, 0.0, G, m, 1, nullptr, KC_SMALL_DENSE, true);
-            ctx.before(KC_SMALL_DENSE, 16.0 * m2, 2.0 * m2);
-            k_ns_factor<<<eg, 256, 0, ctx.stream>>>(m, G, Vm);
-            ctx.after();
+            small_ns_factor(ctx, m, X0, Vm);
             dgemm(ctx, 0, 0, m, m, m, X0, m, Vm, m, 0.0, X1, m, 1, nullptr, KC_SMALL_DENSE);
             std::swap(X0, X1);
         }
@@ -1584,16 +1591,16 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
             if (e != cudaSuccess) return e;
             dgemm(ctx, 0, 0, m, m, m, X0, m, Vm, m, 0.0, X1, m, 1, nullptr, KC_SMALL_DENSE);
             ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-            k_sort_eig<<<(m + 7) / 8, 256, 0, ctx.stream>>>(m, lam0, X1, lam, Q);
+            launch_chained(ctx, k_sort_eig, (m + 7) / 8, 256, 0, m, lam0, X1, lam, Q);
             ctx.after();
             return cudaGetLastError();
         }
         ctx.before(KC_SMALL_DENSE, 24.0 * m2, 4.0 * m2);
-        k_oa_components<<<1, 1024, 0, ctx.stream>>>(m, Tm, normA, X0, lam0, label, csize, (double *)Ag,
+        launch_chained(ctx, k_oa_components, 1, 1024, 0, m, Tm, normA, X0, lam0, label, csize, (double *)Ag,
                                                      (double *)Vg, X1);
         ctx.after();
         ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-        k_sort_eig<<<(m + 7) / 8, 256, 0, ctx.stream>>>(m, lam0, X0, lam, Q);
+        launch_chained(ctx, k_sort_eig, (m + 7) / 8, 256, 0, m, lam0, X0, lam, Q);
         ctx.after();
         return cudaGetLastError();
     }
@@ -1609,7 +1616,7 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
     if (e != cudaSuccess) return e;
     dgemm(ctx, 0, 0, m, m, m, S1, m, Vm, m, 0.0, S0, m, 1, nullptr, KC_SMALL_DENSE);
     ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-    k_sort_eig<<<(m + 7) / 8, 256, 0, ctx.stream>>>(m, lam0, S0, lam, Q);
+    launch_chained(ctx, k_sort_eig, (m + 7) / 8, 256, 0, m, lam0, S0, lam, Q);
     ctx.after();
     return cudaGetLastError();
 }
