@@ -20,10 +20,12 @@
 // identity.  Two launches per block: the panel (T, every block column its own
 // CTA), and the update, one CTA per 64 x 64 tile, whose first CTA takes the
 // next diagonal block and sweeps it in registers while the others work, so
-// the chain of 64 pivots (~11 us) hides behind the update.  Bound by FP32
+// most of the chain of 64 pivots (~15 us) hides behind the update.  Bound by FP32
 // arithmetic: 4 N n^3 flops (n = 1283, N = 4: 34 GF, 0.45 ms at 75 TFLOP/s);
 // cuBLAS complex GEMMs on the whole matrix, with the diagonal blocks and
-// block copies in launches of their own, took 3.9 ms there, this 1.2 ms.
+// block copies in launches of their own, took 3.9 ms there, this 1.15 ms.
+// (The chain in a launch of its own beside the update was slower: it is as long
+// as the update.)
 #include <cublas_v2.h>
 #include <cuda_runtime.h>
 
@@ -60,11 +62,21 @@ __global__ void k_dense_shift(int n, int np, const int32_t *__restrict__ ptr, co
 // one broadcast and the columns' two conflict-free 16-byte shared loads.
 __device__ __forceinline__ int tile_col(int tx, int q) { return 2 * tx + 32 * (q >> 1) + (q & 1); }
 
-// acc += A^T B over the CB rows of two staged CB x CB panels
+// 16-byte asynchronous copies to shared memory
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT> __device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+}
+
+// acc -= A^T B over KR rows of two staged panels of CB columns
+template <int KR>
 __device__ __forceinline__ void tile_product(const float2 (*A)[CB], const float2 (*B)[CB], int ty, int tx,
                                              float2 (&acc)[4][4]) {
 #pragma unroll 4
-    for (int k = 0; k < CB; ++k) {
+    for (int k = 0; k < KR; ++k) {
         const float4 a01 = *reinterpret_cast<const float4 *>(&A[k][4 * ty]);
         const float4 a23 = *reinterpret_cast<const float4 *>(&A[k][4 * ty + 2]);
         const float4 b01 = *reinterpret_cast<const float4 *>(&B[k][2 * tx]);
@@ -76,55 +88,102 @@ __device__ __forceinline__ void tile_product(const float2 (*A)[CB], const float2
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[i][q] = cfma(a[i], b[q], acc[i][q]);
+            for (int q = 0; q < 4; ++q) acc[i][q] = cfma(make_float2(-a[i].x, -a[i].y), b[q], acc[i][q]);
     }
+}
+
+// 1 / x to rounding level for normal x: the correctly rounded routine checks for
+// every special case, in the middle of the chain of pivots
+__device__ __forceinline__ float fast_rcp(float x) {
+    float y;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return fmaf(y, fmaf(-x, y, 1.f), y);
+}
+
+// Pivot k (column k: registers S[.][qk] of lane tx = kx; row k: S[ki][.] of ty =
+// k4) with w = row k / pivot, r = column k, applied to the register rows i
+// (mask), the pivot's own row and column included.
+template <int KI, int QK>
+__device__ __forceinline__ void pivot_rows(float2 (&S)[4][4], const float2 (&w)[4], const float2 (&r)[4], float2 pinv,
+                                           bool own_row, bool own_col, int mask) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (!(mask >> i & 1)) continue;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) S[i][q] = cfma(make_float2(-r[i].x, -r[i].y), w[q], S[i][q]);
+        if (own_col) S[i][QK] = cmul(pinv, r[i]);
+        if (i == KI && own_row) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) S[i][q] = w[q];
+            if (own_col) S[i][QK] = make_float2(-pinv.x, -pinv.y);
+        }
+    }
+}
+
+__device__ __forceinline__ void publish_row(float2 *row, const float2 (&v)[4], int tx) {
+    *reinterpret_cast<float4 *>(row + 2 * tx) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+    *reinterpret_cast<float4 *>(row + 2 * tx + 32) = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
 }
 
 // The symmetric sweep of all CB pivots of a tile in registers: S -> -S^{-1}.
 // Per pivot the owners publish its row (= its column), one barrier, everyone
-// updates, and the owners of the pivot's row and column overwrite theirs (the
-// indices of a column's owners are fixed at compile time but for one lane
-// number, so nothing is selected in the common path).
+// updates.  A chain of 64 such steps, so a step is cut into what the next one
+// needs and the rest: pivot k is applied to the register row that holds row k+1
+// first, which is published; the other three rows follow after the barrier,
+// beside the loads and the reciprocal of pivot k+1: 17 us for the first block
+// against 21.
+struct Pivot {
+    float2 w[4], r[4], pinv;
+};
+template <int HALF, int KI>
+__device__ __forceinline__ void sweep_step(float2 (&S)[4][4], float2 (*row)[CB], int ty, int tx, int k8, Pivot &v) {
+    constexpr int QK = 2 * HALF + (KI & 1), KP = (KI + 3) & 3, NEXT = (KI + 1) & 3;
+    const int k4 = 8 * HALF + k8, k = 4 * k4 + KI;
+    const float2 *rk = row[KI & 1];
+    __syncthreads();
+    const float2 p = rk[k];
+    const float4 c01 = *reinterpret_cast<const float4 *>(rk + 2 * tx);
+    const float4 c23 = *reinterpret_cast<const float4 *>(rk + 2 * tx + 32);
+    const float4 r01 = *reinterpret_cast<const float4 *>(rk + 4 * ty);
+    const float4 r23 = *reinterpret_cast<const float4 *>(rk + 4 * ty + 2);
+    // the rest of pivot k - 1: the register rows other than KI
+    const bool prow = ty == (k - 1) >> 2, pcol = tx == ((k - 1) & 31) >> 1;
+    constexpr int REST = 15 & ~(1 << KI);
+    if constexpr (KI > 0) {
+        pivot_rows<KP, 2 * HALF + (KP & 1)>(S, v.w, v.r, v.pinv, prow, pcol, REST);
+    } else {
+        if (k8 > 0) pivot_rows<3, 2 * HALF + 1>(S, v.w, v.r, v.pinv, prow, pcol, REST);
+        else if (HALF == 1) pivot_rows<3, 1>(S, v.w, v.r, v.pinv, prow, pcol, REST);
+    }
+    const float di = fast_rcp(p.x * p.x + p.y * p.y);
+    v.pinv = make_float2(p.x * di, -p.y * di);
+    v.w[0] = cmul(v.pinv, make_float2(c01.x, c01.y));
+    v.w[1] = cmul(v.pinv, make_float2(c01.z, c01.w));
+    v.w[2] = cmul(v.pinv, make_float2(c23.x, c23.y));
+    v.w[3] = cmul(v.pinv, make_float2(c23.z, c23.w));
+    v.r[0] = make_float2(r01.x, r01.y);
+    v.r[1] = make_float2(r01.z, r01.w);
+    v.r[2] = make_float2(r23.x, r23.y);
+    v.r[3] = make_float2(r23.z, r23.w);
+    pivot_rows<KI, QK>(S, v.w, v.r, v.pinv, ty == k4, tx == (k & 31) >> 1, 1 << NEXT);
+    if (k + 1 < CB && ty == (k + 1) >> 2) publish_row(row[(KI + 1) & 1], S[NEXT], tx);
+}
 __device__ __forceinline__ void tile_sweep(float2 (&S)[4][4], float2 (*row)[CB], int ty, int tx) {
-#pragma unroll
-    for (int half = 0; half < 2; ++half)
-        for (int k8 = 0; k8 < CB / 8; ++k8)
-#pragma unroll
-            for (int ki = 0; ki < 4; ++ki) {
-                const int k4 = 8 * half + k8, k = 4 * k4 + ki;
-                constexpr int Q0[2] = {0, 2};
-                const int qk = Q0[half] + (ki & 1), kx = (k & 31) >> 1;   // column k: registers S[.][qk] of lane tx = kx
-                float2 *rk = row[ki & 1];
-                if (ty == k4) {
-                    *reinterpret_cast<float4 *>(rk + 2 * tx) = make_float4(S[ki][0].x, S[ki][0].y, S[ki][1].x, S[ki][1].y);
-                    *reinterpret_cast<float4 *>(rk + 2 * tx + 32) =
-                        make_float4(S[ki][2].x, S[ki][2].y, S[ki][3].x, S[ki][3].y);
-                }
-                __syncthreads();
-                const float2 p = rk[k];
-                const float4 c01 = *reinterpret_cast<const float4 *>(rk + 2 * tx);
-                const float4 c23 = *reinterpret_cast<const float4 *>(rk + 2 * tx + 32);
-                const float4 r01 = *reinterpret_cast<const float4 *>(rk + 4 * ty);
-                const float4 r23 = *reinterpret_cast<const float4 *>(rk + 4 * ty + 2);
-                const float di = __frcp_rn(p.x * p.x + p.y * p.y);
-                const float2 pinv = make_float2(p.x * di, -p.y * di);
-                const float2 w[4] = {cmul(pinv, make_float2(c01.x, c01.y)), cmul(pinv, make_float2(c01.z, c01.w)),
-                                     cmul(pinv, make_float2(c23.x, c23.y)), cmul(pinv, make_float2(c23.z, c23.w))};
-                const float2 r[4] = {make_float2(r01.x, r01.y), make_float2(r01.z, r01.w), make_float2(r23.x, r23.y),
-                                     make_float2(r23.z, r23.w)};
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) S[i][q] = cfma(make_float2(-r[i].x, -r[i].y), w[q], S[i][q]);
-                if (tx == kx)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) S[i][qk] = cmul(pinv, r[i]);
-                if (ty == k4) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) S[ki][q] = w[q];
-                    if (tx == kx) S[ki][qk] = make_float2(-pinv.x, -pinv.y);
-                }
-            }
+    if (ty == 0) publish_row(row[0], S[0], tx);
+    Pivot v;
+    for (int k8 = 0; k8 < CB / 8; ++k8) {
+        sweep_step<0, 0>(S, row, ty, tx, k8, v);
+        sweep_step<0, 1>(S, row, ty, tx, k8, v);
+        sweep_step<0, 2>(S, row, ty, tx, k8, v);
+        sweep_step<0, 3>(S, row, ty, tx, k8, v);
+    }
+    for (int k8 = 0; k8 < CB / 8; ++k8) {
+        sweep_step<1, 0>(S, row, ty, tx, k8, v);
+        sweep_step<1, 1>(S, row, ty, tx, k8, v);
+        sweep_step<1, 2>(S, row, ty, tx, k8, v);
+        sweep_step<1, 3>(S, row, ty, tx, k8, v);
+    }
+    pivot_rows<3, 3>(S, v.w, v.r, v.pinv, ty == CB / 4 - 1, tx == 15, 14);
 }
 
 // Sweep of the diagonal block at k0: M_KK = -P, and P beside it
@@ -142,6 +201,7 @@ __device__ __forceinline__ void sweep_store(float2 (&S)[4][4], float2 (*row)[CB]
 }
 
 __global__ void __launch_bounds__(256) k_first_block(int np, float2 *__restrict__ M, float2 *__restrict__ P) {
+    chain_wait();
     __shared__ __align__(16) float2 row[2][CB];
     float2 *Mj = M + (int64_t)blockIdx.x * np * np;
     const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
@@ -158,8 +218,9 @@ __global__ void __launch_bounds__(256) k_first_block(int np, float2 *__restrict_
 // one CTA per matrix and 32 columns.
 constexpr int PC = 32, PLD = PC + 2;   // columns of a panel CTA, their pitch
 __global__ void __launch_bounds__(256) k_sweep_panel(int np, int K, float2 *__restrict__ M,
-                                                     const float2 *__restrict__ P, float2 *__restrict__ Cp,
+                                                     const float2 *P, float2 *__restrict__ Cp,
                                                      float2 *__restrict__ Tp) {
+    chain_wait();
     extern __shared__ __align__(16) float2 sm[];
     float2(*sP)[CB] = reinterpret_cast<float2(*)[CB]>(sm);
     float2(*sC)[PLD] = reinterpret_cast<float2(*)[PLD]>(sm + CB * CB);
@@ -168,18 +229,21 @@ __global__ void __launch_bounds__(256) k_sweep_panel(int np, int K, float2 *__re
     float2 *Mj = M + (int64_t)j * np * np;
     float2 *C = Cp + (int64_t)j * CB * np, *T = Tp + (int64_t)j * CB * np;
     const int k0 = K * CB, c0 = J * CB + (blockIdx.y & 1) * PC;
-#pragma unroll 8
-    for (int e = tid; e < CB * CB / 2; e += 256)
-        *reinterpret_cast<float4 *>(&sP[0][0] + 2 * e) =
-            *reinterpret_cast<const float4 *>(P + (int64_t)j * CB * CB + 2 * e);   // symmetric
+#pragma unroll
+    for (int q = 0; q < CB * CB / 2 / 256; ++q)
+        cp_async16(&sP[0][0] + 2 * (tid + 256 * q), P + (int64_t)j * CB * CB + 2 * (tid + 256 * q));   // symmetric
     if (J > K)
 #pragma unroll
-        for (int e = tid; e < CB * PC; e += 256)
-            sC[e / PC][e % PC] = Mj[(int64_t)(k0 + e / PC) * np + c0 + e % PC];
+        for (int q = 0; q < CB * PC / 2 / 256; ++q) {
+            const int e = tid + 256 * q, r = e / (PC / 2), c = e % (PC / 2) * 2;
+            cp_async16(&sC[r][c], Mj + (int64_t)(k0 + r) * np + c0 + c);
+        }
     else
 #pragma unroll
         for (int e = tid; e < CB * PC; e += 256)
             sC[e % CB][e / CB] = Mj[(int64_t)(c0 + e / CB) * np + k0 + e % CB];
+    cp_async_commit();
+    cp_async_wait<0>();
     __syncthreads();
 #pragma unroll
     for (int e = tid; e < CB * PC; e += 256) C[(int64_t)(e / PC) * np + c0 + e % PC] = sC[e / PC][e % PC];
@@ -220,8 +284,9 @@ __global__ void __launch_bounds__(256) k_sweep_panel(int np, int K, float2 *__re
 // M_IJ -= Cp_I^T T_J for the tiles I <= J off block K; the first CTA of each
 // matrix takes the next diagonal block and sweeps it.
 __global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, float2 *__restrict__ M,
-                                                         float2 *__restrict__ P, const float2 *__restrict__ Cp,
-                                                         const float2 *__restrict__ Tp) {
+                                                         float2 *__restrict__ P, const float2 *Cp,
+                                                         const float2 *Tp) {
+    chain_wait();
     extern __shared__ __align__(16) float2 sm[];
     float2(*sA)[CB] = reinterpret_cast<float2(*)[CB]>(sm);
     float2(*sB)[CB] = sA + CB;
@@ -249,6 +314,18 @@ __global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, 
     float2 *Mj = M + (int64_t)j * np * np;
     const float2 *C = Cp + (int64_t)j * CB * np + I * CB, *T = Tp + (int64_t)j * CB * np + J * CB;
     float2 *D = Mj + (int64_t)I * CB * np + J * CB;
+    // both panels by asynchronous copies, in two halves of K: all of a thread's
+    // 16 loads are in flight at once and the product starts on the first half
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int q = 0; q < CB * CB / 4 / 256; ++q) {
+            const int e = tid + 256 * q, r = h * (CB / 2) + e / (CB / 2), c = e % (CB / 2) * 2;
+            cp_async16(&sA[r][c], C + (int64_t)r * np + c);
+            cp_async16(&sB[r][c], T + (int64_t)r * np + c);
+        }
+        cp_async_commit();
+    }
     float2 m[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -258,14 +335,12 @@ __global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, 
             m[i][2 * h] = make_float2(v.x, v.y);
             m[i][2 * h + 1] = make_float2(v.z, v.w);
         }
-    for (int e = tid; e < CB * CB / 2; e += 256) {
-        const int r = e / (CB / 2), c = e % (CB / 2) * 2;
-        *reinterpret_cast<float4 *>(&sA[r][c]) = *reinterpret_cast<const float4 *>(C + (int64_t)r * np + c);
-        float4 v = *reinterpret_cast<const float4 *>(T + (int64_t)r * np + c);
-        *reinterpret_cast<float4 *>(&sB[r][c]) = make_float4(-v.x, -v.y, -v.z, -v.w);
-    }
+    cp_async_wait<1>();
     __syncthreads();
-    tile_product(sA, sB, ty, tx, m);
+    tile_product<CB / 2>(sA, sB, ty, tx, m);
+    cp_async_wait<0>();
+    __syncthreads();
+    tile_product<CB / 2>(sA + CB / 2, sB + CB / 2, ty, tx, m);
     if (next && blockIdx.y == 0) {
         __syncthreads();   // the panels' shared memory holds the pivot rows from here
         sweep_store(m, sA, np, (K + 1) * CB, Mj, P + (int64_t)j * CB * CB, ty, tx);
@@ -280,8 +355,9 @@ __global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, 
 }
 
 // Minv = -M from M's upper triangle (n x n, symmetric), 32 x 32 tiles
-__global__ void __launch_bounds__(256) k_sweep_finish(int n, int np, const float2 *__restrict__ M,
+__global__ void __launch_bounds__(256) k_sweep_finish(int n, int np, const float2 *M,
                                                       float2 *__restrict__ Minv) {
+    chain_wait();
     __shared__ float2 s[32][33];
     if (blockIdx.x < blockIdx.y) return;
     const float2 *Mj = M + (int64_t)blockIdx.z * np * np;
@@ -338,20 +414,20 @@ void coarse_inverse(Ctx &ctx, int n, const PoleSet<float> &ps, const int32_t *pt
     k_dense_shift<<<dim3(np, N), 128, 0, ctx.stream>>>(n, np, ptr, col, ab, ps, M);
     ctx.after();
     ctx.before(KC_MG_COARSE, 16.0 * N * CB * CB, 8.0 * N * CB * CB * CB);
-    k_first_block<<<N, 256, 0, ctx.stream>>>(np, M, P);
+    launch_chained(ctx, k_first_block, N, 256, 0, np, M, P);
     ctx.after();
     if (nb > 1)
         for (int K = 0; K < nb; ++K) {
             ctx.before(KC_MG_COARSE, 24.0 * N * CB * np, 8.0 * N * CB * CB * (double)np);
-            k_sweep_panel<<<dim3(N, 2 * (nb - 1)), 256, PANEL_SMEM, ctx.stream>>>(np, K, M, P, Cp, Tp);
+            launch_chained(ctx, k_sweep_panel, dim3(N, 2 * (nb - 1)), 256, PANEL_SMEM, np, K, M, P, Cp, Tp);
             ctx.after();
             ctx.before(KC_MG_COARSE, 8.0 * N * np * (double)np, 4.0 * N * CB * (double)np * np);
-            k_sweep_update<<<dim3(N, (nb - 1) * nb / 2), 256, SWEEP_SMEM, ctx.stream>>>(np, nb, K, M, P, Cp, Tp);
+            launch_chained(ctx, k_sweep_update, dim3(N, (nb - 1) * nb / 2), 256, SWEEP_SMEM, np, nb, K, M, P, Cp, Tp);
             ctx.after();
         }
     ctx.before(KC_MG_COARSE, 12.0 * N * n * (double)n, 0);
     const unsigned g = (unsigned)((n + 31) / 32);
-    k_sweep_finish<<<dim3(g, g, N), 256, 0, ctx.stream>>>(n, np, M, Minv);
+    launch_chained(ctx, k_sweep_finish, dim3(g, g, N), 256, 0, n, np, M, Minv);
     ctx.after();
 }
 
