@@ -390,8 +390,8 @@ __device__ __forceinline__ void rr_pair(int k, int r, int mp, int &a, int &b) {
 // applied at once, A in shared memory with an odd row pitch.  Bound by shared
 // memory: the 2 x 2 block (k, l) of two pairs takes its row and its column
 // rotation in one visit, so A is read and written once per round (rows, then
-// columns, then the columns of V took three times that: 1.52 ms at m = 150, 1.22 now),
-// and the vectors are not formed here: the rotations are logged and
+// columns, then the columns of V took three times that: 1.52 ms at m = 150, 1.15
+// now, with a thread's column pair and rotation fixed for the round), and the vectors are not formed here: the rotations are logged and
 // k_jacobi_vectors applies them, every row on its own SM.  Two block barriers
 // per round: rotations, update.  A rotation is skipped below rel_tol of
 // sqrt(|a_pp a_qq|); the sweeps stop once every rotation of a sweep was below
@@ -409,16 +409,23 @@ __device__ __forceinline__ void rotate(float c, float s, float &x, float &y) {
     y = s * u + c * v;
 }
 
-// Padded order, row pitch and threads of the one-block Jacobi
+// A rotation (1, 0: none) with its pair p < q
+struct __align__(16) PairRotation {
+    float c, s;
+    int p, q;
+};
+
+// Padded order, row pitch and threads of the one-block Jacobi: in the update
+// thread l + npair * kg takes the blocks (kg + i groups, l)
 struct Jacobi32Shape {
-    int mp, npair, ld, threads;
+    int mp, npair, ld, groups;
     __host__ __device__ explicit Jacobi32Shape(int m) {
         mp = m + (m & 1);
         npair = mp / 2;
         ld = mp + 1;
-        threads = (npair * npair + 31) / 32 * 32;
-        threads = threads < 128 ? 128 : (threads > 1024 ? 1024 : threads);
+        groups = 1024 / npair < npair ? 1024 / npair : npair;
     }
+    __host__ __device__ int threads() const { return (groups * npair + 31) / 32 * 32; }
     size_t bytes() const { return (size_t)mp * ld * sizeof(float); }
 };
 
@@ -432,8 +439,7 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *S, doubl
     float *A = jsm;   // mp x mp: an odd order's last row and column are zero
     const int tid = threadIdx.x, bs = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5, nwarp = bs >> 5;
-    __shared__ float2 cs[JMAX / 2];    // c, s of a pair (1, 0: no rotation)
-    __shared__ int2 pq[JMAX / 2];
+    __shared__ PairRotation par[JMAX / 2];
     __shared__ int maxrel;             // largest relative pivot of the sweep (float bits)
     __shared__ double red[32];
     __shared__ float absmin;
@@ -454,9 +460,7 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *S, doubl
         maxrel = 0;
     }
     __syncthreads();
-    // this thread's blocks (k, l): every bs-th of the npair x npair, l fastest
-    const int k_first = tid / npair, l_first = tid - k_first * npair;
-    const int dk = bs / npair, dl = bs - dk * npair;
+    const int kg = tid / npair, l = tid - kg * npair;
     int64_t g = 0;   // rounds applied
     for (int sweep = 0; sweep < J32_SWEEPS; ++sweep) {
         for (int r = 0; r < mp - 1; ++r, ++g) {
@@ -478,36 +482,30 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *S, doubl
                         atomicMax(&maxrel, __float_as_int(rel));
                     }
                 }
-                cs[tid] = make_float2(c, sv);
-                pq[tid] = make_int2(p, q);
+                par[tid] = PairRotation{c, sv, p, q};
                 rlog[g * npair + tid] = make_float2(a > b ? -c : c, sv);   // the sign: lower row first
             }
             __syncthreads();
-            for (int k = k_first, l = l_first; k < npair;) {
-                const float2 wk = cs[k], wl = cs[l];
-                if (wk.y != 0.f || wl.y != 0.f) {
-                    const int2 ik = pq[k], il = pq[l];
-                    float *Ap = A + ik.x * ld, *Aq = A + ik.y * ld;
-                    float xpp = Ap[il.x], xpq = Ap[il.y], xqp = Aq[il.x], xqq = Aq[il.y];
-                    if (wk.y != 0.f) {
-                        rotate(wk.x, wk.y, xpp, xqp);
-                        rotate(wk.x, wk.y, xpq, xqq);
+            if (kg < sh.groups) {
+                const PairRotation wl = par[l];
+                for (int k = kg; k < npair; k += sh.groups) {
+                    const PairRotation wk = par[k];
+                    if (wk.s == 0.f && wl.s == 0.f) continue;
+                    float *Ap = A + wk.p * ld, *Aq = A + wk.q * ld;
+                    float xpp = Ap[wl.p], xpq = Ap[wl.q], xqp = Aq[wl.p], xqq = Aq[wl.q];
+                    if (wk.s != 0.f) {
+                        rotate(wk.c, wk.s, xpp, xqp);
+                        rotate(wk.c, wk.s, xpq, xqq);
                     }
-                    if (wl.y != 0.f) {
-                        rotate(wl.x, wl.y, xpp, xpq);
-                        rotate(wl.x, wl.y, xqp, xqq);
+                    if (wl.s != 0.f) {
+                        rotate(wl.c, wl.s, xpp, xpq);
+                        rotate(wl.c, wl.s, xqp, xqq);
                     }
                     if (k == l) xpq = xqp = 0.f;
-                    Ap[il.x] = xpp;
-                    Ap[il.y] = xpq;
-                    Aq[il.x] = xqp;
-                    Aq[il.y] = xqq;
-                }
-                k += dk;
-                l += dl;
-                if (l >= npair) {
-                    l -= npair;
-                    ++k;
+                    Ap[wl.p] = xpp;
+                    Ap[wl.q] = xpq;
+                    Aq[wl.p] = xqp;
+                    Aq[wl.q] = xqq;
                 }
             }
             __syncthreads();
@@ -1526,7 +1524,7 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
     if (m <= JMAX) {
         const Jacobi32Shape sh(m);
         ctx.before(KC_SMALL_DENSE, 8.0 * m2, 6.0 * (double)m * m2 * 8);
-        launch_chained(ctx, k_jacobi32, 1, sh.threads, sh.bytes(), m, S, lam0, label, rlog, cnt + 6, 1e-6f);
+        launch_chained(ctx, k_jacobi32, 1, sh.threads(), sh.bytes(), m, S, lam0, label, rlog, cnt + 6, 1e-6f);
         ctx.after();
         jacobi_vectors(ctx, m, rlog, cnt + 6, label, S0);
     } else {
