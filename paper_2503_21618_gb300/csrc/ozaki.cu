@@ -403,7 +403,6 @@ __global__ void __launch_bounds__(256) k_oz_split_panel(int64_t n, int m, int64_
 }
 
 // M = 128, N = 64, bf16 x bf16 -> FP32, both operands K-major
-constexpr uint32_t TC_IDESC = umma_idesc_bf16(TC_TM, TC_TN);
 
 // V 2^e for an int64 V, rounded to nearest even, in integer arithmetic: FP64
 // conversions and FMAs issue at ~1.6 per clock and SM, and four of them per
@@ -457,10 +456,12 @@ __device__ __forceinline__ double oz_combine_f64(const float v[OZ_S]) {
 // 0: the MMAs.  Warps 2..9: epilogue (a warp reads the TMEM lanes of its
 // quarter: rows; the two warps of a quarter take 32 columns each), integer
 // combination, rows staged in shared memory for coalesced stores.
-// Bound by the MMAs (28 digit pairs; at N = 64 an MMA reads 6 KB of shared
-// memory in 48 clocks); the fill, the allocation and the epilogue of a CTA
-// per block were exposed before: 186 -> 175 us per Gram, 319 -> 249 us per
-// tall product at 89 401 x 150.
+// Bound by the MMAs: 28 digit pairs.  One by one, at N = 64, they are bound by
+// shared memory (6 KB in 48 clocks each); the digits of B that share a digit of
+// A are one MMA of up to N = 256 (12 KB in 128 clocks): 175 -> 129 us per Gram,
+// 249 -> 231 us per tall product at 89 401 x 150 (the latter's epilogue shows).
+// Before that the fill, the allocation and the epilogue of a CTA per block were
+// exposed (186 and 319 us).
 struct OzItem {
     int ta, tb;
     int64_t ks0;
@@ -578,15 +579,18 @@ k_oz_gram_tc(int m, int nta, int ntb, int live, int64_t items, int64_t nks, int 
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t a0 = umma_desc(smem_addr(stA + st * TC_STAGE_A));
                     const uint64_t b0 = umma_desc(smem_addr(stB + st * TC_STAGE_B));
+                    // digit s of A times the digits t0 .. of B: their panels follow one another in the
+                    // stage, as the sums d = s + t do in TMEM, so up to four of them are one MMA
 #pragma unroll
-                    for (int d = 0; d < OZ_S; ++d)
+                    for (int k16 = 0; k16 < 2; ++k16)
 #pragma unroll
-                        for (int sd = 0; sd <= d; ++sd)
+                        for (int sd = 0; sd < OZ_S; ++sd)
 #pragma unroll
-                            for (int k16 = 0; k16 < 2; ++k16)
-                                umma_bf16(tmem + (uint32_t)(d * TC_TN),
+                            for (int t0 = 0; t0 < OZ_S - sd; t0 += 4)
+                                umma_bf16(tmem + (uint32_t)((sd + t0) * TC_TN),
                                           umma_desc_at(a0, sd * 2 * TC_PANEL + k16 * 256u),
-                                          umma_desc_at(b0, (d - sd) * TC_PANEL + k16 * 256u), TC_IDESC,
+                                          umma_desc_at(b0, t0 * TC_PANEL + k16 * 256u),
+                                          umma_idesc_bf16(TC_TM, (OZ_S - sd - t0 < 4 ? OZ_S - sd - t0 : 4) * TC_TN),
                                           sd == 0 && k16 == 0 ? (k > 0) : 1u);
                     umma_commit(empty + st);   // stage free once these MMAs have read it
                 }
