@@ -7,10 +7,10 @@
 // that size is solved exactly by its shifted inverses: per solve, with the
 // poles known, every matrix M_j = A_l - sigma_j B_l (complex symmetric,
 // Im M_j = -Im(sigma_j) B_l definite, so every leading block is nonsingular
-// and no pivoting is needed) is formed densely and inverted in place by
-// blocked Gauss-Jordan elimination; the cycle then applies Z_j = M_j^{-1} R_j
-// as one batched complex GEMM per visit.  The inverse is symmetrised, so the
-// cycle stays a complex symmetric operator, as COCG requires.
+// and no pivoting is needed) is formed densely and inverted; the cycle then
+// applies Z_j = M_j^{-1} R_j, one batched product per visit.  The inverse is
+// symmetric to the last bit, so the cycle stays a complex symmetric operator,
+// as COCG requires.
 //
 // The elimination is the symmetric sweep in blocks of CB rows K (the rest R),
 // which keeps M complex symmetric, so only its block upper triangle is held

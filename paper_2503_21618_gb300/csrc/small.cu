@@ -390,8 +390,9 @@ __device__ __forceinline__ void rr_pair(int k, int r, int mp, int &a, int &b) {
 // applied at once, A in shared memory with an odd row pitch.  Bound by shared
 // memory: the 2 x 2 block (k, l) of two pairs takes its row and its column
 // rotation in one visit, so A is read and written once per round (rows, then
-// columns, then the columns of V took three times that: 1.52 ms at m = 150, 1.15
-// now, with a thread's column pair and rotation fixed for the round), and the vectors are not formed here: the rotations are logged and
+// columns, then the columns of V took three times that), and a thread's column
+// pair and its rotation are fixed for the round: 1.52 -> 1.15 ms at m = 150.
+// The vectors are not formed here: the rotations are logged and
 // k_jacobi_vectors applies them, every row on its own SM.  Two block barriers
 // per round: rotations, update.  A rotation is skipped below rel_tol of
 // sqrt(|a_pp a_qq|); the sweeps stop once every rotation of a sweep was below
