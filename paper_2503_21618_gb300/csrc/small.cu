@@ -559,7 +559,8 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *S, doubl
 //             keeps in full (updated in closed form); they go to all CTAs
 // The chain of double-float square roots and divisions (~1 us) thus hides behind
 // the update: 8.3 ms at m = 300 on 16 CTAs, against 11.6 ms on 8 with it, and the
-// rows' move, after the update.
+// rows' move, after the update; 8.0 with the divisions and the root of the skip
+// test as hardware approximations (each first quotient is corrected by a second).
 // The eigenvectors are not formed here: the rotations are logged (FP32) and
 // k_jacobi_vectors applies them to the rows of I afterwards, every row on its
 // own SM.  A rotation is skipped below rel_tol of sqrt(|a_pp a_qq|); the
@@ -615,9 +616,10 @@ __device__ __forceinline__ df df_rot(df c, df x, df s, df z) {
     return df_renorm(d, e);
 }
 __device__ __forceinline__ df df_div(df a, df b) {
-    const float q = a.h / b.h;
+    // both quotients to a few units in the last place: the second corrects the first
+    const float q = __fdividef(a.h, b.h);
     const df r = df_add(a, df_neg(df_mul({q, 0.f}, b)));
-    return df_renorm(q, r.h / b.h);
+    return df_renorm(q, __fdividef(r.h, b.h));
 }
 __device__ __forceinline__ df df_sqrt(df a) {
     const float y = rsqrtf(a.h), s = __fmul_rn(a.h, y);
@@ -711,7 +713,7 @@ k_jacobi_df(int m, const double *__restrict__ S, const double *__restrict__ fro_
         df cc = {1.f, 0.f}, ss = {0.f, 0.f}, da = {0.f, 0.f};
         if (max(a, b) < m) {
             const df app = diag[min(a, b)], aqq = diag[max(a, b)];
-            const float mag = sqrtf(fabsf(app.h * aqq.h));
+            const float prod = fabsf(app.h * aqq.h), mag = prod > 0.f ? prod * rsqrtf(prod) : 0.f;
             if (fabsf(apq.h) > rel_tol * mag && fabsf(apq.h) > absmin) {
                 // t = sign(th) / (|th| + sqrt(1 + th^2)), th = (a_qq - a_pp) / (2 a_pq)
                 const df d = df_add(aqq, df_neg(app)), a2 = {2.f * apq.h, 2.f * apq.l};
@@ -726,7 +728,7 @@ k_jacobi_df(int m, const double *__restrict__ S, const double *__restrict__ fro_
                     ss = df_neg(ss);
                     da = df_neg(da);
                 }
-                atomicMax(&mx[sweep & 1], __float_as_int(fabsf(apq.h) / (mag > 0.f ? mag : 1.f)));
+                atomicMax(&mx[sweep & 1], __float_as_int(__fdividef(fabsf(apq.h), mag > 0.f ? mag : 1.f)));
             }
         }
         const float4 v = make_float4(cc.h, cc.l, ss.h, ss.l);
