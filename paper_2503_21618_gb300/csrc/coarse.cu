@@ -381,7 +381,20 @@ __global__ void __launch_bounds__(256) k_sweep_finish(int n, int np, const float
     }
 }
 
-constexpr size_t SWEEP_SMEM = 2 * CB * CB * sizeof(float2);
+constexpr size_t SWEEP_SMEM = 2 * CB * CB * sizeof(float2);   // three CTAs of the update per SM
+constexpr size_t SWEEP_SMEM_TWO = 100 * 1024;                 // two
+// Three or two CTAs of the update per SM.  The launch ends with the CTAs that
+// sweep the next diagonal blocks, which are faster beside one other CTA than
+// beside two; three per SM pay where they fill the last of several waves (over
+// three quarters of it), and where there are no more than two per SM anyway the
+// larger request only delays their start.  Cycle call, three against two per SM,
+// by the number of tiles on 152 SMs: 112: 370 / 395 us, 264: 711 / 721, 420: 870 /
+// 803, 480: 1073 / 906, 684: 1147 / 1029, 840: 1303 / 1377, 1104: 1764 / 1724.
+size_t sweep_update_smem(int sm_count, int64_t tiles) {
+    const int64_t wave = 3 * (int64_t)sm_count;
+    const bool three = tiles <= 2 * (int64_t)sm_count || (tiles > wave && 4 * (tiles % wave) > 3 * wave);
+    return three ? SWEEP_SMEM : SWEEP_SMEM_TWO;
+}
 constexpr size_t PANEL_SMEM = (CB * CB + CB * PLD) * sizeof(float2);
 
 // The kernels' shared-memory limit, raised once per device
@@ -391,7 +404,7 @@ void raise_sweep_smem() {
     cudaGetDevice(&dev);
     std::call_once(once[dev < 0 || dev >= 64 ? 0 : dev], [] {
         cudaFuncSetAttribute(k_sweep_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PANEL_SMEM);
-        cudaFuncSetAttribute(k_sweep_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SWEEP_SMEM);
+        cudaFuncSetAttribute(k_sweep_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SWEEP_SMEM_TWO);
     });
 }
 
@@ -410,6 +423,7 @@ void coarse_inverse(Ctx &ctx, int n, const PoleSet<float> &ps, const int32_t *pt
     float2 *Tp = Cp + (size_t)N * np * CB;                    // N x (CB x np)
     float2 *P = Tp + (size_t)N * np * CB;                     // N x (CB x CB)
     raise_sweep_smem();
+    const size_t update_smem = sweep_update_smem(ctx.sm_count, (int64_t)N * (nb - 1) * nb / 2);
     ctx.before(KC_MG_COARSE, 8.0 * N * np * np, 0);
     k_dense_shift<<<dim3(np, N), 128, 0, ctx.stream>>>(n, np, ptr, col, ab, ps, M);
     ctx.after();
@@ -422,7 +436,7 @@ void coarse_inverse(Ctx &ctx, int n, const PoleSet<float> &ps, const int32_t *pt
             launch_chained(ctx, k_sweep_panel, dim3(N, 2 * (nb - 1)), 256, PANEL_SMEM, np, K, M, P, Cp, Tp);
             ctx.after();
             ctx.before(KC_MG_COARSE, 8.0 * N * np * (double)np, 4.0 * N * CB * (double)np * np);
-            launch_chained(ctx, k_sweep_update, dim3(N, (nb - 1) * nb / 2), 256, SWEEP_SMEM, np, nb, K, M, P, Cp, Tp);
+            launch_chained(ctx, k_sweep_update, dim3(N, (nb - 1) * nb / 2), 256, update_smem, np, nb, K, M, P, Cp, Tp);
             ctx.after();
         }
     ctx.before(KC_MG_COARSE, 12.0 * N * n * (double)n, 0);
