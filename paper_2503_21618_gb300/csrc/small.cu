@@ -1586,9 +1586,14 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
         if (m > JMAX) {
             // a large group of close eigenvalues is too much for one block:
             // the cooperative Jacobi rotates whatever the refinement left
-            // above rounding level (it returns after one look if nothing is)
+            // above rounding level (it returns after one look if nothing is).
+            // That level is 1/2 eps ||S||_F: the entries of T = X^T S X between
+            // separated pairs are rounding of at most 0.28 eps ||S||_F (m = 161
+            // .. 448, spectra over up to six decades), so these cost no sweep,
+            // and a pair that the refinement took for too close to separate is
+            // rotated to it.
             identity(Vm);
-            const cudaError_t e = coop_jacobi(ctx, m, Tm, Vm, lam0, 60, normA, 2.0 * m, cnt);
+            const cudaError_t e = coop_jacobi(ctx, m, Tm, Vm, lam0, 60, normA, 0.5, cnt);
             if (e != cudaSuccess) return e;
             dgemm(ctx, 0, 0, m, m, m, X0, m, Vm, m, 0.0, X1, m, 1, nullptr, KC_SMALL_DENSE);
             ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
