@@ -396,12 +396,13 @@ __device__ __forceinline__ void rr_pair(int k, int r, int mp, int &a, int &b) {
 // k_jacobi_vectors applies them, every row on its own SM.  Two block barriers
 // per round: rotations, update.  A rotation is skipped below rel_tol of
 // sqrt(|a_pp a_qq|); the sweeps stop once every rotation of a sweep was below
-// sqrt(rel_tol) (quadratic convergence: the next sweep would find nothing).
+// sqrt(rel_tol) (quadratic convergence: the next sweep would find nothing), or
+// when the log is full (max_sweeps: what is left then is the refinement's).
 // Output: lam ascending (FP64), rank (the place of eigenvalue i in lam), the
 // log and *nrounds.
 // ---------------------------------------------------------------------------
 constexpr int JMAX = 160;
-constexpr int J32_SWEEPS = 40;
+constexpr int J32_SWEEPS = 40;   // at most; see log_sweeps
 
 // x' = c x - s y, y' = s x + c y
 __device__ __forceinline__ void rotate(float c, float s, float &x, float &y) {
@@ -432,7 +433,7 @@ struct Jacobi32Shape {
 
 __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *S, double *__restrict__ lam,
                                                   int *__restrict__ rank, float2 *__restrict__ rlog,
-                                                  int *__restrict__ nrounds, float rel_tol) {
+                                                  int *__restrict__ nrounds, int max_sweeps, float rel_tol) {
     chain_wait();
     extern __shared__ float jsm[];
     const Jacobi32Shape sh(m);
@@ -463,7 +464,7 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *S, doubl
     __syncthreads();
     const int kg = tid / npair, l = tid - kg * npair;
     int64_t g = 0;   // rounds applied
-    for (int sweep = 0; sweep < J32_SWEEPS; ++sweep) {
+    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
         for (int r = 0; r < mp - 1; ++r, ++g) {
             if (tid < npair) {
                 int a, b;
@@ -569,7 +570,7 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *S, doubl
 // ---------------------------------------------------------------------------
 constexpr int JDF_MAX = 448;      // a CTA's rows of an 8-CTA cluster in 227 KB
 constexpr int JDF_CTAS = 8, JDF_CTAS_WIDE = 16;
-constexpr int JDF_SWEEPS = 20;
+constexpr int JDF_SWEEPS = 20;    // at most; see log_sweeps
 constexpr int JDF_THREADS = 544;  // 16 warps for the update, one for the rotations
 static_assert(JDF_MAX <= 2 * 32 * JDF_CTAS, "one lane of warp 0 per position of a CTA");
 constexpr int JVEC_ROUNDS = 8;    // rounds of the log per stage of k_jacobi_vectors
@@ -658,7 +659,7 @@ struct JacobiShape {
 
 __global__ void __launch_bounds__(JDF_THREADS, 1)
 k_jacobi_df(int m, const double *__restrict__ S, const double *__restrict__ fro_part, double *__restrict__ lam,
-            float2 *__restrict__ rlog, int *__restrict__ nrounds, float rel_tol) {
+            float2 *__restrict__ rlog, int *__restrict__ nrounds, int max_sweeps, float rel_tol) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     const int C = (int)cl.num_blocks(), c = (int)cl.block_rank();
@@ -746,7 +747,7 @@ k_jacobi_df(int m, const double *__restrict__ S, const double *__restrict__ fro_
 
     int64_t g = 0;   // rounds applied
     int cur = 0;
-    for (int sweep = 0; sweep < JDF_SWEEPS; ++sweep) {
+    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
         for (int r = 0; r < mp - 1; ++r) {
             const float4 *P = par + cur * npair;
             const int *sT = slot_of(cur, 0), *sB = slot_of(cur, 1);
@@ -1152,21 +1153,25 @@ __global__ void __launch_bounds__(256) k_sort_eig(int m, const double *lam_in, c
     for (int j = lane; j < m; j += 32) Q[(int64_t)row * m + rank[j]] = S[(int64_t)row * m + j];
 }
 
-static size_t syev_base_bytes(int m) {
-    const size_t mp = (size_t)(m + (m & 1));
-    const size_t m2 = (size_t)m * m;
-    // group blocks (2 mp^2 doubles) + S0, S1, G, Y, T, V (6 m^2) + lam0, partial norms, counters,
-    // component labels and sizes (2 m ints)
-    const size_t b = 2 * mp * mp * sizeof(double) + 6 * m2 * sizeof(double) +
-                     ((size_t)m + FRO_PARTS + OA_PARTS) * sizeof(double) + 2 * (size_t)m * sizeof(int) + 4096;
-    return (b + 255) / 256 * 256;
+// Matrices of the eigensolver's workspace in front of its vectors and counters:
+// the group blocks (2 mp^2 doubles) and S0, S1, G, Y, T, V (6 m^2)
+static size_t syev_matrix_bytes(int m) {
+    const size_t mp = (size_t)(m + (m & 1)), m2 = (size_t)m * m;
+    return (2 * mp * mp + 6 * m2) * sizeof(double);
 }
 size_t small_syev_work_bytes(int m) {
-    // the rotation log (one entry per pair and round, one round more)
+    // + lam0, partial norms, counters, component labels and sizes (2 m ints)
+    return syev_matrix_bytes(m) + (2 * (size_t)m + 2) * sizeof(double) + 2 * (size_t)m * sizeof(int) + 4096;
+}
+// The rotation log of the Jacobi that precedes the refinement (one entry per
+// pair and round, one round more) takes the matrices' place behind S0, which are
+// written after the vectors are formed.  It holds 13 sweeps, a few less below
+// m = 10; 6 to 9 are the rule.
+static int log_sweeps(int m, int most) {
     const size_t mp = (size_t)(m + (m & 1));
-    const size_t sweeps = m <= JMAX ? J32_SWEEPS : JDF_SWEEPS;
-    const size_t log = m > JDF_MAX ? 0 : (sweeps * (mp - 1) + 1) * (mp / 2) * sizeof(float2);
-    return syev_base_bytes(m) + log + 32;   // the log starts on 16 bytes and is read in 16s
+    const size_t room = syev_matrix_bytes(m) - (size_t)m * m * sizeof(double) - 16;   // the log starts on 16 bytes
+    const size_t rounds = room / (mp / 2 * sizeof(float2)) - 1;
+    return (int)std::min<size_t>(most, rounds / (mp - 1));
 }
 
 // ---------------------------------------------------------------------------
@@ -1483,11 +1488,10 @@ static int jacobi_df_ctas() {
 cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q, double *work, int mode) {
     const size_t m2 = (size_t)m * m;
     const size_t mp = (size_t)(m + (m & 1));
-    char *w = reinterpret_cast<char *>(work);
-    void *Ag = w;
-    void *Vg = w + mp * mp * sizeof(double);
-    double *S0 = reinterpret_cast<double *>(w + 2 * mp * mp * sizeof(double));
-    double *S1 = S0 + m2;
+    double *S0 = work;
+    void *Ag = S0 + m2;
+    void *Vg = S0 + m2 + mp * mp;
+    double *S1 = S0 + m2 + 2 * mp * mp;
     double *G = S1 + m2;
     double *Ym = G + m2;
     double *Tm = Ym + m2;
@@ -1498,8 +1502,8 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
     int *cnt = reinterpret_cast<int *>(oa_part + OA_PARTS);
     int32_t *cst = cnt + 4;   // cnt[6]: rounds of the Jacobi
     int *label = cst + 4, *csize = label + m;   // label: the FP32 Jacobi's ranks first
-    // 16-byte aligned (work is a multiple of 8 bytes) for the vectors' bulk loads
-    float2 *rlog = reinterpret_cast<float2 *>((reinterpret_cast<uintptr_t>(w + syev_base_bytes(m)) + 15) / 16 * 16);
+    // 16-byte aligned (work is a multiple of 8 bytes) for the vectors' 16-byte loads
+    float2 *rlog = reinterpret_cast<float2 *>((reinterpret_cast<uintptr_t>(Ag) + 15) / 16 * 16);
 
     ctx.before(KC_SMALL_DENSE, 8.0 * m2, 2.0 * m2);
     launch_chained(ctx, k_fro, FRO_PARTS, 256, 0, m, S, normA);
@@ -1527,7 +1531,8 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
     if (m <= JMAX) {
         const Jacobi32Shape sh(m);
         ctx.before(KC_SMALL_DENSE, 8.0 * m2, 6.0 * (double)m * m2 * 8);
-        launch_chained(ctx, k_jacobi32, 1, sh.threads(), sh.bytes(), m, S, lam0, label, rlog, cnt + 6, 1e-6f);
+        launch_chained(ctx, k_jacobi32, 1, sh.threads(), sh.bytes(), m, S, lam0, label, rlog, cnt + 6,
+                       log_sweeps(m, J32_SWEEPS), 1e-6f);
         ctx.after();
         jacobi_vectors(ctx, m, rlog, cnt + 6, label, S0);
     } else {
@@ -1545,7 +1550,8 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
         const cudaError_t je =
-            cudaLaunchKernelEx(&cfg, k_jacobi_df, m, S, (const double *)normA, lam0, rlog, cnt + 6, 1e-10f);
+            cudaLaunchKernelEx(&cfg, k_jacobi_df, m, S, (const double *)normA, lam0, rlog, cnt + 6,
+                               log_sweeps(m, JDF_SWEEPS), 1e-10f);
         ctx.after();
         if (je != cudaSuccess) return je;
         jacobi_vectors(ctx, m, rlog, cnt + 6, nullptr, S0);
