@@ -1077,7 +1077,7 @@ slrf_status mg_prepare(slrf_handle *h, const slrf_filter *f, const KrylovDims &d
     mg.Minv = nullptr;
     if (e_inv >= 0) {
         if constexpr (sizeof(T) == 4) {
-            const size_t inv_bytes = (size_t)N * nc * nc * sizeof(cplx<T>);
+            const size_t inv_bytes = (size_t)N * nc * coarse_inverse_ld(nc) * sizeof(cplx<T>);
             const size_t inv_off = (inv_bytes + 255) / 256 * 256;
             CKS(ensure(h, h->mgInv, inv_off + coarse_inverse_work_bytes(nc, N)));
             float2 *Minv = reinterpret_cast<float2 *>(h->mgInv.p);
@@ -1858,7 +1858,7 @@ size_t workspace_estimate(int64_t n, int64_t nnz, int L, int N, int precision, i
         // split vectors and partial sums of their tensor-core application
         if (precision == SLRF_PREC_MIXED) {
             const size_t ne = std::min<size_t>(1536, (size_t)n);
-            mgb += (size_t)N * ne * ne * 8 + coarse_inverse_work_bytes((int)ne, N);
+            mgb += (size_t)N * ne * coarse_inverse_ld((int)ne) * 8 + coarse_inverse_work_bytes((int)ne, N);
             if (coarse_tc_fits((int)Lp))
                 mgb += coarse_tc_panel_bytes((int)ne, N) + coarse_tc_work_bytes((int)ne, N, (int)Lp);
         }

@@ -16,8 +16,10 @@
 // which keeps M complex symmetric, so only its block upper triangle is held
 // and half the arithmetic of Gauss-Jordan is done:
 //   P = M_KK^{-1},  T = P M_KR,  M_RR -= M_KR^T T,  M_KR = T,  M_KK = -P;
-// after the last block M holds -M^{-1}.  M is padded to whole blocks with the
-// identity.  Two launches per block: the panel (T, every block column its own
+// after the last block M holds -M^{-1}.  It runs in the inverses' own storage
+// (a copy padded to whole blocks would double the memory of the level); the
+// last block's padding, the identity, is put in where its tiles are loaded.
+// Two launches per block: the panel (T, every block column its own
 // CTA), and the update, one CTA per 64 x 64 tile, whose first CTA takes the
 // next diagonal block and sweeps it in registers while the others work, so
 // most of the chain of 64 pivots (~15 us) hides behind the update.  Bound by FP32
@@ -40,16 +42,16 @@ namespace {
 
 constexpr int CB = 64;   // block size of the sweep
 
-// M_j = A - sigma_j B on the level's CSR pattern of (a, b) pairs, dense, np x
-// np (rows and columns from n on: the identity)
-__global__ void k_dense_shift(int n, int np, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
+// M_j = A - sigma_j B on the level's CSR pattern of (a, b) pairs, dense, rows
+// of ld = coarse_inverse_ld(n) entries (the one beyond n, if any, is zero and
+// stays so)
+__global__ void k_dense_shift(int n, int ld, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
                               const float2 *__restrict__ ab, PoleSet<float> ps, float2 *__restrict__ M) {
     const int row = blockIdx.x;
     const int j = blockIdx.y;
-    float2 *Mr = M + ((int64_t)j * np + row) * np;
-    for (int c = threadIdx.x; c < np; c += blockDim.x) Mr[c] = make_float2(row >= n && c == row ? 1.f : 0.f, 0.f);
+    float2 *Mr = M + ((int64_t)j * n + row) * ld;
+    for (int c = threadIdx.x; c < ld; c += blockDim.x) Mr[c] = make_float2(0.f, 0.f);
     __syncthreads();
-    if (row >= n) return;
     const float sr = ps.re[j], si = ps.im[j];
     for (int k = ptr[row] + threadIdx.x; k < ptr[row + 1]; k += blockDim.x) {
         const float2 w = ab[k];
@@ -62,9 +64,14 @@ __global__ void k_dense_shift(int n, int np, const int32_t *__restrict__ ptr, co
 // one broadcast and the columns' two conflict-free 16-byte shared loads.
 __device__ __forceinline__ int tile_col(int tx, int q) { return 2 * tx + 32 * (q >> 1) + (q & 1); }
 
-// 16-byte asynchronous copies to shared memory
+// 16-byte asynchronous copies to shared memory; the second form writes zeros
+// (and reads nothing) unless `in`
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool in) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(in ? 16 : 0)
+                 : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int LEFT> __device__ __forceinline__ void cp_async_wait() {
@@ -186,75 +193,81 @@ __device__ __forceinline__ void tile_sweep(float2 (&S)[4][4], float2 (*row)[CB],
     pivot_rows<3, 3>(S, v.w, v.r, v.pinv, ty == CB / 4 - 1, tx == 15, 14);
 }
 
-// Sweep of the diagonal block at k0: M_KK = -P, and P beside it
-__device__ __forceinline__ void sweep_store(float2 (&S)[4][4], float2 (*row)[CB], int np, int k0, float2 *__restrict__ M,
-                                            float2 *__restrict__ P, int ty, int tx) {
+// Sweep of the diagonal block at k0: M_KK = -P
+__device__ __forceinline__ void sweep_store(float2 (&S)[4][4], float2 (*row)[CB], int n, int ld, int k0,
+                                            float2 *__restrict__ M, int ty, int tx) {
     tile_sweep(S, row, ty, tx);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int r = 4 * ty + i, c = tile_col(tx, q);
-            M[(int64_t)(k0 + r) * np + k0 + c] = S[i][q];
-            P[r * CB + c] = make_float2(-S[i][q].x, -S[i][q].y);
+            if (max(r, c) < n - k0) M[(int64_t)(k0 + r) * ld + k0 + c] = S[i][q];
         }
 }
 
-__global__ void __launch_bounds__(256) k_first_block(int np, float2 *__restrict__ M, float2 *__restrict__ P) {
+__global__ void __launch_bounds__(256) k_first_block(int n, int ld, float2 *__restrict__ M) {
     chain_wait();
     __shared__ __align__(16) float2 row[2][CB];
-    float2 *Mj = M + (int64_t)blockIdx.x * np * np;
+    float2 *Mj = M + (int64_t)blockIdx.x * n * ld;
     const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
     float2 S[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) S[i][q] = Mj[(int64_t)(4 * ty + i) * np + tile_col(tx, q)];
-    sweep_store(S, row, np, 0, Mj, P + (int64_t)blockIdx.x * CB * CB, ty, tx);
+        for (int q = 0; q < 4; ++q) {
+            const int r = 4 * ty + i, c = tile_col(tx, q);
+            S[i][q] = r < n && c < n ? Mj[(int64_t)r * ld + c] : make_float2(r == c ? 1.f : 0.f, 0.f);
+        }
+    sweep_store(S, row, n, ld, 0, Mj, ty, tx);
 }
 
 // Panel of block K: the old rows M_K* (from the upper triangle: M_KJ for J >
 // K, M_JK^T for J < K) to Cp, T = P M_K* to Tp and in place of the old block;
-// one CTA per matrix and 32 columns.
+// one CTA per matrix and 32 columns.  Cp and Tp have the columns of the other
+// blocks only (pitch lq).
 constexpr int PC = 32, PLD = PC + 2;   // columns of a panel CTA, their pitch
-__global__ void __launch_bounds__(256) k_sweep_panel(int np, int K, float2 *__restrict__ M,
-                                                     const float2 *P, float2 *__restrict__ Cp,
-                                                     float2 *__restrict__ Tp) {
+__global__ void __launch_bounds__(256) k_sweep_panel(int n, int ld, int lq, int K, float2 *__restrict__ M,
+                                                     float2 *__restrict__ Cp, float2 *__restrict__ Tp) {
     chain_wait();
     extern __shared__ __align__(16) float2 sm[];
     float2(*sP)[CB] = reinterpret_cast<float2(*)[CB]>(sm);
     float2(*sC)[PLD] = reinterpret_cast<float2(*)[PLD]>(sm + CB * CB);
     const int j = blockIdx.x, Jh = blockIdx.y >> 1, J = Jh + (Jh >= K ? 1 : 0);
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    float2 *Mj = M + (int64_t)j * np * np;
-    float2 *C = Cp + (int64_t)j * CB * np, *T = Tp + (int64_t)j * CB * np;
-    const int k0 = K * CB, c0 = J * CB + (blockIdx.y & 1) * PC;
+    float2 *Mj = M + (int64_t)j * n * ld;
+    float2 *C = Cp + (int64_t)j * CB * lq, *T = Tp + (int64_t)j * CB * lq;
+    const int k0 = K * CB, c0 = J * CB + (blockIdx.y & 1) * PC, q0 = Jh * CB + (blockIdx.y & 1) * PC;
 #pragma unroll
-    for (int q = 0; q < CB * CB / 2 / 256; ++q)
-        cp_async16(&sP[0][0] + 2 * (tid + 256 * q), P + (int64_t)j * CB * CB + 2 * (tid + 256 * q));   // symmetric
-    if (J > K)
+    for (int q = 0; q < CB * CB / 2 / 256; ++q) {   // -P, symmetric
+        const int e = tid + 256 * q, r = k0 + e / (CB / 2), c = k0 + e % (CB / 2) * 2;
+        const bool in = r < n && c < n;
+        cp_async16(&sP[0][0] + 2 * e, in ? Mj + (int64_t)r * ld + c : Mj, in);
+    }
+    if (J > K)   // block K is not the last: all its rows are there
 #pragma unroll
         for (int q = 0; q < CB * PC / 2 / 256; ++q) {
             const int e = tid + 256 * q, r = e / (PC / 2), c = e % (PC / 2) * 2;
-            cp_async16(&sC[r][c], Mj + (int64_t)(k0 + r) * np + c0 + c);
+            const bool in = c0 + c < n;
+            cp_async16(&sC[r][c], in ? Mj + (int64_t)(k0 + r) * ld + c0 + c : Mj, in);
         }
-    else
+    else         // all columns of block J are there
 #pragma unroll
         for (int e = tid; e < CB * PC; e += 256)
-            sC[e % CB][e / CB] = Mj[(int64_t)(c0 + e / CB) * np + k0 + e % CB];
+            sC[e % CB][e / CB] = k0 + e % CB < n ? Mj[(int64_t)(c0 + e / CB) * ld + k0 + e % CB] : make_float2(0.f, 0.f);
     cp_async_commit();
     cp_async_wait<0>();
     __syncthreads();
 #pragma unroll
-    for (int e = tid; e < CB * PC; e += 256) C[(int64_t)(e / PC) * np + c0 + e % PC] = sC[e / PC][e % PC];
+    for (int e = tid; e < CB * PC; e += 256) C[(int64_t)(e / PC) * lq + q0 + e % PC] = sC[e / PC][e % PC];
     float2 acc[4][2] = {};
 #pragma unroll 4
     for (int k = 0; k < CB; ++k) {   // P^T = P
         const float4 a01 = *reinterpret_cast<const float4 *>(&sP[k][4 * ty]);
         const float4 a23 = *reinterpret_cast<const float4 *>(&sP[k][4 * ty + 2]);
         const float4 b01 = *reinterpret_cast<const float4 *>(&sC[k][2 * tx]);
-        const float2 a[4] = {make_float2(a01.x, a01.y), make_float2(a01.z, a01.w), make_float2(a23.x, a23.y),
-                             make_float2(a23.z, a23.w)};
+        const float2 a[4] = {make_float2(-a01.x, -a01.y), make_float2(-a01.z, -a01.w), make_float2(-a23.x, -a23.y),
+                             make_float2(-a23.z, -a23.w)};
         const float2 b[2] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w)};
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -263,10 +276,10 @@ __global__ void __launch_bounds__(256) k_sweep_panel(int np, int K, float2 *__re
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const int r = 4 * ty + i, c = c0 + 2 * tx;
+        const int r = 4 * ty + i;
         const float4 v = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
-        *reinterpret_cast<float4 *>(T + (int64_t)r * np + c) = v;
-        if (J > K) *reinterpret_cast<float4 *>(Mj + (int64_t)(k0 + r) * np + c) = v;
+        *reinterpret_cast<float4 *>(T + (int64_t)r * lq + q0 + 2 * tx) = v;
+        if (J > K && c0 + 2 * tx < n) *reinterpret_cast<float4 *>(Mj + (int64_t)(k0 + r) * ld + c0 + 2 * tx) = v;
     }
     if (J < K) {   // transposed, through shared memory
         __syncthreads();
@@ -277,15 +290,14 @@ __global__ void __launch_bounds__(256) k_sweep_panel(int np, int K, float2 *__re
         __syncthreads();
 #pragma unroll
         for (int e = tid; e < CB * PC; e += 256)
-            Mj[(int64_t)(c0 + e / CB) * np + k0 + e % CB] = sC[e % CB][e / CB];
+            if (k0 + e % CB < n) Mj[(int64_t)(c0 + e / CB) * ld + k0 + e % CB] = sC[e % CB][e / CB];
     }
 }
 
 // M_IJ -= Cp_I^T T_J for the tiles I <= J off block K; the first CTA of each
 // matrix takes the next diagonal block and sweeps it.
-__global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, float2 *__restrict__ M,
-                                                         float2 *__restrict__ P, const float2 *Cp,
-                                                         const float2 *Tp) {
+__global__ void __launch_bounds__(256, 3) k_sweep_update(int n, int ld, int lq, int nb, int K, float2 *__restrict__ M,
+                                                         const float2 *Cp, const float2 *Tp) {
     chain_wait();
     extern __shared__ __align__(16) float2 sm[];
     float2(*sA)[CB] = reinterpret_cast<float2(*)[CB]>(sm);
@@ -293,7 +305,7 @@ __global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, 
     const int j = blockIdx.x;   // the matrices fastest: every first CTA starts at once
     // tile t of the upper triangle of the nb - 1 blocks other than K
     const bool next = K + 1 < nb;
-    int I, J;
+    int Ih, Jh;
     {
         int t = blockIdx.y;
         const int q = nb - 1;
@@ -305,15 +317,18 @@ __global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, 
             rem -= q - i;
             ++i;
         }
-        I = i;
-        J = i + rem;
-        if (I >= K) ++I;
-        if (J >= K) ++J;
+        Ih = i;
+        Jh = i + rem;
     }
+    const int I = Ih + (Ih >= K ? 1 : 0), J = Jh + (Jh >= K ? 1 : 0);
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    float2 *Mj = M + (int64_t)j * np * np;
-    const float2 *C = Cp + (int64_t)j * CB * np + I * CB, *T = Tp + (int64_t)j * CB * np + J * CB;
-    float2 *D = Mj + (int64_t)I * CB * np + J * CB;
+    float2 *Mj = M + (int64_t)j * n * ld;
+    const float2 *C = Cp + (int64_t)j * CB * lq + Ih * CB, *T = Tp + (int64_t)j * CB * lq + Jh * CB;
+    float2 *D = Mj + (int64_t)I * CB * ld + J * CB;
+    // whether the thread's rows i (bit i) and column pairs h (bit 4 + h) are inside
+    const int nr = n - I * CB - 4 * ty, nc = n - J * CB - 2 * tx;
+    const unsigned in = (nr >= 4 ? 15u : nr > 0 ? (1u << nr) - 1 : 0u) | (nc > 0 ? 16u : 0u) | (nc > 32 ? 32u : 0u);
+    auto inside = [&](int i, int h) { return (in >> i & 1) && (in >> (4 + h) & 1); };
     // both panels by asynchronous copies, in two halves of K: all of a thread's
     // 16 loads are in flight at once and the product starts on the first half
 #pragma unroll
@@ -321,8 +336,8 @@ __global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, 
 #pragma unroll
         for (int q = 0; q < CB * CB / 4 / 256; ++q) {
             const int e = tid + 256 * q, r = h * (CB / 2) + e / (CB / 2), c = e % (CB / 2) * 2;
-            cp_async16(&sA[r][c], C + (int64_t)r * np + c);
-            cp_async16(&sB[r][c], T + (int64_t)r * np + c);
+            cp_async16(&sA[r][c], C + (int64_t)r * lq + c);
+            cp_async16(&sB[r][c], T + (int64_t)r * lq + c);
         }
         cp_async_commit();
     }
@@ -331,7 +346,10 @@ __global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, 
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const float4 v = *reinterpret_cast<const float4 *>(D + (int64_t)(4 * ty + i) * np + 2 * tx + 32 * h);
+            // outside: the identity, which only the last diagonal block's sweep uses
+            const int r = 4 * ty + i, c = 2 * tx + 32 * h;
+            float4 v = make_float4(r == c ? 1.f : 0.f, 0.f, r == c + 1 ? 1.f : 0.f, 0.f);
+            if (inside(i, h)) v = *reinterpret_cast<const float4 *>(D + (int64_t)r * ld + c);
             m[i][2 * h] = make_float2(v.x, v.y);
             m[i][2 * h + 1] = make_float2(v.z, v.w);
         }
@@ -343,41 +361,39 @@ __global__ void __launch_bounds__(256, 3) k_sweep_update(int np, int nb, int K, 
     tile_product<CB / 2>(sA + CB / 2, sB + CB / 2, ty, tx, m);
     if (next && blockIdx.y == 0) {
         __syncthreads();   // the panels' shared memory holds the pivot rows from here
-        sweep_store(m, sA, np, (K + 1) * CB, Mj, P + (int64_t)j * CB * CB, ty, tx);
+        sweep_store(m, sA, n, ld, (K + 1) * CB, Mj, ty, tx);
         return;
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-            *reinterpret_cast<float4 *>(D + (int64_t)(4 * ty + i) * np + 2 * tx + 32 * h) =
-                make_float4(m[i][2 * h].x, m[i][2 * h].y, m[i][2 * h + 1].x, m[i][2 * h + 1].y);
+            if (inside(i, h))
+                *reinterpret_cast<float4 *>(D + (int64_t)(4 * ty + i) * ld + 2 * tx + 32 * h) =
+                    make_float4(m[i][2 * h].x, m[i][2 * h].y, m[i][2 * h + 1].x, m[i][2 * h + 1].y);
 }
 
-// Minv = -M from M's upper triangle (n x n, symmetric), 32 x 32 tiles
-__global__ void __launch_bounds__(256) k_sweep_finish(int n, int np, const float2 *M,
-                                                      float2 *__restrict__ Minv) {
+// M = -M, the lower triangle from the upper one, in place, 32 x 32 tiles
+__global__ void __launch_bounds__(256) k_sweep_finish(int n, int ld, float2 *M) {
     chain_wait();
     __shared__ float2 s[32][33];
     if (blockIdx.x < blockIdx.y) return;
-    const float2 *Mj = M + (int64_t)blockIdx.z * np * np;
-    float2 *O = Minv + (int64_t)blockIdx.z * n * n;
+    float2 *Mj = M + (int64_t)blockIdx.z * n * ld;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
 #pragma unroll
     for (int i = ty; i < 32; i += 8) {
         const int r = r0 + i, c = c0 + tx;
         // inside a diagonal block both halves are swept; its upper one counts
-        const float2 v = r <= c ? Mj[(int64_t)r * np + c] : Mj[(int64_t)c * np + r];
+        const float2 v = r >= n || c >= n ? make_float2(0.f, 0.f)
+                                          : (r <= c ? Mj[(int64_t)r * ld + c] : Mj[(int64_t)c * ld + r]);
         s[i][tx] = make_float2(-v.x, -v.y);
-        if (r < n && c < n) O[(int64_t)r * n + c] = s[i][tx];
     }
-    if (blockIdx.x == blockIdx.y) return;
     __syncthreads();
 #pragma unroll
     for (int i = ty; i < 32; i += 8) {
-        const int r = c0 + i, c = r0 + tx;
-        if (r < n && c < n) O[(int64_t)r * n + c] = s[tx][i];
+        if (r0 + i < n && c0 + tx < n) Mj[(int64_t)(r0 + i) * ld + c0 + tx] = s[i][tx];
+        if (r0 != c0 && c0 + i < n && r0 + tx < n) Mj[(int64_t)(c0 + i) * ld + r0 + tx] = s[tx][i];
     }
 }
 
@@ -411,37 +427,35 @@ void raise_sweep_smem() {
 }  // namespace
 
 size_t coarse_inverse_work_bytes(int n, int N) {
-    const size_t np = (size_t)(n + CB - 1) / CB * CB;
-    return (size_t)N * (np * np + 2 * np * CB + CB * CB) * sizeof(float2);
+    const size_t nb = (n + CB - 1) / CB;
+    return 2 * (size_t)N * (nb - 1) * CB * CB * sizeof(float2);
 }
 
 void coarse_inverse(Ctx &ctx, int n, const PoleSet<float> &ps, const int32_t *ptr, const int32_t *col,
-                    const float2 *ab, float2 *Minv, void *work) {
-    const int N = ps.N, nb = (n + CB - 1) / CB, np = nb * CB;
-    float2 *M = reinterpret_cast<float2 *>(work);             // N x (np x np), block upper triangle
-    float2 *Cp = M + (size_t)N * np * np;                     // N x (CB x np)
-    float2 *Tp = Cp + (size_t)N * np * CB;                    // N x (CB x np)
-    float2 *P = Tp + (size_t)N * np * CB;                     // N x (CB x CB)
+                    const float2 *ab, float2 *M, void *work) {
+    const int N = ps.N, nb = (n + CB - 1) / CB, ld = coarse_inverse_ld(n), lq = (nb - 1) * CB;
+    float2 *Cp = reinterpret_cast<float2 *>(work);            // N x (CB x lq)
+    float2 *Tp = Cp + (size_t)N * lq * CB;                    // N x (CB x lq)
     raise_sweep_smem();
     const size_t update_smem = sweep_update_smem(ctx.sm_count, (int64_t)N * (nb - 1) * nb / 2);
-    ctx.before(KC_MG_COARSE, 8.0 * N * np * np, 0);
-    k_dense_shift<<<dim3(np, N), 128, 0, ctx.stream>>>(n, np, ptr, col, ab, ps, M);
+    ctx.before(KC_MG_COARSE, 8.0 * N * n * n, 0);
+    k_dense_shift<<<dim3(n, N), 128, 0, ctx.stream>>>(n, ld, ptr, col, ab, ps, M);
     ctx.after();
     ctx.before(KC_MG_COARSE, 16.0 * N * CB * CB, 8.0 * N * CB * CB * CB);
-    launch_chained(ctx, k_first_block, N, 256, 0, np, M, P);
+    launch_chained(ctx, k_first_block, N, 256, 0, n, ld, M);
     ctx.after();
     if (nb > 1)
         for (int K = 0; K < nb; ++K) {
-            ctx.before(KC_MG_COARSE, 24.0 * N * CB * np, 8.0 * N * CB * CB * (double)np);
-            launch_chained(ctx, k_sweep_panel, dim3(N, 2 * (nb - 1)), 256, PANEL_SMEM, np, K, M, P, Cp, Tp);
+            ctx.before(KC_MG_COARSE, 24.0 * N * CB * n, 8.0 * N * CB * CB * (double)n);
+            launch_chained(ctx, k_sweep_panel, dim3(N, 2 * (nb - 1)), 256, PANEL_SMEM, n, ld, lq, K, M, Cp, Tp);
             ctx.after();
-            ctx.before(KC_MG_COARSE, 8.0 * N * np * (double)np, 4.0 * N * CB * (double)np * np);
-            launch_chained(ctx, k_sweep_update, dim3(N, (nb - 1) * nb / 2), 256, update_smem, np, nb, K, M, P, Cp, Tp);
+            ctx.before(KC_MG_COARSE, 8.0 * N * n * (double)n, 4.0 * N * CB * (double)n * n);
+            launch_chained(ctx, k_sweep_update, dim3(N, (nb - 1) * nb / 2), 256, update_smem, n, ld, lq, nb, K, M, Cp, Tp);
             ctx.after();
         }
     ctx.before(KC_MG_COARSE, 12.0 * N * n * (double)n, 0);
     const unsigned g = (unsigned)((n + 31) / 32);
-    launch_chained(ctx, k_sweep_finish, dim3(g, g, N), 256, 0, n, np, M, Minv);
+    launch_chained(ctx, k_sweep_finish, dim3(g, g, N), 256, 0, n, ld, M);
     ctx.after();
 }
 
@@ -455,8 +469,8 @@ int coarse_inverse_apply(Ctx &ctx, void *cublas, const KrylovDims &d, int n, con
     // column-major: Z_j^T (Lp x n, ld W) = R_j^T (Lp x n, ld W) * Minv_j (symmetric)
     ctx.before(KC_MG_COARSE, (double)d.N * n * n * 8 + 2.0 * n * W * 8 * d.frac,
                8.0 * d.N * (double)n * n * d.Lp * d.frac);
-    st = cublasCgemmStridedBatched(hb, CUBLAS_OP_N, CUBLAS_OP_N, d.Lp, n, n, &one, R, W, d.Lp, Minv, n,
-                                   (int64_t)n * n, &zero, Z, W, d.Lp, d.N);
+    st = cublasCgemmStridedBatched(hb, CUBLAS_OP_N, CUBLAS_OP_N, d.Lp, n, n, &one, R, W, d.Lp, Minv,
+                                   coarse_inverse_ld(n), (int64_t)n * coarse_inverse_ld(n), &zero, Z, W, d.Lp, d.N);
     ctx.after();
     return (int)st;
 }

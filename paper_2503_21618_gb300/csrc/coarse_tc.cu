@@ -71,7 +71,8 @@ __global__ void __launch_bounds__(256) k_inv_split_panel(int n, int64_t nks, int
     const int o = blockIdx.x * 32 + (threadIdx.x & 31);
     const int64_t i8 = blockIdx.y * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
     if (o >= ntr * 64 || i8 >= nks * 4) return;
-    const float2 *M = Minv + (int64_t)j * n * n;
+    const int ld = coarse_inverse_ld(n);
+    const float2 *M = Minv + (int64_t)j * n * ld;
     const int oi = o < n ? o : o - n;
     __nv_bfloat16 h[8][CT_PARTS];
 #pragma unroll
@@ -80,7 +81,7 @@ __global__ void __launch_bounds__(256) k_inv_split_panel(int n, int64_t nks, int
         float x = 0.f;
         if (o < 2 * n && k < 2 * n) {
             const int ki = (int)(k < n ? k : k - n);
-            const float2 v = M[(int64_t)ki * n + oi];   // symmetric: (ki, oi) = (oi, ki)
+            const float2 v = M[(int64_t)ki * ld + oi];   // symmetric: (ki, oi) = (oi, ki)
             x = (o < n) == (k < n) ? v.x : (o < n ? -v.y : v.y);
         }
         split3(x, h[t]);

@@ -285,8 +285,10 @@ void mg_dinv(Ctx &ctx, MgSolve<T> &mg, const PoleSet<T> &ps);
 
 // ---------------------------------------------------------------- coarse.cu
 // Dense shifted inverses of one level: Minv_j = (A - sigma_j B)^{-1}, j < N,
-// n x n each (symmetric), from the level's CSR pairs, by a blocked symmetric
-// sweep; work: coarse_inverse_work_bytes.
+// n rows of coarse_inverse_ld(n) entries each (symmetric; even, so that rows
+// start on 16 bytes; the entry beyond n is zero), from the level's CSR pairs,
+// by a blocked symmetric sweep in place; work: coarse_inverse_work_bytes.
+__host__ __device__ inline int coarse_inverse_ld(int n) { return n + (n & 1); }
 size_t coarse_inverse_work_bytes(int n, int N);
 void coarse_inverse(Ctx &ctx, int n, const PoleSet<float> &ps, const int32_t *ptr, const int32_t *col,
                     const float2 *ab, float2 *Minv, void *work);

@@ -32,3 +32,22 @@ def test_syev(api, m, mode, budget):
     h = api.Handle(pencil_1d(600), api.default_opts(mem_budget=budget, eig_refine=mode))
     lam = h.syev(torch.from_numpy(S).cuda())[0].cpu().numpy()
     assert np.abs(lam - np.linalg.eigvalsh(S)).max() <= 1e-13 * np.linalg.norm(S, 2) * max(1, m / 10)
+
+
+# the level solved by its inverses: 200, 333, 833 and 1 533 unknowns
+@pytest.mark.parametrize("n,N,tc,budget", [(600, 1, 0, 1094244), (600, 1, 1, 2551396), (600, 4, 0, 2980116), (600, 4, 1, 8807956),
+                                              (1000, 1, 0, 2154580), (1000, 1, 1, 5541524), (1000, 4, 0, 6312644), (1000, 4, 1, 19859652),
+                                              (2500, 1, 0, 8660872), (2500, 1, 1, 27627848), (2500, 4, 0, 28904920), (2500, 4, 1, 104772056),
+                                              (4600, 1, 0, 24483780), (4600, 1, 1, 82434052), (4600, 4, 0, 87408372), (4600, 4, 1, 319208692)])
+def test_exact_level(api, n, N, tc, budget):
+    m, ldp = 5, 6
+    sig = 0.02 * n * n * (np.linspace(0.1, 1, N) + 1j * np.linspace(0.2, 1, N))
+    R = torch.randn(n, N * ldp * 2, generator=torch.Generator("cuda").manual_seed(n), device="cuda")
+    z = []
+    for b in (budget, 0):
+        h = api.Handle(pencil_1d(n), api.default_opts(precond=api.PRECOND_MG, mg_coarse=16, mg_shift_limit=1e30,
+                                                      mg_exact_tc=tc, mem_budget=b))
+        Z, used = h.precond_apply(api.Filter(sig, np.ones(N)), R, m, ldp)
+        assert used == 2
+        z.append(Z.cpu().numpy())
+    assert np.array_equal(z[0], z[1])
