@@ -106,6 +106,19 @@ __device__ __forceinline__ float fast_rcp(float x) {
     asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return fmaf(y, fmaf(-x, y, 1.f), y);
 }
+// 1 / p of a pivot.  Where the square of its size is near the ends of FP32's range
+// (pencils scaled to 1e-15 and below or 1e15 and above) p is brought to the
+// middle by a power of two first; the same branch for the whole block.
+__device__ __forceinline__ float2 pivot_rcp(float2 p) {
+    const float d = p.x * p.x + p.y * p.y;
+    if (d >= 1e-30f && d <= 1e30f) {
+        const float di = fast_rcp(d);
+        return make_float2(p.x * di, -p.y * di);
+    }
+    const int e = ilogbf(fmaxf(fabsf(p.x), fabsf(p.y)));
+    const float x = scalbnf(p.x, -e), y = scalbnf(p.y, -e), di = fast_rcp(x * x + y * y);
+    return make_float2(scalbnf(x * di, -e), scalbnf(-y * di, -e));
+}
 
 // Pivot k (column k: registers S[.][qk] of lane tx = kx; row k: S[ki][.] of ty =
 // k4) with w = row k / pivot, r = column k, applied to the register rows i
@@ -162,8 +175,7 @@ __device__ __forceinline__ void sweep_step(float2 (&S)[4][4], float2 (*row)[CB],
         if (k8 > 0) pivot_rows<3, 2 * HALF + 1>(S, v.w, v.r, v.pinv, prow, pcol, REST);
         else if (HALF == 1) pivot_rows<3, 1>(S, v.w, v.r, v.pinv, prow, pcol, REST);
     }
-    const float di = fast_rcp(p.x * p.x + p.y * p.y);
-    v.pinv = make_float2(p.x * di, -p.y * di);
+    v.pinv = pivot_rcp(p);
     v.w[0] = cmul(v.pinv, make_float2(c01.x, c01.y));
     v.w[1] = cmul(v.pinv, make_float2(c01.z, c01.w));
     v.w[2] = cmul(v.pinv, make_float2(c23.x, c23.y));
