@@ -35,6 +35,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "sweep_rule.h"
 
 namespace slrf {
 
@@ -411,18 +412,6 @@ __global__ void __launch_bounds__(256) k_sweep_finish(int n, int ld, float2 *M) 
 
 constexpr size_t SWEEP_SMEM = 2 * CB * CB * sizeof(float2);   // three CTAs of the update per SM
 constexpr size_t SWEEP_SMEM_TWO = 100 * 1024;                 // two
-// Three or two CTAs of the update per SM.  The launch ends with the CTAs that
-// sweep the next diagonal blocks, which are faster beside one other CTA than
-// beside two; three per SM pay where they fill the last of several waves (over
-// three quarters of it), and where there are no more than two per SM anyway the
-// larger request only delays their start.  Cycle call, three against two per SM,
-// by the number of tiles on 152 SMs: 112: 370 / 395 us, 264: 711 / 721, 420: 870 /
-// 803, 480: 1073 / 906, 684: 1147 / 1029, 840: 1303 / 1377, 1104: 1764 / 1724.
-size_t sweep_update_smem(int sm_count, int64_t tiles) {
-    const int64_t wave = 3 * (int64_t)sm_count;
-    const bool three = tiles <= 2 * (int64_t)sm_count || (tiles > wave && 4 * (tiles % wave) > 3 * wave);
-    return three ? SWEEP_SMEM : SWEEP_SMEM_TWO;
-}
 constexpr size_t PANEL_SMEM = (CB * CB + CB * PLD) * sizeof(float2);
 
 // The kernels' shared-memory limit, raised once per device
@@ -449,7 +438,8 @@ void coarse_inverse(Ctx &ctx, int n, const PoleSet<float> &ps, const int32_t *pt
     float2 *Cp = reinterpret_cast<float2 *>(work);            // N x (CB x lq)
     float2 *Tp = Cp + (size_t)N * lq * CB;                    // N x (CB x lq)
     raise_sweep_smem();
-    const size_t update_smem = sweep_update_smem(ctx.sm_count, (int64_t)N * (nb - 1) * nb / 2);
+    const size_t update_smem =
+        sweep_three_per_sm(ctx.sm_count, (int64_t)N * (nb - 1) * nb / 2) ? SWEEP_SMEM : SWEEP_SMEM_TWO;
     ctx.before(KC_MG_COARSE, 8.0 * N * n * n, 0);
     k_dense_shift<<<dim3(n, N), 128, 0, ctx.stream>>>(n, ld, ptr, col, ab, ps, M);
     ctx.after();
