@@ -132,7 +132,8 @@ typedef struct {
     int32_t profile;        /* 1: time kernel classes with CUDA events around
                                each launch (those selected by profile_mask)      (0) */
     int32_t spmm_rows;      /* rows per group of the shifted SpMM (1..4); 0 = auto:
-                               3 for 3-dof node-block patterns, else 2             (0) */
+                               3 for 3-dof node-block patterns, else 2 (FP64: 1
+                               where groups of two would be padded)                (0) */
     int32_t gram_ozaki;     /* Grams and tall products (Q1 = U T1, X = Q1 M) of the
                                projection step, FP64-accurate from exact integer
                                digit products (Ozaki splitting): 2 = Grams on the

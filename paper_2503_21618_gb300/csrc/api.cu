@@ -2340,6 +2340,7 @@ slrf_status slrf_create(slrf_handle **out, const slrf_pencil *p, const slrf_opts
             return SLRF_ENOMEM;
         }
         h->A.rg_rows = R;
+        h->A.rg_asked = o->spmm_rows != 0;
         h->A.rg_ngroups = (int)ng;
         h->A.rg_nnz = U;
         h->A.rg_emax = tail[1];

@@ -57,6 +57,7 @@ struct DevPencil {
     // row-group form of the shifted SpMM (rg_rows consecutive rows per group,
     // union column list per group, rg_rows (a, b) pairs per union entry)
     int rg_rows = 1, rg_ngroups = 0;
+    bool rg_asked = false;   // the caller chose rg_rows (slrf_opts.spmm_rows)
     int64_t rg_nnz = 0;
     int32_t *rg_ptr = nullptr, *rg_col = nullptr;
     float2 *rg_ab32 = nullptr;

@@ -1243,8 +1243,9 @@ void krylov_spmm(Ctx &ctx, const KrylovDims &d, const DevPencil &A, const cplx<T
     // FP64 is bound by its FMA pipe, not by the gathers: there the padding
     // pairs of the row groups (12 pairs per row for 9 on the 2D pencils) cost
     // more than the shared gathers save (494 us against 397 at n = 22 201, 240
-    // columns); groups of three have none
-    if (A.rg_rows > 1 && (sizeof(T) == 4 || A.rg_nnz * A.rg_rows == A.nnz)) {
+    // columns); groups of three have none.  A group size that the caller asked
+    // for is taken as it is.
+    if (A.rg_rows > 1 && (sizeof(T) == 4 || A.rg_asked || A.rg_nnz * A.rg_rows == A.nnz)) {
         const int gpb = (A.rg_ngroups + gy - 1) / gy;
         const auto *uab = reinterpret_cast<const typename ABT<T>::type *>(sizeof(T) == 4 ? (const void *)A.rg_ab32
                                                                                           : (const void *)A.rg_ab64);
