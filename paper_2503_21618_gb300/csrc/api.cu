@@ -672,7 +672,7 @@ struct MgStaged {
 
 // Lays out and fills the image of every level but the coarsest level's
 // eigenvectors (mg_stage_v, once they exist).  R0: rows per group of the
-// finest level's row-group form (1 = plain rows).  The folded pairs f_ab
+// finest level's row-group form (1 = plain rows).  The folded pairs
 // come last and are not uploaded: every solve writes them from f_q.
 void mg_stage(const HostHierarchy &H, int R0, MgStaged &S) {
     const int nlev = (int)H.lv.size();
@@ -722,7 +722,7 @@ void mg_stage(const HostHierarchy &H, int R0, MgStaged &S) {
     S.o_fq = take(nq * sizeof(double));
     S.upload_bytes = off;
     S.o_fab32 = take(nslot * sizeof(float2));
-    S.o_fab64 = take(nslot * sizeof(double2));
+    S.o_fab64 = take(FL.down_col.size() * sizeof(double2));   // the FP64 cycle has no up product
     S.total_bytes = off;
     S.fu_nnz = (int64_t)FL.up_col.size();
     S.fd_nnz = (int64_t)FL.down_col.size();
@@ -847,7 +847,8 @@ slrf_status mg_upload(slrf_handle *h, const HostHierarchy &H, const MgStaged &S,
             L0.fd_ptr = reinterpret_cast<const int32_t *>(base + S.o_fdp);
             L0.fd_col = reinterpret_cast<const int32_t *>(base + S.o_fdc);
             L0.f_q = reinterpret_cast<const double2 *>(base + S.o_fq);
-            L0.f_ab = reinterpret_cast<cplx<T> *>(base + (sizeof(T) == 4 ? S.o_fab32 : S.o_fab64));
+            if (sizeof(T) == 4) L0.f_up = reinterpret_cast<cplx<T> *>(base + S.o_fab32);
+            L0.f_down = sizeof(T) == 4 ? L0.f_up + S.fu_nnz * L0.R : reinterpret_cast<cplx<T> *>(base + S.o_fab64);
         }
     };
     fill(h->mg32, 0.0f);
@@ -1460,7 +1461,7 @@ slrf_status krylov_solve(slrf_handle *h, const slrf_filter *f, int m, const doub
             krylov_spmm<T>(ctx, d, h->A, sig, kb.P, kb.Q, kb.s.flag, kb.s.part, kb.gy);
             krylov_reduce_alpha<T>(ctx, d, kb);
             krylov_update<T>(ctx, d, kb);
-            if (use_mg) mg_apply<T>(ctx, d, mg_of<T>(h), sig, kb.s.flag, kb.s.part, kb.gy, kb.R, kb.Z, kb.Q, kb.Q);
+            if (use_mg) mg_apply<T>(ctx, d, mg_of<T>(h), sig, kb.s.flag, kb.s.part, kb.gy, kb.R, kb.Z, kb.Q, true);
             if (use_ilu)
                 ilu_apply<T>(ctx, d, h->ilu_pat, ilu, h->opts.ilu_tri_sweeps, kb.gy, kb.s.flag, kb.R, kb.Z, kb.Q,
                              ilu_y, kb.s.part);

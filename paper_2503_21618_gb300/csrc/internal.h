@@ -256,11 +256,12 @@ template <typename T> struct MgLevel {
     // by fine row groups (the R rows of the level's groups, union coarse
     // columns, R pairs per entry: "up") and by coarse rows (F^T: "down").
     // f_q holds the unfolded FP64 pieces (A P, B P) and (a_ii P, b_ii P) per
-    // stored pair, up entries first; f_ab the folded pairs in that order.
+    // stored pair, up entries first; f_up (FP32 only: the FP64 cycle has no up
+    // product) and f_down the folded pairs.
     int64_t fu_nnz = 0, fd_nnz = 0;
     const int32_t *fu_ptr = nullptr, *fu_col = nullptr, *fd_ptr = nullptr, *fd_col = nullptr;
     const double2 *f_q = nullptr;
-    cplx<T> *f_ab = nullptr;
+    cplx<T> *f_up = nullptr, *f_down = nullptr;   // FP32: f_down follows f_up
 };
 template <typename T> struct MgSolve {
     int nlev = 0, nc = 0;
@@ -310,13 +311,12 @@ void coarse_tc_panels(Ctx &ctx, int n, int N, const float2 *Minv, void *Mpan);
 void coarse_tc_apply(Ctx &ctx, const KrylovDims &d, int n, const void *Mpan, const float2 *R, float2 *Z, void *work,
                      int32_t *err);
 // Z0 = cycle(R0) for all active columns of the state; part receives the
-// partial sums r^T z (slots 0, 1).  Y0 = D R0 with the finest level's
-// damped Jacobi diagonal (mg.lv[0].dinv), if the caller has it (the COCG
-// update forms it); otherwise it is formed into T0, an n x W scratch block
-// (also the scratch of a single-level hierarchy).
+// partial sums r^T z (slots 0, 1).  T0 is an n x W scratch block, overwritten.
+// scaled: it already holds D R0 with the finest level's damped Jacobi diagonal
+// (mg.lv[0].dinv), as the COCG update leaves it; otherwise that is formed here.
 template <typename T>
 void mg_apply(Ctx &ctx, const KrylovDims &d, MgSolve<T> &mg, const cplx<T> *sig, const int32_t *flag, T *part,
-              int gy, const cplx<T> *R0, cplx<T> *Z0, cplx<T> *T0, const cplx<T> *Y0 = nullptr);
+              int gy, const cplx<T> *R0, cplx<T> *Z0, cplx<T> *T0, bool scaled = false);
 // part = partial sums r^T z per column (slots 0, 1) of two state blocks
 template <typename T>
 void mg_rz(Ctx &ctx, const KrylovDims &d, int gy, const cplx<T> *R, const cplx<T> *Z, const int32_t *flag, T *part);

@@ -723,11 +723,11 @@ void mg_dinv(Ctx &ctx, MgSolve<T> &mg, const PoleSet<T> &ps) {
     }
     MgLevel<T> &L0 = mg.lv[0];
     if (mg.nlev > 1) {
-        // the FP64 cycle uses the down pairs (the last) only
-        const int64_t s0 = sizeof(T) == 8 ? L0.fu_nnz * L0.R : 0, ns = L0.fu_nnz * L0.R + L0.fd_nnz - s0;
+        // the FP64 cycle has the down pairs (f_q's last) only
+        const int64_t nup = L0.fu_nnz * L0.R, s0 = L0.f_up ? 0 : nup, ns = nup + L0.fd_nnz - s0;
         ctx.before(KC_KRYLOV_INIT, (double)ns * (32 + sizeof(cplx<T>)), 0);
         k_mg_fold<T><<<(unsigned)((ns + 255) / 256), 256, 0, ctx.stream>>>(ns, L0.f_q + 2 * s0, L0.rho / mg.omega,
-                                                                          L0.f_ab + s0);
+                                                                          L0.f_up ? L0.f_up : L0.f_down);
         ctx.after();
     }
 }
@@ -746,7 +746,7 @@ void mg_scale(Ctx &ctx, const KrylovDims &d, const MgSolve<T> &mg, int gy, const
 
 template <typename T>
 void mg_apply(Ctx &ctx, const KrylovDims &d, MgSolve<T> &mg, const cplx<T> *sig, const int32_t *flag, T *part,
-              int gy, const cplx<T> *R0, cplx<T> *Z0, cplx<T> *T0, const cplx<T> *Y0) {
+              int gy, const cplx<T> *R0, cplx<T> *Z0, cplx<T> *T0, bool scaled) {
     if (mg.nlev == 1) {
         coarse_solve<T>(ctx, d, mg, R0, T0, Z0, flag);
         launch_rz<T>(ctx, d, gy, R0, Z0, flag, part);
@@ -754,25 +754,21 @@ void mg_apply(Ctx &ctx, const KrylovDims &d, MgSolve<T> &mg, const cplx<T> *sig,
     }
     const MgLevel<T> &L = mg.lv[0];
     const MgLevel<T> &Lc = mg.lv[1];
-    if (!Y0) {   // y = D r into the scratch block
-        mg_scale<T>(ctx, d, mg, gy, R0, T0, flag);
-        Y0 = T0;
-    }
+    if (!scaled) mg_scale<T>(ctx, d, mg, gy, R0, T0, flag);   // y = D r
     // r1 = -F^T y
     const int gyd = std::max(1, std::min(gy, (Lc.n + TY - 1) / TY));
-    launch_sspmm<T, MG_DOWN>(ctx, d, KC_MG_FINE, Lc.n, 1, Lc.n, L.fd_ptr, L.fd_col, L.f_ab + L.fu_nnz * L.R,
-                             L.fd_nnz, L.n, gyd, sig, L.dinv, Y0, nullptr, Lc.r, flag, nullptr);
+    launch_sspmm<T, MG_DOWN>(ctx, d, KC_MG_FINE, Lc.n, 1, Lc.n, L.fd_ptr, L.fd_col, L.f_down, L.fd_nnz,
+                             L.n, gyd, sig, L.dinv, T0, nullptr, Lc.r, flag, nullptr);
     cplx<T> *e = cycle<T>(ctx, d, mg, 1, gy, sig, flag);
     if constexpr (sizeof(T) == 8) {
-        // y is scratch (the caller's T0, or the Krylov update's own block)
-        cplx<T> *z1 = const_cast<cplx<T> *>(Y0);
-        launch_xfer<T, MG_PROLONG_ADD>(ctx, d, L.n, Lc.n, L.p_nnz, L.pptr, L.pcol, L.pval, gy, e, z1, flag);
+        // z1 = y + P e in place
+        launch_xfer<T, MG_PROLONG_ADD>(ctx, d, L.n, Lc.n, L.p_nnz, L.pptr, L.pcol, L.pval, gy, e, T0, flag);
         launch_sspmm<T, MG_SMOOTH>(ctx, d, KC_MG_FINE, L.n, 1, L.n, L.row_ptr, L.row_col, L.row_ab, L.row_nnz, L.n, gy,
-                                   sig, L.dinv, z1, R0, Z0, flag, part);
+                                   sig, L.dinv, T0, R0, Z0, flag, part);
     } else {
         // z = D (2 r - M y - F e), r^T z
         launch_sspmm<T, MG_UP>(ctx, d, KC_MG_FINE, L.n, L.R, L.ngroups, L.gptr, L.gcol, L.ab, L.nnz_union, L.n, gy, sig,
-                               L.dinv, Y0, R0, Z0, flag, part, L.fu_ptr, L.fu_col, L.f_ab, L.fu_nnz, e, Lc.n);
+                               L.dinv, T0, R0, Z0, flag, part, L.fu_ptr, L.fu_col, L.f_up, L.fu_nnz, e, Lc.n);
     }
 }
 
@@ -784,7 +780,7 @@ void mg_rz(Ctx &ctx, const KrylovDims &d, int gy, const cplx<T> *R, const cplx<T
 #define INST(T)                                                                                                  \
     template void mg_dinv<T>(Ctx &, MgSolve<T> &, const PoleSet<T> &);                                           \
     template void mg_apply<T>(Ctx &, const KrylovDims &, MgSolve<T> &, const cplx<T> *, const int32_t *, T *,  \
-                              int, const cplx<T> *, cplx<T> *, cplx<T> *, const cplx<T> *);                     \
+                              int, const cplx<T> *, cplx<T> *, cplx<T> *, bool);                                \
     template void mg_rz<T>(Ctx &, const KrylovDims &, int, const cplx<T> *, const cplx<T> *, const int32_t *, T *);
 INST(float)
 INST(double)
