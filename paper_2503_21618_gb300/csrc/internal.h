@@ -133,8 +133,11 @@ int krylov_row_groups(const Ctx &ctx, const KrylovDims &d, int prec_fp32);
 // Launch of a kernel that begins with chain_wait(): overlaps its launch and the
 // scheduling of its blocks with the end of the kernel before it on the stream.
 // The Krylov iteration and the cycle are chains of 15 to 20 short launches, each
-// waiting for the last: plain FP64 solve of the 1D pencil (n = 2000) 19.7 -> 17.5
-// ms, of the 2D pencil (n = 10 000) 102.7 -> 97.8.
+// waiting for the last.  Only grids of at most one CTA per SM overlap: waiting
+// CTAs hold their threads, registers and shared memory, and a large grid that
+// waits behind a short reduction keeps another stream's kernels off the SMs.  64
+// pencils on 64 streams: 2.48 s, with every grid overlapped 2.67, with none 2.47;
+// four requests at once 4.23 s, 4.53 and 4.20.
 template <typename... KA, typename... A>
 inline void launch_chained(Ctx &ctx, void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem,
                            A &&...args) {
@@ -147,7 +150,7 @@ inline void launch_chained(Ctx &ctx, void (*kernel)(KA...), dim3 grid, dim3 bloc
     cfg.dynamicSmemBytes = smem;
     cfg.stream = ctx.stream;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = (int64_t)grid.x * grid.y * grid.z <= ctx.sm_count ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);   // an error stays as the stream's last error
 }
 
