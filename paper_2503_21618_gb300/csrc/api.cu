@@ -260,9 +260,20 @@ cudaError_t dev_alloc(slrf_handle *h, void **ptr, size_t bytes) {
 slrf_status ensure(slrf_handle *h, Buf &b, size_t bytes) {
     if (bytes == 0) bytes = 16;
     if (b.bytes >= bytes) return SLRF_OK;
-    if (h->opts.mem_budget > 0 &&
-        h->pencil_bytes + h->ws_bytes - b.bytes + bytes > (size_t)h->opts.mem_budget)
-        return SLRF_EBUDGET;
+    auto over = [&] {
+        return h->opts.mem_budget > 0 &&
+               h->pencil_bytes + h->ws_bytes - b.bytes + bytes > (size_t)h->opts.mem_budget;
+    };
+    // over the budget: the digit products' scratch, which has a smaller form, goes first
+    if (&b != &h->rOz && &b != &h->rOzT)
+        for (Buf *s : {&h->rOz, &h->rOzT})
+            if (s->p && over()) {
+                cudaFreeAsync(s->p, h->ctx.stream);
+                h->ws_bytes -= s->bytes;
+                s->p = nullptr;
+                s->bytes = 0;
+            }
+    if (over()) return SLRF_EBUDGET;
     // stream-ordered allocation: growing one handle's workspace never waits
     // for work of other handles on other streams
     if (b.p) {
@@ -1513,9 +1524,18 @@ slrf_status gram(slrf_handle *h, int64_t n, int m, const double *X, int64_t ldx,
                  double *G, bool symmetric = false, bool same_x = false) {
     Ctx &ctx = h->ctx;
     if (h->opts.gram_ozaki) {
-        CKS(ensure(h, h->rOz, ozaki_gram_work_bytes(n, m, ctx.sm_count)));
-        ozaki_gram(ctx, n, m, X, ldx, Y, ldy, G, h->rOz.p, symmetric,
-                   h->opts.gram_ozaki == 2 ? h->d_pin + 1 : nullptr, same_x);
+        // a memory budget that does not take the tensor-core form's panels and
+        // partials gets the mma.sync form, which needs half the bytes
+        bool tc = h->opts.gram_ozaki == 2;
+        const void *last = h->rOz.p;
+        slrf_status st = ensure(h, h->rOz, ozaki_gram_work_bytes(n, m, ctx.sm_count));
+        if (st == SLRF_EBUDGET) {
+            tc = false;
+            st = ensure(h, h->rOz, ozaki_gram_work_bytes(n, m, ctx.sm_count, false));
+        }
+        CKS(st);
+        ozaki_gram(ctx, n, m, X, ldx, Y, ldy, G, h->rOz.p, symmetric, tc ? h->d_pin + 1 : nullptr,
+                   same_x && h->rOz.p == last);
         return SLRF_OK;
     }
     const int split = gram_split(ctx, m, n);
@@ -1531,9 +1551,14 @@ slrf_status tall_product(slrf_handle *h, int64_t n, int k, int m, const double *
                          double *B, int64_t ldb, double *C, int64_t ldc) {
     Ctx &ctx = h->ctx;
     if (h->opts.gram_ozaki && ozaki_tall_fits(k)) {
-        CKS(ensure(h, h->rOzT, ozaki_tall_work_bytes(n, k, m)));
-        ozaki_tall(ctx, n, k, m, A, lda, cs, B, ldb, C, ldc, h->rOzT.p, KC_TALL_GEMM,
-                   h->opts.gram_ozaki == 2 ? h->d_pin + 1 : nullptr);
+        bool tc = h->opts.gram_ozaki == 2;   // as in gram()
+        slrf_status st = ensure(h, h->rOzT, ozaki_tall_work_bytes(n, k, m));
+        if (st == SLRF_EBUDGET) {
+            tc = false;
+            st = ensure(h, h->rOzT, ozaki_tall_work_bytes(n, k, m, false));
+        }
+        CKS(st);
+        ozaki_tall(ctx, n, k, m, A, lda, cs, B, ldb, C, ldc, h->rOzT.p, KC_TALL_GEMM, tc ? h->d_pin + 1 : nullptr);
         return SLRF_OK;
     }
     if (cs) small_scale_rows(ctx, k, cs, B);

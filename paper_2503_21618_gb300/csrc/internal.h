@@ -393,7 +393,8 @@ void copy_block(Ctx &ctx, int n, int m, const double *src, int64_t lds, double *
 
 // ---------------------------------------------------------------- ozaki.cu
 // G = X^T Y (m x m, row-major, ld m) from int8 tensor-core digit products.
-size_t ozaki_gram_work_bytes(int64_t n, int m, int sm_count);
+// (tensor_core: of either form, else of the mma.sync form alone)
+size_t ozaki_gram_work_bytes(int64_t n, int m, int sm_count, bool tensor_core = true);
 // symmetric: X^T Y is known to be symmetric (Y = B X with B symmetric): only
 // the tiles on and above the diagonal are computed and mirrored.
 // tc_err != nullptr selects the tensor-core (tcgen05, bf16 digits) form; it
@@ -407,7 +408,7 @@ void ozaki_gram(Ctx &ctx, int64_t n, int m, const double *X, int64_t ldx, const 
 // products.  tc_err != nullptr (and k <= 512) selects the tcgen05 form (bf16
 // digits, FP32 tensor-memory sums); it receives a nonzero code if one of that
 // kernel's bounded waits gives up.  Otherwise int8 mma.sync.
-size_t ozaki_tall_work_bytes(int64_t n, int k, int m);
+size_t ozaki_tall_work_bytes(int64_t n, int k, int m, bool tensor_core = true);
 bool ozaki_tall_fits(int k);
 void ozaki_tall(Ctx &ctx, int64_t n, int k, int m, const double *A, int64_t lda, const double *cs, const double *B,
                 int64_t ldb, double *C, int64_t ldc, void *work, int kc, int32_t *tc_err = nullptr);

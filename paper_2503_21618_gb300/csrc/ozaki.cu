@@ -729,12 +729,13 @@ static void ozaki_gram_tc(Ctx &ctx, int64_t n, int m, const double *X, int64_t l
 }
 
 // ---------------------------------------------------------------------------
-size_t ozaki_gram_work_bytes(int64_t n, int m, int sm_count) {
+size_t ozaki_gram_work_bytes(int64_t n, int m, int sm_count, bool tensor_core) {
     const int64_t npad = (n + 63) / 64 * 64;
     const int mpad = (m + OZ_TM - 1) / OZ_TM * OZ_TM;
     const size_t slices = 2 * (size_t)OZ_S * mpad * npad;
     const size_t split = (size_t)sm_count * 4;
     const size_t mma_sync = slices + split * m * m * sizeof(double) + 2 * (size_t)m * (sizeof(int) + 8) + 1024;
+    if (!tensor_core) return mma_sync;
     // tensor-core form: bf16 digit panels of both operands and one m x m partial per K-slice
     const int64_t nks = (n + TC_KSTEP - 1) / TC_KSTEP;
     const int np = (m + TC_TN - 1) / TC_TN;
@@ -1006,11 +1007,12 @@ static void ozaki_tall_tc(Ctx &ctx, int64_t n, int k, int m, const double *A, in
     ctx.after();
 }
 
-size_t ozaki_tall_work_bytes(int64_t n, int k, int m) {
+size_t ozaki_tall_work_bytes(int64_t n, int k, int m, bool tensor_core) {
     const int64_t npad = (n + OZ_TA - 1) / OZ_TA * OZ_TA;
     const int kpad = (k + 31) / 32 * 32, mpad = (m + OZ_TB - 1) / OZ_TB * OZ_TB;
     const size_t mma_sync = (size_t)OZ_S * npad * kpad + (size_t)OZ_S * mpad * kpad + 256 +
                             (size_t)npad * sizeof(int) + (size_t)m * (sizeof(int) + 8) + 1024;
+    if (!tensor_core) return mma_sync;
     // tensor-core form: bf16 digit panels of A (rows) and B (columns), maxima, scalings, exponents
     const int64_t nks = (k + TC_KSTEP - 1) / TC_KSTEP;
     const int64_t npa = (n + 63) / 64, npb = (m + TC_TN - 1) / TC_TN;

@@ -5,7 +5,7 @@ rearranged."""
 import numpy as np
 import pytest
 
-from workloads import pencil_1d
+from workloads import pencil_1d, pencil_2d_q1, start_block, weyl_gamma
 
 pytestmark = pytest.mark.gpu
 
@@ -51,3 +51,41 @@ def test_exact_level(api, n, N, tc, budget):
         assert used == 2
         z.append(Z.cpu().numpy())
     assert np.array_equal(z[0], z[1])
+
+
+@pytest.mark.parametrize("n,m,budget", [(50021, 127, 208177866), (50021, 211, 412084890)])
+def test_gram(api, n, m, budget):
+    g = torch.Generator("cuda").manual_seed(m)
+    X, Y = (torch.randn(n, m, generator=g, dtype=torch.float64, device="cuda") for _ in range(2))
+    G = api.Handle(pencil_1d(n), api.default_opts(mem_budget=budget)).gram(X, Y)
+    assert (G - X.T @ Y).abs().max() <= 1e-13 * X.abs().max() * Y.abs().max() * n
+
+
+@pytest.mark.parametrize("n,m,budget", [(6400, 298, 32913188)])
+def test_tall_product(api, n, m, budget):
+    g = torch.Generator("cuda").manual_seed(m)
+    A = torch.randn(n, m, generator=g, dtype=torch.float64, device="cuda")
+    B = torch.randn(m, m, generator=g, dtype=torch.float64, device="cuda")
+    C = api.Handle(pencil_1d(n), api.default_opts(mem_budget=budget)).tall_product(A, B)
+    assert (C - A @ B).abs().max() <= 1e-13 * A.abs().max() * B.abs().max() * m
+
+
+# Gram, tall products and their smaller forms within one call
+@pytest.mark.parametrize("n,m,budget", [(50021, 127, 525128286)])
+def test_rayleigh_ritz(api, n, m, budget):
+    p = pencil_1d(n)
+    U = torch.randn(n, m, generator=torch.Generator("cuda").manual_seed(m), dtype=torch.float64, device="cuda")
+    theta, X, resid = api.Handle(p, api.default_opts(mem_budget=budget)).rayleigh_ritz(U)[:3]
+    theta0, X0, resid0 = api.Handle(p).rayleigh_ritz(U)[:3]
+    assert (theta - theta0).abs().max() <= 1e-12 * theta0.abs().max()
+    assert (resid - resid0).abs().max() <= 1e-10
+
+
+# the whole default solve: the Krylov blocks come after the projection's
+@pytest.mark.parametrize("size,nev,cols,budget", [(150, 80, 120, 745270286)])
+def test_solve(api, size, nev, cols, budget):
+    p, gamma = pencil_2d_q1(size), weyl_gamma("2d", nev)
+    V0 = torch.from_numpy(start_block(p.n, cols, 3)).cuda()
+    h = api.Handle(p, api.default_opts(mem_budget=budget))
+    status = h.subspace_iterate(api.design_poles("slrf", 4, gamma, 1.0, 0.01), gamma, V0, tol=1e-8, max_outer=1)[4]
+    assert status in (api.OK, api.NOT_CONVERGED, api.SUBSPACE_TOO_SMALL)
