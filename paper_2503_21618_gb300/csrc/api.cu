@@ -486,15 +486,6 @@ __global__ void k_rg_fill(int64_t n, int R, int64_t ng, const int32_t *rowptr, c
         }
     }
 }
-__global__ void k_symmetrize(int m, double *S) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= (int64_t)m * m) return;
-    const int i = (int)(e / m), j = (int)(e % m);
-    if (j <= i) return;
-    const double v = 0.5 * (S[(int64_t)i * m + j] + S[(int64_t)j * m + i]);
-    S[(int64_t)i * m + j] = v;
-    S[(int64_t)j * m + i] = v;
-}
 // out = (S + S^T) / 2
 __global__ void k_symmetrized(int m, const double *__restrict__ S, double *__restrict__ out) {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -1641,9 +1632,6 @@ slrf_status rr_step(slrf_handle *h, int m, const double *U, int64_t ldu, double 
     CKS(gram(h, n, m, Q1, m, W1, m, Ah1, true, true));   // Q1's digits are those of the last Gram
     dgemm(ctx, 0, 0, m, m, m, Ah1, m, T2, m, 0.0, R1, m, 1, nullptr, KC_SMALL_DENSE);
     dgemm(ctx, 1, 0, m, m, m, T2, m, R1, m, 0.0, Ah, m, 1, nullptr, KC_SMALL_DENSE, true);
-    ctx.before(KC_SMALL_DENSE, 16.0 * m2, 0);
-    k_symmetrize<<<(unsigned)((m2 + 255) / 256), 256, 0, ctx.stream>>>(m, Ah);
-    ctx.after();
     CK(small_syev(ctx, m, Ah, theta, Sm, syw, h->opts.eig_refine));
     // X = Q1 (T2 S); AX, BX by SpMM
     dgemm(ctx, 0, 0, m, m, m, T2, m, Sm, m, 0.0, Mm, m, 1, nullptr, KC_SMALL_DENSE);

@@ -130,7 +130,7 @@ void raise_smem_limits();   // defined after the kernels it configures
 // Blocked Cholesky factor and inverse: G = R^T R, X = R^{-1}, from the
 // elimination of [G | I], whose right part ends as R^{-T}.  Right-looking in
 // CHB x CHB blocks: the diagonal block on one CTA, the panel solves and the
-// trailing updates of both parts spread over the GPU (FP64 issues at ~1.6
+// trailing updates of both parts spread over the GPU (FP64 issues at ~1.7
 // FMAs per clock and SM here, so m^3/6 of them belong on many SMs; what is
 // left is the chain of m pivots).  The right part costs no further steps: a
 // separate triangular inverse by back substitution, one warp per column, was
@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *S, doubl
 // entries are close an FP32 rounding turns a rotation by 45 degrees the other
 // way.  In double-float the path is the FP64 one (a decision differs only
 // where the FP64 one is within ~1e-13), at ten FP32 instructions per
-// operation on a pipe eighty times as fast.
+// operation on a pipe seventy times as fast.
 //
 // All m/2 rotations of a round (rr_pair) are applied at once, A in the shared
 // memory of the C CTAs.  Position k of a round holds the pair (a_k, b_k).  A CTA
@@ -568,8 +568,8 @@ __global__ void __launch_bounds__(1024) k_jacobi32(int m, const double *S, doubl
 // sweeps stop once every rotation of a sweep was below sqrt(rel_tol).
 // Output: lam (FP64, unsorted), the log and *nrounds.
 // ---------------------------------------------------------------------------
-constexpr int JDF_MAX = 448;      // a CTA's rows of an 8-CTA cluster in 227 KB
-constexpr int JDF_CTAS = 8, JDF_CTAS_WIDE = 16;
+constexpr int JDF_MAX = 448;      // 7 positions per lane of k_jacobi_vectors
+constexpr int JDF_CTAS = 16;      // with 8 a solve with 270 columns (n = 26 244) took 185 ms for 169
 constexpr int JDF_SWEEPS = 20;    // at most; see log_sweeps
 constexpr int JDF_THREADS = 544;  // 16 warps for the update, one for the rotations
 static_assert(JDF_MAX <= 2 * 32 * JDF_CTAS, "one lane of warp 0 per position of a CTA");
@@ -674,7 +674,7 @@ k_jacobi_df(int m, const double *__restrict__ S, const double *__restrict__ fro_
     __shared__ int nbfree[2][2];    // free slot of the lower / upper neighbour, by round parity
     __shared__ int myfree[2][2];    // own free slots for an upper / a lower row, by round parity
     __shared__ int mx[2];           // largest relative pivot of a sweep (float bits), by sweep parity
-    __shared__ int allmx[JDF_CTAS_WIDE]; // the CTAs' mx of the sweep that ends
+    __shared__ int allmx[JDF_CTAS]; // the CTAs' mx of the sweep that ends
     __shared__ float absmin;
     __shared__ int scale;           // ||S||_F < 2^scale; A holds S 2^-scale
     const int tid = threadIdx.x, bs = blockDim.x;
@@ -1252,8 +1252,6 @@ __global__ void __launch_bounds__(256) k_oa_step(int m, const double *G, const d
     Ep[e] = v;
 }
 
-// Newton-Schulz orthonormalisation factor: Ep = (3 I - G) / 2
-
 // After the refinement T = Q^T S Q is diagonal up to rounding except inside
 // groups of (nearly) equal eigenvalues.  Indices joined by an off-diagonal
 // entry above tau = 4 m u ||S||_F (about ten times the rounding of the FP64
@@ -1454,13 +1452,12 @@ static cudaError_t coop_jacobi(Ctx &ctx, int m, double *A, double *V, double *la
     return cudaEventSynchronize(done);
 }
 
-// CTAs of the double-float Jacobi's cluster on the current device: 16 if the
-// device places clusters of that size (not a portable one), else 8.  The result
-// does not depend on it.
-static int jacobi_df_ctas() {
+// Whether the current device places the double-float Jacobi's cluster (its size is
+// not a portable one)
+static bool jacobi_df_fits() {
     constexpr int kMaxDevices = 64;
     static std::once_flag once[kMaxDevices];
-    static int ctas[kMaxDevices];
+    static bool fits[kMaxDevices];
     int dev = 0;
     cudaGetDevice(&dev);
     const int i = dev < 0 || dev >= kMaxDevices ? 0 : dev;
@@ -1468,21 +1465,21 @@ static int jacobi_df_ctas() {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = JDF_CTAS_WIDE;
+        attr.val.clusterDim.x = JDF_CTAS;
         attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-        cfg.gridDim = dim3(JDF_CTAS_WIDE);
+        cfg.gridDim = dim3(JDF_CTAS);
         cfg.blockDim = dim3(JDF_THREADS);
-        cfg.dynamicSmemBytes = JacobiShape(JDF_MAX, JDF_CTAS_WIDE).bytes();
+        cfg.dynamicSmemBytes = JacobiShape(JDF_MAX, JDF_CTAS).bytes();
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
         int n = 0;
-        const bool wide =
+        raise_smem_limits();
+        fits[i] =
             cudaFuncSetAttribute(k_jacobi_df, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
             cudaOccupancyMaxActiveClusters(&n, k_jacobi_df, &cfg) == cudaSuccess && n > 0;
-        if (!wide) cudaGetLastError();
-        ctas[i] = wide ? JDF_CTAS_WIDE : JDF_CTAS;
+        if (!fits[i]) cudaGetLastError();
     });
-    return ctas[i];
+    return fits[i];
 }
 
 cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q, double *work, int mode) {
@@ -1513,10 +1510,10 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
         launch_chained(ctx, k_identity, (unsigned)((m2 + 255) / 256), 256, 0, m, V);
         ctx.after();
     };
-    // The one-block FP32 stage takes m <= JMAX (A and V in its shared memory),
-    // the double-float cluster m <= JDF_MAX; beyond that, and without the
-    // refinement, the cooperative FP64 Jacobi.
-    if (mode == 0 || m > JDF_MAX || (mode == 1 && m > JMAX)) {
+    // The one-block FP32 stage takes m <= JMAX (A in its shared memory), the
+    // double-float cluster m <= JDF_MAX; beyond that, without the refinement, and
+    // on a device that does not place the cluster, the cooperative FP64 Jacobi.
+    if (mode == 0 || m > JDF_MAX || (m > JMAX && (mode == 1 || !jacobi_df_fits()))) {
         identity(Vm);
         cudaMemcpyAsync(Tm, S, m2 * sizeof(double), cudaMemcpyDeviceToDevice, ctx.stream);
         const cudaError_t e = coop_jacobi(ctx, m, Tm, Vm, lam0, 60, normA, 0.5 / m, cnt);
@@ -1540,12 +1537,11 @@ cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q,
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
-        const int ctas = jacobi_df_ctas();
-        attr.val.clusterDim.x = ctas;
+        attr.val.clusterDim.x = JDF_CTAS;
         attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-        cfg.gridDim = dim3(ctas);
+        cfg.gridDim = dim3(JDF_CTAS);
         cfg.blockDim = dim3(JDF_THREADS);
-        cfg.dynamicSmemBytes = JacobiShape(m, ctas).bytes();
+        cfg.dynamicSmemBytes = JacobiShape(m, JDF_CTAS).bytes();
         cfg.stream = ctx.stream;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
