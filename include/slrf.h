@@ -124,7 +124,9 @@ typedef struct {
                                or double-float, then three FP64 refinement steps
                                X <- X (I + E) built from the products X^T X and
                                X^T S X (Ogita-Aishima), and FP64 Jacobi inside
-                               groups of nearly equal eigenvalues; 1 (m <= 160;
+                               groups of nearly equal eigenvalues (m > 160: of
+                               every pair with |x_i^T S x_j| above eps ||S||_F / 2;
+                               up to 160: groups joined above 2 m eps ||S||_F); 1 (m <= 160;
                                larger m take 0) = FP32 Jacobi, FP64 re-orthonormal-
                                isation and an FP64 Jacobi polish of the whole
                                matrix; 0 = FP64 Jacobi                          (2) */
@@ -136,10 +138,12 @@ typedef struct {
                                where groups of two would be padded)                (0) */
     int32_t gram_ozaki;     /* Grams and tall products (Q1 = U T1, X = Q1 M) of the
                                projection step, FP64-accurate from exact integer
-                               digit products (Ozaki splitting): 2 = Grams on the
+                               digit products (Ozaki splitting): 2 = on the
                                tcgen05 tensor cores (bf16 digits, FP32 TMEM
-                               accumulators), tall products as with 1; 1 = int8
-                               mma.sync digits for both; 0 = FP64 CUDA cores    (2) */
+                               accumulators; tall products of up to 512 columns),
+                               as with 1 where mem_budget does not take that
+                               form's digits; 1 = int8 mma.sync digits; 0 = FP64
+                               CUDA cores                                       (2) */
     int32_t mg_nu;          /* MG: Jacobi sweeps per side on the levels below the
                                finest (the finest always takes one); 0 = one when
                                the FP32 cycle ends at the mg_exact level, else

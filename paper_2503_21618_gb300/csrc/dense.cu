@@ -185,7 +185,7 @@ __global__ void k_split_reduce(int M, int N, int split, const double *__restrict
 // Small products (the m x m x m GEMMs of the projection) on 8 x 8 output
 // tiles: 64 outputs times a four-way split of each K chunk per CTA, the next
 // chunk's loads in flight during the FMAs, the four sums added in a fixed
-// order.  Bound by the FP64 pipe (~1.6 FMAs per clock and SM), so the tiles
+// order.  Bound by the FP64 pipe (~1.7 FMAs per clock and SM), so the tiles
 // are small enough that the most loaded SM has little more than the average:
 // m = 150 on 100 CTAs of 16 x 16 took 17 us, on 361 of 8 x 8 about 10 us.
 // symmetric: the result is known to be symmetric (X^T X, X^T S X): only the

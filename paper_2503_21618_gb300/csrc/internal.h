@@ -421,8 +421,10 @@ void small_colscale(Ctx &ctx, int m, double *G, double *s);        // s = 1/sqrt
 void small_chol_inv(Ctx &ctx, int m, const double *G, double *R, double *Rinv, int32_t *status, int32_t *out_status,
                     double shift_on_fail);
 void small_scale_rows(Ctx &ctx, int m, const double *s, double *T);  // T = diag(s) T
-// Symmetric eigensolver: lam ascending, Q eigenvectors (columns).  mode 1:
-// FP32 Jacobi followed by FP64 refinement; 0: FP64 Jacobi.
+// Symmetric eigensolver: lam ascending, Q eigenvectors (columns).  mode 2 (m <=
+// 448): Jacobi in FP32 (m <= 160) or double-float, then refinement by FP64 products
+// and FP64 Jacobi on what that leaves; 1 (m <= 160): FP32 Jacobi, FP64
+// re-orthonormalisation and FP64 Jacobi; 0, and beyond those sizes: FP64 Jacobi.
 cudaError_t small_syev(Ctx &ctx, int m, const double *S, double *lam, double *Q, double *work, int mode);
 size_t small_syev_work_bytes(int m);
 

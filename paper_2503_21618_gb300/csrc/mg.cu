@@ -368,7 +368,7 @@ k_mg_scale(int n, int W, int Lp, int N, const cplx<T> *__restrict__ dinv, const 
 // Coarsest solve, one of its two products (n_c x n_c real V times the
 // complex block X, n_c x W):  Out = op(V) X, op(V) = V^T if trans, and if
 // cinv != nullptr each output row k of pole j is scaled by cinv[k*N + j].
-// Bound by the FP64 pipe (two FMAs per clock and SM), so what counts is that
+// Bound by the FP64 pipe (~1.7 FMAs per clock and SM), so what counts is that
 // every SM has the same share.  Two forms:
 //  * k_mg_coarse_gemm: 32-row x 16-column tiles per CTA (16 x 8 threads, four
 //    rows each) from shared memory, where such tiles give every SM two CTAs;
@@ -685,7 +685,7 @@ cplx<T> *cycle(Ctx &ctx, const KrylovDims &d, MgSolve<T> &mg, int l, int gy, con
     {
         const int W = d.W();
         const ColShape cs = col_shape(W / VC, sizeof(T) == 8);
-    dim3 grid(cs.gx, gyl), block(cs.bx, TY);
+        dim3 grid(cs.gx, gyl), block(cs.bx, TY);
         ctx.before(KC_MG_TRANSFER, 2 * vec_bytes<T>(d, L.n) + (double)L.n * d.N * sizeof(cplx<T>), 0);
         launch_chained(ctx, k_mg_jacobi0<T, VC>, grid, block, 0, L.n, W, d.Lp, d.N, L.dinv, L.r, z, flag);
         ctx.after();

@@ -352,7 +352,7 @@ __device__ __forceinline__ long long oz_biased(double x, int e) {
     return ((bits >> 63) ? -(long long)mag : (long long)mag) + BIAS;
 }
 
-// the eight digits' 16-byte groups of eight K-adjacent values
+// the seven digits' 16-byte groups of eight K-adjacent values
 __device__ __forceinline__ void oz_store_digits(const long long v[8], __nv_bfloat16 *__restrict__ out,
                                                 int64_t digit_stride) {
 #pragma unroll
@@ -402,10 +402,8 @@ __global__ void __launch_bounds__(256) k_oz_split_panel(int64_t n, int m, int64_
     oz_store_digits(v, out, nks * np * 2048);
 }
 
-// M = 128, N = 64, bf16 x bf16 -> FP32, both operands K-major
-
 // V 2^e for an int64 V, rounded to nearest even, in integer arithmetic: FP64
-// conversions and FMAs issue at ~1.6 per clock and SM, and four of them per
+// conversions and FMAs issue at ~1.7 per clock and SM, and four of them per
 // output were half of the tall product's time.
 __device__ __forceinline__ double oz_int_to_double(long long V, int e) {
     if (V == 0) return 0.0;
