@@ -1,6 +1,6 @@
 """CPU check of the rule that sets the CTAs per SM of the exact level's sweep
-update (csrc/sweep_rule.h): three where they fill more than three fifths of the
-last of several waves, a full last wave included, and up to two per SM."""
+update (csrc/sweep_rule.h): two in the first wave of three per SM beyond two CTAs per
+SM and in three fifths of the second, three otherwise."""
 import os
 import shutil
 import subprocess
@@ -26,10 +26,8 @@ def test_ctas_per_sm(tmp_path):
     got = subprocess.run([exe], capture_output=True, text=True, check=True).stdout
     wave = 3 * 152
     for t, g in enumerate(got):
-        full, rest = divmod(t, wave)
-        last = rest or wave
-        waves = full + (rest > 0)
-        assert g == ("3" if t <= 304 or (waves > 1 and last > 273) else "2"), t
-    measured = {112: "3", 264: "3", 420: "2", 480: "2", 684: "2", 840: "3", 1104: "2", 1224: "3", 1368: "3"}
+        assert g == ("2" if 2 * 152 < t <= 1.6 * wave else "3"), t
+    measured = {112: "3", 264: "3", 420: "2", 480: "2", 684: "2", 760: "3", 840: "3", 912: "3", 918: "3", 1104: "3",
+                1224: "3", 1368: "3"}
     for t, want in measured.items():
         assert got[t] == want
